@@ -46,6 +46,7 @@
 
 #include "common.cuh"
 #include "gram_tc.cuh"
+#include "tc.cuh"
 
 namespace ssm {
 
@@ -59,9 +60,6 @@ constexpr int kTcDigBits = 5;          // digit width
 constexpr int kTcDigBlock = 2;         // digits per A block and per B block
 constexpr unsigned kTcPlaneBytes = 128u * kTcChunk * 2u;              // 128 pivots x 64 nodes, FP16
 constexpr unsigned kTcBufBytes = 2u * kTcDigBlock * kTcPlaneBytes;    // A and B digit planes of one chunk
-constexpr unsigned long long kTcWaitNs = 200000000ull;                // 200 ms
-
-__device__ __forceinline__ uint32_t tc_smem(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // shared-memory matrix descriptor: K-major, 128-byte swizzle (8 rows x 128
 // bytes per atom, 1024 bytes between atoms along M), version 1
@@ -72,26 +70,6 @@ __device__ __forceinline__ uint64_t tc_desc(uint32_t addr) {
 
 // instruction descriptor: FP16 A and B (K-major), FP32 accumulator, M = N = 128
 constexpr uint32_t kTcIdesc = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-
-__device__ __forceinline__ bool tc_try(uint32_t mbar, unsigned phase) {
-  unsigned done = 0;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(done)
-      : "r"(mbar), "r"(phase)
-      : "memory");
-  return done != 0;
-}
-
-__device__ __forceinline__ bool tc_wait(uint32_t mbar, unsigned phase) {
-  if (tc_try(mbar, phase)) return true;
-  const unsigned long long t0 = globaltimer_ns();
-  for (;;) {
-    if (tc_try(mbar, phase)) return true;
-    if (globaltimer_ns() - t0 > kTcWaitNs) return false;
-  }
-}
 
 // FP16 pair of digit p (bits 5p .. 5p + 4) of two squared distances s0, s1
 // (exact: (1024 + v) - 1024).  L packs bits 0..15 of both, M bits 15..30.

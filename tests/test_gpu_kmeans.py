@@ -92,3 +92,22 @@ def test_kmeans_sp_rejects_sizes_beyond_exact_arithmetic():
     with pytest.raises(ssm.SSMError) as e:
         ssm.ssm_kmeans_pivots(dip, piv)
     assert e.value.code == -1
+
+
+@pytest.mark.parametrize("k,n,dmax,passes", [
+    (1, 5, 3, 3), (16, 127, 1, 6), (17, 128, 9, 6), (33, 129, 40, 6),  # one 16-cluster group, ragged halves, tile edges
+    (96, 20000, 2, 4),                                               # more tiles than SMs, ties in every node
+    (208, 1500, 700, 4), (209, 1500, 700, 4),                        # the largest k of the filter, and one more
+    (200, 1500, 2621, 3), (200, 1500, 2623, 3),                      # the largest distances of the filter, and above
+    (4, 1500, 4096, 5), (4, 1500, 4098, 5),                          # distances that FP16 still holds, and above
+    (64, 900, 20000, 3)])
+def test_kmeans_sp_filter_edges(k, n, dmax, passes):
+    """The tensor-core filter at the edges of its tiles and of its range, and
+    the general kernel just outside: random tables, bit-exact."""
+    dip = I.distance_table(k, n, dmax, 5 + k)
+    piv = np.random.default_rng(k).permutation(n)[:k].astype(np.int32)
+    want_p, want_a, want_it = O.kmeans_sp(dip, piv, passes)
+    got_p, got_a, got_it = ssm.ssm_kmeans_pivots(torch.from_numpy(dip).to(DEV), torch.from_numpy(piv).to(DEV), passes)
+    assert int(got_it.item()) == want_it
+    assert np.array_equal(got_a.cpu().numpy(), want_a)
+    assert np.array_equal(got_p.cpu().numpy(), want_p)
