@@ -270,21 +270,56 @@ __device__ void sssp_block(int32_t n, const int32_t *__restrict__ rowptr, const 
 // band width of the near-far search: kDeltaScale times the mean edge length
 constexpr float kDeltaScale = 8.0f;
 
-__global__ void k_mean_length(int32_t n, const int32_t *__restrict__ rowptr, const float *__restrict__ elen,
-                              float *__restrict__ delta) {
+// delta from the mean edge length: per-block sums, added in block order by the
+// last block (one block over all edges took 1.16 ms on 2.1 M of them)
+constexpr int kMeanBlocks = 28;
+struct MeanWs {
+  float delta;
+  unsigned done;  // zero before the launch
+  double part[kMeanBlocks];
+};
+static_assert(sizeof(MeanWs) <= 256, "the mean's workspace is 256 bytes");
+
+__global__ void __launch_bounds__(1024) k_mean_length(int32_t n, const int32_t *__restrict__ rowptr,
+                                                      const float *__restrict__ elen, MeanWs *__restrict__ ws) {
   __shared__ double red[32];
+  __shared__ unsigned s_ticket;
   const int64_t m2 = rowptr[n];
   double acc = 0.0;
-  for (int64_t t = threadIdx.x; t < m2; t += blockDim.x) acc += (double)elen[t];
+  float sum = 0.0f;
+  int run = 0;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < m2; t += (int64_t)gridDim.x * blockDim.x) {
+    sum += __ldg(elen + t);
+    if (++run == 16) {  // short runs in FP32: the band width needs no more
+      acc += (double)sum;
+      sum = 0.0f;
+      run = 0;
+    }
+  }
+  acc += (double)sum;
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    const float mean = m2 > 0 ? (float)(t / (double)m2) : 1.0f;
-    *delta = mean > 0.0f ? kDeltaScale * mean : 1.0f;
+    ws->part[blockIdx.x] = t;
+    __threadfence();
+    s_ticket = atomicAdd(&ws->done, 1u);
   }
+  __syncthreads();
+  if (s_ticket != gridDim.x - 1 || threadIdx.x != 0) return;
+  __threadfence();
+  double t = 0.0;
+  for (unsigned q = 0; q < gridDim.x; ++q) t += __ldcg(ws->part + q);
+  const float mean = m2 > 0 ? (float)(t / (double)m2) : 1.0f;
+  ws->delta = mean > 0.0f ? kDeltaScale * mean : 1.0f;
+}
+
+static int launch_mean_length(int32_t n, const int32_t *rowptr, const float *elen, MeanWs *ws, cudaStream_t s) {
+  SSM_TRY_CUDA(cudaMemsetAsync(&ws->done, 0, sizeof(unsigned), s));
+  note_launch(), k_mean_length<<<kMeanBlocks, 1024, 0, s>>>(n, rowptr, elen, ws);
+  return SSM_OK;
 }
 
 // d_ip mode: block b takes sources b, b + grid, ...; dist rows [k][n]
@@ -364,10 +399,11 @@ int launch_sssp(int32_t n, const int32_t *rowptr, const int32_t *colidx, const f
   const size_t sb = sssp_slot_bytes(n);
   if (ws_bytes < sssp_ws_bytes(n, k))
     return fail(SSM_E_NOMEM, "sssp: workspace %zu bytes, need %zu", ws_bytes, sssp_ws_bytes(n, k));
-  float *delta = (float *)ws;
+  MeanWs *mean = (MeanWs *)ws;
+  float *delta = &mean->delta;
   char *slots = (char *)ws + 256;
   SSM_TRY_CUDA(cudaMemsetAsync(slots, 0, sb * (size_t)blocks, s));
-  note_launch(), k_mean_length<<<1, 1024, 0, s>>>(n, rowptr, elen, delta);
+  if (int rc = launch_mean_length(n, rowptr, elen, mean, s)) return rc;
   note_launch(), k_sssp_multi<<<blocks, kSsspMultiThreads, 0, s>>>(n, rowptr, colidx, (const unsigned *)elen, k, sources,
                                                             (unsigned *)dist, delta, slots, sb, status);
   const int64_t cnt = (int64_t)k * n;
@@ -800,14 +836,14 @@ namespace ssm {
 struct WmmWs {
   unsigned *mind;
   unsigned long long *keys;
-  float *delta;
-  char *slot;
+  MeanWs *mean;
+  char *slot;  // the single-block search's queues, or the cluster's spill area
 };
 static size_t carve_wmm(Carver &c, WmmWs &w, int32_t n, int32_t k) {
   w.mind = c.take<unsigned>((size_t)n);
   w.keys = c.take<unsigned long long>((size_t)k);
-  w.delta = c.take<float>(1);
-  w.slot = c.take<char>(sssp_slot_bytes(n));
+  w.mean = c.take<MeanWs>(1);
+  w.slot = c.take<char>(std::max(sssp_slot_bytes(n), wmaxmin_spill_entries(n) * sizeof(int32_t)));
   return c.size();
 }
 }  // namespace ssm
@@ -832,17 +868,24 @@ SSM_API int ssm_select_pivots_weighted(int32_t n, int64_t m, const int32_t *rowp
   WmmWs w;
   carve_wmm(c, w, n, k);
   if (!c.ok) return fail(SSM_E_NOMEM, "ssm_select_pivots_weighted: workspace %zu bytes, need %zu", ws_bytes, c.size());
+  if (int rc = launch_mean_length(n, rowptr, elen, w.mean, s)) return rc;
+  float *const delta = &w.mean->delta;
+  // in one cluster when the labels fit its shared memory; larger graphs search
+  // pivot by pivot in one block over global memory
+  bool ran = false;
+  if (int rc = launch_wmaxmin_cluster(n, rowptr, colidx, elen, k, start, pivots, delta, (int32_t *)w.slot, status, s, &ran))
+    return rc;
+  if (ran) return SSM_OK;
   SSM_TRY_CUDA(cudaMemsetAsync(w.keys, 0, (size_t)k * sizeof(unsigned long long), s));
   SSM_TRY_CUDA(cudaMemsetAsync(w.slot, 0, sssp_slot_bytes(n), s));
   const size_t sb = sssp_slot_bytes(n);
-  note_launch(), k_mean_length<<<1, 1024, 0, s>>>(n, rowptr, elen, w.delta);
   note_launch(), k_sssp_maxmin<<<1, kSsspThreads, 0, s>>>(n, rowptr, colidx, (const unsigned *)elen, start, nullptr,
-                                                        pivots, w.mind, w.delta, w.slot, sb, true, status);
+                                                        pivots, w.mind, delta, w.slot, sb, true, status);
   const unsigned ab = (unsigned)std::max(1, std::min((n + 255) / 256, num_sms() * 4));
   for (int a = 1; a < k; ++a) {
     note_launch(), k_wmm_argmax<<<ab, 256, 0, s>>>(n, w.mind, w.keys + a, status);
     note_launch(), k_sssp_maxmin<<<1, kSsspThreads, 0, s>>>(n, rowptr, colidx, (const unsigned *)elen, 0, w.keys + a,
-                                                          pivots + a, w.mind, w.delta, w.slot, sb, false, status);
+                                                          pivots + a, w.mind, delta, w.slot, sb, false, status);
   }
   if (k == 1) note_launch(), k_wmm_argmax<<<ab, 256, 0, s>>>(n, w.mind, w.keys, status);  // reachability check
   SSM_TRY_CUDA(cudaGetLastError());

@@ -16,4 +16,12 @@ size_t sssp_ws_bytes(int32_t n, int32_t k);  // launch_sssp's workspace
 int launch_sssp(int32_t n, const int32_t *rowptr, const int32_t *colidx, const float *elen, int32_t k,
                 const int32_t *sources, float *dist, int32_t *status, void *ws, size_t ws_bytes, cudaStream_t s);
 
+// Weighted max/min pivots in one thread-block cluster (wmaxmin_cluster.cu): *ran
+// is false, and nothing was enqueued, when the graph is too large for one.
+// spill holds wmaxmin_spill_entries(n) words.
+size_t wmaxmin_spill_entries(int32_t n);
+int launch_wmaxmin_cluster(int32_t n, const int32_t *rowptr, const int32_t *colidx, const float *elen, int32_t k,
+                           int32_t start, int32_t *pivots, const float *delta, int32_t *spill, int32_t *status,
+                           cudaStream_t s, bool *ran);
+
 }  // namespace ssm

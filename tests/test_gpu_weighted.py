@@ -212,3 +212,39 @@ def test_layout_weighted_end_to_end_lowers_stress():
     after, _ = ssm.ssm_stress_weighted(g, pos, 256, 256, 3)
     assert torch.isfinite(pos).all()
     assert after[3].item() < before[3].item()
+
+
+def _star(leaves, lengths):
+    s = np.zeros(leaves, np.int32)
+    d = np.arange(1, leaves + 1, dtype=np.int32)
+    return leaves + 1, s, d, np.asarray(lengths, np.float32)
+
+
+MAXMIN = {
+    "one_node_left": lambda: (2, np.array([0], np.int32), np.array([1], np.int32), np.array([0.5], np.float32), 2),
+    "fewer_nodes_than_ctas": lambda: (*(lambda n, s, d: (n, s, d, _mixed_lengths(len(s), 3)))(*I.path(11)), 11),
+    # 60,000 leaves reached in one round: more than the shared-memory part of the near queues
+    "near_queue_spills": lambda: (*_star(60000, I.random_lengths(60000, 9, "uniform", 0.5, 2.0)), 5),
+    # an eighth of 400,000 leaves beyond the first band: the far piles spill
+    "far_pile_spills": lambda: (*_star(400000, np.where(np.arange(400000) % 8 == 0, 90.0 + np.arange(400000) * 1e-4, 0.01)), 4),
+    "equal_path_sums": lambda: (*(lambda n, s, d: (n, s, d, np.ones(len(s), np.float32)))(*I.grid(90, 70)), 60),
+    # labels that do not fit one cluster's shared memory: the single-block search
+    "beyond_one_cluster": lambda: (*I.rgg_lengths(960000, 9.0, 3), 3),
+}
+
+
+@pytest.mark.parametrize("name", list(MAXMIN))
+def test_weighted_maxmin_edges(name):
+    n, s, d, l, k = MAXMIN[name]()
+    g = _gpu_wgraph(n, s, d, l)
+    got = ssm.ssm_select_pivots_weighted(g, k, start=n // 3)
+    want = O.wmaxmin(O.build_wcsr(n, s, d, l), k, n // 3)
+    assert np.array_equal(got.cpu().numpy(), want)
+
+
+def test_weighted_maxmin_disconnected():
+    n, s, d = 40, np.arange(0, 38, dtype=np.int32), np.arange(1, 39, dtype=np.int32)
+    with pytest.raises(ssm.SSMError) as e:
+        g = _gpu_wgraph(n, s, d, np.ones(len(s), np.float32))
+        ssm.ssm_select_pivots_weighted(g, 4)
+    assert e.value.code == -3
