@@ -10,12 +10,13 @@
 //
 //   ssm_edge_lengths        lengths of the CSR edges from the input list
 //                           (a repeated edge keeps its shortest length)
-//   k_sssp                  one block per source: rounds of relaxations of
+//   k_sssp_multi            one block per source: rounds of relaxations of
 //                           a frontier queue, labels lowered by atomicMin
 //                           on their bit patterns (non-negative floats order
 //                           like their bits); with the label row holding
 //                           min over the earlier pivots it is max/min's
-//                           pruned search
+//                           pruned search (k_sssp_maxmin, for graphs whose
+//                           labels do not fit one cluster's shared memory)
 //   k_wmm_argmax            the next max/min pivot: max over v of
 //                           (mind_v, -v) as one 64-bit key
 //   k_wregion_keys, bitonic sort, k_wcounts
@@ -34,8 +35,7 @@
 namespace ssm {
 
 constexpr unsigned kInfBits = 0x7f800000u;
-constexpr int kSsspThreads = 512;       // the max/min search: one block, the whole graph
-constexpr int kSsspMultiThreads = 512;  // one source per block, up to three blocks per SM
+constexpr int kSsspThreads = 512;  // of a search's block (half as many when there are many sources)
 
 // ------------------------------------------------------------ edge lengths
 __global__ void k_fill_u32(int64_t count, unsigned *__restrict__ p, unsigned v) {
@@ -92,178 +92,243 @@ __global__ void k_elen_check(int32_t n, int64_t m2, const unsigned *__restrict__
 }
 
 // ------------------------------------------------------------ SSSP
-// Near-far label-correcting search (two-bucket Delta-stepping): only labels
-// below a threshold T are relaxed in a round ("near"); a node lowered to a
-// label at or above T waits in the far pile; when the near queue is empty
-// T grows by Delta (at least to the smallest far label plus Delta) and the
-// far pile is split again.  Plain rounds over every improved node (the
-// first form) re-relaxed each node about 20 times on a 262K-node geometric
-// graph; the threshold keeps the search close to label-setting order while
-// each round still relaxes a whole band of nodes.  Any order that relaxes
-// until nothing improves reaches the same least path sums.
+// Near-far label-correcting search (two-bucket Delta-stepping), one block per
+// source: only labels below a threshold T are relaxed in a round ("near"); a
+// node lowered to a label at or above T waits in the far pile; when the near
+// queue is empty T grows by Delta (at least to the smallest far label plus
+// Delta) and the far pile is split again.  Plain rounds over every improved
+// node re-relaxed each node about 20 times on a 262K-node geometric graph;
+// the threshold keeps the search close to label-setting order while each round
+// still relaxes a whole band of nodes.  Any order that relaxes until nothing
+// improves reaches the same least path sums.
 //
-// Per block: near queues (current, next), two far piles (ping-pong), and
-// membership bitmaps: one per near queue (the next queue's bits are set by
-// the relaxations of a round, the current queue's bits cleared as its nodes
-// are taken) and one for the far pile.
-struct SsspSlot {
-  int32_t *nq[2];
-  int32_t *fq[2];
-  unsigned *in_near[2], *in_far;
-};
+// While a search runs a node's word holds its label's bits << 1 | queued, so
+// lowering a label and marking the node is one atomicMin with bits << 1 | 1
+// (labels are non-negative floats; an equal label leaves the mark alone), and
+// the value it returns says whether the node has to be queued.  A marked node
+// whose label is below T is in the near queue, one at or above T in the far
+// pile; a far node lowered below T is queued near as well, and its far entry is
+// dropped at the split (the mark is gone by then).  So a node is in each queue
+// at most once.
+//
+// A round is bound by its chain of dependent accesses (a block's search has
+// some 860 rounds of a few hundred nodes on that graph): queue entry, row range
+// and mark, edges, heads' words, atomicMin.  The queues sit in shared memory (a
+// long one goes on in the block's global slot), the rows of a warp's entries
+// are spread over its lanes, and kSsspU edges per lane are in flight at once;
+// heads are read first, and only those that would be lowered see an atomicMin
+// (one in five).  With one edge per lane at a time, queues and membership bits
+// in global memory 200 sources on the 262K-node graph took 18.4 ms, now 8.0 (a
+// round 20,000 cycles, three steps of some 5,500 per warp: the words of 200
+// sources do not fit L2), and 1024 sources 66.9, now 31.
+constexpr int kSsspQ = 1024;  // entries of a queue kept in shared memory
+constexpr int kSsspU = 4;     // edges per lane in flight
 
 __host__ __device__ inline size_t sssp_qbytes(int32_t n) { return (((size_t)n * 4) + 255) & ~size_t(255); }
-__host__ __device__ inline size_t sssp_bbytes(int32_t n) { return ((((size_t)n + 31) / 32) * 4 + 255) & ~size_t(255); }
+size_t sssp_slot_bytes(int32_t n) { return 4 * sssp_qbytes(n); }
 
-__device__ __forceinline__ SsspSlot sssp_slot(char *base, size_t slot_bytes, int b, int32_t n) {
-  char *p = base + (size_t)b * slot_bytes;
-  const size_t qb = sssp_qbytes(n), bb = sssp_bbytes(n);
-  SsspSlot s;
-  s.nq[0] = (int32_t *)p;
-  s.nq[1] = (int32_t *)(p + qb);
-  s.fq[0] = (int32_t *)(p + 2 * qb);
-  s.fq[1] = (int32_t *)(p + 3 * qb);
-  s.in_near[0] = (unsigned *)(p + 4 * qb);
-  s.in_near[1] = (unsigned *)(p + 4 * qb + bb);
-  s.in_far = (unsigned *)(p + 4 * qb + 2 * bb);
-  return s;
+// A block's queues: near by parity, far by parity.  An entry is a node, a near
+// entry in shared memory its row range as well.
+struct SsspQueues {
+  int4 (*near_sm)[kSsspQ];
+  int32_t (*far_sm)[kSsspQ];
+  int32_t *gl;
+  size_t stride;  // of the global parts
+  const int32_t *rowptr;
+  __device__ __forceinline__ int4 get_near(int q, unsigned t) const {
+    if (t < kSsspQ) return near_sm[q][t];
+    const int v = __ldcg(gl + q * stride + t);
+    return make_int4(v, __ldg(rowptr + v), __ldg(rowptr + v + 1), 0);
+  }
+  __device__ __forceinline__ void put_near(int q, unsigned t, int4 e) const {
+    if (t < kSsspQ) near_sm[q][t] = e;
+    else __stcg(gl + q * stride + t, e.x);
+  }
+  __device__ __forceinline__ int32_t get_far(int q, unsigned t) const {
+    return t < kSsspQ ? far_sm[q][t] : __ldcg(gl + (2 + q) * stride + t);
+  }
+  __device__ __forceinline__ void put_far(int q, unsigned t, int32_t v) const {
+    if (t < kSsspQ) far_sm[q][t] = v;
+    else __stcg(gl + (2 + q) * stride + t, v);
+  }
+};
+
+// The whole warp: places in a queue (counter in shared memory) for the flagged
+// (lane, slot) pairs, one atomic for all of them; places[q] is set where flag[q]
+__device__ __forceinline__ void sssp_places(const bool (&flag)[kSsspU], unsigned *counter, unsigned (&place)[kSsspU]) {
+  const unsigned lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
+  unsigned mask[kSsspU], total = 0;
+#pragma unroll
+  for (int q = 0; q < kSsspU; ++q) {
+    mask[q] = __ballot_sync(0xffffffffu, flag[q]);
+    total += __popc(mask[q]);
+  }
+  if (!total) return;
+  unsigned at = 0;
+  if (lane == 0) at = atomicAdd(counter, total);
+  at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+  for (int q = 0; q < kSsspU; ++q) {
+    place[q] = at + __popc(mask[q] & below);
+    at += __popc(mask[q]);
+  }
 }
 
-size_t sssp_slot_bytes(int32_t n) { return 4 * sssp_qbytes(n) + 3 * sssp_bbytes(n); }
-
-__device__ __forceinline__ bool set_bit(unsigned *bm, int v) {
-  const unsigned bit = 1u << (v & 31);
-  return !(atomicOr(bm + (v >> 5), bit) & bit);
-}
-
-// One search from `source` into row (labels as float bits).  init: set every
-// label to +inf first; otherwise the row's labels stay (max/min's pruned
-// search: only nodes the new pivot is strictly closer to change).  delta is
-// the band width.  The bitmaps are clear on entry and on return.
+// One search from `source` into row (words as above).  init: every label is
+// +inf first; otherwise the row's labels stay (max/min's pruned search: only
+// nodes the new pivot is strictly closer to change).  delta is the band width.
+// No word is marked on entry and on return.
 __device__ void sssp_block(int32_t n, const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
                            const unsigned *__restrict__ elen, int32_t source, unsigned *__restrict__ row, bool init,
-                           float delta, SsspSlot sl, int32_t *__restrict__ status) {
-  __shared__ unsigned s_nnext, s_nfar, s_nfar2, s_minfar;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+                           float delta, char *slot, int32_t *__restrict__ status) {
+  __shared__ int4 s_near_q[2][kSsspQ];
+  __shared__ int32_t s_far_q[2][kSsspQ];
+  __shared__ unsigned s_near[2], s_far, s_keep, s_least;
+  const SsspQueues Q{s_near_q, s_far_q, (int32_t *)slot, sssp_qbytes(n) / 4, rowptr};
+  const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  __syncthreads();  // the previous search of this block is over
   if (init)
-    for (int v = threadIdx.x; v < n; v += blockDim.x) row[v] = kInfBits;
+    for (int v = threadIdx.x; v < n; v += blockDim.x) __stcg(row + v, kInfBits << 1);
   __syncthreads();
   if (threadIdx.x == 0) {
-    row[source] = 0u;
-    sl.nq[0][0] = source;
-    s_nfar = 0;
+    __stcg(row + source, 1u);
+    s_near_q[0][0] = make_int4(source, __ldg(rowptr + source), __ldg(rowptr + source + 1), 0);
+    s_near[0] = 1u;
+    s_near[1] = 0u;
+    s_far = 0u;
+    s_least = 0xFFFFFFFFu;
   }
-  __syncthreads();
-  unsigned nnear = 1, nfar = 0;
-  int cur = 0, fcur = 0;
   float T = delta;
-  // every pass relaxes at least one node whose label is then final for the
-  // band, so the passes are bounded; the cap only guards against a fault
+  int cur = 0, fcur = 0;
+  // every round relaxes at least one node whose label is then final for the
+  // band, so the rounds are bounded; the cap only guards against a fault
   const int64_t cap = 64ll * ((int64_t)n + 16);
-  for (int64_t pass = 0;; ++pass) {
-    if (pass > cap) {
+  for (int64_t round = 0;; ++round) {
+    __syncthreads();  // the queue of this round is complete
+    unsigned count = s_near[cur];
+    if (count == 0) {
+      const unsigned nfar = s_far, least = s_least;
+      if (nfar == 0) break;
+      // next band: T >= smallest far label + delta (least is at or below it);
+      // the marked entries of the far pile go to the near queue or the other pile
+      T = fmaxf(T + delta, least == 0xFFFFFFFFu ? 0.0f : __uint_as_float(least) + delta);
+      // where delta vanishes against the labels, take the next float above
+      // the smallest far label so that at least that node moves on
+      if (least != 0xFFFFFFFFu && !(T > __uint_as_float(least))) T = __uint_as_float(least + 1u);
+      const unsigned tbits = __float_as_uint(T);
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        s_keep = 0u;
+        s_least = 0xFFFFFFFFu;
+      }
+      __syncthreads();
+      for (unsigned t = threadIdx.x; t < nfar; t += blockDim.x) {
+        const int v = Q.get_far(fcur, t);
+        const unsigned w = __ldcg(row + v);
+        if (!(w & 1u)) continue;
+        if ((w >> 1) < tbits) {
+          Q.put_near(cur, atomicAdd(&s_near[cur], 1u), make_int4(v, __ldg(rowptr + v), __ldg(rowptr + v + 1), 0));
+        } else {
+          Q.put_far(fcur ^ 1, atomicAdd(&s_keep, 1u), v);
+          atomicMin(&s_least, w >> 1);
+        }
+      }
+      __syncthreads();
+      if (threadIdx.x == 0) s_far = s_keep;
+      fcur ^= 1;
+      count = s_near[cur];
+      if (count == 0) continue;
+      __syncthreads();
+    }
+    if (round > cap) {
       if (threadIdx.x == 0) dev_fail(status, SSM_E_NUMERIC);
       break;
     }
-    if (nnear == 0) {
-      if (nfar == 0) break;
-      // next band: T >= smallest far label + delta; split the far pile
-      const int32_t *fq = fcur ? sl.fq[1] : sl.fq[0];
-      int32_t *fq2 = fcur ? sl.fq[0] : sl.fq[1];
-      int32_t *nq = cur ? sl.nq[1] : sl.nq[0];
-      if (threadIdx.x == 0) {
-        s_minfar = kInfBits;
-        s_nnext = 0;
-        s_nfar2 = 0;
-      }
-      __syncthreads();
-      for (unsigned t = threadIdx.x; t < nfar; t += blockDim.x) atomicMin(&s_minfar, __ldcg(row + fq[t]));
-      __syncthreads();
-      T = fmaxf(T + delta, __uint_as_float(s_minfar) + delta);
-      // where delta vanishes against the labels, take the next float above
-      // the smallest far label so that at least that node moves on
-      if (!(T > __uint_as_float(s_minfar))) T = __uint_as_float(s_minfar + 1u);
-      for (unsigned t = threadIdx.x; t < nfar; t += blockDim.x) {
-        const int v = fq[t];
-        atomicAnd(sl.in_far + (v >> 5), ~(1u << (v & 31)));
-        if (__uint_as_float(__ldcg(row + v)) < T) nq[atomicAdd(&s_nnext, 1u)] = v;
-        else {
-          set_bit(sl.in_far, v);
-          fq2[atomicAdd(&s_nfar2, 1u)] = v;
-        }
-      }
-      __syncthreads();
-      nnear = s_nnext;
-      nfar = s_nfar2;
-      fcur ^= 1;
-      __syncthreads();
-      continue;
-    }
-    if (threadIdx.x == 0) {
-      s_nnext = 0;
-      s_nfar = nfar;
-    }
-    __syncthreads();
-    const int32_t *qc = cur ? sl.nq[1] : sl.nq[0];
-    int32_t *qn = cur ? sl.nq[0] : sl.nq[1];
-    unsigned *inc = cur ? sl.in_near[1] : sl.in_near[0];
-    unsigned *inn = cur ? sl.in_near[0] : sl.in_near[1];
-    int32_t *fq = fcur ? sl.fq[1] : sl.fq[0];
-    // a warp takes 32 near entries at a time and walks their rows together,
-    // 32 edge slots per step (hubs spread over the lanes)
-    for (unsigned base = (unsigned)warp * 32u; base < nnear; base += blockDim.x) {
-      const unsigned idx = base + (unsigned)lane;
+    const unsigned tbits = __float_as_uint(T);
+    unsigned *const next = &s_near[cur ^ 1];
+    // entries per warp and step: a small round is spread over all warps
+    const unsigned ipw = min(32u, (count + nwarps - 1u) / nwarps);
+    for (unsigned base = warp * ipw; base < count; base += nwarps * ipw) {
       int b = 0, e = 0;
-      unsigned dvb = kInfBits;
-      if (idx < nnear) {
-        const int v = qc[idx];
-        atomicAnd(inc + (v >> 5), ~(1u << (v & 31)));
-        b = __ldg(rowptr + v);
-        e = __ldg(rowptr + v + 1);
-        dvb = __ldcg(row + v);
+      unsigned dv = 0;
+      if (lane < ipw && base + lane < count) {
+        // the edges need the row range only: they are on their way together
+        // with the label (a near entry's node is always marked)
+        const int4 en = Q.get_near(cur, base + lane);
+        b = en.y;
+        e = en.z;
+        dv = atomicAnd(row + en.x, ~1u) >> 1;
       }
-      const int deg = e - b;
-      int incl = deg;
+      int incl = e - b;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
+        if ((int)lane >= o) incl += t;
       }
       const int total = __shfl_sync(0xffffffffu, incl, 31);
-      for (int s0 = 0; s0 < total; s0 += 32) {
-        const int slot = s0 + lane;
-        int lo = 0;
+      for (int s0 = 0; s0 < total; s0 += 32 * kSsspU) {
+        int u[kSsspU], at[kSsspU];
+        unsigned nb[kSsspU], len[kSsspU];
+        bool act[kSsspU];
 #pragma unroll
-        for (int step = 16; step >= 1; step >>= 1) {
-          const int pv = __shfl_sync(0xffffffffu, incl, lo + step - 1);
-          if (pv <= slot) lo += step;
-        }
-        const int owner = lo > 31 ? 31 : lo;
-        const int o_incl = __shfl_sync(0xffffffffu, incl, owner);
-        const int o_deg = __shfl_sync(0xffffffffu, deg, owner);
-        const int o_beg = __shfl_sync(0xffffffffu, b, owner);
-        const unsigned o_d = __shfl_sync(0xffffffffu, dvb, owner);
-        if (slot < total) {
-          const int t = o_beg + (slot - (o_incl - o_deg));
-          const int u = __ldg(colidx + t);
-          const float nd = __fadd_rn(__uint_as_float(o_d), __uint_as_float(__ldg(elen + t)));
-          const unsigned ndb = __float_as_uint(nd);
-          const unsigned old = atomicMin(row + u, ndb);
-          if (ndb < old) {
-            if (nd < T) {
-              if (set_bit(inn, u)) qn[atomicAdd(&s_nnext, 1u)] = u;
-            } else if (set_bit(sl.in_far, u)) {
-              fq[atomicAdd(&s_nfar, 1u)] = u;
-            }
+        for (int q = 0; q < kSsspU; ++q) {
+          const int t = s0 + 32 * q + (int)lane;
+          act[q] = t < total;
+          int lo = 0;  // row = first lane whose inclusive prefix exceeds t
+#pragma unroll
+          for (int step = 16; step >= 1; step >>= 1) {
+            const int pv = __shfl_sync(0xffffffffu, incl, lo + step - 1);
+            if (pv <= t) lo += step;
           }
+          at[q] = lo > 31 ? 31 : lo;
+          const int o_end = __shfl_sync(0xffffffffu, e, at[q]), o_incl = __shfl_sync(0xffffffffu, incl, at[q]);
+          const int pos = o_end - (o_incl - t);
+          u[q] = act[q] ? __ldg(colidx + pos) : 0;
+          len[q] = act[q] ? __ldg(elen + pos) : 0u;
         }
+        unsigned old[kSsspU];
+#pragma unroll
+        for (int q = 0; q < kSsspU; ++q) old[q] = act[q] ? __ldcg(row + u[q]) : 0u;
+#pragma unroll
+        for (int q = 0; q < kSsspU; ++q) {
+          nb[q] = __float_as_uint(__fadd_rn(__uint_as_float(__shfl_sync(0xffffffffu, dv, at[q])), __uint_as_float(len[q])));
+          act[q] = act[q] && (old[q] >> 1) > nb[q];
+        }
+#pragma unroll
+        for (int q = 0; q < kSsspU; ++q)
+          if (act[q]) old[q] = atomicMin(row + u[q], 2u * nb[q] + 1u);
+        // the lowered heads' row ranges, should they be queued (asked for with the
+        // words, for every head, they cost 10 % more than their latency hid)
+        int rb[kSsspU], re[kSsspU];
+#pragma unroll
+        for (int q = 0; q < kSsspU; ++q) {
+          rb[q] = act[q] ? __ldg(rowptr + u[q]) : 0;
+          re[q] = act[q] ? __ldg(rowptr + u[q] + 1) : 0;
+        }
+        unsigned least = 0xFFFFFFFFu, place[kSsspU] = {};
+        bool near[kSsspU], far[kSsspU];
+#pragma unroll
+        for (int q = 0; q < kSsspU; ++q) {
+          const bool lower = act[q] && (old[q] >> 1) > nb[q], was = (old[q] & 1u) != 0u, below = nb[q] < tbits;
+          near[q] = lower && below && (!was || (old[q] >> 1) >= tbits);
+          far[q] = lower && !below && !was;
+          if (lower && !below) least = min(least, nb[q]);
+        }
+        sssp_places(near, next, place);
+#pragma unroll
+        for (int q = 0; q < kSsspU; ++q)
+          if (near[q]) Q.put_near(cur ^ 1, place[q], make_int4(u[q], rb[q], re[q], 0));
+        sssp_places(far, &s_far, place);
+#pragma unroll
+        for (int q = 0; q < kSsspU; ++q)
+          if (far[q]) Q.put_far(fcur, place[q], u[q]);
+        least = __reduce_min_sync(0xffffffffu, least);
+        if (lane == 0 && least != 0xFFFFFFFFu) atomicMin(&s_least, least);
       }
     }
     __syncthreads();
-    nnear = s_nnext;
-    nfar = s_nfar;
+    if (threadIdx.x == 0) s_near[cur] = 0u;
     cur ^= 1;
-    __syncthreads();
   }
 }
 
@@ -275,7 +340,7 @@ constexpr float kDeltaScale = 8.0f;
 constexpr int kMeanBlocks = 28;
 struct MeanWs {
   float delta;
-  unsigned done;  // zero before the launch
+  unsigned done, next;  // zero before the launch; blocks finished, sources handed out
   double part[kMeanBlocks];
 };
 static_assert(sizeof(MeanWs) <= 256, "the mean's workspace is 256 bytes");
@@ -317,28 +382,34 @@ __global__ void __launch_bounds__(1024) k_mean_length(int32_t n, const int32_t *
 }
 
 static int launch_mean_length(int32_t n, const int32_t *rowptr, const float *elen, MeanWs *ws, cudaStream_t s) {
-  SSM_TRY_CUDA(cudaMemsetAsync(&ws->done, 0, sizeof(unsigned), s));
+  SSM_TRY_CUDA(cudaMemsetAsync(&ws->done, 0, 2 * sizeof(unsigned), s));
   note_launch(), k_mean_length<<<kMeanBlocks, 1024, 0, s>>>(n, rowptr, elen, ws);
   return SSM_OK;
 }
 
-// d_ip mode: block b takes sources b, b + grid, ...; dist rows [k][n]
-__global__ void __launch_bounds__(kSsspMultiThreads, 3) k_sssp_multi(int32_t n, const int32_t *__restrict__ rowptr,
+// d_ip mode: a block takes one source after another; dist rows [k][n] hold words
+// (k_sssp_labels turns them into labels)
+__global__ void __launch_bounds__(kSsspThreads, 2) k_sssp_multi(int32_t n, const int32_t *__restrict__ rowptr,
                                                              const int32_t *__restrict__ colidx,
                                                              const unsigned *__restrict__ elen, int32_t k,
                                                              const int32_t *__restrict__ sources,
-                                                             unsigned *__restrict__ dist, const float *__restrict__ delta,
+                                                             unsigned *__restrict__ dist, MeanWs *__restrict__ ws,
                                                              char *slots, size_t slot_bytes,
                                                              int32_t *__restrict__ status) {
-  const SsspSlot sl = sssp_slot(slots, slot_bytes, blockIdx.x, n);
-  const float dl = *delta;
-  for (int a = blockIdx.x; a < k; a += gridDim.x) {
+  __shared__ int s_a;
+  const float dl = ws->delta;
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_a = (int)atomicAdd(&ws->next, 1u);
+    __syncthreads();
+    const int a = s_a;
+    if (a >= k) break;
     const int s = sources[a];
     if (s < 0 || s >= n) {
       if (threadIdx.x == 0) dev_fail(status, SSM_E_ARG);
       continue;
     }
-    sssp_block(n, rowptr, colidx, elen, s, dist + (size_t)a * n, true, dl, sl, status);
+    sssp_block(n, rowptr, colidx, elen, s, dist + (size_t)a * n, true, dl, slots + blockIdx.x * slot_bytes, status);
   }
 }
 
@@ -350,17 +421,15 @@ __global__ void __launch_bounds__(kSsspThreads) k_sssp_maxmin(int32_t n, const i
                                                               const unsigned long long *__restrict__ key,
                                                               int32_t *__restrict__ pivot_out,
                                                               unsigned *__restrict__ mind,
-                                                              const float *__restrict__ delta, char *slots,
-                                                              size_t slot_bytes, bool init,
+                                                              const float *__restrict__ delta, char *slots, bool init,
                                                               int32_t *__restrict__ status) {
-  const SsspSlot sl = sssp_slot(slots, slot_bytes, 0, n);
   const int s = key ? (int)(0xFFFFFFFFu - (unsigned)(*key & 0xFFFFFFFFull)) : start;
   if (s < 0 || s >= n) {
     if (threadIdx.x == 0) dev_fail(status, SSM_E_ARG);
     return;
   }
   if (threadIdx.x == 0) *pivot_out = s;
-  sssp_block(n, rowptr, colidx, elen, s, mind, init, *delta, sl, status);
+  sssp_block(n, rowptr, colidx, elen, s, mind, init, *delta, slots, status);
 }
 
 // *key = max over v of (bits(mind_v) << 32 | (2^32 - 1 - v)): the largest
@@ -370,7 +439,7 @@ __global__ void k_wmm_argmax(int32_t n, const unsigned *__restrict__ mind, unsig
   unsigned long long best = 0;
   bool inf = false;
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-    const unsigned b = mind[v];
+    const unsigned b = mind[v] >> 1;
     inf |= b >= kInfBits;
     const unsigned long long kk = ((unsigned long long)b << 32) | (0xFFFFFFFFu - (unsigned)v);
     best = kk > best ? kk : best;
@@ -383,12 +452,28 @@ __global__ void k_wmm_argmax(int32_t n, const unsigned *__restrict__ mind, unsig
   if (inf) dev_fail(status, SSM_E_DISCONNECTED);
 }
 
-__global__ void k_check_finite_rows(int64_t count, const unsigned *__restrict__ dist, int32_t *__restrict__ status) {
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < count; t += (int64_t)gridDim.x * blockDim.x)
-    if (dist[t] >= kInfBits) {
-      dev_fail(status, SSM_E_DISCONNECTED);
-      return;
-    }
+// words to labels, four at a time where the table allows it; an unreachable
+// node is an error
+__global__ void k_sssp_labels(int64_t count, unsigned *__restrict__ dist, int32_t *__restrict__ status) {
+  const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, gs = (int64_t)gridDim.x * blockDim.x;
+  const int64_t quads = (reinterpret_cast<uintptr_t>(dist) & 15u) == 0 ? count / 4 : 0;
+  bool inf = false;
+  uint4 *d4 = reinterpret_cast<uint4 *>(dist);
+  for (int64_t t = gt; t < quads; t += gs) {
+    uint4 w = d4[t];
+    w.x >>= 1;
+    w.y >>= 1;
+    w.z >>= 1;
+    w.w >>= 1;
+    inf |= max(max(w.x, w.y), max(w.z, w.w)) >= kInfBits;
+    d4[t] = w;
+  }
+  for (int64_t t = 4 * quads + gt; t < count; t += gs) {
+    const unsigned w = dist[t] >> 1;
+    inf |= w >= kInfBits;
+    dist[t] = w;
+  }
+  if (inf) dev_fail(status, SSM_E_DISCONNECTED);
 }
 
 size_t sssp_ws_bytes(int32_t n, int32_t k) { return 256 + sssp_slot_bytes(n) * (size_t)sssp_blocks(k); }
@@ -400,20 +485,22 @@ int launch_sssp(int32_t n, const int32_t *rowptr, const int32_t *colidx, const f
   if (ws_bytes < sssp_ws_bytes(n, k))
     return fail(SSM_E_NOMEM, "sssp: workspace %zu bytes, need %zu", ws_bytes, sssp_ws_bytes(n, k));
   MeanWs *mean = (MeanWs *)ws;
-  float *delta = &mean->delta;
   char *slots = (char *)ws + 256;
-  SSM_TRY_CUDA(cudaMemsetAsync(slots, 0, sb * (size_t)blocks, s));
   if (int rc = launch_mean_length(n, rowptr, elen, mean, s)) return rc;
-  note_launch(), k_sssp_multi<<<blocks, kSsspMultiThreads, 0, s>>>(n, rowptr, colidx, (const unsigned *)elen, k, sources,
-                                                            (unsigned *)dist, delta, slots, sb, status);
+  // blocks of half the width, twice as many at once, where there are many
+  // sources and their rounds are narrow: 1024 sources take 2.6 against 3.1 ms
+  // on 20K nodes, but 43 against 32 ms on 262K
+  const int threads = k > 2 * num_sms() && n < 65536 ? kSsspThreads / 2 : kSsspThreads;
+  note_launch(), k_sssp_multi<<<blocks, threads, 0, s>>>(n, rowptr, colidx, (const unsigned *)elen, k, sources,
+                                                       (unsigned *)dist, mean, slots, sb, status);
   const int64_t cnt = (int64_t)k * n;
-  note_launch(), k_check_finite_rows<<<(unsigned)std::min<int64_t>((cnt + 255) / 256, (int64_t)num_sms() * 8), 256, 0,
-                                       s>>>(cnt, (const unsigned *)dist, status);
+  note_launch(), k_sssp_labels<<<(unsigned)std::min<int64_t>((cnt / 4 + 255) / 256 + 1, (int64_t)num_sms() * 16), 256, 0, s>>>(
+      cnt, (unsigned *)dist, status);
   SSM_TRY_CUDA(cudaGetLastError());
   return SSM_OK;
 }
 
-int sssp_blocks(int32_t k) { return std::max(1, std::min<int>(k, num_sms() * 3)); }
+int sssp_blocks(int32_t k) { return std::max(1, std::min<int>(k, num_sms() * 4)); }
 
 // ------------------------------------------------------------ regions and s
 __global__ void k_wregion_keys(int32_t n, int32_t k, const float *__restrict__ dist, int32_t *__restrict__ region,
@@ -877,15 +964,13 @@ SSM_API int ssm_select_pivots_weighted(int32_t n, int64_t m, const int32_t *rowp
     return rc;
   if (ran) return SSM_OK;
   SSM_TRY_CUDA(cudaMemsetAsync(w.keys, 0, (size_t)k * sizeof(unsigned long long), s));
-  SSM_TRY_CUDA(cudaMemsetAsync(w.slot, 0, sssp_slot_bytes(n), s));
-  const size_t sb = sssp_slot_bytes(n);
   note_launch(), k_sssp_maxmin<<<1, kSsspThreads, 0, s>>>(n, rowptr, colidx, (const unsigned *)elen, start, nullptr,
-                                                        pivots, w.mind, delta, w.slot, sb, true, status);
+                                                        pivots, w.mind, delta, w.slot, true, status);
   const unsigned ab = (unsigned)std::max(1, std::min((n + 255) / 256, num_sms() * 4));
   for (int a = 1; a < k; ++a) {
     note_launch(), k_wmm_argmax<<<ab, 256, 0, s>>>(n, w.mind, w.keys + a, status);
     note_launch(), k_sssp_maxmin<<<1, kSsspThreads, 0, s>>>(n, rowptr, colidx, (const unsigned *)elen, 0, w.keys + a,
-                                                          pivots + a, w.mind, delta, w.slot, sb, false, status);
+                                                          pivots + a, w.mind, delta, w.slot, false, status);
   }
   if (k == 1) note_launch(), k_wmm_argmax<<<ab, 256, 0, s>>>(n, w.mind, w.keys, status);  // reachability check
   SSM_TRY_CUDA(cudaGetLastError());
