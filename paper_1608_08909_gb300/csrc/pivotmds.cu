@@ -1103,65 +1103,129 @@ SSM_API int ssm_pivotmds(int32_t n, const int32_t *rowptr, const int32_t *colidx
 
 
 // ------------------------------------------------------------- weighted
-// PivotMDS on a float32 distance table (weighted graphs).  delta_ia = d_ia^2
-// is formed in FP64 (exactly); with cbar_a the column means,
+// PivotMDS on a float32 distance table (weighted graphs).  With delta_ia =
+// d_ia^2 and cbar_a the column means,
 //   C^T C = 1/4 J_k G' J_k,  G'_ab = sum_i (delta_ia - cbar_a)(delta_ib - cbar_b),
-// the column centring applied before the product so that nothing cancels;
-// G' is summed in FP64 per fixed node chunk and the chunk partials are added
-// in chunk order.
+// the column centring applied before the product so that nothing cancels.
+//
+// The squares are taken to fixed point: X_ia = d_ia^2 2^f rounded to an
+// integer (the square of a 24-bit mantissa shifted), f the largest with every
+// X below 2^48.  Rounding is at most 2^-47 of the largest square (2^-49 where
+// that lies just below a power of four), unbiased, so a sum over n nodes is off
+// by about 2^-48 / sqrt(n) of its terms' range -- below what FP64 additions
+// lose.  Column sums are exact integer sums.  For the product the centred value
+// V = X - C (C the mean rounded to an integer; |V| < 2^48) is split into
+// V = H 2^20 + L, |L| <= 2^19, and a pair costs three 32 x 32 -> 64-bit integer
+// multiply-adds, H H' and H L' + L H', exact over kWFlush nodes, where FP64 at
+// 1/64 of the FP32 rate costs 16 issue cycles a multiply-add.  L L' is formed on
+// the diagonal only, where it does not average out (elsewhere it is 2^-52 / sqrt(n)
+// of the entry).  The 64-bit sums go to FP64 per fixed node chunk and the chunk
+// partials are added in chunk order.
+// Measured (262K nodes, k = 200): the FP64 product took 16.2 ms, this one
+// 4.0; the column sums 0.26 -> 0.09 (and 0.04 for the largest distance); the
+// projection for a float layout 0.50 -> 0.09.
 namespace ssm {
 
-constexpr int kWTile = 32;
+constexpr int kWStage = 64;     // nodes staged in shared memory at a time
+constexpr int kWFlush = 512;    // nodes per 64-bit sum: 2^54 2^9 < 2^63
+constexpr int kWSplit = 20;     // bits of L
 
 static int64_t wgram_chunk(int32_t n) {
   int64_t c = ((int64_t)n + 63) / 64;
   c = std::max<int64_t>(1024, std::min<int64_t>(16384, c));
-  return (c + kWTile - 1) / kWTile * kWTile;
+  return (c + kWFlush - 1) / kWFlush * kWFlush;
 }
 
-// partc[a * nchunks + c] = sum over the nodes of chunk c of d_ia^2 (fixed tree)
+// the exponent f from the largest |distance| (its bits): dmax < 2^(E+1), so
+// dmax^2 2^f < 2^48 with f = 46 - 2 E.  A table with an infinity or a NaN gives
+// a NaN product, which the eigen-solve refuses.
+__device__ __forceinline__ bool wfix_bad(unsigned dmax_bits) { return dmax_bits >= 0x7F800000u; }
+__device__ __forceinline__ int wfix_f(unsigned dmax_bits) { return 46 - 2 * ((int)(dmax_bits >> 23) - 127); }
+
+// round(d^2 2^f), d a normal float (below that: 0)
+__device__ __forceinline__ long long wfix(float d, int f) {
+  const unsigned b = __float_as_uint(d) & 0x7FFFFFFFu;
+  const int e = (int)(b >> 23);
+  if (e == 0) return 0ll;
+  const unsigned long long m = (b & 0x7FFFFFu) | 0x800000u;
+  const int sh = -(2 * (e - 150) + f);  // d^2 = m^2 2^(2 (e - 150)); at least 0 for d <= dmax
+  if (sh > 48) return 0ll;
+  return (long long)((m * m + ((1ull << sh) >> 1)) >> sh);
+}
+
+__global__ void k_wdmax(int64_t count, const float *__restrict__ dist, unsigned *__restrict__ out) {
+  unsigned m = 0u;
+  const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, gs = (int64_t)gridDim.x * blockDim.x;
+  const int64_t quads = (reinterpret_cast<uintptr_t>(dist) & 15u) == 0 ? count / 4 : 0;
+  const uint4 *d4 = reinterpret_cast<const uint4 *>(dist);
+#pragma unroll 4
+  for (int64_t t = gt; t < quads; t += gs) {
+    const uint4 v = __ldg(d4 + t);
+    m = max(max(m, max(v.x & 0x7FFFFFFFu, v.y & 0x7FFFFFFFu)), max(v.z & 0x7FFFFFFFu, v.w & 0x7FFFFFFFu));
+  }
+  for (int64_t t = 4 * quads + gt; t < count; t += gs) m = max(m, __float_as_uint(__ldg(dist + t)) & 0x7FFFFFFFu);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+}
+
+// partc[a * nchunks + c] = sum over the nodes of chunk c of d_ia^2 (an exact
+// integer sum, rounded once)
 __global__ void __launch_bounds__(256) k_wcolsum_part(int32_t n, int32_t k, const float *__restrict__ dist,
-                                                      int64_t chunk, int64_t nchunks, double *__restrict__ partc) {
-  __shared__ double red[8];
+                                                      const unsigned *__restrict__ dmax, int64_t chunk, int64_t nchunks,
+                                                      double *__restrict__ partc) {
+  __shared__ unsigned long long red[8];
+  const int f = wfix_f(*dmax);
   for (int64_t task = blockIdx.x; task < (int64_t)k * nchunks; task += gridDim.x) {
     const int a = (int)(task / nchunks);
     const int64_t c = task - (int64_t)a * nchunks;
     const int64_t i0 = c * chunk, i1 = min((int64_t)n, i0 + chunk);
-    double acc = 0.0;
-    for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-      const double d = (double)__ldg(dist + (size_t)a * n + i);
-      acc += d * d;
+    const float *row = dist + (size_t)a * n;
+    unsigned long long acc = 0ull;  // at most 16384 values below 2^48
+    for (int64_t ib = i0 + threadIdx.x; ib < i1; ib += 4 * blockDim.x) {
+      float d[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) d[q] = ib + q * blockDim.x < i1 ? __ldg(row + ib + q * blockDim.x) : 0.0f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc += (unsigned long long)wfix(d[q], f);
     }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {
-      double t = 0.0;
+      unsigned long long t = 0ull;
       for (int w = 0; w < 8; ++w) t += red[w];
-      partc[task] = t;
+      partc[task] = scalbn((double)t, -f);
     }
     __syncthreads();
   }
 }
 
-__global__ void k_wcolsum_final(int32_t k, int64_t nchunks, const double *__restrict__ partc,
-                                double *__restrict__ colsum) {
+__global__ void k_wcolsum_final(int32_t n, int32_t k, int64_t nchunks, const double *__restrict__ partc,
+                                const unsigned *__restrict__ dmax, double *__restrict__ colsum,
+                                long long *__restrict__ centre) {
   for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < k; a += gridDim.x * blockDim.x) {
     double t = 0.0;
+#pragma unroll 8
     for (int64_t c = 0; c < nchunks; ++c) t += partc[(size_t)a * nchunks + c];
     colsum[a] = t;
+    centre[a] = __double2ll_rn(scalbn(t, wfix_f(*dmax)) / (double)n);
   }
 }
 
-// one 32 x 32 tile (ta <= tb) of G' over one node chunk; 16 x 16 threads,
-// 2 x 2 outputs each; partials into partg[c][a][b]
-__global__ void __launch_bounds__(256) k_wgram(int32_t n, int32_t k, const float *__restrict__ dist,
-                                               const double *__restrict__ colsum, int64_t chunk, int64_t nchunks,
-                                               int32_t ntiles, double *__restrict__ partg) {
-  __shared__ double sa[kWTile][kWTile + 1], sb[kWTile][kWTile + 1];  // [node][pivot]
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+// One T x T tile (ta <= tb) of G' over one node chunk; (T / 2)^2 threads, 2 x 2
+// outputs each; partials into partg[c][a][b].  Bound by the integer
+// multiply-adds (four issue cycles each); T = 32 or 40, whichever pads k less.
+template <int T>
+__global__ void __launch_bounds__(T *T / 4) k_wgram(int32_t n, int32_t k, const float *__restrict__ dist,
+                                                    const unsigned *__restrict__ dmax,
+                                                    const long long *__restrict__ centre, int64_t chunk,
+                                                    int64_t nchunks, int32_t ntiles, double *__restrict__ partg) {
+  constexpr int kThreads = T * T / 4, kHalf = T / 2;
+  __shared__ __align__(16) int sh[2][kWStage][T], sl[2][kWStage][T];  // H and L of both sides, [node][pivot]
+  const int tx = threadIdx.x % kHalf, ty = threadIdx.x / kHalf;
   const int64_t npairs = (int64_t)ntiles * (ntiles + 1) / 2;
-  const double inv_n = 1.0 / (double)n;
+  const int f = wfix_f(*dmax);
+  const double unit = wfix_bad(*dmax) ? __longlong_as_double(0x7FF8000000000000ll) : scalbn(1.0, -2 * f);
   for (int64_t task = blockIdx.x; task < npairs * nchunks; task += gridDim.x) {
     const int64_t c = task / npairs;
     int64_t pr = task - c * npairs;
@@ -1171,39 +1235,59 @@ __global__ void __launch_bounds__(256) k_wgram(int32_t n, int32_t k, const float
       ++ta;
     }
     const int tb = ta + (int)pr;
-    const int a0 = ta * kWTile, b0 = tb * kWTile;
+    const bool diag = ta == tb;
+    const int a0 = ta * T, b0 = tb * T;
     const int64_t i0 = c * chunk, i1 = min((int64_t)n, i0 + chunk);
-    double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-    for (int64_t ib = i0; ib < i1; ib += kWTile) {
-      // stage 32 nodes x 32 pivots of each side, centred by the column means
-      for (int e = threadIdx.x; e < kWTile * kWTile; e += blockDim.x) {
-        const int pv = e / kWTile, nd = e % kWTile;
-        const int64_t i = ib + nd;
-        double va = 0.0, vb = 0.0;
-        if (i < i1) {
-          if (a0 + pv < k) {
-            const double d = (double)__ldg(dist + (size_t)(a0 + pv) * n + i);
-            va = d * d - colsum[a0 + pv] * inv_n;
+    double g[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+    for (int64_t fb = i0; fb < i1; fb += kWFlush) {
+      long long hh[2][2] = {{0ll, 0ll}, {0ll, 0ll}}, hl[2][2] = {{0ll, 0ll}, {0ll, 0ll}}, ll[2] = {0ll, 0ll};
+      const int64_t fe = min(i1, fb + kWFlush);
+      for (int64_t ib = fb; ib < fe; ib += kWStage) {
+        __syncthreads();  // the staged nodes are consumed
+        for (int e = threadIdx.x; e < (diag ? 1 : 2) * kWStage * T; e += kThreads) {
+          const int side = e / (kWStage * T), r = e - side * (kWStage * T), pv = r / kWStage, nd = r % kWStage;
+          const int p = (side ? b0 : a0) + pv;
+          const int64_t i = ib + nd;
+          int H = 0, L = 0;
+          if (p < k && i < fe) {
+            const long long v = wfix(__ldg(dist + (size_t)p * n + i), f) - __ldg(centre + p);
+            H = (int)((v + (1ll << (kWSplit - 1))) >> kWSplit);
+            L = (int)(v - ((long long)H << kWSplit));
           }
-          if (b0 + pv < k) {
-            const double d = (double)__ldg(dist + (size_t)(b0 + pv) * n + i);
-            vb = d * d - colsum[b0 + pv] * inv_n;
-          }
+          sh[side][nd][pv] = H;
+          sl[side][nd][pv] = L;
         }
-        sa[nd][pv] = va;
-        sb[nd][pv] = vb;
-      }
-      __syncthreads();
+        __syncthreads();
+        const int sb = diag ? 0 : 1;
 #pragma unroll 4
-      for (int nd = 0; nd < kWTile; ++nd) {
-        const double x0 = sa[nd][2 * ty], x1 = sa[nd][2 * ty + 1];
-        const double y0 = sb[nd][2 * tx], y1 = sb[nd][2 * tx + 1];
-        acc[0][0] += x0 * y0;
-        acc[0][1] += x0 * y1;
-        acc[1][0] += x1 * y0;
-        acc[1][1] += x1 * y1;
+        for (int nd = 0; nd < kWStage; ++nd) {
+          const int2 xh = *reinterpret_cast<const int2 *>(&sh[0][nd][2 * ty]), xl = *reinterpret_cast<const int2 *>(&sl[0][nd][2 * ty]);
+          const int2 yh = *reinterpret_cast<const int2 *>(&sh[sb][nd][2 * tx]), yl = *reinterpret_cast<const int2 *>(&sl[sb][nd][2 * tx]);
+          hh[0][0] += (long long)xh.x * yh.x;
+          hh[0][1] += (long long)xh.x * yh.y;
+          hh[1][0] += (long long)xh.y * yh.x;
+          hh[1][1] += (long long)xh.y * yh.y;
+          hl[0][0] += (long long)xh.x * yl.x;
+          hl[0][1] += (long long)xh.x * yl.y;
+          hl[1][0] += (long long)xh.y * yl.x;
+          hl[1][1] += (long long)xh.y * yl.y;
+          hl[0][0] += (long long)xl.x * yh.x;
+          hl[0][1] += (long long)xl.x * yh.y;
+          hl[1][0] += (long long)xl.y * yh.x;
+          hl[1][1] += (long long)xl.y * yh.y;
+        }
+        if (diag && tx == ty)
+          for (int nd = 0; nd < kWStage; ++nd) {
+            ll[0] += (long long)sl[0][nd][2 * tx] * sl[0][nd][2 * tx];
+            ll[1] += (long long)sl[0][nd][2 * tx + 1] * sl[0][nd][2 * tx + 1];
+          }
       }
-      __syncthreads();
+#pragma unroll
+      for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          g[p][q] += ((double)hh[p][q] * (double)(1 << kWSplit) + (double)hl[p][q]) * (double)(1 << kWSplit) +
+                     (p == q ? (double)ll[p] : 0.0);
     }
     double *pg = partg + (size_t)c * k * k;
 #pragma unroll
@@ -1211,7 +1295,7 @@ __global__ void __launch_bounds__(256) k_wgram(int32_t n, int32_t k, const float
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         const int a = a0 + 2 * ty + p, b = b0 + 2 * tx + q;
-        if (a < k && b < k) pg[(size_t)a * k + b] = acc[p][q];
+        if (a < k && b < k) pg[(size_t)a * k + b] = g[p][q] * unit;
       }
   }
 }
@@ -1230,33 +1314,72 @@ __global__ void k_wgram_reduce(int32_t k, int64_t nchunks, const double *__restr
 }
 
 
-// x_i = C v = -1/2 (sum_a d_ia^2 v_a - rbar_i sigma - kappa), FP64
+// x_i = C v = -1/2 (sum_a d_ia^2 v_a - rbar_i sigma - kappa): in FP64 for a
+// double layout; for a float one the sum over pivots in two-float FP32 (d^2 as
+// an exact pair, 2^-45 or better, 0.5 ms of FP64 before)
+template <bool F64>
 __global__ void __launch_bounds__(256) k_wproject(int32_t n, int32_t k, const float *__restrict__ dist,
                                                   const double *__restrict__ vv, const EigOut *__restrict__ eo,
-                                                  void *__restrict__ pos, int precision) {
-  extern __shared__ __align__(16) double svv[];  // v0[k], v1[k]
-  for (int a = threadIdx.x; a < 2 * k; a += blockDim.x) svv[a] = vv[a];
+                                                  void *__restrict__ pos) {
+  extern __shared__ __align__(16) double svv[];  // FP64: v0[k], v1[k]; FP32: per pivot (v0 hi, v1 hi, v0 lo, v1 lo)
+  float4 *sv = reinterpret_cast<float4 *>(svv);
+  if (F64) {
+    for (int a = threadIdx.x; a < 2 * k; a += blockDim.x) svv[a] = vv[a];
+  } else {
+    for (int a = threadIdx.x; a < k; a += blockDim.x) {
+      const double v0 = vv[a], v1 = vv[k + a];
+      const float h0 = (float)v0, h1 = (float)v1;
+      sv[a] = make_float4(h0, h1, (float)(v0 - (double)h0), (float)(v1 - (double)h1));
+    }
+  }
   __syncthreads();
   const double sig0 = eo->sigma[0], sig1 = eo->sigma[1], kap0 = eo->kappa[0], kap1 = eo->kappa[1];
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     double x = 0.0, y = 0.0, rs = 0.0;
-    for (int a = 0; a < k; ++a) {
-      const double d = (double)__ldg(dist + (size_t)a * n + i);
-      const double dd = d * d;
-      rs += dd;
-      x += dd * svv[a];
-      y += dd * svv[k + a];
+    if (F64) {
+      for (int a = 0; a < k; ++a) {
+        const double d = (double)__ldg(dist + (size_t)a * n + i);
+        const double dd = d * d;
+        rs += dd;
+        x += dd * svv[a];
+        y += dd * svv[k + a];
+      }
+    } else {
+      float2 hi = make_float2(0.f, 0.f), lo = make_float2(0.f, 0.f);
+      float rh = 0.f, rl = 0.f;
+      for (int a0 = 0; a0 < k; a0 += 8) {
+        float dq[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) dq[q] = a0 + q < k ? __ldg(dist + (size_t)(a0 + q) * n + i) : 0.f;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          if (a0 + q >= k) break;
+          const float ph = dq[q] * dq[q], pl = fmaf(dq[q], dq[q], -ph);  // ph + pl = d^2
+          const float4 v = sv[a0 + q];
+          ff_madd2(hi, lo, ph, make_float2(v.x, v.y), make_float2(v.z, v.w));
+          lo.x = fmaf(pl, v.x, lo.x);
+          lo.y = fmaf(pl, v.y, lo.y);
+          const float t = rh + ph, z = t - rh;  // two-sum
+          rl += ((rh - (t - z)) + (ph - z)) + pl;
+          rh = t;
+        }
+      }
+      x = (double)hi.x + (double)lo.x;
+      y = (double)hi.y + (double)lo.y;
+      rs = (double)rh + (double)rl;
     }
     const double rbar = rs / (double)k;
     x = -0.5 * (x - rbar * sig0 - kap0);
     y = -0.5 * (y - rbar * sig1 - kap1);
-    if (precision == 64) reinterpret_cast<double2 *>(pos)[i] = make_double2(x, y);
+    if (F64) reinterpret_cast<double2 *>(pos)[i] = make_double2(x, y);
     else reinterpret_cast<float2 *>(pos)[i] = make_float2((float)x, (float)y);
   }
 }
 
 struct WMdsWs {
   double *colsum, *partc, *partg;
+  long long *centre;
+  unsigned *wmax;
 };
 
 static size_t carve_wmds(Carver &c, MdsWs &w, WMdsWs &x, int32_t n, int32_t k) {
@@ -1265,6 +1388,8 @@ static size_t carve_wmds(Carver &c, MdsWs &w, WMdsWs &x, int32_t n, int32_t k) {
   x.colsum = c.take<double>((size_t)k);
   x.partc = c.take<double>((size_t)k * nch);
   x.partg = c.take<double>((size_t)nch * k * k);
+  x.centre = c.take<long long>((size_t)k);
+  x.wmax = c.take<unsigned>(1);
   return c.size();
 }
 
@@ -1294,14 +1419,20 @@ SSM_API int ssm_pivotmds_weighted(int32_t n, const int32_t *rowptr, const int32_
   if (!c.ok) return fail(SSM_E_NOMEM, "ssm_pivotmds_weighted: workspace %zu bytes, need %zu", ws_bytes, c.size());
   const int sms = num_sms();
   const int64_t ch = wgram_chunk(n), nch = ((int64_t)n + ch - 1) / ch;
-  const int ntiles = (k + kWTile - 1) / kWTile;
   SSM_TRY_CUDA(cudaMemsetAsync(w.done, 0, sizeof(unsigned), s));
+  SSM_TRY_CUDA(cudaMemsetAsync(x.wmax, 0, sizeof(unsigned), s));
+  note_launch(), k_wdmax<<<sms * 8, 256, 0, s>>>((int64_t)k * n, dist, x.wmax);
   note_launch(), k_wcolsum_part<<<(unsigned)std::min<int64_t>((int64_t)k * nch, (int64_t)sms * 8), 256, 0, s>>>(
-      n, k, dist, ch, nch, x.partc);
-  note_launch(), k_wcolsum_final<<<std::max(1, (k + 255) / 256), 256, 0, s>>>(k, nch, x.partc, x.colsum);
-  const int64_t gtasks = (int64_t)ntiles * (ntiles + 1) / 2 * nch;
-  note_launch(), k_wgram<<<(unsigned)std::min<int64_t>(gtasks, (int64_t)sms * 8), 256, 0, s>>>(
-      n, k, dist, x.colsum, ch, nch, ntiles, x.partg);
+      n, k, dist, x.wmax, ch, nch, x.partc);
+  note_launch(), k_wcolsum_final<<<(k + 31) / 32, 32, 0, s>>>(n, k, nch, x.partc, x.wmax, x.colsum, x.centre);
+  auto tiles = [&](int T) { return (k + T - 1) / T; };
+  auto work = [&](int T) { return (int64_t)tiles(T) * (tiles(T) + 1) / 2 * T * T; };
+  const int T = work(40) < work(32) ? 40 : 32;
+  const unsigned gtasks = (unsigned)std::min<int64_t>((int64_t)tiles(T) * (tiles(T) + 1) / 2 * nch, (int64_t)sms * 64);
+  if (T == 40)
+    note_launch(), k_wgram<40><<<gtasks, 400, 0, s>>>(n, k, dist, x.wmax, x.centre, ch, nch, tiles(T), x.partg);
+  else
+    note_launch(), k_wgram<32><<<gtasks, 256, 0, s>>>(n, k, dist, x.wmax, x.centre, ch, nch, tiles(T), x.partg);
   const int64_t kk = (int64_t)k * k;
   note_launch(), k_wgram_reduce<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((kk + 255) / 256, sms * 4)), 256, 0,
                                   s>>>(k, nch, x.partg, w.B);
@@ -1311,7 +1442,11 @@ SSM_API int ssm_pivotmds_weighted(int32_t n, const int32_t *rowptr, const int32_
       k, w.B, w.rowmean);
   if (int rc = launch_eigen(n, k, w, (const double *)x.colsum, eig, status, s)) return rc;
   const int pb = (int)std::min<int64_t>(((int64_t)n + 255) / 256, (int64_t)sms * 8);
-  note_launch(), k_wproject<<<pb, 256, 2 * (size_t)k * sizeof(double), s>>>(n, k, dist, w.vv, w.eo, pos, precision);
+  const size_t psm = 2 * (size_t)k * sizeof(double);
+  if (precision == 64)
+    note_launch(), k_wproject<true><<<pb, 256, psm, s>>>(n, k, dist, w.vv, w.eo, pos);
+  else
+    note_launch(), k_wproject<false><<<pb, 256, psm, s>>>(n, k, dist, w.vv, w.eo, pos);
   if (rescale) return launch_rescale(n, rowptr, colidx, elen, pos, precision, w, status, s);
   SSM_TRY_CUDA(cudaGetLastError());
   return SSM_OK;

@@ -610,34 +610,98 @@ __global__ void k_seg_start(int32_t k, const unsigned long long *__restrict__ ke
   }
 }
 
-__global__ void k_wcounts(int32_t n, int32_t k, const int32_t *__restrict__ rowptr,
-                          const int32_t *__restrict__ colidx, const int32_t *__restrict__ pivots,
-                          const float *__restrict__ dist, const unsigned long long *__restrict__ keys,
-                          const int64_t *__restrict__ seg, uint32_t *__restrict__ s_out) {
-  const int64_t total = (int64_t)k * n;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int a = (int)(t / n), i = (int)(t - (int64_t)a * n);
-    const int p = __ldg(pivots + a);
-    uint32_t c = 0;
-    if (p != i && find_in_row(colidx, __ldg(rowptr + i), __ldg(rowptr + i + 1), p) < 0) {
-      const float d = __ldg(dist + t);
-      // entries of region a with 2 * d_ja <= d_ia: a prefix of the sorted segment
-      int64_t lo = seg[a], hi = seg[a + 1];
-      const int64_t b0 = lo;
-      while (lo < hi) {
-        const int64_t mid = lo + ((hi - lo) >> 1);
-        const float dj = __uint_as_float((unsigned)(keys[mid] & 0xFFFFFFFFull));
-        if (__fmul_rn(2.0f, dj) <= d) lo = mid + 1;
-        else hi = mid;
-      }
-      c = (uint32_t)(lo - b0);
+// s_ia for one pivot (blockIdx.x) and a range of nodes: the entries of region a
+// with 2 d_ja <= d_ia are a prefix of its sorted segment, found by binary search
+// in shared memory (a segment of more than kCountSeg entries: in global memory).
+// One search over global memory per (pivot, node), with a binary search of the
+// node's row for the pivot, took 1.62 ms on 52 M pairs, now 0.26; the pivot and its
+// neighbours, where s is 0, are cleared afterwards (k_wcounts_near).
+constexpr int kCountSeg = 8192;
+__global__ void __launch_bounds__(256) k_wcounts(int32_t n, const float *__restrict__ dist,
+                                                 const unsigned long long *__restrict__ keys,
+                                                 const int64_t *__restrict__ seg, uint32_t *__restrict__ s_out) {
+  __shared__ float sd[kCountSeg];
+  const int a = blockIdx.x;
+  const int64_t lo = seg[a];
+  const int len = (int)(seg[a + 1] - lo);
+  const bool staged = len <= kCountSeg;
+  if (staged)
+    for (int t = threadIdx.x; t < len; t += blockDim.x) sd[t] = __fmul_rn(2.0f, __uint_as_float((unsigned)keys[lo + t]));
+  __syncthreads();
+  const float *d = dist + (size_t)a * n;
+  uint32_t *out = s_out + (size_t)a * n;
+  for (int64_t i = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.y * blockDim.x) {
+    const float di = __ldg(d + i);
+    int b = 0, e = len;
+    while (b < e) {
+      const int mid = (b + e) >> 1;
+      const float v = staged ? sd[mid] : __fmul_rn(2.0f, __uint_as_float((unsigned)keys[lo + mid]));
+      if (v <= di) b = mid + 1;
+      else e = mid;
     }
-    s_out[t] = c;
+    out[i] = (uint32_t)b;
   }
+}
+
+__global__ void k_wcounts_near(int32_t n, const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
+                               const int32_t *__restrict__ pivots, uint32_t *__restrict__ s_out) {
+  const int p = pivots[blockIdx.x];
+  if ((unsigned)p >= (unsigned)n) return;
+  uint32_t *out = s_out + (size_t)blockIdx.x * n;
+  if (threadIdx.x == 0) out[p] = 0u;
+  for (int t = rowptr[p] + threadIdx.x; t < rowptr[p + 1]; t += blockDim.x) out[colidx[t]] = 0u;
 }
 
 // ------------------------------------------------------------ the sweep
 constexpr int kWSweepThreads = 256;
+
+// relative change: block sums; the last block adds them, a fixed share per
+// thread and a fixed tree (added by one thread they took 45 us of a 183 us
+// iteration on 1,023 blocks)
+__device__ void wsweep_change(double dn, double dd, double *__restrict__ part, unsigned *__restrict__ done,
+                              double *__restrict__ rel) {
+  __shared__ double red[2][kWSweepThreads / 32];
+  __shared__ unsigned s_ticket;
+  auto block_sum = [&](double &x, double &y) {  // in thread 0
+    for (int o = 16; o > 0; o >>= 1) {
+      x += __shfl_xor_sync(0xffffffffu, x, o);
+      y += __shfl_xor_sync(0xffffffffu, y, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+      red[0][threadIdx.x >> 5] = x;
+      red[1][threadIdx.x >> 5] = y;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      x = y = 0.0;
+      for (int w = 0; w < kWSweepThreads / 32; ++w) {
+        x += red[0][w];
+        y += red[1][w];
+      }
+    }
+    __syncthreads();
+  };
+  block_sum(dn, dd);
+  if (threadIdx.x == 0) {
+    part[2 * blockIdx.x] = dn;
+    part[2 * blockIdx.x + 1] = dd;
+    __threadfence();
+    s_ticket = atomicAdd(done, 1u);
+  }
+  __syncthreads();
+  if (s_ticket != gridDim.x - 1) return;
+  __threadfence();
+  double a0 = 0.0, a1 = 0.0;
+  for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
+    a0 += __ldcg(part + 2 * b);
+    a1 += __ldcg(part + 2 * b + 1);
+  }
+  block_sum(a0, a1);
+  if (threadIdx.x == 0) {
+    *rel = a1 > 0.0 ? sqrt(a0) / sqrt(a1) : 0.0;
+    *done = 0;
+  }
+}
 
 // Eq. 4 for one node in FP64, every operation rounded on its own in the
 // order of the plain FP64 definition (bit-identical to it)
@@ -717,39 +781,7 @@ __global__ void __launch_bounds__(kWSweepThreads) k_wsweep(int32_t n, const int3
     dn += ex * ex + ey * ey;
     dd += (double)xi.x * (double)xi.x + (double)xi.y * (double)xi.y;
   }
-  // relative change: block sums, then the last block adds them in block order
-  __shared__ double red[2][kWSweepThreads / 32];
-  __shared__ unsigned s_ticket;
-  for (int o = 16; o > 0; o >>= 1) {
-    dn += __shfl_xor_sync(0xffffffffu, dn, o);
-    dd += __shfl_xor_sync(0xffffffffu, dd, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    red[0][threadIdx.x >> 5] = dn;
-    red[1][threadIdx.x >> 5] = dd;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a0 = 0.0, a1 = 0.0;
-    for (int w = 0; w < kWSweepThreads / 32; ++w) {
-      a0 += red[0][w];
-      a1 += red[1][w];
-    }
-    part[2 * blockIdx.x] = a0;
-    part[2 * blockIdx.x + 1] = a1;
-    __threadfence();
-    s_ticket = atomicAdd(done, 1u);
-  }
-  __syncthreads();
-  if (s_ticket != gridDim.x - 1 || threadIdx.x != 0) return;
-  __threadfence();
-  double a0 = 0.0, a1 = 0.0;
-  for (unsigned b = 0; b < gridDim.x; ++b) {
-    a0 += __ldcg(part + 2 * b);
-    a1 += __ldcg(part + 2 * b + 1);
-  }
-  *rel = a1 > 0.0 ? sqrt(a0) / sqrt(a1) : 0.0;
-  *done = 0;
+  wsweep_change(dn, dd, part, done, rel);
 }
 
 // FP32 form: w'_ia = s_ia / d_ia^2 formed once per call into wtab (0 where
@@ -759,11 +791,17 @@ __global__ void __launch_bounds__(kWSweepThreads) k_wsweep(int32_t n, const int3
 // owns one node; eight pivots' (d, w') pairs are loaded before they are used.
 __global__ void k_wprep(int64_t count, const float *__restrict__ dist, const uint32_t *__restrict__ s_tab,
                         float *__restrict__ wtab) {
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < count; t += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t sc = s_tab[t];
-    const float d = dist[t];
-    wtab[t] = sc ? (float)sc / (d * d) : 0.0f;
+  auto weight = [](uint32_t sc, float d) { return sc ? (float)sc / (d * d) : 0.0f; };
+  const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, gs = (int64_t)gridDim.x * blockDim.x;
+  const bool quads_ok = ((reinterpret_cast<uintptr_t>(dist) | reinterpret_cast<uintptr_t>(s_tab)) & 15u) == 0;
+  const int64_t quads = quads_ok ? count / 4 : 0;  // wtab is 256-byte aligned
+#pragma unroll 2
+  for (int64_t t = gt; t < quads; t += gs) {
+    const float4 d = __ldg(reinterpret_cast<const float4 *>(dist) + t);
+    const uint4 c = __ldg(reinterpret_cast<const uint4 *>(s_tab) + t);
+    reinterpret_cast<float4 *>(wtab)[t] = make_float4(weight(c.x, d.x), weight(c.y, d.y), weight(c.z, d.z), weight(c.w, d.w));
   }
+  for (int64_t t = 4 * quads + gt; t < count; t += gs) wtab[t] = weight(s_tab[t], dist[t]);
 }
 
 constexpr int kWPrefetch = 8;
@@ -847,38 +885,7 @@ __global__ void __launch_bounds__(kWSweepThreads) k_wsweep_f32(int32_t n, const 
     dn += ex * ex + ey * ey;
     dd += (double)xi.x * (double)xi.x + (double)xi.y * (double)xi.y;
   }
-  __shared__ double red[2][kWSweepThreads / 32];
-  __shared__ unsigned s_ticket;
-  for (int o = 16; o > 0; o >>= 1) {
-    dn += __shfl_xor_sync(0xffffffffu, dn, o);
-    dd += __shfl_xor_sync(0xffffffffu, dd, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    red[0][threadIdx.x >> 5] = dn;
-    red[1][threadIdx.x >> 5] = dd;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a0 = 0.0, a1 = 0.0;
-    for (int w = 0; w < kWSweepThreads / 32; ++w) {
-      a0 += red[0][w];
-      a1 += red[1][w];
-    }
-    part[2 * blockIdx.x] = a0;
-    part[2 * blockIdx.x + 1] = a1;
-    __threadfence();
-    s_ticket = atomicAdd(done, 1u);
-  }
-  __syncthreads();
-  if (s_ticket != gridDim.x - 1 || threadIdx.x != 0) return;
-  __threadfence();
-  double a0 = 0.0, a1 = 0.0;
-  for (unsigned b = 0; b < gridDim.x; ++b) {
-    a0 += __ldcg(part + 2 * b);
-    a1 += __ldcg(part + 2 * b + 1);
-  }
-  *rel = a1 > 0.0 ? sqrt(a0) / sqrt(a1) : 0.0;
-  *done = 0;
+  wsweep_change(dn, dd, part, done, rel);
 }
 
 }  // namespace ssm
@@ -1017,9 +1024,8 @@ SSM_API int ssm_weighted_counts(int32_t n, const int32_t *rowptr, const int32_t 
       n, k, dist, region, w.keys, npad);
   if (int rc = launch_sort(w.keys, npad, s)) return rc;
   note_launch(), k_seg_start<<<std::max(1, (k + 256) / 256), 256, 0, s>>>(k, w.keys, npad, w.seg);
-  const int64_t total = (int64_t)k * n;
-  note_launch(), k_wcounts<<<(unsigned)std::min<int64_t>((total + 255) / 256, (int64_t)sms * 16), 256, 0, s>>>(
-      n, k, rowptr, colidx, pivots, dist, w.keys, w.seg, s_tab);
+  note_launch(), k_wcounts<<<dim3((unsigned)k, (unsigned)std::min((n + 8191) / 8192, 65535)), 256, 0, s>>>(n, dist, w.keys, w.seg, s_tab);
+  note_launch(), k_wcounts_near<<<k, 128, 0, s>>>(n, rowptr, colidx, pivots, s_tab);
   SSM_TRY_CUDA(cudaGetLastError());
   return SSM_OK;
 }

@@ -30,7 +30,8 @@
 // those of every other correct search.  Entries beyond a queue's
 // shared-memory part go to a global spill area (an owner's node is in each
 // queue at most once, so `slots` entries per queue always suffice).
-// Measured (262K-node geometric graph, k = 200): kTIMES
+// Measured (262K-node geometric graph, k = 200): 123 ms in one block, 23.4 ms here
+// (about 2.9 us a round; 16 CTAs of 512 threads: 23.4, of 256: 26.6, of 1024: 25.8).
 #include <algorithm>
 
 #include "cluster.cuh"

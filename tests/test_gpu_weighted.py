@@ -248,3 +248,42 @@ def test_weighted_maxmin_disconnected():
         g = _gpu_wgraph(n, s, d, np.ones(len(s), np.float32))
         ssm.ssm_select_pivots_weighted(g, 4)
     assert e.value.code == -3
+
+
+@pytest.mark.parametrize("n,k", [(40, 2), (513, 31), (700, 40), (1025, 41), (3000, 65)])
+def test_weighted_pivotmds_tile_edges(n, k):
+    """The fixed-point Gram at the edges of its tiles and node ranges, lengths
+    spread over four decades: eigenvalues to 1e-10, double layout to 1e-9."""
+    rng = np.random.default_rng(n)
+    s, d = (lambda t: (t[1], t[2]))(I.random_btree(n, 3))
+    s, d = np.concatenate([s, rng.integers(0, n, n).astype(np.int32)]), np.concatenate([d, rng.integers(0, n, n).astype(np.int32)])
+    l = _mixed_lengths(len(s), n)
+    og = O.build_wcsr(n, s, d, l)
+    dip = O.wpivot_dist(og, rng.permutation(n)[:k].astype(np.int32))
+    opos, oeig = O.wpivotmds(dip)
+    g = _gpu_wgraph(n, s, d, l)
+    pos, eig = ssm.ssm_pivotmds_weighted(g, torch.from_numpy(dip).to(DEV), precision=64, rescale=False)
+    eig = eig.cpu().numpy()
+    np.testing.assert_allclose(eig[0], oeig[0], rtol=1e-10)
+    # two pivots have one axis (the second eigenvalue is zero but for rounding)
+    # whose two entries tie: either sign
+    axes = 2 if oeig[1] > 1e-6 * oeig[0] else 1
+    if axes == 2:
+        np.testing.assert_allclose(eig[1], oeig[1], rtol=1e-10)
+    got = pos.cpu().numpy()[:, :axes]
+    if k == 2 and (got * opos[:, :1]).sum() < 0:
+        got = -got
+    assert _norm_err(got, opos[:, :axes]) < 1e-9
+
+
+def test_weighted_counts_of_a_large_region():
+    """Regions longer than the part of a segment kept in shared memory."""
+    n, s, d, l = I.rgg_lengths(30000, 8.0, 11)
+    og = O.build_wcsr(n, s, d, l)
+    piv = O.wmaxmin(og, 2)
+    dip = O.wpivot_dist(og, piv)
+    reg = O.wregions(dip)
+    g = _gpu_wgraph(n, s, d, l)
+    greg, gs = ssm.ssm_weighted_counts(g, torch.from_numpy(piv).to(DEV), torch.from_numpy(dip).to(DEV))
+    assert np.array_equal(greg.cpu().numpy(), reg)
+    assert np.array_equal(gs.cpu().numpy(), O.wcounts(og, piv, dip, reg, threads=8))
