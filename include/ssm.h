@@ -82,9 +82,10 @@ unsigned long long ssm_set_wait_limit_ns(unsigned long long ns);
  *   out[0] the sweep kernel: 0 FP32 with the clamped s table in shared memory,
  *          1 FP32 with the clamped s table in global memory, 2 FP32 with the
  *          full (w', w' d) table, 3 FP64 with the counts in shared memory,
- *          4 FP64 with the counts in global memory (-1: no call yet);
+ *          4 FP64 with the counts in global memory, 5 FP32 in one thread-block
+ *          cluster (small graphs, at least four iterations) (-1: no call yet);
  *   out[1] pivot ranges per 128-node tile (1: a warp takes whole tiles);
- *   out[2] blocks of the sweep grid;  out[3] the largest d_ip entry (FP32) or -1.
+ *   out[2] blocks of the sweep grid (of the cluster);  out[3] the largest d_ip entry (FP32) or -1.
  * A diagnostic with no counterpart in the paper. */
 void ssm_last_sweep_config(int32_t *out);
 

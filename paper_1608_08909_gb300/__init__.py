@@ -141,7 +141,7 @@ def ssm_last_sweep_config() -> dict:
     out = (ctypes.c_int32 * 4)()
     lib().ssm_last_sweep_config(ctypes.cast(out, ctypes.c_void_p))
     kinds = {-1: None, 0: "f32_clamped_smem", 1: "f32_clamped_global", 2: "f32_full_table", 3: "f64_counts_smem",
-             4: "f64_counts_global"}
+             4: "f64_counts_global", 5: "f32_cluster"}
     return {"kernel": kinds.get(out[0], out[0]), "nsplit": out[1], "blocks": out[2], "dmax": out[3]}
 
 

@@ -56,6 +56,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "sweep.cuh"
 
 namespace ssm {
 
@@ -969,17 +970,40 @@ SSM_API int ssm_iterate(int32_t n, int64_t m, const int32_t *rowptr, const int32
     // clamped s table; the row lengths decide the neighbour-kernel grid
     // (from the caller's hints when given; otherwise read back once)
     SSM_TRY_CUDA(cudaMemsetAsync(w.meta, 0, 4 * sizeof(unsigned), s));
-    note_launch(), k_nbr_classify<<<nb, 256, 0, s>>>(n, rowptr, w.meta + 1, w.mid_rows, w.long_rows);
     if (hints) {
       if (hints[0] < 0 || hints[0] > 65534 || hints[1] < 0 || hints[2] < 0 || hints[1] + hints[2] > n)
         return fail(SSM_E_ARG, "ssm_iterate: bad hints");
       for (int q = 0; q < 3; ++q) meta[q] = (unsigned)hints[q];
-    } else {
+    }
+    // small graphs: all iterations in one cluster launch
+    auto in_cluster = [&](int *blocks) {
+      return launch_sweep_cluster(n, m, rowptr, colidx, k, pivots, dip, cnt_off, cnt, (int32_t)meta[0], (float2 *)pos, iters,
+                                  tol, iters_done, rel_change, status, s, blocks);
+    };
+    auto note_cluster = [&](int blocks) {
+      const int32_t config[4] = {5, 1, blocks, (int32_t)meta[0]};
+      std::copy(config, config + 4, g_last_config);
+    };
+    int cluster = 0;
+    if (hints) {
+      if (int rc = in_cluster(&cluster)) return rc;
+      if (cluster) {
+        note_cluster(cluster);
+        return SSM_OK;
+      }
+    }
+    note_launch(), k_nbr_classify<<<nb, 256, 0, s>>>(n, rowptr, w.meta + 1, w.mid_rows, w.long_rows);
+    if (!hints) {
       const int64_t kn = (int64_t)k * n;
       note_launch(), k_dip_max<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((kn + 255) / 256, sms * 8)), 256, 0,
                                  s>>>(kn, dip, w.meta);
       SSM_TRY_CUDA(cudaMemcpyAsync(meta, w.meta, 3 * sizeof(unsigned), cudaMemcpyDeviceToHost, s));
       SSM_TRY_CUDA(cudaStreamSynchronize(s));
+      if (int rc = in_cluster(&cluster)) return rc;
+      if (cluster) {
+        note_cluster(cluster);
+        return SSM_OK;
+      }
     }
     const unsigned dmax = meta[0];
     const bool full = (size_t)k * ((size_t)dmax + 1) <= (size_t)kFullPlane;

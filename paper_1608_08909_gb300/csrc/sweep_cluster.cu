@@ -1,0 +1,387 @@
+// The FP32 Jacobi sweeps of Eq. 4 for a small graph, all iterations in one
+// launch of one thread-block cluster.
+//
+// On a graph of a few thousand nodes an iteration on the whole GPU is two
+// kernels that each wait for the other (14 us at n = 1024, k = 50, of which the
+// arithmetic is well below one).  Here a cluster of C CTAs (16 or 8) keeps
+// everything in shared memory: every CTA holds the positions of all nodes (two
+// buffers), the (w', w' d) table of every pivot and distance, and for the nodes
+// it owns (every C-th, so that the hubs of a heavy-tailed graph are spread) the
+// table places of their d_ip and their neighbours.  Positions are kept CTA by
+// CTA: node v at (v mod C) per + v div C.  A lane has two consecutive nodes (packed FP32x2), so a pivot's
+// position is one broadcast and its table row is shared by 64 nodes; the warps
+// of a 64-node block share its pivots and neighbours (warp w every W-th), rows
+// above kScLong entries are a warp's work each, and a node's W + 1 partial sums
+// are added in order.  (Lanes sharing a node, each with its own pivots, took
+// 1.4 to 5 times as long: every pivot position and table entry was a gather.)
+// At the end of an iteration a CTA copies its new positions into the other
+// buffer of every CTA (bulk copies through distributed shared memory, which
+// complete on an mbarrier of the receiver), and goes on when all of the others'
+// have arrived: no cluster barrier.  A CTA sends X^{t+1} after it has read X^t
+// for the last time, so a sender that has received everybody's X^{t+1} may write
+// X^{t+2} over X^t; barriers alternate with the buffers for the same reason.
+//
+// The update is the single-graph sweep's form about x_i: x_i + (sum_a (B - w)
+// (x_i - x_p) + sum_j (x_j - x_i)(1 - 1/r)) / den, B = w d / r, with r^2 + 1e-24
+// so that coincident points add nothing; only the order of a node's sum differs
+// (fixed here too).  Bound by latency: shared-memory gathers, two block
+// barriers and the copies.  Measured (us an iteration, two kernels on the whole
+// GPU before, here): grid of 1,024 nodes, k = 50: 14.4, 2.1; Barabasi-Albert
+// graph of 8,000 nodes, k = 60: 18.3, 6.8; of 4,096 nodes, k = 200: 24, 7.2.
+#include <algorithm>
+
+#include "cluster.cuh"
+#include "common.cuh"
+#include "sweep.cuh"
+#include "tc.cuh"
+
+namespace ssm {
+
+constexpr int kScThreads = 1024;  // half as many where a CTA has fewer than kScWide (node, pivot) pairs
+constexpr int kScWide = 8192;
+constexpr int kScLong = 16;       // longest row that one lane per warp walks
+constexpr int kScMaxCluster = 16;
+constexpr int kScMaxN = 8192;     // node ids in 16 bits
+constexpr int kScMaxD = 4095;     // d^2 exact in FP32
+constexpr int kScMinIters = 4;    // the tables are formed by every launch
+constexpr float kScR2Floor = 1e-24f;
+
+struct ScArgs {
+  int32_t n, k, dmax, per, perp, warps, iters;  // nodes per CTA (perp: up to whole blocks), warps per 64-node block
+  int32_t ecap;  // neighbour ids of a CTA kept in shared memory
+  const int32_t *rowptr, *colidx, *pivots, *cnt_off;
+  const uint32_t *cnt;
+  const uint16_t *dip;
+  float2 *pos;
+  double tol;
+  int32_t *iters_done;
+  double *rel_change;
+  int32_t *status;
+};
+
+__device__ __forceinline__ float sc_rsqrt(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// one thread: `bytes` (a multiple of 16) of this CTA's shared memory to the
+// address dst of another CTA, completing on that CTA's mbarrier
+__device__ __forceinline__ void dsmem_bulk_copy(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t mbar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "r"(src), "r"(bytes), "r"(mbar)
+               : "memory");
+}
+
+__device__ __forceinline__ void dsmem_st_d2(uint32_t a, double x, double y) {
+  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(x), "d"(y) : "memory");
+}
+
+// the term of a neighbour at place j about x
+__device__ __forceinline__ void sc_edge(const float2 *Xc, int j, float2 x, float &sx, float &sy) {
+  const float2 q = Xc[j];
+  const float ex = q.x - x.x, ey = q.y - x.y;
+  const float r2 = fmaf(ex, ex, ey * ey);
+  const float f = r2 > 0.f ? 1.f - sc_rsqrt(r2) : 0.f;
+  sx = fmaf(ex, f, sx);
+  sy = fmaf(ey, f, sy);
+}
+
+__global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
+  extern __shared__ __align__(16) unsigned char sc_smem[];
+  __shared__ double s_red[2][kScThreads / 32];
+  __shared__ __align__(16) double2 s_part[2][kScMaxCluster];
+  __shared__ __align__(8) uint64_t s_bar[2];  // X^t of the other CTAs has arrived, by parity of t
+  const int n = A.n, k = A.k, D = A.dmax + 1;
+  unsigned C;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+  const size_t stride = (size_t)A.per * C;  // the last CTAs' places may be one short
+  float2 *X = reinterpret_cast<float2 *>(sc_smem);            // [2][stride]
+  float2 *tab = X + 2 * stride;                               // [k][D] (-w, w d)
+  float2 *part = tab + (size_t)k * D;                         // [warps + 1][perp] partial sums; the last: long rows
+  float *den = reinterpret_cast<float *>(part + (size_t)(A.warps + 1) * A.perp);  // [perp]
+  int32_t *rows = reinterpret_cast<int32_t *>(den + A.perp);  // [perp + 1] row starts, local
+  int32_t *lrows = rows + A.perp + 2;                         // [perp] long rows
+  int32_t *start = lrows + A.perp;                            // [perp] entry of the graph's rows less the local one
+  int32_t *pnode = start + A.perp;                            // [k]
+  uint16_t *place = reinterpret_cast<uint16_t *>(pnode + ((k + 1) & ~1));  // [k][perp]
+  uint16_t *cols = place + (size_t)k * A.perp;                // [ecap]
+  __shared__ int s_nlong;
+  const unsigned r = cluster_rank();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int T = (int)blockDim.x;
+  const int i0 = (int)r * A.per, own = n > (int)r ? (n - 1 - (int)r) / (int)C + 1 : 0;  // nodes r, r + C, ...
+  auto at = [&](int v) { return (v % (int)C) * A.per + v / (int)C; };
+
+  for (int i = tid; i < n; i += T) X[at(i)] = A.pos[i];
+  // w = s / d^2, w d = s / d from exact operands (s <= n, d^2 < 2^24), each rounded once
+  for (int t = tid; t < k * D; t += T) {
+    const int a = t / D, d = t - a * D;
+    const int o = __ldg(A.cnt_off + a), ecc = __ldg(A.cnt_off + a + 1) - o - 1;
+    float2 w = make_float2(0.f, 0.f);
+    if (d >= 2) {
+      const float s = (float)__ldg(A.cnt + o + min(d >> 1, ecc)), fd = (float)d;
+      w = make_float2(-__fdiv_rn(s, fd * fd), __fdiv_rn(s, fd));
+    }
+    tab[t] = w;
+  }
+  for (int a = tid; a < k; a += T) {
+    int p = __ldg(A.pivots + a);
+    if ((unsigned)p >= (unsigned)n) {  // a pivot id outside the graph: recorded, read as node 0
+      dev_fail(A.status, SSM_E_ARG);
+      p = 0;
+    }
+    pnode[a] = at(p);
+  }
+  if (tid == 0) {
+    s_nlong = 0;
+    rows[0] = 0;
+  }
+  if (warp == 0) {  // local row starts
+    int sum = 0;
+    for (int b = 0; b < A.perp; b += 32) {
+      const int li = b + lane, v = li * (int)C + (int)r;
+      int deg = li < own ? __ldg(A.rowptr + v + 1) - __ldg(A.rowptr + v) : 0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, deg, o);
+        if (lane >= o) deg += t;
+      }
+      rows[li + 1] = sum + deg;
+      sum += __shfl_sync(0xffffffffu, deg, 31);
+    }
+  }
+  __syncthreads();
+  const bool cols_here = rows[own] <= A.ecap;  // else read from the graph, entry by entry
+  for (int li = tid; li < own; li += T) {
+    const int e = __ldg(A.rowptr + li * (int)C + (int)r), t0 = rows[li], len = rows[li + 1] - t0;
+    start[li] = e - t0;
+    if (cols_here && len <= kScLong)
+      for (int t = 0; t < len; ++t) cols[t0 + t] = (uint16_t)at(__ldg(A.colidx + e + t));
+  }
+  __syncthreads();
+  if (cols_here)  // long rows, a warp each
+    for (int li = warp; li < own; li += T / 32) {
+      const int t0 = rows[li], len = rows[li + 1] - t0;
+      if (len > kScLong)
+        for (int t = lane; t < len; t += 32) cols[t0 + t] = (uint16_t)at(__ldg(A.colidx + start[li] + t0 + t));
+    }
+  for (int t = tid; t < A.perp * k; t += T) {
+    const int a = t / A.perp, li = t - a * A.perp;
+    unsigned d = li < own ? __ldg(A.dip + (size_t)a * n + li * (int)C + (int)r) : 0u;
+    if (d > (unsigned)A.dmax) {  // a wrong dmax hint: recorded, clamped
+      dev_fail(A.status, SSM_E_ARG);
+      d = (unsigned)A.dmax;
+    }
+    place[t] = (uint16_t)(a * D + (int)d);
+  }
+  __syncthreads();
+  for (int li = tid; li < A.perp; li += T) {  // denominators: they do not change between iterations
+    const int deg = rows[li + 1] - rows[li];
+    float acc = 0.f;
+    for (int a = 0; a < k; ++a) acc -= tab[place[a * A.perp + li]].x;
+    den[li] = acc + (float)deg;
+    part[(size_t)A.warps * A.perp + li] = make_float2(0.f, 0.f);
+    if (deg > kScLong) lrows[atomicAdd(&s_nlong, 1)] = li;  // in any order: every row is a sum of its own
+  }
+  const int W = A.warps, blocks = A.perp / 64, blk = warp / W, wb = warp - blk * W;
+  const int l0 = 64 * blk + 2 * lane;  // this lane's nodes l0, l0 + 1 (blk < blocks)
+  // bytes of the others' positions (every CTA sends an even number of nodes)
+  unsigned expect = 0;
+  for (unsigned c = 0; c < C; ++c)
+    if (c != r && n > (int)c) expect += 8u * (unsigned)(((n - 1 - (int)c) / (int)C + 2) & ~1);
+  if (tid == 0) {
+    for (int q = 0; q < 2; ++q) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_smem(&s_bar[q])));
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  cluster_sync();  // every CTA of the cluster runs, and has read pos, before any remote write
+
+  int it = 0;
+  bool ok = true;
+  for (; it < A.iters; ++it) {
+    const float2 *Xc = X + (size_t)(it & 1) * stride;
+    float2 *Xn = X + (size_t)((it & 1) ^ 1) * stride;
+    const uint32_t bar = tc_smem(&s_bar[(it + 1) & 1]);
+    const bool change = A.tol > 0.0 || it + 1 == A.iters;
+    if (blk < blocks) {
+      const float2 x0 = l0 < own ? Xc[i0 + l0] : make_float2(0.f, 0.f), x1 = l0 + 1 < own ? Xc[i0 + l0 + 1] : make_float2(0.f, 0.f);
+      const float2 xi = make_float2(x0.x, x1.x), yi = make_float2(x0.y, x1.y), tiny = make_float2(kScR2Floor, kScR2Floor);
+      float2 ax = make_float2(0.f, 0.f), ay = ax;
+#pragma unroll 4
+      for (int a = wb; a < k; a += W) {
+        const unsigned pl = *reinterpret_cast<const unsigned *>(place + a * A.perp + l0);
+        const float2 w0 = tab[pl & 0xFFFFu], w1 = tab[pl >> 16], p = Xc[pnode[a]];
+        const float2 dx = __fadd2_rn(xi, make_float2(-p.x, -p.x)), dy = __fadd2_rn(yi, make_float2(-p.y, -p.y));
+        const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, tiny));
+        const float2 c = __ffma2_rn(make_float2(w0.y, w1.y), make_float2(sc_rsqrt(r2.x), sc_rsqrt(r2.y)),
+                                    make_float2(w0.x, w1.x));  // B - w
+        ax = __ffma2_rn(c, dx, ax);
+        ay = __ffma2_rn(c, dy, ay);
+      }
+      float sx[2] = {ax.x, ax.y}, sy[2] = {ay.x, ay.y};
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int rb = rows[l0 + q], re = rows[l0 + q + 1];
+        if (re - rb <= kScLong)
+          for (int t = rb + wb; t < re; t += W) sc_edge(Xc, cols_here ? cols[t] : at(__ldg(A.colidx + start[l0 + q] + t)), q ? x1 : x0, sx[q], sy[q]);
+        part[(size_t)wb * A.perp + l0 + q] = make_float2(sx[q], sy[q]);
+      }
+    }
+    for (int q = warp; q < s_nlong; q += T / 32) {
+      const int li = lrows[q];
+      const float2 x = Xc[i0 + li];
+      float sx = 0.f, sy = 0.f;
+      for (int t = rows[li] + lane; t < rows[li + 1]; t += 32) sc_edge(Xc, cols_here ? cols[t] : at(__ldg(A.colidx + start[li] + t)), x, sx, sy);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        sx += __shfl_xor_sync(0xffffffffu, sx, o);
+        sy += __shfl_xor_sync(0xffffffffu, sy, o);
+      }
+      if (lane == 0) part[(size_t)W * A.perp + li] = make_float2(sx, sy);
+    }
+    __syncthreads();
+    float cn = 0.f, cd = 0.f;
+    for (int li = tid; li < own; li += T) {
+      const float2 x = Xc[i0 + li];
+      float ax = 0.f, ay = 0.f;
+#pragma unroll 4
+      for (int w = 0; w <= W; ++w) {
+        const float2 v = part[(size_t)w * A.perp + li];
+        ax += v.x;
+        ay += v.y;
+      }
+      const float dn = den[li], chk = ax + ay;
+      if (!(chk == chk)) dev_fail(A.status, SSM_E_NUMERIC);
+      const float ex = dn > 0.f ? ax / dn : 0.f, ey = dn > 0.f ? ay / dn : 0.f;
+      Xn[i0 + li] = make_float2(x.x + ex, x.y + ey);
+      cn = fmaf(ex, ex, fmaf(ey, ey, cn));
+      cd = fmaf(x.x, x.x, fmaf(x.y, x.y, cd));
+    }
+    if (change) {  // ||X^{t+1} - X^t||_F / ||X^t||_F: lanes, warps and CTAs in a fixed order
+      double tn = (double)cn, td = (double)cd;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        tn += __shfl_xor_sync(0xffffffffu, tn, o);
+        td += __shfl_xor_sync(0xffffffffu, td, o);
+      }
+      if (lane == 0) {
+        s_red[0][warp] = tn;
+        s_red[1][warp] = td;
+      }
+      __syncthreads();
+      if (warp == 0) {
+        tn = lane < T / 32 ? s_red[0][lane] : 0.0;
+        td = lane < T / 32 ? s_red[1][lane] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          tn += __shfl_xor_sync(0xffffffffu, tn, o);
+          td += __shfl_xor_sync(0xffffffffu, td, o);
+        }
+        if ((unsigned)lane < C) dsmem_st_d2(dsmem_addr(&s_part[it & 1][r], (unsigned)lane), tn, td);
+      }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the copies read what was just written
+    __syncthreads();
+    if (warp == 0) {
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(expect) : "memory");
+      __syncwarp();
+      if ((unsigned)lane < C && (unsigned)lane != r && own > 0)
+        dsmem_bulk_copy(dsmem_addr(Xn + i0, (unsigned)lane), tc_smem(Xn + i0), 8u * (unsigned)((own + 1) & ~1),
+                        dsmem_addr(&s_bar[(it + 1) & 1], (unsigned)lane));
+    }
+    // the (it / 2)-th use of this barrier; a CTA that gives up takes the others,
+    // whose waits then run out, with it
+    ok = tc_wait(bar, (unsigned)(it >> 1) & 1u);
+    if (!__syncthreads_and(ok ? 1 : 0)) {
+      ok = false;
+      break;
+    }
+    if (change) {
+      cluster_sync();  // the partial sums
+      double num = 0.0, dn = 0.0;
+      for (unsigned c = 0; c < C; ++c) {
+        num += s_part[it & 1][c].x;
+        dn += s_part[it & 1][c].y;
+      }
+      const double rel = dn > 0.0 ? sqrt(num) / sqrt(dn) : 0.0;
+      if (r == 0 && tid == 0) {
+        *A.rel_change = rel;
+        *A.iters_done = it + 1;
+      }
+      if (A.tol > 0.0 && rel < A.tol) {  // the same sums in every CTA: uniform
+        ++it;
+        break;
+      }
+    }
+  }
+  if (!ok) dev_fail(A.status, SSM_E_TIMEOUT);
+  const float2 *Xf = X + (size_t)(it & 1) * stride;
+  for (int t = tid; t < own; t += T) A.pos[t * (int)C + (int)r] = Xf[i0 + t];
+  cluster_sync();  // no CTA leaves while another may still write its shared memory
+}
+
+static size_t sc_smem_bytes(int32_t C, int32_t per, int32_t k, int32_t D, int32_t perp, int32_t warps) {
+  return ((size_t)2 * per * C + (size_t)k * D + (size_t)(warps + 1) * perp) * sizeof(float2) + (size_t)perp * 4 +
+         (size_t)(3 * perp + 2) * 4 + (size_t)((k + 1) & ~1) * 4 + (size_t)perp * k * 2;
+}
+
+int launch_sweep_cluster(int32_t n, int64_t m, const int32_t *rowptr, const int32_t *colidx, int32_t k,
+                         const int32_t *pivots, const uint16_t *dip, const int32_t *cnt_off, const uint32_t *cnt,
+                         int32_t dmax, float2 *pos, int32_t iters, double tol, int32_t *iters_done, double *rel_change,
+                         int32_t *status, cudaStream_t s, int *blocks) {
+  *blocks = 0;
+  if (n > kScMaxN || dmax > kScMaxD || iters < kScMinIters || (int64_t)k * (dmax + 1) > 65535) return SSM_OK;
+  int dev = 0, smem_max = 0;
+  SSM_TRY_CUDA(cudaGetDevice(&dev));
+  SSM_TRY_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  const size_t budget = (size_t)smem_max - 2 * 1024;  // static shared memory of the kernel
+  const void *kern = (const void *)k_sweep_cluster;
+  for (int C : {16, 8}) {
+    ScArgs A;
+    A.per = ((n + C - 1) / C + 1) & ~1;  // even: copies start on 16 bytes
+    A.perp = (A.per + 63) / 64 * 64;
+    const int threads = (int64_t)A.per * k < kScWide ? kScThreads / 2 : kScThreads;
+    A.warps = std::max(1, threads / 32 / (A.perp / 64));
+    if (A.perp / 64 > threads / 32) continue;  // a warp has one block of nodes
+    // fewer partial sums where the table leaves no room for them
+    while (A.warps > 1 && sc_smem_bytes(C, A.per, k, dmax + 1, A.perp, A.warps) > budget) A.warps /= 2;
+    const size_t fixed = sc_smem_bytes(C, A.per, k, dmax + 1, A.perp, A.warps);
+    if (fixed > budget) continue;
+    A.ecap = (int32_t)std::min<size_t>((budget - fixed) / 2, (size_t)(2 * m));
+    const size_t smem = fixed + (size_t)A.ecap * 2;
+    A.n = n; A.k = k; A.dmax = dmax; A.iters = iters; A.rowptr = rowptr; A.colidx = colidx; A.pivots = pivots;
+    A.cnt_off = cnt_off; A.cnt = cnt; A.dip = dip; A.pos = pos; A.tol = tol; A.iters_done = iters_done;
+    A.rel_change = rel_change; A.status = status;
+    if (C > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+      (void)cudaGetLastError();
+      continue;
+    }
+    SSM_TRY_CUDA(allow_dynamic_smem(kern));
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)C);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess) {
+      (void)cudaGetLastError();
+      continue;
+    }
+    if (clusters < 1) continue;
+    note_launch();
+    SSM_TRY_CUDA(cudaLaunchKernelEx(&cfg, k_sweep_cluster, A));
+    *blocks = C;
+    return SSM_OK;
+  }
+  return SSM_OK;
+}
+
+}  // namespace ssm

@@ -154,3 +154,63 @@ def test_sweep_coincident_positions(name, k, kernel):
     pos = torch.from_numpy(x0.copy()).to(DEV)
     ssm.ssm_batch_iterate([(g, P, pos)], 1)
     assert _norm_err(pos.cpu().numpy(), want) < 1e-5
+
+
+# ------------------------------------------------------------------ small graphs in one cluster
+def _clique(n):
+    s, d = np.triu_indices(n, 1)
+    return n, s.astype(np.int32), d.astype(np.int32)
+
+
+CLUSTER = {
+    "fewer_nodes_than_ctas": (lambda: I.path(5), 2),
+    "one_node_per_cta_and_one_more": (lambda: I.path(17), 17),
+    "ragged_blocks": (lambda: I.grid(33, 31), 12),
+    "long_rows": (lambda: I.ba(1025, 6, 3), 33),
+    "neighbours_beyond_shared_memory": (lambda: _clique(1500), 2),
+    "few_partial_sums": (lambda: I.grid(64, 64), 100),
+    "largest": (lambda: I.ba(8192, 4, 5), 60),
+    "one_too_large": (lambda: I.ba(8193, 4, 5), 60),
+}
+
+
+@pytest.mark.parametrize("name", list(CLUSTER))
+def test_sweep_fp32_small_graph_cluster(name):
+    """The fifth iteration of a cluster launch against the oracle's step from the
+    fourth (two launches that agree on the first four), at the single step's
+    bound of 1e-5; a spread-out random start."""
+    make, k = CLUSTER[name]
+    n, s, d = make()
+    prep = O.prepare(n, s, d, k)
+    x0 = (np.random.default_rng(n).standard_normal((n, 2)) * np.sqrt(n)).astype(np.float32)
+    g, P = _gpu_graph(n, s, d), _gpu_pivots(k, prep)
+    four, five = torch.from_numpy(x0.copy()).to(DEV), torch.from_numpy(x0.copy()).to(DEV)
+    ssm.ssm_iterate(g, P, four, 4)
+    done, rel = ssm.ssm_iterate(g, P, five, 5)
+    assert (ssm.ssm_last_sweep_config()["kernel"] == "f32_cluster") == (name != "one_too_large")
+    x4 = four.cpu().numpy().astype(np.float64)
+    want, orel = O.sweep_jacobi(prep.g, prep.pivots, prep.dip, prep.w, x4)
+    assert int(done.item()) == 5
+    assert _norm_err(five.cpu().numpy(), want) < 1e-5
+    assert rel.item() == pytest.approx(orel, rel=1e-4)
+
+
+def test_sweep_fp32_cluster_tolerance_and_wrong_hint():
+    """tol > 0 stops at the same iteration as single sweeps do; a largest
+    distance below the true one is refused."""
+    n, s, d = I.grid(32, 32)
+    g, P, pos, _ = ssm.prepare(n, s, d, 20)
+    one, x = 0, pos.clone()
+    while True:
+        _, rel = ssm.ssm_iterate(g, P, x, 1)
+        one += 1
+        if rel.item() < 3e-3:
+            break
+        assert one < 200
+    done, rel = ssm.ssm_iterate(g, P, pos, 200, tol=3e-3)
+    assert int(done.item()) == one > 4 and rel.item() < 3e-3
+    assert _norm_err(pos.cpu().numpy(), x.cpu().numpy().astype(np.float64)) < one * 1e-5
+    P.dmax -= 1
+    with pytest.raises(ssm.SSMError) as e:
+        ssm.ssm_iterate(g, P, pos, 4)
+    assert e.value.code == -1
