@@ -24,6 +24,7 @@
 
 #include "common.cuh"
 #include "gram_tc.cuh"
+#include "wgram_tc.cuh"
 
 namespace ssm {
 
@@ -1109,20 +1110,18 @@ SSM_API int ssm_pivotmds(int32_t n, const int32_t *rowptr, const int32_t *colidx
 // the column centring applied before the product so that nothing cancels.
 //
 // The squares are taken to fixed point: X_ia = d_ia^2 2^f rounded to an
-// integer (the square of a 24-bit mantissa shifted), f the largest with every
-// X below 2^48.  Rounding is at most 2^-47 of the largest square (2^-49 where
-// that lies just below a power of four), unbiased, so a sum over n nodes is off
-// by about 2^-48 / sqrt(n) of its terms' range -- below what FP64 additions
-// lose.  Column sums are exact integer sums.  For the product the centred value
-// V = X - C (C the mean rounded to an integer; |V| < 2^48) is split into
-// V = H 2^20 + L, |L| <= 2^19, and a pair costs three 32 x 32 -> 64-bit integer
-// multiply-adds, H H' and H L' + L H', exact over kWFlush nodes, where FP64 at
-// 1/64 of the FP32 rate costs 16 issue cycles a multiply-add.  L L' is formed on
-// the diagonal only, where it does not average out (elsewhere it is 2^-52 / sqrt(n)
-// of the entry).  The 64-bit sums go to FP64 per fixed node chunk and the chunk
-// partials are added in chunk order.
+// integer (the square of a 24-bit mantissa shifted).  Column sums are exact sums
+// of X below 2^49 (the rounding, unbiased, is 2^-49 / sqrt(n) of the range).  The
+// product is that of the centred integers V = X - C, C the mean rounded: on the
+// tensor cores for up to 208 pivots, X below 2^55 (wgram_tc.cu); for more of
+// them here, X below 2^47: V = H 2^20 + L, |L| <= 2^19, and a pair costs three 32 x 32 -> 64-bit
+// integer multiply-adds, H H' and H L' + L H', exact over kWFlush nodes, where
+// FP64 at 1/64 of the FP32 rate costs 16 issue cycles a multiply-add.  L L' is
+// formed on the diagonal only, where it does not average out (elsewhere it is
+// 2^-52 / sqrt(n) of the entry).  The 64-bit sums go to FP64 per fixed node
+// chunk and the chunk partials are added in chunk order.
 // Measured (262K nodes, k = 200): the FP64 product took 16.2 ms, this one
-// 4.0; the column sums 0.26 -> 0.09 (and 0.04 for the largest distance); the
+// 3.9, the tensor cores 1.7; the column sums 0.26 -> 0.09 (and 0.04 for the largest distance); the
 // projection for a float layout 0.50 -> 0.09.
 namespace ssm {
 
@@ -1134,23 +1133,6 @@ static int64_t wgram_chunk(int32_t n) {
   int64_t c = ((int64_t)n + 63) / 64;
   c = std::max<int64_t>(1024, std::min<int64_t>(16384, c));
   return (c + kWFlush - 1) / kWFlush * kWFlush;
-}
-
-// the exponent f from the largest |distance| (its bits): dmax < 2^(E+1), so
-// dmax^2 2^f < 2^48 with f = 46 - 2 E.  A table with an infinity or a NaN gives
-// a NaN product, which the eigen-solve refuses.
-__device__ __forceinline__ bool wfix_bad(unsigned dmax_bits) { return dmax_bits >= 0x7F800000u; }
-__device__ __forceinline__ int wfix_f(unsigned dmax_bits) { return 46 - 2 * ((int)(dmax_bits >> 23) - 127); }
-
-// round(d^2 2^f), d a normal float (below that: 0)
-__device__ __forceinline__ long long wfix(float d, int f) {
-  const unsigned b = __float_as_uint(d) & 0x7FFFFFFFu;
-  const int e = (int)(b >> 23);
-  if (e == 0) return 0ll;
-  const unsigned long long m = (b & 0x7FFFFFu) | 0x800000u;
-  const int sh = -(2 * (e - 150) + f);  // d^2 = m^2 2^(2 (e - 150)); at least 0 for d <= dmax
-  if (sh > 48) return 0ll;
-  return (long long)((m * m + ((1ull << sh) >> 1)) >> sh);
 }
 
 __global__ void k_wdmax(int64_t count, const float *__restrict__ dist, unsigned *__restrict__ out) {
@@ -1174,13 +1156,13 @@ __global__ void __launch_bounds__(256) k_wcolsum_part(int32_t n, int32_t k, cons
                                                       const unsigned *__restrict__ dmax, int64_t chunk, int64_t nchunks,
                                                       double *__restrict__ partc) {
   __shared__ unsigned long long red[8];
-  const int f = wfix_f(*dmax);
+  const int f = wfix_f(*dmax) + kWfix49;
   for (int64_t task = blockIdx.x; task < (int64_t)k * nchunks; task += gridDim.x) {
     const int a = (int)(task / nchunks);
     const int64_t c = task - (int64_t)a * nchunks;
     const int64_t i0 = c * chunk, i1 = min((int64_t)n, i0 + chunk);
     const float *row = dist + (size_t)a * n;
-    unsigned long long acc = 0ull;  // at most 16384 values below 2^48
+    unsigned long long acc = 0ull;  // at most 16384 values below 2^49
     for (int64_t ib = i0 + threadIdx.x; ib < i1; ib += 4 * blockDim.x) {
       float d[4];
 #pragma unroll
@@ -1201,14 +1183,14 @@ __global__ void __launch_bounds__(256) k_wcolsum_part(int32_t n, int32_t k, cons
 }
 
 __global__ void k_wcolsum_final(int32_t n, int32_t k, int64_t nchunks, const double *__restrict__ partc,
-                                const unsigned *__restrict__ dmax, double *__restrict__ colsum,
-                                long long *__restrict__ centre) {
+                                const unsigned *__restrict__ dmax, int bits, double *__restrict__ colsum,
+                                long long *__restrict__ centre) {  // the centre in X of exponent f + bits
   for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < k; a += gridDim.x * blockDim.x) {
     double t = 0.0;
 #pragma unroll 8
     for (int64_t c = 0; c < nchunks; ++c) t += partc[(size_t)a * nchunks + c];
     colsum[a] = t;
-    centre[a] = __double2ll_rn(scalbn(t, wfix_f(*dmax)) / (double)n);
+    centre[a] = __double2ll_rn(scalbn(t, wfix_f(*dmax) + bits) / (double)n);
   }
 }
 
@@ -1221,10 +1203,12 @@ __global__ void __launch_bounds__(T *T / 4) k_wgram(int32_t n, int32_t k, const 
                                                     const long long *__restrict__ centre, int64_t chunk,
                                                     int64_t nchunks, int32_t ntiles, double *__restrict__ partg) {
   constexpr int kThreads = T * T / 4, kHalf = T / 2;
-  __shared__ __align__(16) int sh[2][kWStage][T], sl[2][kWStage][T];  // H and L of both sides, [node][pivot]
+  // H and L of both sides, [node][pivot], rows two words longer so that a
+  // warp's stores (one pivot, consecutive nodes) meet in two lanes a bank at most
+  __shared__ __align__(16) int sh[2][kWStage][T + 2], sl[2][kWStage][T + 2];
   const int tx = threadIdx.x % kHalf, ty = threadIdx.x / kHalf;
   const int64_t npairs = (int64_t)ntiles * (ntiles + 1) / 2;
-  const int f = wfix_f(*dmax);
+  const int f = wfix_f(*dmax) + kWfix47;
   const double unit = wfix_bad(*dmax) ? __longlong_as_double(0x7FF8000000000000ll) : scalbn(1.0, -2 * f);
   for (int64_t task = blockIdx.x; task < npairs * nchunks; task += gridDim.x) {
     const int64_t c = task / npairs;
@@ -1380,6 +1364,7 @@ struct WMdsWs {
   double *colsum, *partc, *partg;
   long long *centre;
   unsigned *wmax;
+  unsigned long long *acc;  // tensor-core product (k <= kWgMaxK)
 };
 
 static size_t carve_wmds(Carver &c, MdsWs &w, WMdsWs &x, int32_t n, int32_t k) {
@@ -1387,7 +1372,8 @@ static size_t carve_wmds(Carver &c, MdsWs &w, WMdsWs &x, int32_t n, int32_t k) {
   const int64_t ch = wgram_chunk(n), nch = ((int64_t)n + ch - 1) / ch;
   x.colsum = c.take<double>((size_t)k);
   x.partc = c.take<double>((size_t)k * nch);
-  x.partg = c.take<double>((size_t)nch * k * k);
+  x.partg = k > kWgMaxK ? c.take<double>((size_t)nch * k * k) : nullptr;
+  x.acc = k > kWgMaxK ? nullptr : c.take<unsigned long long>(wgram_tc_acc_words(k));
   x.centre = c.take<long long>((size_t)k);
   x.wmax = c.take<unsigned>(1);
   return c.size();
@@ -1424,18 +1410,24 @@ SSM_API int ssm_pivotmds_weighted(int32_t n, const int32_t *rowptr, const int32_
   note_launch(), k_wdmax<<<sms * 8, 256, 0, s>>>((int64_t)k * n, dist, x.wmax);
   note_launch(), k_wcolsum_part<<<(unsigned)std::min<int64_t>((int64_t)k * nch, (int64_t)sms * 8), 256, 0, s>>>(
       n, k, dist, x.wmax, ch, nch, x.partc);
-  note_launch(), k_wcolsum_final<<<(k + 31) / 32, 32, 0, s>>>(n, k, nch, x.partc, x.wmax, x.colsum, x.centre);
-  auto tiles = [&](int T) { return (k + T - 1) / T; };
-  auto work = [&](int T) { return (int64_t)tiles(T) * (tiles(T) + 1) / 2 * T * T; };
-  const int T = work(40) < work(32) ? 40 : 32;
-  const unsigned gtasks = (unsigned)std::min<int64_t>((int64_t)tiles(T) * (tiles(T) + 1) / 2 * nch, (int64_t)sms * 64);
-  if (T == 40)
-    note_launch(), k_wgram<40><<<gtasks, 400, 0, s>>>(n, k, dist, x.wmax, x.centre, ch, nch, tiles(T), x.partg);
-  else
-    note_launch(), k_wgram<32><<<gtasks, 256, 0, s>>>(n, k, dist, x.wmax, x.centre, ch, nch, tiles(T), x.partg);
+  note_launch(), k_wcolsum_final<<<(k + 31) / 32, 32, 0, s>>>(n, k, nch, x.partc, x.wmax,
+                                                       k <= kWgMaxK ? 0 : kWfix47, x.colsum, x.centre);
   const int64_t kk = (int64_t)k * k;
-  note_launch(), k_wgram_reduce<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((kk + 255) / 256, sms * 4)), 256, 0,
-                                  s>>>(k, nch, x.partg, w.B);
+  if (k <= kWgMaxK) {
+    if (int rc = launch_wgram_tc(n, k, dist, x.wmax, x.centre, x.acc, w.B, status, s)) return rc;
+  } else {
+    // tiles of 32 or 40 pivots, whichever pad k less
+    auto tiles = [&](int T) { return (k + T - 1) / T; };
+    auto work = [&](int T) { return (int64_t)tiles(T) * (tiles(T) + 1) / 2 * T * T; };
+    const int T = work(40) < work(32) ? 40 : 32;
+    const unsigned gtasks = (unsigned)std::min<int64_t>((int64_t)tiles(T) * (tiles(T) + 1) / 2 * nch, (int64_t)sms * 64);
+    if (T == 40)
+      note_launch(), k_wgram<40><<<gtasks, 400, 0, s>>>(n, k, dist, x.wmax, x.centre, ch, nch, tiles(T), x.partg);
+    else
+      note_launch(), k_wgram<32><<<gtasks, 256, 0, s>>>(n, k, dist, x.wmax, x.centre, ch, nch, tiles(T), x.partg);
+    note_launch(), k_wgram_reduce<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((kk + 255) / 256, sms * 4)), 256, 0,
+                                    s>>>(k, nch, x.partg, w.B);
+  }
   // B = 1/4 (G' - rowmean_a - rowmean_b + grand mean)
   note_launch(), k_row_means<<<1, 1024, 0, s>>>(k, w.B, w.rowmean);
   note_launch(), k_center<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((kk + 255) / 256, sms * 4)), 256, 0, s>>>(

@@ -250,9 +250,10 @@ def test_weighted_maxmin_disconnected():
     assert e.value.code == -3
 
 
-@pytest.mark.parametrize("n,k", [(40, 2), (513, 31), (700, 40), (1025, 41), (3000, 65)])
+@pytest.mark.parametrize("n,k", [(40, 2), (513, 31), (700, 40), (1025, 128), (3000, 129), (2500, 208), (1500, 209), (1100, 240)])
 def test_weighted_pivotmds_tile_edges(n, k):
-    """The fixed-point Gram at the edges of its tiles and node ranges, lengths
+    """The fixed-point Gram at the edges of its tiles and node ranges, on the
+    tensor cores (up to 208 pivots) and in integer multiply-adds, lengths
     spread over four decades: eigenvalues to 1e-10, double layout to 1e-9."""
     rng = np.random.default_rng(n)
     s, d = (lambda t: (t[1], t[2]))(I.random_btree(n, 3))
