@@ -384,7 +384,7 @@ typedef struct {
 } ssm_batch_graph;
 size_t ssm_batch_iterate_workspace(int32_t G, const ssm_batch_graph *graphs);
 /* Batched preparation of the graphs above (Algorithm 1 lines 1-4 for G
- * small graphs in two launches, one block per graph): from edge lists to
+ * small graphs in three launches): from edge lists to
  * the packed arrays ssm_batch_iterate reads.  Graph g has n nodes (1..12288),
  * k max/min-sp pivots (2 <= k <= min(n, 100); start node 0), and m_in edges
  * src/dst[edge_off .. edge_off + m_in) with local ids.
@@ -396,8 +396,8 @@ size_t ssm_batch_iterate_workspace(int32_t G, const ssm_batch_graph *graphs);
  * m_out[g] (host, edges after deduplication; may be NULL).  Device errors
  * are read back and returned: SSM_E_GRAPH, SSM_E_DISCONNECTED.
  * ssm_batch_layout_init (asynchronous): from those, cnt_off / cnt (as
- * ssm_aggregate), PivotMDS (exact integer Gram matrix, FP64 eigenpairs by a
- * parallel cyclic Jacobi method) and the rescale to unit mean edge length
+ * ssm_aggregate), PivotMDS (exact integer Gram matrix, FP64 eigenpairs by
+ * Householder reduction and bisection) and the rescale to unit mean edge length
  * into pos (float x, y pairs at 2 node_off); eig (device double [2G], may be
  * NULL) gets the two eigenvalues.  m[g] (host) = the edge counts.  Both use
  * a workspace of ssm_batch_prepare_workspace(G, in) bytes (the same one).

@@ -21,7 +21,7 @@ __device__ __forceinline__ long long wfix(float d, int f) {
   const int e = (int)(b >> 23);
   if (e == 0) return 0ll;
   const unsigned long long m = (b & 0x7FFFFFu) | 0x800000u;
-  const int sh = -(2 * (e - 150) + f);  // d^2 = m^2 2^(2 (e - 150)); at least -7 for d <= dmax
+  const int sh = -(2 * (e - 150) + f);  // d^2 = m^2 2^(2 (e - 150)); at least -8 for d <= dmax
   if (sh > 48) return 0ll;
   return sh <= 0 ? (long long)((m * m) << -sh) : (long long)((m * m + (1ull << (sh - 1))) >> sh);
 }

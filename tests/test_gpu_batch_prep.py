@@ -138,3 +138,40 @@ def test_batch_prepare_errors():
     with pytest.raises(ssm.SSMError) as e:
         ssm.ssm_batch_prepare([(n, np.array([0, 70], np.int32), np.array([1, 2], np.int32), 5)])
     assert e.value.code == -2
+
+
+def _edges():
+    """Graphs at the edges of the preparation's kernels: word and chunk
+    boundaries, a hub, a path as long as allowed, neighbour lists that shared
+    memory does not hold (with and without repeated edges)."""
+    rng = np.random.default_rng(11)
+    out = []
+    for n, k in [(2, 2), (31, 31), (32, 32), (33, 33), (97, 64), (513, 65), (700, 96), (1025, 97)]:
+        n, s, d = _messy(n, n, max(60, 2 * n))
+        out.append((n, s, d, k))
+    hub = np.zeros(8000, np.int32)
+    out.append((8001, hub, np.arange(1, 8001, dtype=np.int32), 40))
+    n, s, d = I.path(12288)
+    out.append((n, s, d, 5))
+    n, s, d = _messy(5, 12288, 40000)
+    out.append((n, s, d, 34))
+    out.append((n, np.concatenate([s, s, d]), np.concatenate([d, d, s]), 100))
+    full = np.stack(np.triu_indices(400, 1)).astype(np.int32)
+    full = full[:, rng.permutation(full.shape[1])]
+    out.append((400, full[0], full[1], 100))
+    return out
+
+
+def test_batch_pivots_edges():
+    batch = _edges()
+    bp = ssm.ssm_batch_prepare(batch)
+    for g, (n, s, d, k) in enumerate(batch):
+        v = bp.graph(g)
+        og = O.build_csr(n, s, d)
+        assert np.array_equal(v["rowptr"].cpu().numpy(), og.rowptr), g
+        assert np.array_equal(v["colidx"].cpu().numpy(), og.colidx), g
+        piv = O.maxmin(og, k, 0)
+        assert np.array_equal(v["pivots"].cpu().numpy(), piv), g
+        dip = O.pivot_dist(og, piv)
+        assert np.array_equal(v["dip"].cpu().numpy(), dip), g
+        assert np.array_equal(v["region"].cpu().numpy(), O.regions(dip)), g
