@@ -8,13 +8,13 @@
 // shared memory; the running minimum names the regions, whose eccentricities
 // and the count-table length close the launch.  k_prep_dist searches from the
 // pivots, 32 of a graph at a time.  The host reads the lengths once for the
-// whole batch and places the tables.  k_prep_layout then fills the cumulative counts, forms
-// the exact integer Gram matrix Delta^T Delta of the squared distances
-// (128-bit sums over 32-node chunks staged in shared memory), the FP64
-// matrix B = 1/4 J (G - s s^T / n) J, its top two eigenpairs (Householder
-// reduction, bisection, inverse iteration; one block), projects, signs and rescales the
-// layout.  Every reduction has a fixed order: results do not depend on
-// timing.
+// whole batch and places the tables.  k_prep_gram forms the exact integer
+// Gram matrices Delta^T Delta of the squared distances; k_prep_layout, a block
+// per graph, fills the cumulative counts, forms the FP64 matrix
+// B = 1/4 J (G - s s^T / n) J and its top two eigenpairs (Householder
+// reduction, bisection, inverse iteration), projects, signs and rescales the
+// layout.  Sums are of whole numbers or in a fixed order: results do not
+// depend on timing.
 #include <algorithm>
 #include <vector>
 
@@ -25,7 +25,6 @@ namespace ssm {
 constexpr int kPrepMaxN = 12288;
 constexpr int kPrepMaxK = 100;
 constexpr int kPrepThreads = 512;
-constexpr int kPrepChunk = 32;     // nodes per staged chunk of the Gram
 
 struct PrepDev {
   int32_t n, k;
@@ -374,14 +373,16 @@ struct LayoutDev {
   int32_t n, k;
   int64_t m;
   int64_t node_off, row_off, col_off, piv_off, dip_off, cnt_off_off, cnt_base;
+  int64_t gram_off;  // words
 };
 
 struct LayoutArgs {
   int32_t G;
   const LayoutDev *desc;
-  const int32_t *order;
+  const int32_t *order, *task0;  // task0 [G + 1]: first Gram task by place in the order
   const int32_t *rowptr, *colidx, *region, *ecc;
   const uint16_t *dip;
+  unsigned long long *gram;  // per graph: column sums [k], then 32-bit parts (low, high) of the sums per pair
   int32_t *cnt_off;
   uint32_t *cnt;
   float2 *pos;
@@ -389,6 +390,90 @@ struct LayoutArgs {
   unsigned *ctr;
   int32_t *status;
 };
+
+static int64_t gram_words(int64_t k) { return k + 2 * k * k; }
+
+// The exact Gram matrix Delta^T Delta of the squared distances, over the whole
+// GPU: the unit of work is kGramNodes nodes of one graph, so that one large
+// graph's products are spread over the SMs (as part of the graph's own block
+// they were 4.6 M cycles of the longest chain of a batch).  A thread owns an
+// 8 x 8 tile of pivot pairs (91 tiles of the upper triangle at k = 100) in 64
+// registers pairs: per node 4 loads of 16 bytes and 64 multiply-adds of 32 x 32
+// bits, which bound it (0.9 ms for 512 graphs of 64 to 8192 nodes, 5 G
+// products).  A unit's sums (512 products below 2^55) are exact in
+// 64 bits; their 32-bit halves are added to the graph's sums by atomics, whole
+// numbers, so the order does not show.
+constexpr int kGramNodes = 512, kGramStage = 32, kGramThreads = 96, kGramLd = (kPrepMaxK + 7) / 8 * 8;
+__global__ void __launch_bounds__(kGramThreads) k_prep_gram(LayoutArgs L) {
+  __shared__ __align__(16) uint32_t st[kGramStage][kGramLd];
+  // this block's graph: the last place in the order whose tasks start here or before
+  int lo = 0, hi = L.G;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (L.task0[mid] <= (int)blockIdx.x) lo = mid; else hi = mid;
+  }
+  const LayoutDev D = L.desc[L.order[lo]];
+  const int n = D.n, k = D.k, T = (k + 7) / 8, k8 = 8 * T;
+  const int n0 = ((int)blockIdx.x - L.task0[lo]) * kGramNodes, n1 = min(n, n0 + kGramNodes);
+  const uint16_t *dip = L.dip + D.dip_off;
+  unsigned long long *sums = L.gram + D.gram_off;
+  int ta = -1, tb = 0;
+  if ((int)threadIdx.x < T * (T + 1) / 2) {
+    int p = threadIdx.x;
+    for (ta = 0; p >= T - ta; ++ta) p -= T - ta;
+    tb = ta + p;
+  }
+  unsigned long long acc[8][8];
+#pragma unroll
+  for (int x = 0; x < 8; ++x)
+#pragma unroll
+    for (int y = 0; y < 8; ++y) acc[x][y] = 0ull;
+  unsigned long long cs[(kGramLd + kGramThreads - 1) / kGramThreads] = {};
+  for (int i0 = n0; i0 < n1; i0 += kGramStage) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < k8 * kGramStage; e += kGramThreads) {
+      const int a = e / kGramStage, t = e % kGramStage;
+      const uint32_t d = a < k && i0 + t < n1 ? dip[(int64_t)a * n + i0 + t] : 0u;
+      st[t][a] = d * d;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < (kGramLd + kGramThreads - 1) / kGramThreads; ++q) {
+      const int a = threadIdx.x + q * kGramThreads;
+      if (a < k8)
+        for (int t = 0; t < kGramStage; ++t) cs[q] += st[t][a];
+    }
+    if (ta < 0) continue;
+#pragma unroll 1
+    for (int t = 0; t < kGramStage; ++t) {
+      uint32_t va[8], vb[8];
+      *reinterpret_cast<uint4 *>(va) = *reinterpret_cast<const uint4 *>(&st[t][8 * ta]);
+      *reinterpret_cast<uint4 *>(va + 4) = *reinterpret_cast<const uint4 *>(&st[t][8 * ta + 4]);
+      *reinterpret_cast<uint4 *>(vb) = *reinterpret_cast<const uint4 *>(&st[t][8 * tb]);
+      *reinterpret_cast<uint4 *>(vb + 4) = *reinterpret_cast<const uint4 *>(&st[t][8 * tb + 4]);
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+#pragma unroll
+        for (int y = 0; y < 8; ++y) acc[x][y] += (unsigned long long)va[x] * vb[y];
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < (kGramLd + kGramThreads - 1) / kGramThreads; ++q) {
+    const int a = threadIdx.x + q * kGramThreads;
+    if (a < k) atomicAdd(sums + a, cs[q]);
+  }
+  if (ta < 0) return;
+#pragma unroll
+  for (int x = 0; x < 8; ++x)
+#pragma unroll
+    for (int y = 0; y < 8; ++y) {
+      const int a = 8 * ta + x, b = 8 * tb + y;
+      if (a > b || b >= k) continue;
+      unsigned long long *o = sums + k + 2 * ((int64_t)a * k + b);
+      atomicAdd(o, acc[x][y] & 0xFFFFFFFFull);
+      if (acc[x][y] >> 32) atomicAdd(o + 1, acc[x][y] >> 32);
+    }
+}
 
 // fixed-order block sum of one double per thread
 __device__ double block_sum_d(double v, double *s_red) {
@@ -401,23 +486,48 @@ __device__ double block_sum_d(double v, double *s_red) {
   __syncthreads();
   return t;
 }
+__device__ __forceinline__ double warp_sum_d(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
 
-__global__ void __launch_bounds__(kPrepThreads) k_prep_layout(LayoutArgs L) {
+// 1 / sqrt(s) for a normal s > 0, from FP32's reciprocal square root by two
+// Newton steps (2^-22 -> 2^-43 -> FP64 rounding); the exponent is halved apart
+__device__ __forceinline__ double rsqrt_newton(double s) {
+  const int h = (__double2hiint(s) >> 21) - 511;  // half the exponent (of 2^0: 0)
+  const double t = __hiloint2double(__double2hiint(s) - (h << 21), __double2loint(s));  // in [1/2, 2)
+  double y = (double)rsqrtf((float)t);
+  y = fma(0.5 * y, fma(-t * y, y, 1.0), y);
+  y = fma(0.5 * y, fma(-t * y, y, 1.0), y);
+  return __hiloint2double(__double2hiint(y) - (h << 20), __double2loint(y));
+}
+
+// PivotMDS and the rescale of one graph per block.  FP64 runs at a 64th of
+// FP32's rate here and a dependent step takes 60 cycles or more, so the
+// eigen-solve is a chain of FP64 latencies: the matrix holds the reflectors
+// in the rows it no longer needs (81 KB, two blocks per SM fill each other's
+// gaps), only a triangle is updated, four threads share a row of a product,
+// square roots are two Newton steps, loops over k are a warp's, and the node
+// loop of the projection is integer arithmetic.  2.5 ms for 512 graphs of 64 to
+// 8192 nodes, k = 100 (with the Gram and an FP64 projection in the block, one
+// block per SM and single-thread loops over k: 6.5 ms).
+constexpr int kLayLd = kPrepMaxK + 1;  // odd: columns and rows without bank conflicts
+__global__ void __launch_bounds__(kPrepThreads, 2) k_prep_layout(LayoutArgs L) {
   extern __shared__ __align__(16) unsigned char lsm[];
-  double *Am = reinterpret_cast<double *>(lsm);              // [kPrepMaxK^2]
-  double *V = Am + kPrepMaxK * kPrepMaxK;                     // [kPrepMaxK^2]
-  uint32_t *chunk = reinterpret_cast<uint32_t *>(V + kPrepMaxK * kPrepMaxK);  // [kPrepChunk][kPrepMaxK]
+  double *Am = reinterpret_cast<double *>(lsm);  // [kPrepMaxK][kLayLd]
   __shared__ double s_red[kPrepThreads / 32];
-  __shared__ unsigned long long s_col[kPrepMaxK];
-  __shared__ double s_rm[kPrepMaxK], s_v[2][kPrepMaxK];
+  __shared__ double s_rm[kPrepMaxK], s_gm;
   __shared__ int s_off[kPrepMaxK + 1];
-  __shared__ double s_dg[kPrepMaxK], s_e[kPrepMaxK], s_p[kPrepMaxK], s_w[kPrepMaxK], s_lam[2];
+  __shared__ double s_dg[kPrepMaxK], s_e[kPrepMaxK], s_p[4][kPrepMaxK], s_w[kPrepMaxK], s_lam[2];
   __shared__ double s_y[2][kPrepMaxK], s_fd[2][kPrepMaxK], s_fu[2][kPrepMaxK], s_fu2[2][kPrepMaxK], s_fl[2][kPrepMaxK];
   __shared__ double s_e2[kPrepMaxK];
   __shared__ int s_piv[2][kPrepMaxK];
-  __shared__ int s_task, s_big[2];
+  __shared__ int s_task;
   __shared__ double s_sig[2], s_kap[2];
+  __shared__ int4 s_fix[kPrepMaxK];  // (low, high) parts of an eigenvector pair's entries in fixed point
   __shared__ int s_done;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int kWarps = kPrepThreads / 32;
   for (;;) {
     if (threadIdx.x == 0) s_task = (int)atomicAdd(L.ctr, 1u);
     __syncthreads();
@@ -456,139 +566,111 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_layout(LayoutArgs L) {
         cnt[t] = acc;
       }
     }
-    // ---- exact Gram G = Delta^T Delta (upper triangle, 128-bit) and s_a
-    const int npairs = k * (k + 1) / 2;
-    constexpr int kPairsPerThread = (kPrepMaxK * (kPrepMaxK + 1) / 2 + kPrepThreads - 1) / kPrepThreads;
-    unsigned __int128 acc[kPairsPerThread];
-    int pa[kPairsPerThread], pb[kPairsPerThread];
-#pragma unroll
-    for (int j = 0; j < kPairsPerThread; ++j) {
-      acc[j] = 0;
-      int p = threadIdx.x + j * blockDim.x;
-      int a = 0;
-      if (p < npairs) {
-        while (p >= k - a) {
-          p -= k - a;
-          ++a;
-        }
-        pa[j] = a;
-        pb[j] = a + p;
-      } else {
-        pa[j] = -1;
-        pb[j] = -1;
-      }
-    }
-    unsigned long long colsum = 0;
-    for (int i0 = 0; i0 < n; i0 += kPrepChunk) {
-      __syncthreads();
-      for (int e = threadIdx.x; e < kPrepChunk * k; e += blockDim.x) {
-        const int a = e / kPrepChunk, t = e % kPrepChunk;
-        const int i = i0 + t;
-        const uint32_t d = i < n ? dip[(int64_t)a * n + i] : 0u;
-        chunk[t * kPrepMaxK + a] = d * d;
-      }
-      __syncthreads();
-      if (threadIdx.x < k)
-        for (int t = 0; t < kPrepChunk; ++t) colsum += chunk[t * kPrepMaxK + threadIdx.x];
-#pragma unroll
-      for (int j = 0; j < kPairsPerThread; ++j) {
-        if (pa[j] < 0) continue;
-        const int a = pa[j], b = pb[j];
-        // a chunk's 32 products (each below 2^52) sum exactly in 64 bits;
-        // the chunk sums go into the 128-bit total
-        unsigned long long cs = 0;
-        for (int t = 0; t < kPrepChunk; ++t)
-          cs += (unsigned long long)chunk[t * kPrepMaxK + a] * (unsigned long long)chunk[t * kPrepMaxK + b];
-        acc[j] += cs;
-      }
-    }
-    if (threadIdx.x < k) s_col[threadIdx.x] = colsum;
-    __syncthreads();
     // B = G - s s^T / n, then 1/4 J B J
+    const unsigned long long *col = L.gram + D.gram_off, *pairs = col + k;
     const double inv_n = 1.0 / (double)n;
-    const double two64 = 18446744073709551616.0;
-#pragma unroll
-    for (int j = 0; j < kPairsPerThread; ++j) {
-      if (pa[j] < 0) continue;
-      const int a = pa[j], b = pb[j];
-      const double g = (double)(unsigned long long)(acc[j] >> 64) * two64 + (double)(unsigned long long)acc[j];
-      const double v = g - ((double)s_col[a] * (double)s_col[b]) * inv_n;
-      Am[a * kPrepMaxK + b] = v;
-      Am[b * kPrepMaxK + a] = v;
-    }
-    __syncthreads();
-    for (int a = threadIdx.x; a < k; a += blockDim.x) {
-      double r = 0.0;
-      for (int b = 0; b < k; ++b) r += Am[a * kPrepMaxK + b];
-      s_rm[a] = r / (double)k;
-    }
-    __syncthreads();
-    double gm = 0.0;
-    for (int a = 0; a < k; ++a) gm += s_rm[a];
-    gm /= (double)k;
-    for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
+    for (int e = threadIdx.x; e < k * k; e += kPrepThreads) {
       const int a = e / k, b = e % k;
-      Am[a * kPrepMaxK + b] = 0.25 * (Am[a * kPrepMaxK + b] - s_rm[a] - s_rm[b] + gm);
-      V[a * kPrepMaxK + b] = a == b ? 1.0 : 0.0;
+      if (a > b) continue;
+      const unsigned long long plo = pairs[2 * e], phi = pairs[2 * e + 1];
+      const unsigned __int128 g128 = ((unsigned __int128)phi << 32) + plo;
+      const double g = (double)(unsigned long long)(g128 >> 64) * 18446744073709551616.0 + (double)(unsigned long long)g128;
+      const double v = g - ((double)col[a] * (double)col[b]) * inv_n;
+      Am[a * kLayLd + b] = v;
+      Am[b * kLayLd + a] = v;
+    }
+    __syncthreads();
+    for (int a = warp; a < k; a += kWarps) {
+      double r = 0.0;
+      for (int b = lane; b < k; b += 32) r += Am[a * kLayLd + b];
+      r = warp_sum_d(r);
+      if (lane == 0) s_rm[a] = r / (double)k;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      double g = 0.0;
+      for (int a = lane; a < k; a += 32) g += s_rm[a];
+      g = warp_sum_d(g);
+      if (lane == 0) s_gm = g / (double)k;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < k * k; e += kPrepThreads) {
+      const int a = e / k, b = e % k;
+      if (a > b) continue;
+      const double v = 0.25 * (Am[a * kLayLd + b] - s_rm[a] - s_rm[b] + s_gm);
+      Am[a * kLayLd + b] = v;
+      Am[b * kLayLd + a] = v;
     }
     __syncthreads();
     // ---- top-2 eigenpairs: Householder reduction of B to a tridiagonal T
-    // (Q^T B Q = T, reflector vectors kept in V), the two largest
-    // eigenvalues of T by Sturm-count bisection, their eigenvectors by
-    // inverse iteration on T, and back through the reflectors
-    double *Hv = V;  // row j: the unit reflector of step j (entries j+1 .. k-1)
+    // (Q^T B Q = T; row j keeps the unit reflector of step j in its entries
+    // j + 1 .. k - 1), the two largest eigenvalues of T by Sturm-count
+    // bisection, their eigenvectors by inverse iteration on T, and back
+    // through the reflectors
     for (int j = 0; j + 2 < k; ++j) {
-      // warp 0: the reflector of column j (norm by shuffles)
-      if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
+      double *hv = Am + j * kLayLd;
+      if (warp == 0) {  // the reflector of row j (the matrix is symmetric)
         double sig = 0.0;
-        for (int r = j + 2 + lane; r < k; r += 32) sig += Am[r * kPrepMaxK + j] * Am[r * kPrepMaxK + j];
-        for (int o = 16; o > 0; o >>= 1) sig += __shfl_xor_sync(0xffffffffu, sig, o);
-        const double x0 = Am[(j + 1) * kPrepMaxK + j];
-        if (sig == 0.0) {  // the column is already tridiagonal: H = I
-          for (int r = lane; r < k; r += 32) Hv[j * kPrepMaxK + r] = 0.0;
-          if (lane == 0) s_e[j] = x0;
-        } else {
-          const double nrm = sqrt(x0 * x0 + sig);
-          const double alpha = x0 >= 0.0 ? -nrm : nrm;
-          const double v0 = x0 - alpha;
-          const double vinv = 1.0 / sqrt(v0 * v0 + sig);
-          for (int r = lane; r < k; r += 32)
-            Hv[j * kPrepMaxK + r] = r <= j ? 0.0 : (r == j + 1 ? v0 : Am[r * kPrepMaxK + j]) * vinv;
-          if (lane == 0) s_e[j] = alpha;
+        for (int r = j + 2 + lane; r < k; r += 32) sig = fma(hv[r], hv[r], sig);
+        sig = warp_sum_d(sig);
+        const double x0 = hv[j + 1];
+        // a row that is tridiagonal already (or whose square vanishes): H = I
+        const bool none = !(sig >= 1e-290);
+        double v0 = 0.0, vinv = 0.0, e = x0;
+        if (!none) {
+          const double s2 = fma(x0, x0, sig);
+          const double nrm = s2 * rsqrt_newton(s2);
+          e = x0 >= 0.0 ? -nrm : nrm;
+          v0 = x0 - e;
+          vinv = rsqrt_newton(fma(v0, v0, sig));
         }
+        __syncwarp();
+        for (int r = j + 1 + lane; r < k; r += 32) hv[r] = (r == j + 1 ? v0 : hv[r]) * vinv;
+        if (lane == 0) s_e[j] = e;
       }
       __syncthreads();
-      const double *hv = Hv + j * kPrepMaxK;
       if (hv[j + 1] == 0.0) continue;  // H = I (the same decision in every thread)
-      // p = A v over the trailing block (read down the columns: A is
-      // symmetric and consecutive threads then touch consecutive words)
-      for (int r = j + 1 + threadIdx.x; r < k; r += blockDim.x) {
+      // p = A v over the trailing block, a quarter of the sum per thread
+      for (int r = j + 1 + (threadIdx.x & 127); r < k; r += 128) {
         double t = 0.0;
-        for (int c = j + 1; c < k; ++c) t += Am[c * kPrepMaxK + r] * hv[c];
-        s_p[r] = t;
+        for (int c = j + 1 + (threadIdx.x >> 7); c < k; c += kPrepThreads / 128) t = fma(Am[c * kLayLd + r], hv[c], t);
+        s_p[threadIdx.x >> 7][r] = t;
       }
       __syncthreads();
       // warp 0: K = v . p, w = 2 (p - K v)
-      if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
-        double kk = 0.0;
-        for (int r = j + 1 + lane; r < k; r += 32) kk += hv[r] * s_p[r];
-        for (int o = 16; o > 0; o >>= 1) kk += __shfl_xor_sync(0xffffffffu, kk, o);
-        for (int r = j + 1 + lane; r < k; r += 32) s_w[r] = 2.0 * (s_p[r] - kk * hv[r]);
+      if (warp == 0) {
+        double kk = 0.0, p[(kPrepMaxK + 31) / 32];
+#pragma unroll
+        for (int q = 0; q < (kPrepMaxK + 31) / 32; ++q) {
+          const int r = j + 1 + lane + 32 * q;
+          p[q] = r < k ? (s_p[0][r] + s_p[1][r]) + (s_p[2][r] + s_p[3][r]) : 0.0;
+          if (r < k) kk = fma(hv[r], p[q], kk);
+        }
+        kk = warp_sum_d(kk);
+#pragma unroll
+        for (int q = 0; q < (kPrepMaxK + 31) / 32; ++q) {
+          const int r = j + 1 + lane + 32 * q;
+          if (r < k) s_w[r] = 2.0 * fma(-kk, hv[r], p[q]);
+        }
       }
       __syncthreads();
-      const int L = k - j - 1;
-      for (int e2 = threadIdx.x; e2 < L * L; e2 += blockDim.x) {
-        const int r = j + 1 + e2 / L, c = j + 1 + e2 % L;
-        Am[r * kPrepMaxK + c] -= hv[r] * s_w[c] + s_w[r] * hv[c];
-      }
+      // A -= v w^T + w v^T, the lower triangle and its mirror image: a warp
+      // takes a short and a long row
+      const int M = k - j - 1;
+      for (int h = warp; 2 * h < M; h += kWarps)
+        for (int side = 0; side < (2 * h == M - 1 ? 1 : 2); ++side) {
+          const int r = j + 1 + (side == 0 ? h : M - 1 - h);
+          const double vr = hv[r], wr = s_w[r];
+          for (int c = j + 1 + lane; c <= r; c += 32) {
+            const double v = fma(-wr, hv[c], fma(-vr, s_w[c], Am[r * kLayLd + c]));
+            Am[r * kLayLd + c] = v;
+            Am[c * kLayLd + r] = v;
+          }
+        }
       __syncthreads();
     }
-    if (threadIdx.x == 0) {
-      for (int a = 0; a < k; ++a) s_dg[a] = Am[a * kPrepMaxK + a];
-      if (k >= 2) s_e[k - 2] = Am[(k - 1) * kPrepMaxK + (k - 2)];
-    }
+    for (int a = threadIdx.x; a < k; a += kPrepThreads) s_dg[a] = Am[a * kLayLd + a];
+    if (threadIdx.x == 0) s_e[k - 2] = Am[(k - 1) * kLayLd + (k - 2)];
     __syncthreads();
     // eigenvalues number k-1 and k-2 (ascending) by bisection on Sturm counts,
     // 32 points per step evaluated by the lanes of warp 0 (the largest) and
@@ -615,15 +697,15 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_layout(LayoutArgs L) {
         cnt += q < 0.0;
         for (int a = 1; a < k; ++a) {
           double r;
-          const double aq = fabs(q);
-          if (aq > 1e-30 && aq < 1e30) {
+          const unsigned aq = (unsigned)__double2hiint(q) & 0x7FFFFFFFu;
+          if (aq - 0x39B00000u < 0x0C900000u) {  // 2^-100 <= |q| < 2^101
             const double r0 = (double)__frcp_rn((float)q);
             r = r0 * fma(-q, r0, 2.0);
           } else {
             r = 1.0 / (q == 0.0 ? 1e-300 : q);
           }
           q = fma(-s_e2[a - 1], r, s_dg[a] - x);
-          cnt += q < 0.0;
+          cnt += (unsigned)__double2hiint(q) >> 31;  // its sign (no q here is -0)
         }
         // the smallest lane point with more than idx eigenvalues below it
         const unsigned above = __ballot_sync(0xffffffffu, cnt > idx);
@@ -637,147 +719,180 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_layout(LayoutArgs L) {
     }
     __syncthreads();
     // inverse iteration on T - lambda I (tridiagonal LU with partial
-    // pivoting, factored once, two solves), one thread per eigenvalue; the
-    // second vector is then made orthogonal to the first
-    if (threadIdx.x == 0 || threadIdx.x == 32) {
-      const int want = threadIdx.x >> 5;
+    // pivoting, factored once, two solves), one warp per eigenvalue (the
+    // recurrences on its first lane); the second vector is then made
+    // orthogonal to the first
+    if (warp < 2) {
+      const int want = warp;
       double *y = s_y[want];
       double *dd = s_fd[want], *du = s_fu[want], *du2 = s_fu2[want], *dl = s_fl[want];
       int *piv = s_piv[want];
       const double lam = s_lam[want];
       const double pert = 1e-14 * (fabs(lam) + 1e-300);
-      for (int a = 0; a < k; ++a) {
+      for (int a = lane; a < k; a += 32) {
         y[a] = 1.0 + 0.01 * (double)((a * 37) % 11);
         dd[a] = s_dg[a] - lam;
         du[a] = a + 1 < k ? s_e[a] : 0.0;
         dl[a] = a + 1 < k ? s_e[a] : 0.0;
         du2[a] = 0.0;
       }
-      for (int a = 0; a + 1 < k; ++a) {
-        if (fabs(dd[a]) >= fabs(dl[a])) {
-          if (dd[a] == 0.0) dd[a] = pert;
-          const double f = dl[a] / dd[a];
-          dl[a] = f;
-          dd[a + 1] -= f * du[a];
-          piv[a] = 0;
-        } else {
-          const double f = dd[a] / dl[a];
-          dd[a] = dl[a];
-          dl[a] = f;
-          const double t = du[a];
-          du[a] = dd[a + 1];
-          dd[a + 1] = t - f * dd[a + 1];
-          if (a + 2 < k) {
-            du2[a] = du[a + 1];
-            du[a + 1] = -f * du[a + 1];
-          }
-          piv[a] = 1;
-        }
-      }
-      if (dd[k - 1] == 0.0) dd[k - 1] = pert;
-      for (int a = 0; a < k; ++a) dd[a] = 1.0 / dd[a];  // reciprocals for the solves
-      for (int it = 0; it < 2; ++it) {
+      __syncwarp();
+      if (lane == 0) {
         for (int a = 0; a + 1 < k; ++a) {
-          if (piv[a] == 0) {
-            y[a + 1] -= dl[a] * y[a];
+          if (fabs(dd[a]) >= fabs(dl[a])) {
+            if (dd[a] == 0.0) dd[a] = pert;
+            const double f = dl[a] / dd[a];
+            dl[a] = f;
+            dd[a + 1] -= f * du[a];
+            piv[a] = 0;
           } else {
-            const double t = y[a];
-            y[a] = y[a + 1];
-            y[a + 1] = t - dl[a] * y[a];
+            const double f = dd[a] / dl[a];
+            dd[a] = dl[a];
+            dl[a] = f;
+            const double t = du[a];
+            du[a] = dd[a + 1];
+            dd[a + 1] = t - f * dd[a + 1];
+            if (a + 2 < k) {
+              du2[a] = du[a + 1];
+              du[a + 1] = -f * du[a + 1];
+            }
+            piv[a] = 1;
           }
         }
-        y[k - 1] *= dd[k - 1];
-        if (k >= 2) y[k - 2] = (y[k - 2] - du[k - 2] * y[k - 1]) * dd[k - 2];
-        for (int a = k - 3; a >= 0; --a) y[a] = (y[a] - du[a] * y[a + 1] - du2[a] * y[a + 2]) * dd[a];
+        if (dd[k - 1] == 0.0) dd[k - 1] = pert;
+      }
+      __syncwarp();
+      for (int a = lane; a < k; a += 32) dd[a] = 1.0 / dd[a];  // reciprocals for the solves
+      __syncwarp();
+      for (int it = 0; it < 2; ++it) {
+        if (lane == 0) {
+          double ya = y[0];
+          for (int a = 0; a + 1 < k; ++a) {
+            const double yb = y[a + 1];
+            if (piv[a] == 0) {
+              y[a] = ya;
+              ya = fma(-dl[a], ya, yb);
+            } else {
+              y[a] = yb;
+              ya = fma(-dl[a], yb, ya);
+            }
+          }
+          double y1 = ya * dd[k - 1], y2 = 0.0;
+          y[k - 1] = y1;
+          for (int a = k - 2; a >= 0; --a) {
+            const double t = fma(-du[a], y1, fma(-du2[a], y2, y[a])) * dd[a];
+            y2 = y1;
+            y1 = t;
+            y[a] = t;
+          }
+        }
+        __syncwarp();
         double nr = 0.0;
-        for (int a = 0; a < k; ++a) nr += y[a] * y[a];
+        for (int a = lane; a < k; a += 32) nr = fma(y[a], y[a], nr);
+        nr = warp_sum_d(nr);
         nr = nr > 0.0 ? 1.0 / sqrt(nr) : 0.0;
-        for (int a = 0; a < k; ++a) y[a] *= nr;
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double dt = 0.0;
-      for (int a = 0; a < k; ++a) dt += s_y[1][a] * s_y[0][a];
-      double nr = 0.0;
-      for (int a = 0; a < k; ++a) {
-        s_y[1][a] -= dt * s_y[0][a];
-        nr += s_y[1][a] * s_y[1][a];
-      }
-      nr = nr > 0.0 ? 1.0 / sqrt(nr) : 0.0;
-      for (int a = 0; a < k; ++a) s_y[1][a] *= nr;
-      s_done = s_lam[0] > 0.0;
-      if (L.eig) {
-        L.eig[2 * gi] = s_lam[0];
-        L.eig[2 * gi + 1] = s_lam[1];
-      }
-    }
-    __syncthreads();
-    // z = H_0 H_1 ... H_{k-3} y, the reflectors applied last to first (one
-    // warp: k <= 100 entries, dot products by shuffles, no block barrier)
-    if (threadIdx.x < 32) {
-      const int lane = threadIdx.x;
-      for (int j = k - 3; j >= 0; --j) {
-        const double *hv = Hv + j * kPrepMaxK;
-        double d0 = 0.0, d1 = 0.0;
-        for (int r = j + 1 + lane; r < k; r += 32) {
-          d0 += hv[r] * s_y[0][r];
-          d1 += hv[r] * s_y[1][r];
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          d0 += __shfl_xor_sync(0xffffffffu, d0, o);
-          d1 += __shfl_xor_sync(0xffffffffu, d1, o);
-        }
-        for (int r = j + 1 + lane; r < k; r += 32) {
-          s_y[0][r] -= 2.0 * d0 * hv[r];
-          s_y[1][r] -= 2.0 * d1 * hv[r];
-        }
+        for (int a = lane; a < k; a += 32) y[a] *= nr;
         __syncwarp();
       }
     }
     __syncthreads();
-    if (!s_done) dev_fail(L.status, SSM_E_NUMERIC);
-    // each vector signed so that its largest-magnitude entry (lowest index on a tie) is positive
-    if (threadIdx.x == 0)
-      for (int r = 0; r < 2; ++r) {
-        int big = 0;
-        for (int a = 1; a < k; ++a)
-          if (fabs(s_y[r][a]) > fabs(s_y[r][big])) big = a;
-        s_big[r] = big;
+    if (warp == 0) {
+      double dt = 0.0, nr = 0.0;
+      for (int a = lane; a < k; a += 32) dt = fma(s_y[1][a], s_y[0][a], dt);
+      dt = warp_sum_d(dt);
+      for (int a = lane; a < k; a += 32) {
+        s_y[1][a] = fma(-dt, s_y[0][a], s_y[1][a]);
+        nr = fma(s_y[1][a], s_y[1][a], nr);
       }
-    __syncthreads();
-    for (int a = threadIdx.x; a < k; a += blockDim.x)
-      for (int r = 0; r < 2; ++r) s_v[r][a] = (s_y[r][s_big[r]] < 0 ? -1.0 : 1.0) * s_y[r][a];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double sg0 = 0.0, sg1 = 0.0, cv0 = 0.0, cv1 = 0.0, cb = 0.0;
-      for (int a = 0; a < k; ++a) {
-        const double cbar = (double)s_col[a] * inv_n;
-        sg0 += s_v[0][a];
-        sg1 += s_v[1][a];
-        cv0 += cbar * s_v[0][a];
-        cv1 += cbar * s_v[1][a];
-        cb += cbar;
+      nr = warp_sum_d(nr);
+      nr = nr > 0.0 ? 1.0 / sqrt(nr) : 0.0;
+      for (int a = lane; a < k; a += 32) s_y[1][a] *= nr;
+      if (lane == 0) {
+        s_done = s_lam[0] > 0.0;
+        if (L.eig) {
+          L.eig[2 * gi] = s_lam[0];
+          L.eig[2 * gi + 1] = s_lam[1];
+        }
       }
-      const double gbar = cb / (double)k;
-      s_sig[0] = sg0;
-      s_sig[1] = sg1;
-      s_kap[0] = cv0 - gbar * sg0;
-      s_kap[1] = cv1 - gbar * sg1;
     }
     __syncthreads();
-    // ---- x_i = -1/2 (sum_a d_ia^2 v_a - rbar_i sigma - kappa), FP64
-    float2 *pos = L.pos + D.node_off;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      double x = 0.0, y = 0.0, rs = 0.0;
-      for (int a = 0; a < k; ++a) {
-        const double d = (double)dip[(int64_t)a * n + i];
-        const double dd = d * d;
-        rs += dd;
-        x += dd * s_v[0][a];
-        y += dd * s_v[1][a];
+    // z = H_0 H_1 ... H_{k-3} y, the reflectors applied last to first, a warp
+    // per vector; each is then signed so that its largest-magnitude entry
+    // (lowest index on a tie) is positive
+    if (warp < 2) {
+      double *y = s_y[warp];
+      for (int j = k - 3; j >= 0; --j) {
+        const double *hv = Am + j * kLayLd;
+        double dt = 0.0;
+        for (int r = j + 1 + lane; r < k; r += 32) dt = fma(hv[r], y[r], dt);
+        dt = -2.0 * warp_sum_d(dt);
+        for (int r = j + 1 + lane; r < k; r += 32) y[r] = fma(dt, hv[r], y[r]);
+        __syncwarp();
       }
-      const double rbar = rs / (double)k;
+      double big = -1.0;
+      int at = 0;
+      for (int a = lane; a < k; a += 32)
+        if (fabs(y[a]) > big) {
+          big = fabs(y[a]);
+          at = a;
+        }
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, big, o);
+        const int oa = __shfl_xor_sync(0xffffffffu, at, o);
+        if (ob > big || (ob == big && oa < at)) {
+          big = ob;
+          at = oa;
+        }
+      }
+      const double sgn = y[at] < 0 ? -1.0 : 1.0;
+      __syncwarp();
+      // fixed point for the node loop: round(v 2^54) = high 2^27 + low, |v| <= 1
+      // (a NaN or an infinity, of a matrix that was none, fails the batch)
+      double sg = 0.0, cv = 0.0, cb = 0.0;
+      bool bad = false;
+      for (int a = lane; a < k; a += 32) {
+        const double v = sgn * y[a], cbar = (double)col[a] * inv_n;
+        y[a] = v;
+        sg += v;
+        cv = fma(cbar, v, cv);
+        cb += cbar;
+        bad |= !(fabs(v) <= 1.0 + 1e-9);
+        const long long f = __double2ll_rn(v * 18014398509481984.0);
+        int *o = reinterpret_cast<int *>(s_fix + a) + 2 * warp;
+        o[0] = (int)(f & 0x7FFFFFF);
+        o[1] = (int)(f >> 27);
+      }
+      sg = warp_sum_d(sg);
+      cv = warp_sum_d(cv);
+      cb = warp_sum_d(cb);
+      if (__any_sync(0xffffffffu, bad) && lane == 0) dev_fail(L.status, SSM_E_NUMERIC);
+      if (lane == 0) {
+        s_sig[warp] = sg;
+        s_kap[warp] = cv - cb / (double)k * sg;
+      }
+    }
+    __syncthreads();
+    if (!s_done) dev_fail(L.status, SSM_E_NUMERIC);
+    // ---- x_i = -1/2 (sum_a d_ia^2 v_a - rbar_i sigma - kappa): whole
+    // numbers, exact (d^2 < 2^28, 100 terms: below 2^63), then FP64
+    float2 *pos = L.pos + D.node_off;
+    for (int i = threadIdx.x; i < n; i += kPrepThreads) {
+      long long xl = 0, xh = 0, yl = 0, yh = 0;
+      unsigned long long rs = 0;
+#pragma unroll 4
+      for (int a = 0; a < k; ++a) {
+        const int d = (int)dip[(int64_t)a * n + i];
+        const int dd = d * d;
+        const int4 f = s_fix[a];
+        rs += (unsigned)dd;
+        xl += (long long)dd * f.x;
+        xh += (long long)dd * f.y;
+        yl += (long long)dd * f.z;
+        yh += (long long)dd * f.w;
+      }
+      const double x = fma((double)xh, 134217728.0, (double)xl) * 0x1p-54;
+      const double y = fma((double)yh, 134217728.0, (double)yl) * 0x1p-54;
+      const double rbar = (double)rs / (double)k;
       pos[i] = make_float2((float)(-0.5 * (x - rbar * s_sig[0] - s_kap[0])),
                            (float)(-0.5 * (y - rbar * s_sig[1] - s_kap[1])));
     }
@@ -815,16 +930,20 @@ struct PrepWs {
   LayoutDev *ld;
   int32_t *order;
   unsigned *ctr;  // [3]
+  int32_t *task0;  // [G + 1]
+  unsigned long long *gram;
   int64_t *lens;  // [2 G]: table lengths, then edge counts
   int32_t *tmp;
 };
 
-// cap < 0: the prefix only (what the layout call uses)
-static void carve_prep(Carver &c, PrepWs &w, int32_t G, int64_t cap) {
+// gram: words of the Gram sums; cap < 0: the prefix only (what the layout call uses)
+static void carve_prep(Carver &c, PrepWs &w, int32_t G, int64_t gram, int64_t cap) {
   w.pd = c.take<PrepDev>((size_t)G);
   w.ld = c.take<LayoutDev>((size_t)G);
   w.order = c.take<int32_t>((size_t)G);
   w.ctr = c.take<unsigned>(3);
+  w.task0 = c.take<int32_t>((size_t)G + 1);
+  w.gram = c.take<unsigned long long>((size_t)gram);
   w.lens = c.take<int64_t>(2 * (size_t)G);
   w.tmp = cap >= 0 ? c.take<int32_t>((size_t)std::max<int64_t>(cap, 1)) : nullptr;
 }
@@ -841,20 +960,21 @@ static void prep_smem(int32_t G, const ssm_batch_input *in, int64_t &pivots, int
   }
 }
 
-static size_t layout_smem() {
-  return 2 * (size_t)kPrepMaxK * kPrepMaxK * sizeof(double) + (size_t)kPrepChunk * kPrepMaxK * sizeof(uint32_t);
-}
+static size_t layout_smem() { return (size_t)kPrepMaxK * kLayLd * sizeof(double); }
 
 }  // namespace ssm
 
 // =========================================================== C ABI
 SSM_API size_t ssm_batch_prepare_workspace(int32_t G, const ssm_batch_input *in) {
   if (G < 1 || !in) return 0;
-  int64_t cap = 0;
-  for (int32_t g = 0; g < G; ++g) cap += 2 * std::max<int64_t>(0, in[g].m_in);
+  int64_t cap = 0, gram = 0;
+  for (int32_t g = 0; g < G; ++g) {
+    cap += 2 * std::max<int64_t>(0, in[g].m_in);
+    gram += ssm::gram_words(std::max(in[g].k, 0));
+  }
   ssm::Carver c(nullptr, 0);
   ssm::PrepWs w;
-  ssm::carve_prep(c, w, G, cap);
+  ssm::carve_prep(c, w, G, gram, cap);
   return c.size();
 }
 
@@ -867,7 +987,7 @@ SSM_API int ssm_batch_pivots(int32_t G, const ssm_batch_input *in, const int32_t
     return fail(SSM_E_ARG, "ssm_batch_pivots: null pointer or G < 1");
   std::vector<PrepDev> pd((size_t)G);
   std::vector<int32_t> order((size_t)G);
-  int64_t node = 0, row = 0, col = 0, piv = 0, dipo = 0, offo = 0, edges = 0;
+  int64_t node = 0, row = 0, col = 0, piv = 0, dipo = 0, offo = 0, edges = 0, gram = 0;
   for (int32_t g = 0; g < G; ++g) {
     const ssm_batch_input &x = in[g];
     if (x.n < 1 || x.n > kPrepMaxN) return fail(SSM_E_ARG, "ssm_batch_pivots: graph %d has n = %d (1..%d)", g, x.n, kPrepMaxN);
@@ -884,6 +1004,7 @@ SSM_API int ssm_batch_pivots(int32_t G, const ssm_batch_input *in, const int32_t
     o.cnt_base = 0;
     node += x.n; row += x.n + 1; col += 2 * x.m_in; piv += x.k; dipo += (int64_t)x.k * x.n; offo += x.k + 1;
     edges = std::max(edges, x.edge_off + x.m_in);
+    gram += gram_words(x.k);
     order[(size_t)g] = g;
   }
   std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
@@ -891,7 +1012,7 @@ SSM_API int ssm_batch_pivots(int32_t G, const ssm_batch_input *in, const int32_t
   });
   Carver c(ws, ws_bytes);
   PrepWs w;
-  carve_prep(c, w, G, col);
+  carve_prep(c, w, G, gram, col);
   if (!c.ok) return fail(SSM_E_NOMEM, "ssm_batch_pivots: workspace %zu bytes, need %zu", ws_bytes, c.size());
   SSM_TRY_CUDA(cudaMemcpyAsync(w.pd, pd.data(), pd.size() * sizeof(PrepDev), cudaMemcpyHostToDevice, s));
   SSM_TRY_CUDA(cudaMemcpyAsync(w.order, order.data(), order.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
@@ -940,7 +1061,8 @@ SSM_API int ssm_batch_layout_init(int32_t G, const ssm_batch_graph *graphs, cons
       !status || !ws)
     return fail(SSM_E_ARG, "ssm_batch_layout_init: null pointer or G < 1");
   std::vector<LayoutDev> ld((size_t)G);
-  std::vector<int32_t> order((size_t)G);
+  std::vector<int32_t> order((size_t)G), task0((size_t)G + 1);
+  int64_t gram = 0, tasks = 0;
   for (int32_t g = 0; g < G; ++g) {
     const ssm_batch_graph &x = graphs[g];
     if (x.n < 1 || x.n > kPrepMaxN || x.k < 2 || x.k > kPrepMaxK || x.k > x.n || x.cnt_len < x.k)
@@ -950,24 +1072,33 @@ SSM_API int ssm_batch_layout_init(int32_t G, const ssm_batch_graph *graphs, cons
     d.n = x.n; d.k = x.k; d.m = m[g];
     d.node_off = x.node_off; d.row_off = x.row_off; d.col_off = x.col_off; d.piv_off = x.piv_off;
     d.dip_off = x.dip_off; d.cnt_off_off = x.cnt_off_off; d.cnt_base = x.cnt_base;
+    d.gram_off = gram;
+    gram += gram_words(x.k);
     order[(size_t)g] = g;
   }
   std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
     const LayoutDev &x = ld[(size_t)a], &y = ld[(size_t)b];
     return (int64_t)x.n * x.k * x.k > (int64_t)y.n * y.k * y.k;
   });
+  for (int32_t q = 0; q < G; ++q) {
+    task0[(size_t)q] = (int32_t)tasks;
+    tasks += (ld[(size_t)order[(size_t)q]].n + kGramNodes - 1) / kGramNodes;
+  }
+  task0[(size_t)G] = (int32_t)tasks;
   Carver c(ws, ws_bytes);
   PrepWs w;
-  carve_prep(c, w, G, -1);
+  carve_prep(c, w, G, gram, -1);
   if (!c.ok) return fail(SSM_E_NOMEM, "ssm_batch_layout_init: workspace %zu bytes, need %zu", ws_bytes, c.size());
   LayoutDev *dd = w.ld;
   int32_t *dorder = w.order;
   unsigned *ctr = w.ctr + 1;
   SSM_TRY_CUDA(cudaMemcpyAsync(dd, ld.data(), ld.size() * sizeof(LayoutDev), cudaMemcpyHostToDevice, s));
   SSM_TRY_CUDA(cudaMemcpyAsync(dorder, order.data(), order.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+  SSM_TRY_CUDA(cudaMemcpyAsync(w.task0, task0.data(), task0.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
   SSM_TRY_CUDA(cudaMemsetAsync(ctr, 0, sizeof(unsigned), s));
+  SSM_TRY_CUDA(cudaMemsetAsync(w.gram, 0, (size_t)gram * sizeof(unsigned long long), s));
   LayoutArgs L;
-  L.G = G; L.desc = dd; L.order = dorder; L.rowptr = rowptr; L.colidx = colidx; L.region = region; L.ecc = ecc;
+  L.G = G; L.desc = dd; L.order = dorder; L.task0 = w.task0; L.gram = w.gram; L.rowptr = rowptr; L.colidx = colidx; L.region = region; L.ecc = ecc;
   L.dip = dip; L.cnt_off = cnt_off; L.cnt = cnt; L.pos = reinterpret_cast<float2 *>(pos); L.eig = eig; L.ctr = ctr;
   L.status = status;
   const size_t smem = layout_smem();
@@ -976,6 +1107,8 @@ SSM_API int ssm_batch_layout_init(int32_t G, const ssm_batch_graph *graphs, cons
   SSM_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_prep_layout, kPrepThreads, smem));
   if (per_sm < 1) return fail(SSM_E_ARG, "ssm_batch_layout_init: %zu bytes of shared memory do not fit", smem);
   const int blocks = std::max(1, std::min(G, per_sm * num_sms()));
+  note_launch(), k_prep_gram<<<(int)tasks, kGramThreads, 0, s>>>(L);
+  SSM_TRY_CUDA(cudaGetLastError());
   note_launch(), k_prep_layout<<<blocks, kPrepThreads, smem, s>>>(L);
   SSM_TRY_CUDA(cudaGetLastError());
   return SSM_OK;
