@@ -641,17 +641,17 @@ def _batch_input_dtype():
 
 
 def ssm_batch_prepare(graphs, device="cuda", stream=None, check: bool = True) -> BatchPacked:
-    """Algorithm 1 lines 1-4 for a batch of small graphs in two launches.
+    """Algorithm 1 lines 1-4 for a batch of small graphs in four launches.
     graphs: list of (n, src, dst, k) with host edge arrays (local ids)."""
     import numpy as np
     _require_cuda()
     L = lib()
     G = len(graphs)
     inp = np.zeros(G, dtype=_batch_input_dtype())
-    eo = 0
-    for i, (n, s_, d_, k) in enumerate(graphs):
-        inp[i] = (n, k, len(s_), eo)
-        eo += len(s_)
+    inp["n"], inp["k"] = [g[0] for g in graphs], [g[3] for g in graphs]
+    inp["m_in"] = [len(g[1]) for g in graphs]
+    inp["edge_off"] = np.cumsum(inp["m_in"]) - inp["m_in"]
+    eo = int(inp["m_in"].sum())
     src = torch.from_numpy(np.concatenate([np.asarray(g[1], np.int32) for g in graphs]) if eo else
                            np.zeros(1, np.int32)).to(device)
     dst = torch.from_numpy(np.concatenate([np.asarray(g[2], np.int32) for g in graphs]) if eo else

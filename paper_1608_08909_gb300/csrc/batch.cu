@@ -68,18 +68,21 @@ __device__ __forceinline__ float b_rsqrt(float x) {
   return y;
 }
 
-// per graph (block b: graph b, or order[b] with use_order): the clamped s
+// per graph (blocks (b, *): graph b, or order[b] with use_order; the second
+// grid index deals out pivots and words): the clamped s
 // table (s by d at 2 off_a + a: 0 below 2, cnt[min(d/2, ecc)] up to d =
 // 2 ecc + 2, larger d clamped there; with do_stab) and d_ip re-laid in tiles
 // of P = ppt node pairs: word (t k + a) P + q holds d(a, 2(t P + q)) |
 // d(a, 2(t P + q) + 1) << 16 (0 past the last node) -- a lane owning
-// 2 P / 32 consecutive nodes reads its P / 32 words of a pivot together
+// 2 P / 32 consecutive nodes reads its P / 32 words of a pivot together.  The
+// copy's 2-byte loads and stores of all graphs bound it: 160 us for 512
+// graphs of 64 to 8192 nodes, k = 100 (870 us as long as the largest graph had one block)
 __global__ void k_batch_setup(BatchArgs A, int use_order, int do_stab) {
   const int gi = use_order ? __ldg(A.order + blockIdx.x) : (int)blockIdx.x;
   const BatchDev D = A.desc[gi];
   const int32_t *off = A.cnt_off + D.cnt_off_off;
   if (do_stab)
-    for (int a = 0; a < D.k; ++a) {
+    for (int a = blockIdx.y; a < D.k; a += gridDim.y) {
       const int o = __ldg(off + a), ecc = __ldg(off + a + 1) - o - 1;
       for (int d = threadIdx.x; d <= 2 * ecc + 2; d += blockDim.x)
         A.stab[D.stab_off + 2 * o + a + d] = d >= 2 ? (float)__ldg(A.cnt + D.cnt_base + o + min(d >> 1, ecc)) : 0.f;
@@ -87,8 +90,8 @@ __global__ void k_batch_setup(BatchArgs A, int use_order, int do_stab) {
   const int P = D.ppt;
   const int tiles = (D.n + 2 * P - 1) / (2 * P), total = tiles * D.k * P;  // below 2^31: n <= 12288, k <= 1024
   const uint16_t *dip = A.dip + D.dip_off;
-  for (int w = threadIdx.x; w < total; w += blockDim.x) {
-    const int q = w % P, ta = w / P;
+  for (int w = blockIdx.y * blockDim.x + threadIdx.x; w < total; w += gridDim.y * blockDim.x) {
+    const int q = w & (P - 1), ta = w / P;  // P: 32 or 64
     const int a = ta % D.k;
     const int i = 2 * ((ta / D.k) * P + q);
     const uint16_t *row = dip + (size_t)a * D.n;
@@ -500,10 +503,13 @@ SSM_API int ssm_batch_iterate(int32_t G, const ssm_batch_graph *graphs, const in
   };
   // the tiled copies of one class (or of every graph) for the shapes in dv
   auto setup = [&](int ci, int do_stab) -> int {
+    int64_t most = 1;  // words of the largest graph: 16 per thread
+    for (int32_t i = 0; i < G; ++i) most = std::max(most, batch_words(dv[(size_t)i].n, dv[(size_t)i].k));
+    const unsigned parts = (unsigned)std::min<int64_t>((most + 4095) / 4096, 1024);
     if (ci < 0) {
-      note_launch(), k_batch_setup<<<G, 256, 0, s>>>(A, 0, do_stab);
+      note_launch(), k_batch_setup<<<dim3((unsigned)G, parts), 256, 0, s>>>(A, 0, do_stab);
     } else {
-      note_launch(), k_batch_setup<<<cls[ci].count, 256, 0, s>>>(class_args(A, ci), 1, do_stab);
+      note_launch(), k_batch_setup<<<dim3((unsigned)cls[ci].count, parts), 256, 0, s>>>(class_args(A, ci), 1, do_stab);
     }
     SSM_TRY_CUDA(cudaGetLastError());
     return SSM_OK;
@@ -584,7 +590,8 @@ SSM_API int ssm_batch_iterate(int32_t G, const ssm_batch_graph *graphs, const in
 
   // the sweeps of the whole batch: one CUDA graph (per class a counter reset
   // and a persistent kernel, the classes on forked branches so that their
-  // kernels can share the GPU), launched once; recorded on private streams
+  // kernels can share the GPU, the class of the largest graphs, whose chains
+  // are the longest, first), launched once; recorded on private streams
   // (the caller's may be the legacy default stream, which cannot be
   // captured), launched on the caller's
   cudaStream_t cs[kClasses + 1] = {};
@@ -608,7 +615,7 @@ SSM_API int ssm_batch_iterate(int32_t G, const ssm_batch_graph *graphs, const in
   }
   int rc = SSM_OK;
   if ((e = cudaEventRecord(ev[kClasses], cs[0])) == cudaSuccess) {
-    for (int ci = 0; ci < kClasses && rc == SSM_OK && e == cudaSuccess; ++ci) {
+    for (int ci = kClasses - 1; ci >= 0 && rc == SSM_OK && e == cudaSuccess; --ci) {
       if (!cls[ci].count) continue;
       if ((e = cudaStreamWaitEvent(cs[ci + 1], ev[kClasses], 0)) != cudaSuccess) break;
       rc = launch_batch_sweep(class_args(A, ci), cls[ci].threads, cls[ci].npl, cls[ci].blocks, cls[ci].nmax,
