@@ -39,6 +39,7 @@ constexpr int kEigP = SSM_EIG_P;  // subspace dimension
 // eigenvalue pairs but drown the second pair below FP64 precision when
 // lambda_2 / lambda_1 is small, so the fourth power is kept
 constexpr int kEigPowerLog2 = SSM_EIG_POWER_LOG2;
+constexpr int kEigMaxProducts = 8;  // products with that power between two orthonormalisations, at most
 constexpr int kEigThreads = 256;
 constexpr int kMaxPivotsMds = 1024;
 constexpr int kEigScratch = (kEigThreads / 32 + 1) * (kEigP * (kEigP + 1) / 2);  // doubles for block_sum
@@ -281,6 +282,7 @@ __device__ __forceinline__ void tiny_jacobi_warp(int P, double *H, double *Q) {
   const int lane = threadIdx.x & 31;
   if (lane < P * P) Q[lane] = (lane / P == lane % P) ? 1.0 : 0.0;
   __syncwarp();
+  double last = 1e300;
   for (int sweep = 0; sweep < 60; ++sweep) {
     double off = 0.0, tot = 0.0;
     if (lane < P * P) {
@@ -293,7 +295,11 @@ __device__ __forceinline__ void tiny_jacobi_warp(int P, double *H, double *Q) {
       off += __shfl_xor_sync(0xffffffffu, off, o);
       tot += __shfl_xor_sync(0xffffffffu, tot, o);
     }
-    if (off <= 1e-32 * tot || off == 0.0) break;  // the same sums in every lane
+    // (the same sums in every lane.)  The rotations' own rounding leaves up to
+    // some 1e-31 of tot: at that level a sweep that does not halve `off` is the
+    // last (rgg256k, weighted: such sweeps were 280 of k_eigen's 455 us)
+    if (off <= 1e-32 * tot || off == 0.0 || (off <= 1e-30 * tot && off >= 0.5 * last)) break;
+    last = off;
     for (int r = 0; r < 3; ++r) {
       double c = 1.0, sn = 0.0;
       if (lane < 2) {
@@ -606,7 +612,23 @@ __global__ void __launch_bounds__(kEigThreads) k_eigen(int32_t n, int32_t k, con
     }
     __syncthreads();
     if (s_done || s_stuck) break;
-    for (int t = threadIdx.x; t < k * P; t += blockDim.x) V[t] = Y[t];  // next basis: orthonormalised M W
+    // next basis: M^p W, orthonormalised.  A product with M is a tenth of an
+    // iteration's Rayleigh-Ritz step, test and Gram-Schmidt (4 of 40 us at
+    // k = 200), so a flat spectrum takes several: as many as keep the first
+    // vector's growth over the second below 2^8 (Gram-Schmidt then leaves
+    // 2^8 of FP64's rounding in it, far below tol) and over the last below
+    // 2^32.  ba1m, k = 200: 0.69 ms, with one product each 1.94 ms.
+    const double g2 = H[0] / H[(P > 1 ? 1 : 0) * (P + 1)], gP = H[0] / H[(P - 1) * (P + 1)];
+    double a2 = g2, aP = gP;
+    for (int p = 1; p < kEigMaxProducts; ++p) {
+      a2 *= g2;
+      aP *= gP;
+      if (!(a2 <= 256.0 && aP <= 4294967296.0)) break;  // (a Ritz value of zero: no)
+      for (int t = threadIdx.x; t < k * P; t += blockDim.x) V[t] = Y[t];
+      __syncthreads();
+      if (!product(M, P)) return;
+    }
+    for (int t = threadIdx.x; t < k * P; t += blockDim.x) V[t] = Y[t];
     __syncthreads();
     orthonormalise(k, P, V, scratch, 0x9e37ull + (unsigned long long)it);
   }

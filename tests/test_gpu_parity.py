@@ -434,6 +434,22 @@ def test_pivotmds_matches_oracle(name, k):
         assert _norm_err(pos.cpu().numpy(), O.rescale(og, opos)) < 1e-9
 
 
+@pytest.mark.parametrize("n,k", [(500, 3), (3000, 4), (3000, 5), (6000, 200)])
+def test_pivotmds_flat_spectrum(n, k):
+    """Heavy-tailed graphs, whose eigenvalues lie close together (several
+    products between two orthonormalisations): eigenvalues to 1e-10, positions
+    to the stopping residual 1e-12 lambda_1 over the second pair's gap."""
+    n, s, d = I.ba(n, 4, 7)
+    og = O.build_csr(n, s, d)
+    dip = O.pivot_dist(og, O.maxmin(og, k, 0))
+    opos, oeig, B = O.pivotmds(dip, return_b=True)
+    lam = np.linalg.eigvalsh(B)[::-1]
+    pos, eig = ssm.ssm_pivotmds(_gpu_graph(n, s, d), torch.from_numpy(dip).to(DEV), precision=64, rescale=False)
+    np.testing.assert_allclose(eig.cpu().numpy()[:2], oeig, rtol=1e-10)
+    gap = min(lam[0] - lam[1], lam[1] - lam[2])
+    assert _norm_err(pos.cpu().numpy(), opos) < 1e-9 + 4e-12 * lam[0] / gap
+
+
 @pytest.mark.parametrize("n0,seed", [(83, 2573530203214907681), (725, 3306426093002437330)])
 def test_pivotmds_small_second_eigenvalue(n0, seed):
     """Small RGGs whose lambda_2 / lambda_1 is below 1e-2: the second pair sinks
