@@ -90,8 +90,9 @@ unsigned long long ssm_set_wait_limit_ns(unsigned long long ns);
 void ssm_last_sweep_config(int32_t *out);
 
 /* What the last max/min pivot selection on this host thread chose, in out[2]
- * (host): out[0] the thread-block cluster size of the cluster kernel (0: the
- * cooperative grid kernel; -1: no call yet), out[1] bytes of the distance to
+ * (host): out[0] the thread-block cluster size of the cluster kernel (1: one
+ * block, for graphs that its shared memory holds; 0: the cooperative grid
+ * kernel; -1: no call yet), out[1] bytes of the distance to
  * the closest pivot per node (4, or 2 for graphs whose 4-byte array does not
  * fit the cluster; a search deeper than 65534 levels then hands the whole
  * selection to the grid kernel on the device).  A diagnostic with no

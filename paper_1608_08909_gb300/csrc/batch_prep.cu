@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "block_search.cuh"
 #include "common.cuh"
 
 namespace ssm {
@@ -48,10 +49,7 @@ struct PrepArgs {
   int32_t *status;
 };
 
-constexpr int kPrepInf = 0x7FFFFFFF;  // the key of a node that no search has reached
-
-// shared memory of a graph, without its neighbour lists
-__host__ __device__ constexpr int64_t prep_node_bytes(int64_t n) { return 8 * (n + 1) + 4 * n; }
+// shared memory of a graph's searches from its pivots, without its neighbour lists
 __host__ __device__ constexpr int64_t dist_node_bytes(int64_t n) { return 12 * n + 4 * (n + 1) + (n + 31) / 32 * 64; }
 
 // exclusive block scan of a[0..len) in place, total returned; s_part holds a
@@ -93,10 +91,8 @@ __device__ int block_exclusive_scan(int *a, int len, int *s_part) {
 
 // CSR, max/min pivots, regions, eccentricities and table lengths of one graph
 // per block.  The searches are chains of short levels (10 to 30 nodes wide
-// after the first few pivots), so a level's latency is all that counts: eight
-// lanes per frontier node, offsets and neighbours (16 bits) in shared memory
-// where they fit, one block barrier per level (three rotating queue lengths)
-// and one queue atomic per warp.  512 graphs of 64 to 8192 nodes, k = 100: a
+// after the first few pivots): block_search, the offsets in shared memory and
+// the neighbours too where they fit.  512 graphs of 64 to 8192 nodes, k = 100: a
 // batch takes as long as its largest graph (1,700 levels), 1.38 ms; with a lane
 // per node, neighbours in global memory and a queue atomic per node a level
 // took 4,500 cycles, and the searches below were part of the same block: 18.4 ms.
@@ -105,7 +101,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_pivots(PrepArgs A) {
   __shared__ int s_part[kPrepThreads / 32 + 1], s_ecc[kPrepMaxK];
   __shared__ int s_task, s_len[3];
   __shared__ unsigned s_key[2];
-  const int lane = threadIdx.x & 31, sub = threadIdx.x & 7;
+  const int lane = threadIdx.x & 31;
   for (;;) {
     if (threadIdx.x == 0) s_task = (int)atomicAdd(A.ctr, 1u);
     __syncthreads();
@@ -126,7 +122,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_pivots(PrepArgs A) {
     // duplicates and gaps, for the searches from the pivots
     uint16_t *const tmp = reinterpret_cast<uint16_t *>(A.tmp + D.col_off);
     uint16_t *const packed = tmp + 2 * D.m_in;
-    uint16_t *const col = prep_node_bytes(n) + 4 * D.m_in <= A.ubytes ? qb + n : tmp;
+    uint16_t *const col = block_search_bytes(n) + 4 * D.m_in <= A.ubytes ? qb + n : tmp;
     // ---- CSR: degrees, scatter, rows sorted and deduplicated
     for (int i = threadIdx.x; i <= n; i += blockDim.x) off[i] = 0;
     __syncthreads();
@@ -200,11 +196,12 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_pivots(PrepArgs A) {
     }
     const uint16_t *const nbr = gaps && col == tmp ? packed : col;
     __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) key[i] = kPrepInf;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) key[i] = kBsInf;
     if (threadIdx.x < 3) s_len[threadIdx.x] = 0;
     if (threadIdx.x < 2) s_key[threadIdx.x] = 0u;
     __syncthreads();
-    int slot = 0;  // the queue length in use
+    const BlockSearch B{key, off, nbr, qa, qb, s_len};
+    int slot = 0;
     for (int a = 0; a < k; ++a) {
       int p = 0;
       if (a > 0) {
@@ -218,57 +215,18 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_pivots(PrepArgs A) {
       }
       if (threadIdx.x == 0) {
         A.pivots[D.piv_off + a] = p;
-        key[p] = a;
-        qa[0] = (uint16_t)p;
-        s_len[slot] = 1;
         s_key[(a + 1) & 1] = 0u;
       }
-      __syncthreads();
-      for (int level = 1;; ++level) {
-        const int ncur = s_len[slot], nslot = slot == 2 ? 0 : slot + 1;
-        if (ncur == 0) break;
-        if (threadIdx.x == 0) s_len[nslot == 2 ? 0 : nslot + 1] = 0;
-        const uint16_t *qc = level & 1 ? qa : qb;
-        uint16_t *qn = level & 1 ? qb : qa;
-        const int nk = level * 128 + a;
-        // whole warps: four nodes of eight lanes each
-        for (int t0 = (threadIdx.x >> 5) * 4; t0 < ncur; t0 += kPrepThreads / 8) {
-          const int t = t0 + (lane >> 3);
-          int j = 0, e = 0;
-          if (t < ncur) {
-            const int v = qc[t];
-            j = off[v] + sub;
-            e = off[v + 1];
-          }
-          while (__any_sync(0xffffffffu, j < e)) {
-            bool lowered = false;
-            int u = 0;
-            if (j < e) {
-              u = nbr[j];
-              lowered = key[u] > nk && atomicMin(key + u, nk) > nk;
-            }
-            const unsigned m = __ballot_sync(0xffffffffu, lowered);
-            if (m) {
-              int base = 0;
-              if (lane == 0) base = atomicAdd(s_len + nslot, __popc(m));
-              base = __shfl_sync(0xffffffffu, base, 0);
-              if (lowered) qn[base + __popc(m & ((1u << lane) - 1u))] = (uint16_t)u;
-            }
-            j += 8;
-          }
-        }
-        __syncthreads();
-        slot = nslot;
-      }
+      block_search(B, p, 7, a, slot);
       if (a == 0)
         for (int i = threadIdx.x; i < n; i += blockDim.x)
-          if (key[i] == kPrepInf) dev_fail(A.status, SSM_E_DISCONNECTED);
+          if (key[i] == kBsInf) dev_fail(A.status, SSM_E_DISCONNECTED);
     }
     // ---- regions and eccentricities
     for (int a = threadIdx.x; a < k; a += blockDim.x) s_ecc[a] = 0;
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const int c = key[i] == kPrepInf ? 0 : key[i];  // (the status then refuses the batch)
+      const int c = key[i] == kBsInf ? 0 : key[i];  // (the status then refuses the batch)
       A.region[D.node_off + i] = c & 127;
       atomicMax(s_ecc + (c & 127), c >> 7);
     }
@@ -954,7 +912,7 @@ static void prep_smem(int32_t G, const ssm_batch_input *in, int64_t &pivots, int
   const int64_t cap = 227 * 1024 - 2048;
   pivots = dist = 0;
   for (int32_t g = 0; g < G; ++g) {
-    const int64_t p = prep_node_bytes(in[g].n), d = dist_node_bytes(in[g].n), nb = 4 * in[g].m_in;
+    const int64_t p = block_search_bytes(in[g].n), d = dist_node_bytes(in[g].n), nb = 4 * in[g].m_in;
     pivots = std::max(pivots, p + nb <= cap ? p + nb : p);
     dist = std::max(dist, d + nb <= cap ? d + nb : d);
   }

@@ -1,4 +1,5 @@
 // Breadth-first searches on the device:
+// (graphs that one block's shared memory holds: small_graph.cu)
 //   * ssm_select_pivots: max/min-sp pivot sampling (Section 4.1), one pruned
 //     level-synchronous BFS per new pivot inside one cooperative persistent
 //     kernel; small frontiers are expanded by one block without device-wide
@@ -482,6 +483,8 @@ int launch_maxmin(int32_t n, int64_t m2, const int32_t *rowptr, const int32_t *c
   unsigned *spill = nullptr;
   carve_maxmin(c, A, &spill, n, m2);
   if (!c.ok) return fail(SSM_E_NOMEM, "max/min pivots: workspace %zu bytes, need %zu", ws_bytes, c.size());
+  // a level in one block's shared memory costs a sixth of the cluster's
+  if (small_graph_fits(n, m2)) return launch_small_maxmin(n, m2, rowptr, colidx, k, start, pivots, status, s);
   int rc = expand_adj(m2, rowptr, colidx, const_cast<int4 *>(A.adj), s);
   if (rc) return rc;
   unsigned *fallback = const_cast<unsigned *>(A.run_if);
@@ -967,6 +970,9 @@ int launch_msbfs(int32_t n, int64_t m2, const int32_t *rowptr, const int32_t *co
     void *pws = c.take<char>(pw);
     B.run_if = gaveup;
     if (!c.ok) return fail(SSM_E_NOMEM, "BFS: workspace %zu bytes, need %zu", ws_bytes, c.size());
+    // (not where the pulled BFS hands its levels on: that writes no distances)
+    if (!after_pass && small_bfs_fits(n, m2, k))
+      return launch_small_bfs(n, m2, rowptr, colidx, k, sources, dist, status, s);
     SSM_TRY_CUDA(cudaMemsetAsync(gaveup, 0, sizeof(unsigned), s));
     int rc = launch_msbfs_pull(n, rowptr, colidx, k, sources, dist, status, gaveup, pws, pw, s, after_pass);
     if (rc) return rc;

@@ -15,6 +15,15 @@ size_t maxmin_workspace(int32_t n, int64_t m2);
 int launch_maxmin(int32_t n, int64_t m2, const int32_t *rowptr, const int32_t *colidx, int32_t k, int32_t start,
                   int32_t *pivots, int32_t *status, void *ws, size_t ws_bytes, cudaStream_t s);
 
+// max/min pivots and distances of graphs that one block's shared memory holds
+// (small_graph.cu)
+bool small_graph_fits(int32_t n, int64_t m2);
+bool small_bfs_fits(int32_t n, int64_t m2, int32_t k);
+int launch_small_maxmin(int32_t n, int64_t m2, const int32_t *rowptr, const int32_t *colidx, int32_t k, int32_t start,
+                        int32_t *pivots, int32_t *status, cudaStream_t s);
+int launch_small_bfs(int32_t n, int64_t m2, const int32_t *rowptr, const int32_t *colidx, int32_t k,
+                     const int32_t *sources, uint16_t *dist, int32_t *status, cudaStream_t s);
+
 // max/min pivots inside one thread-block cluster (maxmin_cluster.cu), for
 // graphs whose mind array fits the cluster's shared memory.  Sets
 // *mind_bytes to 4 or 2 when the cluster kernel was enqueued (0: the caller

@@ -235,6 +235,38 @@ def test_select_pivots_deep_search_hands_over_to_the_grid_kernel():
     assert np.array_equal(got, O.maxmin(og, 3, 450000))
 
 
+def _complete(n):
+    a, b = np.triu_indices(n, 1)
+    return n, a.astype(np.int32), b.astype(np.int32)
+
+
+def _star(n):
+    return n, np.zeros(n - 1, np.int32), np.arange(1, n, dtype=np.int32)
+
+
+@pytest.mark.parametrize("graph,k,cluster", [
+    (lambda: I.path(2), 2, 1), (lambda: I.grid(3, 11), 33, 1), (lambda: I.path(14463), 4, 1),
+    (lambda: I.path(14464), 4, 16),                      # 16 bytes per node: past the shared memory
+    (lambda: _star(9000), 40, 1),                        # a row of many warps, a frontier of all nodes
+    (lambda: _complete(335), 30, 1), (lambda: _complete(340), 30, 16),
+    (lambda: I.ba(7000, 4, 3), 150, 1), (lambda: I.rgg(5000, 8.0, 2), 200, 1)])
+def test_small_graph_searches(graph, k, cluster):
+    """Max/min pivots and distances of graphs that one block's shared memory
+    holds, and just past it: the same numbers as the oracle's; also a search
+    from every source that many blocks share."""
+    n, s, d = graph()
+    og = O.build_csr(n, s, d)
+    g = _gpu_graph(n, s, d)
+    got = ssm.ssm_select_pivots(g, k, n // 2)
+    assert ssm.ssm_last_pivot_config()["cluster"] == cluster
+    piv = O.maxmin(og, k, n // 2)
+    assert np.array_equal(got.cpu().numpy(), piv)
+    assert np.array_equal(ssm.ssm_pivot_bfs(g, got).cpu().numpy(), O.pivot_dist(og, piv))
+    if n <= 9000:
+        src = (np.arange(700) * 37 % n).astype(np.int32)
+        assert np.array_equal(ssm.ssm_pivot_bfs(g, torch.from_numpy(src).to(DEV)).cpu().numpy(), O.pivot_dist(og, src))
+
+
 # ------------------------------------------------------------------ a2 d_ip
 
 @pytest.mark.parametrize("name,k", [("grid32", 50), ("path", 7), ("btree", 33), ("rgg", 100), ("ba", 64),
