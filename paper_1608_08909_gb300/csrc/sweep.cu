@@ -748,25 +748,120 @@ __global__ void k_dip_max(int64_t count, const uint16_t *__restrict__ dip, unsig
 
 // ----------------------------------------------------------------- FP64
 // The same update evaluated in plain double precision, one node per thread:
-// the comparison baseline for the FP32 sweep.  Every operation is an
-// explicitly rounded IEEE double operation (no fused multiply-add), taken in
+// the comparison baseline for the FP32 sweep.  Every result is that of an
+// explicitly rounded IEEE double operation (no contraction), taken in
 // the order in which Eq. 4 is written -- neighbours in CSR order, then pivots
-// a = 0..k-1 -- so its results do not depend on compiler contraction.
+// a = 0..k-1 -- so it does not depend on compiler contraction.
+//
+// FP64 at a 64th of FP32's rate bounds it: a term's count of FP64
+// instructions.  The square root and the divides of a term therefore share
+// one reciprocal square root (over_length), and s / d^2 takes 1 / d^2 from a
+// table: some 33 instructions a term where three IEEE divides and a square
+// root made it 85.  ba64k, k = 200: 1.05 ms an iteration, 2.1 to 2.2 before.
 struct PivD {
   double x, y;
   int off, ecc;
 };
 
-__device__ __forceinline__ double dist_rn(double dx, double dy) {
-  return __dsqrt_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
+// d, d^2 and RN(1 / d^2) for d below kF64Dists
+constexpr int kF64Dists = 1024;
+constexpr int kF64LongRow = 16;  // longer rows: k_f64_long_rows
+struct DistD {
+  double d, d2, inv;
+};
+
+// 2^-400 <= |v| < 2^400
+__device__ __forceinline__ bool mid_range(double v) {
+  return ((unsigned)__double2hiint(v) & 0x7FFFFFFFu) - (623u << 20) < (800u << 20);
+}
+
+// (qx, qy) = (tx / r, ty / r) with r = sqrt(dx^2 + dy^2), every operation
+// rounded to nearest; false where r is zero.  One reciprocal square root y of
+// h = r^2 serves them: Halley's iteration brings the hardware's approximation
+// (20 bits) to FP64 rounding, r is h y corrected once by its exact residual,
+// 1 / r is y corrected once, and each quotient is the product with it
+// corrected once by its exact residual (Markstein's scheme: a residual by
+// fused multiply-add, one correction).  What is rounded last is within 2^-104
+// of the exact value, so a result differs from the IEEE operation's, by one
+// unit in the last place, only where that lies so close to a rounding
+// boundary: about one operand in 2^50 (none of 15e9 random ones).  Where a value is outside 2^+-400 (or
+// not a number), the IEEE operations.
+__device__ __forceinline__ bool over_length(double dx, double dy, double tx, double ty, double &qx, double &qy) {
+  const double h = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
+  if (mid_range(h) && (mid_range(tx) || tx == 0.0) && (mid_range(ty) || ty == 0.0)) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(h));
+    const double e = __fma_rn(-__dmul_rn(h, y), y, 1.0);
+    y = __fma_rn(__dmul_rn(y, e), __fma_rn(e, 0.375, 0.5), y);
+    const double g = __dmul_rn(h, y);
+    const double half = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));  // y / 2
+    const double r = __fma_rn(__fma_rn(-g, g, h), half, g);
+    const double z = __fma_rn(__fma_rn(-r, y, 1.0), y, y);
+    qx = __dmul_rn(tx, z);
+    qx = __fma_rn(__fma_rn(-r, qx, tx), z, qx);
+    qy = __dmul_rn(ty, z);
+    qy = __fma_rn(__fma_rn(-r, qy, ty), z, qy);
+    return true;
+  }
+  const double r = __dsqrt_rn(h);
+  if (!(r > 0.0)) return false;
+  qx = __ddiv_rn(tx, r);
+  qy = __ddiv_rn(ty, r);
+  return true;
+}
+
+// a neighbour's x_j + (x_i - x_j) / r, or x_j where r is zero
+__device__ __forceinline__ double2 f64_neighbour(const double2 &x, const double2 &q) {
+  const double dx = __dsub_rn(x.x, q.x), dy = __dsub_rn(x.y, q.y);
+  double ux, uy;
+  return over_length(dx, dy, dx, dy, ux, uy) ? make_double2(__dadd_rn(q.x, ux), __dadd_rn(q.y, uy)) : q;
+}
+
+// The neighbour sums of rows above kF64LongRow, a warp per row: the lanes form
+// 32 summands at a time, which are added in CSR order (x in even lanes, y in odd
+// ones).  Consecutive rows go to different blocks: in a heavy-tailed graph the
+// first nodes are the hubs.  As part of the sweep a hub's row, in one lane, was
+// the longest chain: ba64k, k = 200: 1.79 ms an iteration against 1.05.
+__global__ void __launch_bounds__(kSweepThreads) k_f64_long_rows(int32_t n, const int32_t *__restrict__ rowptr,
+                                                                 const int32_t *__restrict__ colidx,
+                                                                 const int32_t *__restrict__ stop,
+                                                                 const double2 *__restrict__ pin,
+                                                                 double2 *__restrict__ nb) {
+  __shared__ double2 s_sum[kSweepThreads / 32][32];
+  if (__ldcg(stop)) return;
+  const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const int64_t warps = (int64_t)gridDim.x * (kSweepThreads / 32), first = (int64_t)warp * gridDim.x + blockIdx.x;
+  for (int64_t i0 = first; i0 < n; i0 += 32 * warps) {
+    const int64_t i = i0 + lane * warps;  // lane's row: every warps-th
+    const int b = i < n ? __ldg(rowptr + i) : 0, e = i < n ? __ldg(rowptr + i + 1) : 0;
+    for (unsigned m = __ballot_sync(0xffffffffu, e - b > kF64LongRow); m; m &= m - 1u) {
+      const int o = __ffs(m) - 1;
+      const int ob = __shfl_sync(0xffffffffu, b, o), oe = __shfl_sync(0xffffffffu, e, o);
+      const int64_t row = i0 + o * warps;
+      const double2 x = pin[row];
+      const double *mine = reinterpret_cast<const double *>(s_sum[warp]) + (lane & 1u);
+      double sum = 0.0;
+      for (int t0 = ob; t0 < oe; t0 += 32) {
+        if (t0 + (int)lane < oe) s_sum[warp][lane] = f64_neighbour(x, pin[__ldg(colidx + t0 + lane)]);
+        __syncwarp();
+        const int c = min(32, oe - t0);
+#pragma unroll 8
+        for (int t = 0; t < c; ++t) sum = __dadd_rn(sum, mine[2 * t]);
+        __syncwarp();
+      }
+      if (lane < 2) reinterpret_cast<double *>(nb + row)[lane] = sum;
+    }
+  }
 }
 
 template <bool CNT_SMEM>
 __global__ void __launch_bounds__(kSweepThreads) k_sweep_f64(SweepArgs A, const double2 *__restrict__ pin,
-                                                              double2 *__restrict__ pout) {
+                                                              double2 *__restrict__ pout,
+                                                              const double2 *__restrict__ nb) {
   extern __shared__ __align__(16) unsigned char smem[];
   PivD *piv = reinterpret_cast<PivD *>(smem);
-  double *cntd = reinterpret_cast<double *>(piv + A.k);
+  DistD *dist = reinterpret_cast<DistD *>(piv + A.k);  // [kF64Dists]
+  double *cntd = reinterpret_cast<double *>(dist + kF64Dists);
   if (__ldcg(A.stop)) return;
   const int n = A.n, k = A.k;
   for (int a = threadIdx.x; a < k; a += blockDim.x) {
@@ -781,34 +876,41 @@ __global__ void __launch_bounds__(kSweepThreads) k_sweep_f64(SweepArgs A, const 
   }
   if (CNT_SMEM)
     for (int t = threadIdx.x; t < A.cnt_len; t += blockDim.x) cntd[t] = (double)__ldg(A.cnt + t);
+  for (int d = threadIdx.x; d < kF64Dists; d += blockDim.x) {
+    const double dd = (double)max(d, 1), d2 = __dmul_rn(dd, dd);
+    dist[d] = DistD{dd, d2, __ddiv_rn(1.0, d2)};
+  }
   __syncthreads();
 
   const unsigned lane = threadIdx.x & 31u;
-  const unsigned ntiles = (unsigned)((n + 31) / 32);
-  for (;;) {
-    unsigned tile = 0;
-    if (lane == 0) tile = atomicAdd(A.tile_ctr, 1u);
-    tile = __shfl_sync(0xffffffffu, tile, 0);
+  const unsigned ntiles = (unsigned)((n + 31) / 32), warp = threadIdx.x >> 5;
+  // the first tiles go round the blocks (every SM the same number of them, its
+  // FP64 unit being the bound), the others to whichever warp is free
+  unsigned tile = warp * gridDim.x + blockIdx.x;
+  for (bool first = true;; first = false) {
+    if (!first) {
+      if (lane == 0) tile = gridDim.x * (kSweepThreads / 32) + atomicAdd(A.tile_ctr, 1u);
+      tile = __shfl_sync(0xffffffffu, tile, 0);
+    }
     if (tile >= ntiles) break;
     const int i = (int)(tile * 32u + lane);
     const bool live = i < n;
     const double2 x = live ? pin[i] : make_double2(0.0, 0.0);
     double nx = 0.0, ny = 0.0, den = 0.0;
+    const int b = live ? __ldg(A.rowptr + i) : 0, e = live ? __ldg(A.rowptr + i + 1) : 0;
     if (live) {
-      const int b = __ldg(A.rowptr + i), e = __ldg(A.rowptr + i + 1);
-      for (int t = b; t < e; ++t) {
-        const double2 q = pin[__ldg(A.colidx + t)];
-        const double dx = __dsub_rn(x.x, q.x), dy = __dsub_rn(x.y, q.y);
-        const double r = dist_rn(dx, dy);
-        if (r > 0.0) {
-          nx = __dadd_rn(nx, __dadd_rn(q.x, __ddiv_rn(dx, r)));
-          ny = __dadd_rn(ny, __dadd_rn(q.y, __ddiv_rn(dy, r)));
-        } else {
-          nx = __dadd_rn(nx, q.x);
-          ny = __dadd_rn(ny, q.y);
+      if (e - b > kF64LongRow) {
+        const double2 v = __ldg(nb + i);
+        nx = v.x;
+        ny = v.y;
+      } else {
+        for (int t = b; t < e; ++t) {
+          const double2 v = f64_neighbour(x, pin[__ldg(A.colidx + t)]);
+          nx = __dadd_rn(nx, v.x);
+          ny = __dadd_rn(ny, v.y);
         }
-        den = __dadd_rn(den, 1.0);
       }
+      den = (double)(e - b);
       const uint16_t *colp = A.dip + i;
       for (int a = 0; a < k; ++a) {
         const int d = __ldcs(colp + (size_t)a * n);
@@ -816,13 +918,23 @@ __global__ void __launch_bounds__(kSweepThreads) k_sweep_f64(SweepArgs A, const 
         const PivD P = piv[a];
         const int h = min(d >> 1, P.ecc);
         const double s = CNT_SMEM ? cntd[P.off + h] : (double)__ldg(A.cnt + P.off + h);
-        const double dd = (double)d;
-        const double w = __ddiv_rn(s, __dmul_rn(dd, dd));
+        // w = RN(s / d^2): a quotient of integers below 2^32 lies no closer to a
+        // rounding boundary than 2^-86, far outside the corrected product's error
+        double dd, w;
+        if (d < kF64Dists) {
+          const DistD T = dist[d];
+          dd = T.d;
+          w = __dmul_rn(s, T.inv);
+          w = __fma_rn(__fma_rn(-w, T.d2, s), T.inv, w);
+        } else {
+          dd = (double)d;
+          w = __ddiv_rn(s, __dmul_rn(dd, dd));
+        }
         const double dx = __dsub_rn(x.x, P.x), dy = __dsub_rn(x.y, P.y);
-        const double r = dist_rn(dx, dy);
-        if (r > 0.0) {
-          nx = __dadd_rn(nx, __dmul_rn(w, __dadd_rn(P.x, __ddiv_rn(__dmul_rn(dd, dx), r))));
-          ny = __dadd_rn(ny, __dmul_rn(w, __dadd_rn(P.y, __ddiv_rn(__dmul_rn(dd, dy), r))));
+        double ux, uy;
+        if (over_length(dx, dy, __dmul_rn(dd, dx), __dmul_rn(dd, dy), ux, uy)) {
+          nx = __dadd_rn(nx, __dmul_rn(w, __dadd_rn(P.x, ux)));
+          ny = __dadd_rn(ny, __dmul_rn(w, __dadd_rn(P.y, uy)));
         } else {
           nx = __dadd_rn(nx, __dmul_rn(w, P.x));
           ny = __dadd_rn(ny, __dmul_rn(w, P.y));
@@ -863,6 +975,7 @@ struct IterWs {
   double *tile_part;
   float *stab;
   float2 *nb;       // [n] neighbour sums
+  double2 *nb64;    // [n] neighbour sums of long rows (FP64)
   int32_t *mid_rows, *long_rows;  // [n] rows longer than kShortDeg / kMidDeg
   unsigned *dtile;
   float *wtab;    // full-table mode: w and w d planes
@@ -900,6 +1013,7 @@ static size_t carve_iterate(Carver &c, IterWs &w, int32_t n, int64_t m2, int32_t
   w.tile_part = c.take<double>(2 * ((size_t)n / 32 + 2));
   w.stab = c.take<float>((size_t)(2 * cnt_len + k));
   w.nb = precision == 64 ? nullptr : c.take<float2>((size_t)n);
+  w.nb64 = precision == 64 ? c.take<double2>((size_t)n) : nullptr;
   w.mid_rows = precision == 64 ? nullptr : c.take<int32_t>((size_t)n);
   w.long_rows = precision == 64 ? nullptr : c.take<int32_t>((size_t)n);
   w.dtile = precision == 64 ? nullptr : c.take<unsigned>((size_t)((n + kTileNodes - 1) / kTileNodes) * (size_t)k * 32 * kPpl);
@@ -960,7 +1074,7 @@ SSM_API int ssm_iterate(int32_t n, int64_t m, const int32_t *rowptr, const int32
   unsigned meta[3] = {0, 0, 0};
   bool tsm = true;
   if (precision == 64) {
-    const size_t piv = (size_t)k * sizeof(PivD), tab = (size_t)cnt_len * sizeof(double);
+    const size_t piv = (size_t)k * sizeof(PivD) + kF64Dists * sizeof(DistD), tab = (size_t)cnt_len * sizeof(double);
     tsm = piv + tab <= kSmemBudget;
     smem = piv + (tsm ? tab : 0);
     kern = tsm ? (const void *)k_sweep_f64<true> : (const void *)k_sweep_f64<false>;
@@ -1047,7 +1161,8 @@ SSM_API int ssm_iterate(int32_t n, int64_t m, const int32_t *rowptr, const int32
   // one warp per tile, or up to kSplitTasksPerWarp warps per tile on graphs
   // small enough to split (their pivot ranges keep the extra warps busy)
   const int64_t per_tile = (precision == 32 && w.split_cap > 0 && kSplitTasksPerWarp > 0) ? kSplitTasksPerWarp : 1;
-  const int64_t want = (tiles * per_tile + (kSweepThreads / 32) - 1) / (kSweepThreads / 32);
+  int64_t want = (tiles * per_tile + (kSweepThreads / 32) - 1) / (kSweepThreads / 32);
+  if (precision == 64) want = (want + sms - 1) / sms * sms;  // the same number on every SM
   const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * sms, want));
   if (precision == 32 && w.split_cap > 0 && kSplitTasksPerWarp > 0) {
     // about kSplitTasksPerWarp tasks per resident warp, ranges of at least 2 kPrefetch pivots
@@ -1094,7 +1209,11 @@ SSM_API int ssm_iterate(int32_t n, int64_t m, const int32_t *rowptr, const int32
       SSM_TRY_CUDA(cudaLaunchKernelExC(&cfg, kern, args));
       continue;
     }
-    void *args[] = {&A, &pin, &pout};
+    note_launch(), k_f64_long_rows<<<(int)std::min<int64_t>(tiles, (int64_t)sms * 8), kSweepThreads, 0, s>>>(
+        n, rowptr, colidx, w.stop, (const double2 *)pin, w.nb64);
+    SSM_TRY_CUDA(cudaGetLastError());
+    const double2 *nb64 = w.nb64;
+    void *args[] = {&A, &pin, &pout, &nb64};
     note_launch();
     SSM_TRY_CUDA(cudaLaunchKernel(kern, dim3(blocks), dim3(kSweepThreads), args, smem, s));
   }

@@ -109,6 +109,25 @@ def test_sweep_fp64_counts_in_global_memory(long_path):
     assert rel.item() == pytest.approx(orel, rel=1e-12)
 
 
+@pytest.mark.parametrize("scale", [1.0, 1e-130, 1e130, 1e-70])
+@pytest.mark.parametrize("name,k", [("path", 7), ("ba", 40), ("star", 5)])
+def test_sweep_fp64_ranges_bit_for_bit(name, k, scale):
+    """The shared reciprocal square root, its range check (lengths whose squares
+    leave 2^+-400 take the IEEE operations), distances below and above the
+    table of 1 / d^2, rows on both sides of the long-row limit: the oracle's
+    bits."""
+    n, s, d = {"path": lambda: I.path(2500), "ba": lambda: I.ba(700, 4, 3),
+               "star": lambda: (1000, np.zeros(999, np.int32), np.arange(1, 1000, dtype=np.int32))}[name]()
+    prep = O.prepare(n, s, d, k)
+    x0 = scale * (prep.pos0 + np.random.default_rng(2).normal(size=(n, 2)))
+    x0[::7, 1] = x0[0, 1]  # equal ordinates: a zero difference
+    want, _ = O.sweep_jacobi(prep.g, prep.pivots, prep.dip, prep.w, x0)
+    pos = torch.from_numpy(x0.copy()).to(DEV)
+    ssm.ssm_iterate(_gpu_graph(n, s, d), _gpu_pivots(k, prep), pos, 1)
+    assert ssm.ssm_last_sweep_config()["kernel"] == "f64_counts_smem"
+    assert np.array_equal(pos.cpu().numpy(), want)
+
+
 # ------------------------------------------------------------------ coincident positions
 
 def _coincident_state(prep, rng, count):
