@@ -531,7 +531,8 @@ size_t maxmin_workspace(int32_t n, int64_t m2) {
 #ifndef SSM_ADJ2_MAX_MB
 #define SSM_ADJ2_MAX_MB 48
 #endif
-constexpr int kCtaThreads = 512;
+constexpr int kCtaThreads = 512;      // two blocks per SM
+constexpr int kCtaManyThreads = 384, kCtaManyBlocks = 4;  // many sources, or a small graph
 constexpr int kCtaStep = SSM_CTA_STEP;         // edges whose loads a lane has in flight at once
 constexpr int kCtaLaneRow = SSM_CTA_LANE_ROW;  // rows up to this length: one lane; longer: the warp
 constexpr int kCtaQMax = SSM_CTA_QMAX;         // frontier entries per level kept in shared memory (at most)
@@ -572,8 +573,14 @@ struct CtaBfsArgs {
 // walked by the whole warp, one row at a time.  Each step claims its nodes,
 // compacts the appends with warp ballots and reserves their slots with one
 // shared-memory atomic, so a round costs about one global-memory latency.
-template <bool ADJ, int MINB>
-__global__ void __launch_bounds__(kCtaThreads, MINB) k_bfs_cta(CtaBfsArgs A) {
+// The instructions of a step bound it (issue slots 58 % busy, a third of the
+// stalls at the level's barrier; DRAM 21 %, L2 42 %): only an eighth of the
+// edges claim a node, so the append goes through the lanes' claims one by one
+// (mostly two rounds) and not through the step's four edges: 1,024 sources on
+// rgg256k 13.0 -> 12.1 ms.  Wider adjacency loads do not help: aligning them
+// costs more steps than they save.
+template <bool ADJ, bool MANY>
+__global__ void __launch_bounds__(MANY ? kCtaManyThreads : kCtaThreads, MANY ? kCtaManyBlocks : 2) k_bfs_cta(CtaBfsArgs A) {
   extern __shared__ __align__(16) unsigned cta_smem[];
   __shared__ unsigned s_cnt[3];
   const unsigned n = (unsigned)A.n, nwords = (n + 31u) / 32u;
@@ -627,35 +634,35 @@ __global__ void __launch_bounds__(kCtaThreads, MINB) k_bfs_cta(CtaBfsArgs A) {
       // ok[u]) and append the new ones to the next frontier
       auto step = [&](const int (&idx)[kCtaStep], const bool (&ok)[kCtaStep]) {
         int2 ed[kCtaStep];
-        bool push[kCtaStep];
 #pragma unroll
         for (int u = 0; u < kCtaStep; ++u) ed[u] = ok[u] ? __ldg(A.adj + idx[u]) : make_int2(0, 0);
-        unsigned tot = 0;
+        unsigned won = 0;  // bit u: this lane claimed edge u's node
 #pragma unroll
-        for (int u = 0; u < kCtaStep; ++u) {
-          push[u] = false;
+        for (int u = 0; u < kCtaStep; ++u)
           if (ok[u]) {
             const unsigned v = (unsigned)ed[u].x & ((1u << kAdj2NodeBits) - 1u);
             const unsigned bit = 1u << (v & 31u);
             unsigned *wp = vis + (v >> 5);
-            push[u] = !(*wp & bit) && !(atomicOr(wp, bit) & bit);
+            if (!(*wp & bit) && !(atomicOr(wp, bit) & bit)) won |= 1u << u;
           }
-          tot += __popc(__ballot_sync(0xffffffffu, push[u]));
-        }
+        const unsigned tot = __reduce_add_sync(0xffffffffu, (unsigned)__popc(won));
         if (tot == 0) return;
         unsigned pos = 0;
         if (lane == 0) pos = atomicAdd(cnt_next, tot);
         pos = __shfl_sync(0xffffffffu, pos, 0);
+        // one claimed node per lane at a time: an eighth of the edges are claims
+        for (unsigned mk; (mk = __ballot_sync(0xffffffffu, won != 0u)) != 0u; won &= won - 1u) {
+          if (won) {
+            int2 c = ed[0];
 #pragma unroll
-        for (int u = 0; u < kCtaStep; ++u) {
-          const unsigned mk = __ballot_sync(0xffffffffu, push[u]);
-          if (push[u]) {
-            const unsigned v = (unsigned)ed[u].x & ((1u << kAdj2NodeBits) - 1u);
-            unsigned dg = (unsigned)ed[u].x >> kAdj2NodeBits;
-            if (dg == kAdj2DegEsc) dg = (unsigned)(__ldg(A.rowptr + v + 1) - ed[u].y);
+            for (int u = 1; u < kCtaStep; ++u)
+              if ((won & ((1u << u) - 1u)) == 0u) c = ed[u];
+            const unsigned v = (unsigned)c.x & ((1u << kAdj2NodeBits) - 1u);
+            unsigned dg = (unsigned)c.x >> kAdj2NodeBits;
+            if (dg == kAdj2DegEsc) dg = (unsigned)(__ldg(A.rowptr + v + 1) - c.y);
             row[v] = nd;
             const unsigned q = pos + __popc(mk & lt);
-            const int2 ent = make_int2(ed[u].y, (int)dg);
+            const int2 ent = make_int2(c.y, (int)dg);
             if (q < qsm) sout[q] = ent; else gout[q] = ent;
           }
           pos += __popc(mk);
@@ -736,19 +743,21 @@ __global__ void k_pack_adj(int64_t m2, const int32_t *__restrict__ rowptr, const
 static bool cta_bfs_fits(int32_t n) { return (size_t)((n + 31) / 32) * 4 <= kCtaBitmapMax; }
 
 struct CtaBfsShape {
-  bool many;  // four blocks per SM (32 registers a thread), else two (64)
-  int slots, qsm;
+  bool many;  // four blocks per SM (384 threads of 40 registers), else two (512 of 64)
+  int slots, qsm, threads;
   size_t smem;
 };
 
 static const void *cta_bfs_kernel(bool packed, bool many) {
-  if (packed) return many ? (const void *)k_bfs_cta<true, 4> : (const void *)k_bfs_cta<true, 2>;
-  return many ? (const void *)k_bfs_cta<false, 4> : (const void *)k_bfs_cta<false, 2>;
+  if (packed) return many ? (const void *)k_bfs_cta<true, true> : (const void *)k_bfs_cta<true, false>;
+  return many ? (const void *)k_bfs_cta<false, true> : (const void *)k_bfs_cta<false, false>;
 }
 
-// Blocks of 512 threads: on a large graph whose sources fit two per SM, two
+// On a large graph whose sources fit two per SM, two blocks of 512 threads
 // per SM, with the shared memory an SM can give each beyond the bitmap holding
-// the first qsm frontier entries of both levels; otherwise four per SM, with
+// the first qsm frontier entries of both levels; otherwise four of 384 per SM
+// (1,024 sources on rgg256k 11.1 ms; of 512 threads, whose 32 registers spill,
+// 12.1; five of 320 or six of 256, which leave L1 less room, 15.0), with
 // the bitmap alone (measured: a shared-memory frontier at four blocks per SM
 // leaves less L1 for the adjacency reads and was slower on rgg256k, and two
 // fat blocks per SM cost concurrent requests of mid-size graphs 7 % of the
@@ -758,7 +767,8 @@ static CtaBfsShape cta_bfs_shape(int32_t n, int32_t nsrc) {
   CtaBfsShape S;
   const int sms = num_sms();
   S.many = nsrc > 2 * sms || n < kCtaFewMinNodes;
-  const int want = S.many ? 4 : 2;
+  const int want = S.many ? kCtaManyBlocks : 2;
+  S.threads = S.many ? kCtaManyThreads : kCtaThreads;
   const size_t bitmap = (size_t)(((n + 31) / 32 + 3) & ~3) * 4;
   int dev = 0, per_sm_smem = 0, per_block_max = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -776,7 +786,7 @@ static CtaBfsShape cta_bfs_shape(int32_t n, int32_t nsrc) {
   int per_sm = 0;
   const void *kern = cta_bfs_kernel(true, S.many);
   if (allow_dynamic_smem(kern) != cudaSuccess || allow_dynamic_smem(cta_bfs_kernel(false, S.many)) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kCtaThreads, S.smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, S.threads, S.smem) != cudaSuccess ||
       per_sm < 1) {
     (void)cudaGetLastError();
     per_sm = 1;
@@ -991,7 +1001,7 @@ int launch_msbfs(int32_t n, int64_t m2, const int32_t *rowptr, const int32_t *co
     }
     void *args[] = {&B};
     note_launch();
-    SSM_TRY_CUDA(cudaLaunchKernel(cta_bfs_kernel(packed, S.many), dim3(S.slots), dim3(kCtaThreads), args, S.smem, s));
+    SSM_TRY_CUDA(cudaLaunchKernel(cta_bfs_kernel(packed, S.many), dim3(S.slots), dim3(S.threads), args, S.smem, s));
     return SSM_OK;
   }
   MsBfsArgs A;
