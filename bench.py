@@ -657,7 +657,7 @@ def run_batch(args):
     torch.cuda.synchronize()
     t_prep = time.perf_counter() - t0
 
-    # the same batch prepared in two launches (ssm_batch_prepare): timed with
+    # the same batch prepared in four launches (ssm_batch_prepare): timed with
     # CUDA events around both calls (the edge lists already on the host, their
     # copy to the device inside the timing), after one untimed warm-up
     ssm.ssm_batch_prepare(graphs)
@@ -713,7 +713,7 @@ def run_batch(args):
         "ms_sweeps": round(ms, 3), "wall_ms_call": round(wall * 1e3, 3), "prepare_s": round(t_prep, 3),
         "batched_prepare": {"ms": round(t_bprep, 3), "wall_ms": round(t_bprep_wall * 1e3, 3),
                             "note": "ssm_batch_prepare: CSR, max/min pivots, d_ip, counts, PivotMDS and rescale "
-                                    "for the whole batch in two launches (one host read of the table lengths); "
+                                    "for the whole batch in four launches (one host read of the table lengths); "
                                     "prepare_s is the per-graph pipeline on 8 streams"},
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                      "frac": round(achieved / peak, 4), "traffic": None,

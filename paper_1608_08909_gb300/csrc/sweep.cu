@@ -623,58 +623,111 @@ __global__ void __launch_bounds__(kSweepThreads, MODE == 2 ? SSM_SWEEP_FULL_MIN_
 // of the node's entry in the shared-memory table.  A distance above the table
 // (a wrong dmax hint) is recorded as SSM_E_ARG and clamped, so no table read
 // leaves the table
-__global__ void k_tile_dip(int32_t n, int32_t k, int32_t row, const uint16_t *__restrict__ dip,
-                           unsigned *__restrict__ dtile, int32_t *__restrict__ status, int32_t pair_loads) {
-  // node pair p = (2p, 2p + 1) of pivot a lands in word (t k + a) P + (p mod P), t = p div P,
-  // P = kTileNodes / 2 pairs per tile; blocks step over pivots in y, pairs in x
+//
+// loads of d_ip: 16 bytes at a time (2: n a multiple of 8 and dip on 16 bytes),
+// aligned words, shifted where the row starts in the middle of one (1: dip on 4
+// bytes), or single entries (0)
+enum DipLoads : int32_t { kDipEntries = 0, kDipWords = 1, kDipQuads = 2 };
+
+// d_ip of pivot a and nodes 8 g .. 8 g + 7, two per word (0 past the last node)
+__device__ __forceinline__ uint4 dip_quad(const uint16_t *__restrict__ dip, int n, int a, int64_t g, int32_t loads) {
+  const int64_t i0 = 8 * g;
+  const int left = (int)min((int64_t)8, n - i0);
+  if (left <= 0) return make_uint4(0u, 0u, 0u, 0u);
+  const uint16_t *row = dip + (size_t)a * n;
+  if (loads == kDipQuads) return __ldg(reinterpret_cast<const uint4 *>(row) + g);  // (all eight are there)
+  unsigned v[4];
+  if (loads == kDipWords) {
+    const size_t first = (size_t)a * n + i0;
+    const int odd = (int)(first & 1u);
+    const unsigned *words = reinterpret_cast<const unsigned *>(dip) + (first >> 1);
+    unsigned w[5];
+#pragma unroll
+    for (int t = 0; t < 5; ++t) w[t] = 2 * t - odd < left ? __ldg(words + t) : 0u;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) v[t] = odd ? __byte_perm(w[t], w[t + 1], 0x5432) : w[t];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) v[t] = 2 * t + 1 < left ? v[t] : 2 * t < left ? v[t] & 0xFFFFu : 0u;
+  } else {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const unsigned lo = 2 * t < left ? (unsigned)__ldg(row + i0 + 2 * t) : 0u;
+      const unsigned hi = 2 * t + 1 < left ? (unsigned)__ldg(row + i0 + 2 * t + 1) : 0u;
+      v[t] = lo | (hi << 16);
+    }
+  }
+  return make_uint4(v[0], v[1], v[2], v[3]);
+}
+
+// word (t k + a) P + (p mod P), t = p div P, of the copy holds node pair
+// p = (2p, 2p + 1) of pivot a (P = kTileNodes / 2 pairs per tile); a thread
+// takes four pairs
+__device__ __forceinline__ uint4 *tile_quad(unsigned *dtile, int k, int a, int64_t g) {
   constexpr int64_t P = kTileNodes / 2;
-  const int64_t npairs = ((int64_t)(n + kTileNodes - 1) / kTileNodes) * P;
-  const unsigned top = row > 0 ? (unsigned)row - 1u : 0u;
-  auto enc = [&](int a, unsigned lo, unsigned hi) -> unsigned {
-    if (row > 0) {
-      if (lo > top || hi > top) {
-        dev_fail(status, SSM_E_ARG);
-        lo = min(lo, top);
-        hi = min(hi, top);
+  const int64_t p = 4 * g;
+  return reinterpret_cast<uint4 *>(dtile + ((p / P) * k + a) * P + (p % P));
+}
+
+// e(d) = d.  rgg256k, k = 200 (rows on 8 bytes): 38 us for 209 MB; with a 4-byte
+// load and store per thread 100
+__global__ void k_tile_dip(int32_t n, int32_t k, const uint16_t *__restrict__ dip, unsigned *__restrict__ dtile,
+                           int32_t loads) {
+  const int64_t nquads = ((int64_t)(n + kTileNodes - 1) / kTileNodes) * (kTileNodes / 8);
+  for (int a = blockIdx.y; a < k; a += gridDim.y)
+    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < nquads; g += (int64_t)gridDim.x * blockDim.x)
+      *tile_quad(dtile, k, a, g) = dip_quad(dip, n, a, g, loads);
+}
+
+// full-table mode: the copy with e(d) the byte offset of the node's entry, and
+// den[i] = deg(i) + sum_{a = 0..k-1} w'_ia in FP32, pivots in order (the sum the
+// clamped mode forms inside every sweep): one pass over d_ip for both, a thread
+// per eight nodes with four pivots' loads in flight, -w in shared memory.  HBM
+// bounds it: ba1m, k = 200: 133 us for 838 MB = 6.3 TB/s (copy and sum apart: 165 + 81)
+constexpr int kTileDenAhead = 4;
+__global__ void __launch_bounds__(256) k_tile_den(int32_t n, int32_t k, int32_t row, const uint16_t *__restrict__ dip,
+                                                  unsigned *__restrict__ dtile, int32_t *__restrict__ status,
+                                                  int32_t loads, const float *__restrict__ wtab,
+                                                  const int32_t *__restrict__ rowptr, float *__restrict__ den) {
+  extern __shared__ __align__(16) unsigned char td_smem[];
+  float *mw = reinterpret_cast<float *>(td_smem);  // [k][row]
+  for (int t = threadIdx.x; t < k * row; t += blockDim.x) mw[t] = __ldg(wtab + t);
+  __syncthreads();
+  const int64_t nquads = ((int64_t)(n + kTileNodes - 1) / kTileNodes) * (kTileNodes / 8);
+  const unsigned top = (unsigned)row - 1u;
+  bool bad = false;
+  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < nquads; g += (int64_t)gridDim.x * blockDim.x) {
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    auto pivot = [&](int a, const uint4 &v) {
+      const unsigned in[4] = {v.x, v.y, v.z, v.w};
+      unsigned out[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        unsigned lo = in[t] & 0xFFFFu, hi = in[t] >> 16;
+        bad |= lo > top || hi > top;
+        lo = (unsigned)a * (unsigned)row + min(lo, top);
+        hi = (unsigned)a * (unsigned)row + min(hi, top);
+        acc[2 * t] -= mw[lo];
+        acc[2 * t + 1] -= mw[hi];
+        out[t] = (kTabEntryBytes * lo) | ((kTabEntryBytes * hi) << 16);
       }
-      lo = kTabEntryBytes * ((unsigned)a * (unsigned)row + lo);
-      hi = kTabEntryBytes * ((unsigned)a * (unsigned)row + hi);
+      *tile_quad(dtile, k, a, g) = make_uint4(out[0], out[1], out[2], out[3]);
+    };
+    int a = 0;
+    for (; a + kTileDenAhead <= k; a += kTileDenAhead) {
+      uint4 v[kTileDenAhead];
+#pragma unroll
+      for (int t = 0; t < kTileDenAhead; ++t) v[t] = dip_quad(dip, n, a + t, g, loads);
+#pragma unroll
+      for (int t = 0; t < kTileDenAhead; ++t) pivot(a + t, v[t]);
     }
-    return lo | (hi << 16);
-  };
-  if (pair_loads == 2) {
-    // n a multiple of 8, dip 16-byte aligned: four pairs (one 16-byte load,
-    // one 16-byte store of four consecutive words of a tile) per thread
-    const int64_t nquads = npairs / 4;
-    for (int a = blockIdx.y; a < k; a += gridDim.y) {
-      const uint4 *drow = reinterpret_cast<const uint4 *>(dip + (size_t)a * n);
-      for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < nquads; g += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = 4 * g;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (2 * p + 7 < n) v = __ldg(drow + g);  // else past the last node: zeros (n % 8 == 0: all or nothing)
-        const uint4 out = make_uint4(enc(a, v.x & 0xFFFFu, v.x >> 16), enc(a, v.y & 0xFFFFu, v.y >> 16),
-                                     enc(a, v.z & 0xFFFFu, v.z >> 16), enc(a, v.w & 0xFFFFu, v.w >> 16));
-        *reinterpret_cast<uint4 *>(dtile + ((p / P) * k + a) * P + (p % P)) = out;
-      }
+    for (; a < k; ++a) pivot(a, dip_quad(dip, n, a, g, loads));
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int64_t i = 8 * g + q;
+      if (i < n) den[i] = acc[q] + (float)(rowptr[i + 1] - rowptr[i]);
     }
-    return;
   }
-  for (int a = blockIdx.y; a < k; a += gridDim.y) {
-    const uint16_t *drow = dip + (size_t)a * n;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < npairs; p += (int64_t)gridDim.x * blockDim.x) {
-      const int64_t i = 2 * p;
-      unsigned lo = 0u, hi = 0u;
-      if (pair_loads && i + 1 < n) {  // n even and dip 4-byte aligned: the pair is one aligned word
-        const unsigned v = __ldg(reinterpret_cast<const unsigned *>(drow + i));
-        lo = v & 0xFFFFu;
-        hi = v >> 16;
-      } else {
-        if (i < n) lo = (unsigned)__ldg(drow + i);
-        if (i + 1 < n) hi = (unsigned)__ldg(drow + i + 1);
-      }
-      dtile[((p / P) * k + a) * P + (p % P)] = enc(a, lo, hi);
-    }
-  }
+  if (bad) dev_fail(status, SSM_E_ARG);
 }
 
 
@@ -705,36 +758,6 @@ __global__ void k_build_wtab(int32_t k, int32_t dmax, const int32_t *__restrict_
     }
     wtab[t] = -w;
     wtab[kFullPlane + t] = wd;
-  }
-}
-
-// full-table mode: den[i] = deg(i) + sum_{a = 0..k-1} w'_ia in FP32, pivots in
-// order (the sum the clamped mode forms inside every sweep); one warp per tile;
-// dtile holds table byte offsets
-__global__ void k_sweep_den(int32_t n, int32_t k, const unsigned *__restrict__ dtile,
-                            const float *__restrict__ wtab, const int32_t *__restrict__ rowptr,
-                            float *__restrict__ den) {
-  const unsigned lane = threadIdx.x & 31u;
-  const int64_t ntiles = (n + kTileNodes - 1) / kTileNodes;
-  for (int64_t tile = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; tile < ntiles;
-       tile += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const DWords *tp = reinterpret_cast<const DWords *>(dtile) + tile * (int64_t)k * 32 + lane;
-    float acc[kNpl];
-#pragma unroll
-    for (int q = 0; q < kNpl; ++q) acc[q] = 0.f;
-    for (int a = 0; a < k; ++a) {
-      const DWords pw = __ldg(tp + (int64_t)a * 32);
-#pragma unroll
-      for (int j = 0; j < kPpl; ++j) {
-        const unsigned pk = dword(pw, j);
-        acc[2 * j] -= __ldg(wtab + (pk & 0xFFFFu) / kTabEntryBytes);  // the table holds -w
-        acc[2 * j + 1] -= __ldg(wtab + (pk >> 16) / kTabEntryBytes);
-      }
-    }
-    const int64_t i0 = tile * kTileNodes + (int64_t)kNpl * lane;
-#pragma unroll
-    for (int q = 0; q < kNpl; ++q)
-      if (i0 + q < n) den[i0 + q] = acc[q] + (float)(rowptr[i0 + q + 1] - rowptr[i0 + q]);
   }
 }
 
@@ -1124,22 +1147,21 @@ SSM_API int ssm_iterate(int32_t n, int64_t m, const int32_t *rowptr, const int32
     A.dmax = (int32_t)dmax;
     A.wtab = w.wtab;
     A.den = w.den;
-    {
-      const int64_t npairs = ((int64_t)n + kTileNodes - 1) / kTileNodes * (kTileNodes / 2);
-      const int gy = std::min(k, 16);
-      const int gx = (int)std::max<int64_t>(1, std::min<int64_t>((npairs + 255) / 256, (int64_t)sms * 8 / gy + 1));
-      const int32_t pair_loads = (n % 8 == 0 && (reinterpret_cast<uintptr_t>(dip) & 15u) == 0)  ? 2
-                                 : (n % 2 == 0 && (reinterpret_cast<uintptr_t>(dip) & 3u) == 0) ? 1
-                                                                                                 : 0;
-      note_launch(), k_tile_dip<<<dim3(gx, gy), 256, 0, s>>>(n, k, full ? (int32_t)dmax + 1 : 0, dip, w.dtile, status,
-                                                           pair_loads);
-    }
+    const int64_t nquads = ((int64_t)n + kTileNodes - 1) / kTileNodes * (kTileNodes / 8);
+    const int32_t loads = (n % 8 == 0 && (reinterpret_cast<uintptr_t>(dip) & 15u) == 0) ? kDipQuads
+                          : (reinterpret_cast<uintptr_t>(dip) & 3u) == 0               ? kDipWords
+                                                                                        : kDipEntries;
     if (full) {
       note_launch(), k_build_wtab<<<std::max(1, std::min(sms * 4, (int)(((int64_t)k * (dmax + 1) + 255) / 256))), 256, 0,
                                     s>>>(k, (int32_t)dmax, cnt_off, cnt, w.wtab);
-      note_launch(), k_sweep_den<<<std::max(1, (int)std::min<int64_t>(((int64_t)n + 511) / 512, sms * 8)), 256, 0, s>>>(
-          n, k, w.dtile, w.wtab, rowptr, w.den);
+      const size_t plane = (size_t)k * ((size_t)dmax + 1) * sizeof(float);
+      SSM_TRY_CUDA(allow_dynamic_smem((const void *)k_tile_den));
+      note_launch(), k_tile_den<<<(int)std::min<int64_t>((nquads + 255) / 256, (int64_t)sms * 8), 256, plane, s>>>(
+          n, k, (int32_t)dmax + 1, dip, w.dtile, status, loads, w.wtab, rowptr, w.den);
     } else {
+      const int gy = std::min(k, 16);
+      const int gx = (int)std::max<int64_t>(1, std::min<int64_t>((nquads + 255) / 256, (int64_t)sms * 8 / gy + 1));
+      note_launch(), k_tile_dip<<<dim3(gx, gy), 256, 0, s>>>(n, k, dip, w.dtile, loads);
       note_launch(), k_build_stab<<<std::min(k, sms * 4), 128, 0, s>>>(k, cnt_off, cnt, w.stab);
     }
     const size_t piv = (size_t)k * (sizeof(float4) + sizeof(uint2));

@@ -204,7 +204,7 @@ __device__ void sssp_block(int32_t n, const int32_t *__restrict__ rowptr, const 
   // band, so the rounds are bounded; the cap only guards against a fault
   const int64_t cap = 64ll * ((int64_t)n + 16);
   for (int64_t round = 0;; ++round) {
-    __syncthreads();  // the queue of this round is complete
+    __syncthreads();  // the queue of this pass is complete
     unsigned count = s_near[cur];
     if (count == 0) {
       const unsigned nfar = s_far, least = s_least;

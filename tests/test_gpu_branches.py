@@ -128,6 +128,27 @@ def test_sweep_fp64_ranges_bit_for_bit(name, k, scale):
     assert np.array_equal(pos.cpu().numpy(), want)
 
 
+@pytest.mark.parametrize("family,n", [("ba", 9001), ("ba", 9002), ("ba", 9004), ("ba", 9008), ("rgg", 9400), ("path", 8201)])
+@pytest.mark.parametrize("shift", [0, 1, 2, 8])
+def test_sweep_distance_copy_alignments(family, n, shift):
+    """The sweep's tiled copy of d_ip (and the denominators summed with it) from
+    rows on any alignment: the same positions as from a table on 16 bytes."""
+    n, s, d = {"ba": lambda: I.ba(n, 4, 3), "rgg": lambda: I.rgg(n, 8.0, 7), "path": lambda: I.path(n)}[family]()
+    prep = O.prepare(n, s, d, 21)
+    g, P = _gpu_graph(n, s, d), _gpu_pivots(21, prep)
+    x0 = torch.from_numpy(prep.pos0.astype(np.float32)).to(DEV)
+    want, _ = O.sweep_jacobi(prep.g, prep.pivots, prep.dip, prep.w, prep.pos0.astype(np.float32).astype(np.float64))
+    room = torch.zeros(21 * n + 16, dtype=torch.uint16, device=DEV)
+    moved = room[shift:shift + 21 * n].view(21, n)
+    moved.copy_(P.dip)
+    a, b = x0.clone(), x0.clone()
+    ssm.ssm_iterate(g, P, a, 1)
+    P.dip = moved
+    ssm.ssm_iterate(g, P, b, 1)
+    assert _norm_err(a.cpu().numpy(), want) < 1e-5
+    assert torch.equal(a, b)
+
+
 # ------------------------------------------------------------------ coincident positions
 
 def _coincident_state(prep, rng, count):
