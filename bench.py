@@ -286,7 +286,7 @@ def run_gpu(args):
         macs = npass * n * k * k
         kmeans = {"passes": npass, "max_passes": 50, "ms": round(km_ms, 3),
                   "int_mac_per_s": macs / (km_ms * 1e-3), "moved_pivots": int((newp != P.pivots).sum().item()),
-                  "note": "exact 64-bit integer dot products of the assignment (n k^2 per pass) on CUDA cores"}
+                  "note": "dot products of the assignment (n k^2 per pass): tensor-core filter with a proven bound, exact integer products for the candidates it leaves"}
 
     weighted = None
     if not args.no_weighted:
