@@ -629,43 +629,61 @@ __global__ void __launch_bounds__(kSweepThreads, MODE == 2 ? SSM_SWEEP_FULL_MIN_
 // bytes), or single entries (0)
 enum DipLoads : int32_t { kDipEntries = 0, kDipWords = 1, kDipQuads = 2 };
 
-// d_ip of pivot a and nodes 8 g .. 8 g + 7, two per word (0 past the last node)
-__device__ __forceinline__ uint4 dip_quad(const uint16_t *__restrict__ dip, int n, int a, int64_t g, int32_t loads) {
-  const int64_t i0 = 8 * g;
-  const int left = (int)min((int64_t)8, n - i0);
-  if (left <= 0) return make_uint4(0u, 0u, 0u, 0u);
-  const uint16_t *row = dip + (size_t)a * n;
-  if (loads == kDipQuads) return __ldg(reinterpret_cast<const uint4 *>(row) + g);  // (all eight are there)
-  unsigned v[4];
-  if (loads == kDipWords) {
-    const size_t first = (size_t)a * n + i0;
+// the 2 W entries of d_ip from entry `first` on, two per word (0 from the left-th on)
+template <int W>
+struct DipPart {
+  unsigned w[W];
+};
+template <int W>
+__device__ __forceinline__ DipPart<W> dip_part(const uint16_t *__restrict__ dip, size_t first, int left, int32_t loads) {
+  DipPart<W> v;
+  if (loads == kDipQuads) {  // all of them are there, or none
+    if constexpr (W == 4) {
+      const uint4 q = left ? __ldg(reinterpret_cast<const uint4 *>(dip + first)) : make_uint4(0u, 0u, 0u, 0u);
+      v.w[0] = q.x; v.w[1] = q.y; v.w[2] = q.z; v.w[3] = q.w;
+    } else {
+      v.w[0] = left ? __ldg(reinterpret_cast<const unsigned *>(dip + first)) : 0u;
+    }
+  } else if (loads == kDipWords) {
     const int odd = (int)(first & 1u);
     const unsigned *words = reinterpret_cast<const unsigned *>(dip) + (first >> 1);
-    unsigned w[5];
+    unsigned w[W + 1];
 #pragma unroll
-    for (int t = 0; t < 5; ++t) w[t] = 2 * t - odd < left ? __ldg(words + t) : 0u;
+    for (int t = 0; t < W + 1; ++t) w[t] = left > 0 && 2 * t - odd < left ? __ldg(words + t) : 0u;
 #pragma unroll
-    for (int t = 0; t < 4; ++t) v[t] = odd ? __byte_perm(w[t], w[t + 1], 0x5432) : w[t];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) v[t] = 2 * t + 1 < left ? v[t] : 2 * t < left ? v[t] & 0xFFFFu : 0u;
+    for (int t = 0; t < W; ++t) {
+      const unsigned x = odd ? __byte_perm(w[t], w[t + 1], 0x5432) : w[t];
+      v.w[t] = 2 * t + 1 < left ? x : 2 * t < left ? x & 0xFFFFu : 0u;
+    }
   } else {
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const unsigned lo = 2 * t < left ? (unsigned)__ldg(row + i0 + 2 * t) : 0u;
-      const unsigned hi = 2 * t + 1 < left ? (unsigned)__ldg(row + i0 + 2 * t + 1) : 0u;
-      v[t] = lo | (hi << 16);
+    for (int t = 0; t < W; ++t) {
+      const unsigned lo = 2 * t < left ? (unsigned)__ldg(dip + first + 2 * t) : 0u;
+      const unsigned hi = 2 * t + 1 < left ? (unsigned)__ldg(dip + first + 2 * t + 1) : 0u;
+      v.w[t] = lo | (hi << 16);
     }
   }
-  return make_uint4(v[0], v[1], v[2], v[3]);
+  return v;
+}
+
+// how many of the nodes 2 W g .. 2 W (g + 1) - 1 there are
+template <int W>
+__device__ __forceinline__ int part_left(int n, int64_t g) {
+  return (int)max((int64_t)0, min((int64_t)(2 * W), n - 2 * W * g));
 }
 
 // word (t k + a) P + (p mod P), t = p div P, of the copy holds node pair
 // p = (2p, 2p + 1) of pivot a (P = kTileNodes / 2 pairs per tile); a thread
-// takes four pairs
-__device__ __forceinline__ uint4 *tile_quad(unsigned *dtile, int k, int a, int64_t g) {
+// takes W pairs
+template <int W>
+__device__ __forceinline__ void tile_store(unsigned *dtile, int k, int a, int64_t g, const DipPart<W> &v) {
   constexpr int64_t P = kTileNodes / 2;
-  const int64_t p = 4 * g;
-  return reinterpret_cast<uint4 *>(dtile + ((p / P) * k + a) * P + (p % P));
+  const int64_t p = W * g;
+  unsigned *o = dtile + ((p / P) * k + a) * P + (p % P);
+  if constexpr (W == 4)
+    *reinterpret_cast<uint4 *>(o) = make_uint4(v.w[0], v.w[1], v.w[2], v.w[3]);
+  else
+    *o = v.w[0];
 }
 
 // e(d) = d.  rgg256k, k = 200 (rows on 8 bytes): 38 us for 209 MB; with a 4-byte
@@ -675,15 +693,19 @@ __global__ void k_tile_dip(int32_t n, int32_t k, const uint16_t *__restrict__ di
   const int64_t nquads = ((int64_t)(n + kTileNodes - 1) / kTileNodes) * (kTileNodes / 8);
   for (int a = blockIdx.y; a < k; a += gridDim.y)
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < nquads; g += (int64_t)gridDim.x * blockDim.x)
-      *tile_quad(dtile, k, a, g) = dip_quad(dip, n, a, g, loads);
+      tile_store<4>(dtile, k, a, g, dip_part<4>(dip, (size_t)a * n + 8 * g, part_left<4>(n, g), loads));
 }
 
 // full-table mode: the copy with e(d) the byte offset of the node's entry, and
 // den[i] = deg(i) + sum_{a = 0..k-1} w'_ia in FP32, pivots in order (the sum the
 // clamped mode forms inside every sweep): one pass over d_ip for both, a thread
-// per eight nodes with four pivots' loads in flight, -w in shared memory.  HBM
-// bounds it: ba1m, k = 200: 133 us for 838 MB = 6.3 TB/s (copy and sum apart: 165 + 81)
-constexpr int kTileDenAhead = 4;
+// per 2 W nodes with four or eight pivots' loads in flight, -w in shared memory.  HBM
+// bounds it with W = 4: ba1m, k = 200: 133 us for 838 MB = 6.3 TB/s (copy and sum apart: 165 + 81)
+// W = 1 below this many nodes, where the chain over the pivots is the bound and
+// threads are few: n = 20,000: 19 against 37 us, 100,000: 30 against 54, 2^20:
+// 164 against 130
+constexpr int kTileDenSmall = 1 << 18;
+template <int W>
 __global__ void __launch_bounds__(256) k_tile_den(int32_t n, int32_t k, int32_t row, const uint16_t *__restrict__ dip,
                                                   unsigned *__restrict__ dtile, int32_t *__restrict__ status,
                                                   int32_t loads, const float *__restrict__ wtab,
@@ -692,38 +714,42 @@ __global__ void __launch_bounds__(256) k_tile_den(int32_t n, int32_t k, int32_t 
   float *mw = reinterpret_cast<float *>(td_smem);  // [k][row]
   for (int t = threadIdx.x; t < k * row; t += blockDim.x) mw[t] = __ldg(wtab + t);
   __syncthreads();
-  const int64_t nquads = ((int64_t)(n + kTileNodes - 1) / kTileNodes) * (kTileNodes / 8);
+  const int64_t parts = ((int64_t)(n + kTileNodes - 1) / kTileNodes) * (kTileNodes / (2 * W));
   const unsigned top = (unsigned)row - 1u;
   bool bad = false;
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < nquads; g += (int64_t)gridDim.x * blockDim.x) {
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    auto pivot = [&](int a, const uint4 &v) {
-      const unsigned in[4] = {v.x, v.y, v.z, v.w};
-      unsigned out[4];
+  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < parts; g += (int64_t)gridDim.x * blockDim.x) {
+    float acc[2 * W];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        unsigned lo = in[t] & 0xFFFFu, hi = in[t] >> 16;
+    for (int q = 0; q < 2 * W; ++q) acc[q] = 0.f;
+    auto pivot = [&](int a, const DipPart<W> &v) {
+      DipPart<W> out;
+#pragma unroll
+      for (int t = 0; t < W; ++t) {
+        unsigned lo = v.w[t] & 0xFFFFu, hi = v.w[t] >> 16;
         bad |= lo > top || hi > top;
         lo = (unsigned)a * (unsigned)row + min(lo, top);
         hi = (unsigned)a * (unsigned)row + min(hi, top);
         acc[2 * t] -= mw[lo];
         acc[2 * t + 1] -= mw[hi];
-        out[t] = (kTabEntryBytes * lo) | ((kTabEntryBytes * hi) << 16);
+        out.w[t] = (kTabEntryBytes * lo) | ((kTabEntryBytes * hi) << 16);
       }
-      *tile_quad(dtile, k, a, g) = make_uint4(out[0], out[1], out[2], out[3]);
+      tile_store<W>(dtile, k, a, g, out);
     };
+    constexpr int kAhead = W == 4 ? 4 : 8;
+    const int left = part_left<W>(n, g);
+    size_t first = (size_t)(2 * W * g);
     int a = 0;
-    for (; a + kTileDenAhead <= k; a += kTileDenAhead) {
-      uint4 v[kTileDenAhead];
+    for (; a + kAhead <= k; a += kAhead) {
+      DipPart<W> v[kAhead];
 #pragma unroll
-      for (int t = 0; t < kTileDenAhead; ++t) v[t] = dip_quad(dip, n, a + t, g, loads);
+      for (int t = 0; t < kAhead; ++t, first += (size_t)n) v[t] = dip_part<W>(dip, first, left, loads);
 #pragma unroll
-      for (int t = 0; t < kTileDenAhead; ++t) pivot(a + t, v[t]);
+      for (int t = 0; t < kAhead; ++t) pivot(a + t, v[t]);
     }
-    for (; a < k; ++a) pivot(a, dip_quad(dip, n, a, g, loads));
+    for (; a < k; ++a, first += (size_t)n) pivot(a, dip_part<W>(dip, first, left, loads));
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int64_t i = 8 * g + q;
+    for (int q = 0; q < 2 * W; ++q) {
+      const int64_t i = 2 * W * g + q;
       if (i < n) den[i] = acc[q] + (float)(rowptr[i + 1] - rowptr[i]);
     }
   }
@@ -1155,8 +1181,12 @@ SSM_API int ssm_iterate(int32_t n, int64_t m, const int32_t *rowptr, const int32
       note_launch(), k_build_wtab<<<std::max(1, std::min(sms * 4, (int)(((int64_t)k * (dmax + 1) + 255) / 256))), 256, 0,
                                     s>>>(k, (int32_t)dmax, cnt_off, cnt, w.wtab);
       const size_t plane = (size_t)k * ((size_t)dmax + 1) * sizeof(float);
-      SSM_TRY_CUDA(allow_dynamic_smem((const void *)k_tile_den));
-      note_launch(), k_tile_den<<<(int)std::min<int64_t>((nquads + 255) / 256, (int64_t)sms * 8), 256, plane, s>>>(
+      const bool small = n < kTileDenSmall;
+      auto den_kernel = small ? k_tile_den<1> : k_tile_den<4>;
+      const int64_t parts = small ? 4 * nquads : nquads;
+      const int threads = small ? 128 : 256;
+      SSM_TRY_CUDA(allow_dynamic_smem((const void *)den_kernel));
+      note_launch(), den_kernel<<<(int)std::min<int64_t>((parts + threads - 1) / threads, (int64_t)sms * 8), threads, plane, s>>>(
           n, k, (int32_t)dmax + 1, dip, w.dtile, status, loads, w.wtab, rowptr, w.den);
     } else {
       const int gy = std::min(k, 16);
