@@ -94,7 +94,7 @@ __device__ int block_exclusive_scan(int *a, int len, int *s_part) {
 // per block.  The searches are chains of short levels (10 to 30 nodes wide
 // after the first few pivots): block_search, the offsets in shared memory and
 // the neighbours too where they fit.  512 graphs of 64 to 8192 nodes, k = 100: a
-// batch takes as long as its largest graph (1,700 levels), 1.38 ms; with a lane
+// batch takes as long as its largest graph (1,700 levels), 1.53 ms; with a lane
 // per node, neighbours in global memory and a queue atomic per node a level
 // took 4,500 cycles, and the searches below were part of the same block: 18.4 ms.
 __global__ void __launch_bounds__(kPrepThreads) k_prep_pivots(PrepArgs A) {
