@@ -26,7 +26,7 @@ namespace ssm {
 constexpr int kPrepMaxN = 12288;
 constexpr int kPrepMaxK = 100;
 constexpr int kPrepThreads = 512;
-constexpr int kDistThreads = 1024;  // (512: 2.3 ms against 1.7 on the batch at k_prep_dist)
+constexpr int kDistThreads = 1024;
 
 struct PrepDev {
   int32_t n, k;
@@ -253,7 +253,10 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_pivots(PrepArgs A) {
 // lanes per listed node store its distances and pass the bits on to neighbours
 // that do not have them (shared-memory reductions that return nothing).  The
 // work of a level is the nodes that changed, so that long thin graphs pay for
-// their two or three nodes per level and a scan of n / 512 words per thread.
+// their two or three nodes per level and a scan of n / 1024 words per thread.
+// 1.7 ms for the batch at k_prep_pivots, 2.3 with 512 threads; a queue of single
+// (pivot, node) pairs in global memory took 18 M cycles (9 ms) of the largest
+// graph's block alone.
 __global__ void __launch_bounds__(kDistThreads) k_prep_dist(PrepArgs A) {
   extern __shared__ __align__(16) unsigned char psm[];
   __shared__ int s_task;
