@@ -14,26 +14,24 @@
 // above kScLong entries are a warp's work each, and a node's W + 1 partial sums
 // are added in order.  (Lanes sharing a node, each with its own pivots, took
 // 1.4 to 5 times as long: every pivot position and table entry was a gather.)
-// At the end of an iteration a CTA copies its new positions into the other
-// buffer of every CTA (bulk copies through distributed shared memory, which
-// complete on an mbarrier of the receiver), and goes on when all of the others'
-// have arrived: no cluster barrier.  A CTA sends X^{t+1} after it has read X^t
-// for the last time, so a sender that has received everybody's X^{t+1} may write
-// X^{t+2} over X^t; barriers alternate with the buffers for the same reason.
+// A CTA stores its new positions into the other buffer of every CTA (distributed
+// shared memory; warps that would be idle each serve some of the receivers), and
+// an iteration ends at the hardware's cluster barrier: every CTA makes the same
+// number of them, also one that owns no node, and none writes to another after
+// the last.  X^{t+1} goes into the buffer that was read before the last barrier.
 //
 // The update is the single-graph sweep's form about x_i: x_i + (sum_a (B - w)
 // (x_i - x_p) + sum_j (x_j - x_i)(1 - 1/r)) / den, B = w d / r, with r^2 + 1e-24
 // so that coincident points add nothing; only the order of a node's sum differs
-// (fixed here too).  Bound by latency: shared-memory gathers, two block
-// barriers and the copies.  Measured (us an iteration, two kernels on the whole
-// GPU before, here): grid of 1,024 nodes, k = 50: 14.4, 2.1; Barabasi-Albert
-// graph of 8,000 nodes, k = 60: 18.3, 6.8; of 4,096 nodes, k = 200: 24, 7.2.
+// (fixed here too).  Bound by latency: shared-memory gathers, a block barrier,
+// the stores and the cluster barrier.  Measured (us an iteration, two kernels on
+// the whole GPU, here): grid of 1,024 nodes, k = 50: 14.1, 2.2; Barabasi-Albert
+// graph of 8,000 nodes, k = 60: 18.8, 8.0; of 4,096 nodes, k = 200: 25.2, 7.6.
 #include <algorithm>
 
 #include "cluster.cuh"
 #include "common.cuh"
 #include "sweep.cuh"
-#include "tc.cuh"
 
 namespace ssm {
 
@@ -65,12 +63,8 @@ __device__ __forceinline__ float sc_rsqrt(float x) {
   return y;
 }
 
-// one thread: `bytes` (a multiple of 16) of this CTA's shared memory to the
-// address dst of another CTA, completing on that CTA's mbarrier
-__device__ __forceinline__ void dsmem_bulk_copy(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t mbar) {
-  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "r"(src), "r"(bytes), "r"(mbar)
-               : "memory");
+__device__ __forceinline__ void dsmem_st_f2(uint32_t a, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
 }
 
 __device__ __forceinline__ void dsmem_st_d2(uint32_t a, double x, double y) {
@@ -91,7 +85,6 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
   extern __shared__ __align__(16) unsigned char sc_smem[];
   __shared__ double s_red[2][kScThreads / 32];
   __shared__ __align__(16) double2 s_part[2][kScMaxCluster];
-  __shared__ __align__(8) uint64_t s_bar[2];  // X^t of the other CTAs has arrived, by parity of t
   const int n = A.n, k = A.k, D = A.dmax + 1;
   unsigned C;
   asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
@@ -186,22 +179,14 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
   }
   const int W = A.warps, blocks = A.perp / 64, blk = warp / W, wb = warp - blk * W;
   const int l0 = 64 * blk + 2 * lane;  // this lane's nodes l0, l0 + 1 (blk < blocks)
-  // bytes of the others' positions (every CTA sends an even number of nodes)
-  unsigned expect = 0;
-  for (unsigned c = 0; c < C; ++c)
-    if (c != r && n > (int)c) expect += 8u * (unsigned)(((n - 1 - (int)c) / (int)C + 2) & ~1);
-  if (tid == 0) {
-    for (int q = 0; q < 2; ++q) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_smem(&s_bar[q])));
-    asm volatile("fence.mbarrier_init.release.cluster;");
-  }
+  // warps of own nodes, and how many warps share the stores of one of them
+  const int nw = (own + 31) / 32, share = nw > 0 ? max(1, min((int)C, T / 32 / nw)) : 1;
   cluster_sync();  // every CTA of the cluster runs, and has read pos, before any remote write
 
   int it = 0;
-  bool ok = true;
   for (; it < A.iters; ++it) {
     const float2 *Xc = X + (size_t)(it & 1) * stride;
     float2 *Xn = X + (size_t)((it & 1) ^ 1) * stride;
-    const uint32_t bar = tc_smem(&s_bar[(it + 1) & 1]);
     const bool change = A.tol > 0.0 || it + 1 == A.iters;
     if (blk < blocks) {
       const float2 x0 = l0 < own ? Xc[i0 + l0] : make_float2(0.f, 0.f), x1 = l0 + 1 < own ? Xc[i0 + l0 + 1] : make_float2(0.f, 0.f);
@@ -241,7 +226,9 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
     }
     __syncthreads();
     float cn = 0.f, cd = 0.f;
-    for (int li = tid; li < own; li += T) {
+    for (int u = warp; u < nw * share; u += T / 32) {
+      const int sh = u / nw, li = (u - sh * nw) * 32 + lane;
+      if (li >= own) continue;
       const float2 x = Xc[i0 + li];
       float ax = 0.f, ay = 0.f;
 #pragma unroll 4
@@ -250,13 +237,17 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
         ax += v.x;
         ay += v.y;
       }
-      const float dn = den[li], chk = ax + ay;
-      if (!(chk == chk)) dev_fail(A.status, SSM_E_NUMERIC);
+      const float dn = den[li];
       const float ex = dn > 0.f ? ax / dn : 0.f, ey = dn > 0.f ? ay / dn : 0.f;
-      Xn[i0 + li] = make_float2(x.x + ex, x.y + ey);
+      for (unsigned c = (unsigned)sh; c < C; c += (unsigned)share)
+        dsmem_st_f2(dsmem_addr(Xn + i0 + li, c), make_float2(x.x + ex, x.y + ey));
+      if (sh > 0) continue;
+      const float chk = ax + ay;
+      if (!(chk == chk)) dev_fail(A.status, SSM_E_NUMERIC);
       cn = fmaf(ex, ex, fmaf(ey, ey, cn));
       cd = fmaf(x.x, x.x, fmaf(x.y, x.y, cd));
     }
+    __syncwarp();
     if (change) {  // ||X^{t+1} - X^t||_F / ||X^t||_F: lanes, warps and CTAs in a fixed order
       double tn = (double)cn, td = (double)cd;
 #pragma unroll
@@ -280,25 +271,9 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
         if ((unsigned)lane < C) dsmem_st_d2(dsmem_addr(&s_part[it & 1][r], (unsigned)lane), tn, td);
       }
     }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the copies read what was just written
-    __syncthreads();
-    if (warp == 0) {
-      if (lane == 0)
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(expect) : "memory");
-      __syncwarp();
-      if ((unsigned)lane < C && (unsigned)lane != r && own > 0)
-        dsmem_bulk_copy(dsmem_addr(Xn + i0, (unsigned)lane), tc_smem(Xn + i0), 8u * (unsigned)((own + 1) & ~1),
-                        dsmem_addr(&s_bar[(it + 1) & 1], (unsigned)lane));
-    }
-    // the (it / 2)-th use of this barrier; a CTA that gives up takes the others,
-    // whose waits then run out, with it
-    ok = tc_wait(bar, (unsigned)(it >> 1) & 1u);
-    if (!__syncthreads_and(ok ? 1 : 0)) {
-      ok = false;
-      break;
-    }
+    __syncwarp();
+    cluster_sync();  // X^{t+1} and the partial sums are everywhere
     if (change) {
-      cluster_sync();  // the partial sums
       double num = 0.0, dn = 0.0;
       for (unsigned c = 0; c < C; ++c) {
         num += s_part[it & 1][c].x;
@@ -315,10 +290,8 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
       }
     }
   }
-  if (!ok) dev_fail(A.status, SSM_E_TIMEOUT);
   const float2 *Xf = X + (size_t)(it & 1) * stride;
   for (int t = tid; t < own; t += T) A.pos[t * (int)C + (int)r] = Xf[i0 + t];
-  cluster_sync();  // no CTA leaves while another may still write its shared memory
 }
 
 static size_t sc_smem_bytes(int32_t C, int32_t per, int32_t k, int32_t D, int32_t perp, int32_t warps) {
@@ -339,7 +312,7 @@ int launch_sweep_cluster(int32_t n, int64_t m, const int32_t *rowptr, const int3
   const void *kern = (const void *)k_sweep_cluster;
   for (int C : {16, 8}) {
     ScArgs A;
-    A.per = ((n + C - 1) / C + 1) & ~1;  // even: copies start on 16 bytes
+    A.per = (n + C - 1) / C;
     A.perp = (A.per + 63) / 64 * 64;
     const int threads = (int64_t)A.per * k < kScWide ? kScThreads / 2 : kScThreads;
     A.warps = std::max(1, threads / 32 / (A.perp / 64));

@@ -254,3 +254,31 @@ def test_sweep_fp32_cluster_tolerance_and_wrong_hint():
     with pytest.raises(ssm.SSMError) as e:
         ssm.ssm_iterate(g, P, pos, 4)
     assert e.value.code == -1
+
+
+@pytest.mark.parametrize("n", [2, 7, 8, 15, 16, 17])
+def test_sweep_fp32_cluster_of_few_nodes(n):
+    """Clusters in which some CTAs own no node, over many iterations: every one
+    of them takes part in every exchange, so a run gives the same bits again,
+    cut in two, and stopped by the tolerance."""
+    s, d = np.arange(n - 1, dtype=np.int32), np.arange(1, n, dtype=np.int32)
+    g = _gpu_graph(n, s, d)
+    piv = torch.arange(n, dtype=torch.int32, device=DEV)
+    dip = ssm.ssm_pivot_bfs(g, piv)
+    cnt_len, dmax = ssm.ssm_aggregate_size(dip, with_dmax=True)
+    P = ssm.Pivots(n, piv, dip, *ssm.ssm_aggregate(dip, cnt_len), dmax)
+    x0 = torch.from_numpy((np.random.default_rng(n).standard_normal((n, 2)) * n).astype(np.float32)).to(DEV)
+
+    def run(*cuts, tol=0.0):
+        x = x0.clone()
+        for iters in cuts:
+            done, rel = ssm.ssm_iterate(g, P, x, iters, tol)
+        assert ssm.ssm_last_sweep_config()["kernel"] == "f32_cluster"
+        return x, int(done.item()), rel.item()
+
+    x, done, _ = run(400)
+    assert done == 400 and torch.isfinite(x).all()
+    assert torch.equal(run(400)[0], x) and torch.equal(run(150, 250)[0], x)
+    y, done, rel = run(400, tol=1e-2)
+    assert done == 400 or rel < 1e-2
+    assert done < 4 or torch.equal(run(done)[0], y)
