@@ -1140,7 +1140,8 @@ SSM_API int ssm_iterate(int32_t n, int64_t m, const int32_t *rowptr, const int32
     }
     // small graphs: all iterations in one cluster launch
     auto in_cluster = [&](int *blocks) {
-      return launch_sweep_cluster(n, m, rowptr, colidx, k, pivots, dip, cnt_off, cnt, (int32_t)meta[0], (float2 *)pos, iters,
+      return launch_sweep_cluster(n, m, rowptr, colidx, k, pivots, dip, cnt_off, cnt, (int32_t)meta[0], (int32_t)meta[2],
+                                  (float2 *)pos, iters,
                                   tol, iters_done, rel_change, status, s, blocks);
     };
     auto note_cluster = [&](int blocks) {

@@ -11,7 +11,7 @@
 // CTA: node v at (v mod C) per + v div C.  A lane has two consecutive nodes (packed FP32x2), so a pivot's
 // position is one broadcast and its table row is shared by 64 nodes; the warps
 // of a 64-node block share its pivots and neighbours (warp w every W-th), rows
-// above kScLong entries are a warp's work each, and a node's W + 1 partial sums
+// above kScLong entries are a warp's work each (hubs: below), and a node's W + 1 partial sums
 // are added in order.  (Lanes sharing a node, each with its own pivots, took
 // 1.4 to 5 times as long: every pivot position and table entry was a gather.)
 // A CTA stores its new positions into the other buffer of every CTA (distributed
@@ -25,8 +25,14 @@
 // so that coincident points add nothing; only the order of a node's sum differs
 // (fixed here too).  Bound by latency: shared-memory gathers, a block barrier,
 // the stores and the cluster barrier.  Measured (us an iteration, two kernels on
-// the whole GPU, here): grid of 1,024 nodes, k = 50: 14.1, 2.2; Barabasi-Albert
-// graph of 8,000 nodes, k = 60: 18.8, 8.0; of 4,096 nodes, k = 200: 25.2, 7.6.
+// the whole GPU, here): grid of 1,024 nodes, k = 50: 14.1, 2.3; Barabasi-Albert
+// graph of 8,000 nodes, k = 60: 18.8, 8.6; of 4,096 nodes, k = 200: 25.2, 7.8.
+//
+// Rows above kScHub entries, where a CTA has few of them, are cut into segments
+// that all its warps share (star of 8,000 nodes: 20.5, and 21 with a warp per
+// row; 6.9 so).  A CTA keeps the neighbours that its shared memory has room for
+// and reads the others from L2 in every iteration, which 16 SMs of one GPC do at
+// some 0.5 TB/s: the limit to this form on dense graphs (kScMaxRead).
 #include <algorithm>
 
 #include "cluster.cuh"
@@ -38,15 +44,25 @@ namespace ssm {
 constexpr int kScThreads = 1024;  // half as many where a CTA has fewer than kScWide (node, pivot) pairs
 constexpr int kScWide = 8192;
 constexpr int kScLong = 16;       // longest row that one lane per warp walks
+constexpr int kScHub = kMidDeg;   // longest row that one warp walks, if a CTA has few that are longer
+constexpr int kScMaxHubs = 64;    // (above this many they fill the warps as they are)
+constexpr int kScHubSegs = 128;   // a hub's entries per warp: so that these and one per hub are enough,
+constexpr int kScMinSeg = 256;    // and at least this many
 constexpr int kScMaxCluster = 16;
 constexpr int kScMaxN = 8192;     // node ids in 16 bits
 constexpr int kScMaxD = 4095;     // d^2 exact in FP32
 constexpr int kScMinIters = 4;    // the tables are formed by every launch
+// Neighbours per CTA, on average, beyond its shared memory: with 55,000 (8,000
+// nodes of degree 200, k = 3) 25 us an iteration against 15 in two kernels; with
+// 45,000 (clique of 1,500, k = 2) 16.0 against 15.5; with 12,000 (clique of 1,300,
+// k = 50) 13.9 against 18.3
+constexpr int64_t kScMaxRead = 49152;
 constexpr float kScR2Floor = 1e-24f;
 
 struct ScArgs {
   int32_t n, k, dmax, per, perp, warps, iters;  // nodes per CTA (perp: up to whole blocks), warps per 64-node block
   int32_t ecap;  // neighbour ids of a CTA kept in shared memory
+  int32_t hubs;  // there are rows above kScHub: the hubs' lists are part of the shared memory
   const int32_t *rowptr, *colidx, *pivots, *cnt_off;
   const uint32_t *cnt;
   const uint16_t *dip;
@@ -55,6 +71,13 @@ struct ScArgs {
   int32_t *iters_done;
   double *rel_change;
   int32_t *status;
+};
+
+// rows of a CTA that all its warps share, in segments
+struct ScHubs {
+  float2 sum[kScHubSegs + kScMaxHubs];
+  int seg[kScHubSegs + kScMaxHubs];  // node | number of the segment << 16
+  int node[kScMaxHubs], first[kScMaxHubs];  // a hub, and the place of its first segment
 };
 
 __device__ __forceinline__ float sc_rsqrt(float x) {
@@ -81,6 +104,53 @@ __device__ __forceinline__ void sc_edge(const float2 *Xc, int j, float2 x, float
   sy = fmaf(ey, f, sy);
 }
 
+// the whole warp: the terms of the neighbours whose places are place[b .. e - 1],
+// or (place null) those of the graph's entries col[b .. e - 1], at(id) their
+// places, about the node at place `self` (whose own term, past the end, is
+// zero); the sum in every lane
+template <class At>
+__device__ __forceinline__ float2 sc_row(const float2 *Xc, const uint16_t *place, const int32_t *__restrict__ col, int b,
+                                         int e, int self, At at) {
+  constexpr int U = 8;  // neighbours per lane in flight
+  const float2 x = Xc[self];
+  float sx = 0.f, sy = 0.f;
+  const int lane = (int)(threadIdx.x & 31u);
+  auto edges = [&](const int (&j)[U]) {
+#pragma unroll
+    for (int q = 0; q < U; ++q) sc_edge(Xc, j[q], x, sx, sy);
+  };
+  if (place && e - b <= 16 * U) {
+    for (int t = b + lane; t < e; t += 32) sc_edge(Xc, place[t], x, sx, sy);
+  } else if (place) {
+    for (int t0 = b; t0 < e; t0 += 32 * U) {
+      int j[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) j[q] = t0 + 32 * q + lane < e ? place[t0 + 32 * q + lane] : self;
+      edges(j);
+    }
+  } else {
+    int v[U];  // the next ids are on their way while these are used
+#pragma unroll
+    for (int q = 0; q < U; ++q) v[q] = __ldg(col + min(b + lane + 32 * q, e - 1));
+    for (int t0 = b; t0 < e; t0 += 32 * U) {
+      int j[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        j[q] = t0 + 32 * q + lane < e ? at(v[q]) : self;
+        v[q] = __ldg(col + min(t0 + 32 * (U + q) + lane, e - 1));
+      }
+      edges(j);
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    sx += __shfl_xor_sync(0xffffffffu, sx, o);
+    sy += __shfl_xor_sync(0xffffffffu, sy, o);
+  }
+  return make_float2(sx, sy);
+}
+
 __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
   extern __shared__ __align__(16) unsigned char sc_smem[];
   __shared__ double s_red[2][kScThreads / 32];
@@ -98,13 +168,15 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
   int32_t *start = lrows + A.perp;                            // [perp] entry of the graph's rows less the local one
   int32_t *pnode = start + A.perp;                            // [k]
   uint16_t *place = reinterpret_cast<uint16_t *>(pnode + ((k + 1) & ~1));  // [k][perp]
-  uint16_t *cols = place + (size_t)k * A.perp;                // [ecap]
-  __shared__ int s_nlong;
+  ScHubs *hub = reinterpret_cast<ScHubs *>(place + (size_t)k * A.perp);
+  uint16_t *cols = reinterpret_cast<uint16_t *>(hub + (A.hubs ? 1 : 0));  // [ecap]
+  __shared__ int s_nlong, s_nhub, s_hubsum, s_nseg;
   const unsigned r = cluster_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int T = (int)blockDim.x;
   const int i0 = (int)r * A.per, own = n > (int)r ? (n - 1 - (int)r) / (int)C + 1 : 0;  // nodes r, r + C, ...
-  auto at = [&](int v) { return (v % (int)C) * A.per + v / (int)C; };
+  const int cs = 31 - __clz((int)C);
+  auto at = [&](int v) { return (v & ((int)C - 1)) * A.per + (v >> cs); };
 
   for (int i = tid; i < n; i += T) X[at(i)] = A.pos[i];
   // w = s / d^2, w d = s / d from exact operands (s <= n, d^2 < 2^24), each rounded once
@@ -127,7 +199,7 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
     pnode[a] = at(p);
   }
   if (tid == 0) {
-    s_nlong = 0;
+    s_nlong = s_nhub = s_hubsum = s_nseg = 0;
     rows[0] = 0;
   }
   if (warp == 0) {  // local row starts
@@ -145,20 +217,51 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
     }
   }
   __syncthreads();
-  const bool cols_here = rows[own] <= A.ecap;  // else read from the graph, entry by entry
+  auto here = [&](int li) { return rows[li + 1] <= A.ecap; };  // a row's neighbours are kept; else read from the graph
   for (int li = tid; li < own; li += T) {
     const int e = __ldg(A.rowptr + li * (int)C + (int)r), t0 = rows[li], len = rows[li + 1] - t0;
     start[li] = e - t0;
-    if (cols_here && len <= kScLong)
+    if (len <= kScLong && here(li))
       for (int t = 0; t < len; ++t) cols[t0 + t] = (uint16_t)at(__ldg(A.colidx + e + t));
+    if (len > kScHub) {
+      atomicAdd(&s_nhub, 1);
+      atomicAdd(&s_hubsum, len);
+    }
   }
   __syncthreads();
-  if (cols_here)  // long rows, a warp each
-    for (int li = warp; li < own; li += T / 32) {
-      const int t0 = rows[li], len = rows[li + 1] - t0;
-      if (len > kScLong)
-        for (int t = lane; t < len; t += 32) cols[t0 + t] = (uint16_t)at(__ldg(A.colidx + start[li] + t0 + t));
+  const int nhub = A.hubs && s_nhub <= kScMaxHubs ? s_nhub : 0, hublen = nhub ? kScHub : 0x7FFFFFFF;
+  const int seg = max(kScMinSeg, (s_hubsum + kScHubSegs - 1) / kScHubSegs);
+  __syncthreads();
+  if (tid == 0) s_nhub = 0;
+  __syncthreads();
+  // long rows and hubs, in any order: every row is a sum of its own
+  for (int li = tid; li < own; li += T) {
+    const int len = rows[li + 1] - rows[li];
+    if (len > hublen) {
+      const int h = atomicAdd(&s_nhub, 1), c = (len + seg - 1) / seg, first = atomicAdd(&s_nseg, c);
+      hub->node[h] = li;
+      hub->first[h] = first;
+      for (int q = 0; q < c; ++q) hub->seg[first + q] = li | q << 16;
+    } else if (len > kScLong) {
+      lrows[atomicAdd(&s_nlong, 1)] = li;
     }
+  }
+  __syncthreads();
+  auto keep = [&](int li, int first, int step) {  // a row's neighbours, eight loads in flight
+    if (!here(li)) return;
+    const int32_t *col = A.colidx + start[li];
+    const int e = rows[li + 1];
+    for (int t = rows[li] + first; t < e; t += 8 * step) {
+      int v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = __ldg(col + min(t + q * step, e - 1));
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (t + q * step < e) cols[t + q * step] = (uint16_t)at(v[q]);
+    }
+  };
+  for (int q = warp; q < s_nlong; q += T / 32) keep(lrows[q], lane, 32);  // long rows, a warp each
+  for (int h = 0; h < nhub; ++h) keep(hub->node[h], tid, T);              // hubs, all threads
   for (int t = tid; t < A.perp * k; t += T) {
     const int a = t / A.perp, li = t - a * A.perp;
     unsigned d = li < own ? __ldg(A.dip + (size_t)a * n + li * (int)C + (int)r) : 0u;
@@ -175,7 +278,6 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
     for (int a = 0; a < k; ++a) acc -= tab[place[a * A.perp + li]].x;
     den[li] = acc + (float)deg;
     part[(size_t)A.warps * A.perp + li] = make_float2(0.f, 0.f);
-    if (deg > kScLong) lrows[atomicAdd(&s_nlong, 1)] = li;  // in any order: every row is a sum of its own
   }
   const int W = A.warps, blocks = A.perp / 64, blk = warp / W, wb = warp - blk * W;
   const int l0 = 64 * blk + 2 * lane;  // this lane's nodes l0, l0 + 1 (blk < blocks)
@@ -207,22 +309,41 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         const int rb = rows[l0 + q], re = rows[l0 + q + 1];
-        if (re - rb <= kScLong)
-          for (int t = rb + wb; t < re; t += W) sc_edge(Xc, cols_here ? cols[t] : at(__ldg(A.colidx + start[l0 + q] + t)), q ? x1 : x0, sx[q], sy[q]);
+        if (re - rb <= kScLong) {
+          const bool in = re <= A.ecap;
+          for (int t = rb + wb; t < re; t += W)
+            sc_edge(Xc, in ? cols[t] : at(__ldg(A.colidx + start[l0 + q] + t)), q ? x1 : x0, sx[q], sy[q]);
+        }
         part[(size_t)wb * A.perp + l0 + q] = make_float2(sx[q], sy[q]);
       }
     }
     for (int q = warp; q < s_nlong; q += T / 32) {
       const int li = lrows[q];
-      const float2 x = Xc[i0 + li];
-      float sx = 0.f, sy = 0.f;
-      for (int t = rows[li] + lane; t < rows[li + 1]; t += 32) sc_edge(Xc, cols_here ? cols[t] : at(__ldg(A.colidx + start[li] + t)), x, sx, sy);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        sx += __shfl_xor_sync(0xffffffffu, sx, o);
-        sy += __shfl_xor_sync(0xffffffffu, sy, o);
+      const float2 v = sc_row(Xc, here(li) ? cols : nullptr, A.colidx + start[li], rows[li], rows[li + 1], i0 + li, at);
+      if (lane == 0) part[(size_t)W * A.perp + li] = v;
+    }
+    if (nhub) {  // a segment per warp, then a hub per warp
+      for (int q = warp; q < s_nseg; q += T / 32) {
+        const int li = hub->seg[q] & 0xFFFF, b = rows[li] + (hub->seg[q] >> 16) * seg;
+        const float2 v = sc_row(Xc, here(li) ? cols : nullptr, A.colidx + start[li], b, min(b + seg, rows[li + 1]), i0 + li, at);
+        if (lane == 0) hub->sum[q] = v;
       }
-      if (lane == 0) part[(size_t)W * A.perp + li] = make_float2(sx, sy);
+      __syncthreads();
+      for (int h = warp; h < nhub; h += T / 32) {
+        const int li = hub->node[h], c = (rows[li + 1] - rows[li] + seg - 1) / seg;
+        float sx = 0.f, sy = 0.f;
+        for (int q = lane; q < c; q += 32) {
+          sx += hub->sum[hub->first[h] + q].x;
+          sy += hub->sum[hub->first[h] + q].y;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          sx += __shfl_xor_sync(0xffffffffu, sx, o);
+          sy += __shfl_xor_sync(0xffffffffu, sy, o);
+        }
+        if (lane == 0) part[(size_t)W * A.perp + li] = make_float2(sx, sy);
+      }
     }
     __syncthreads();
     float cn = 0.f, cd = 0.f;
@@ -294,15 +415,15 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
   for (int t = tid; t < own; t += T) A.pos[t * (int)C + (int)r] = Xf[i0 + t];
 }
 
-static size_t sc_smem_bytes(int32_t C, int32_t per, int32_t k, int32_t D, int32_t perp, int32_t warps) {
-  return ((size_t)2 * per * C + (size_t)k * D + (size_t)(warps + 1) * perp) * sizeof(float2) + (size_t)perp * 4 +
+static size_t sc_smem_bytes(int32_t C, int32_t per, int32_t k, int32_t D, int32_t perp, int32_t warps, int32_t hubs) {
+  return (hubs ? sizeof(ScHubs) : 0) + ((size_t)2 * per * C + (size_t)k * D + (size_t)(warps + 1) * perp) * sizeof(float2) + (size_t)perp * 4 +
          (size_t)(3 * perp + 2) * 4 + (size_t)((k + 1) & ~1) * 4 + (size_t)perp * k * 2;
 }
 
 int launch_sweep_cluster(int32_t n, int64_t m, const int32_t *rowptr, const int32_t *colidx, int32_t k,
                          const int32_t *pivots, const uint16_t *dip, const int32_t *cnt_off, const uint32_t *cnt,
-                         int32_t dmax, float2 *pos, int32_t iters, double tol, int32_t *iters_done, double *rel_change,
-                         int32_t *status, cudaStream_t s, int *blocks) {
+                         int32_t dmax, int32_t long_rows, float2 *pos, int32_t iters, double tol, int32_t *iters_done,
+                         double *rel_change, int32_t *status, cudaStream_t s, int *blocks) {
   *blocks = 0;
   if (n > kScMaxN || dmax > kScMaxD || iters < kScMinIters || (int64_t)k * (dmax + 1) > 65535) return SSM_OK;
   int dev = 0, smem_max = 0;
@@ -312,16 +433,18 @@ int launch_sweep_cluster(int32_t n, int64_t m, const int32_t *rowptr, const int3
   const void *kern = (const void *)k_sweep_cluster;
   for (int C : {16, 8}) {
     ScArgs A;
+    A.hubs = long_rows > 0;
     A.per = (n + C - 1) / C;
     A.perp = (A.per + 63) / 64 * 64;
     const int threads = (int64_t)A.per * k < kScWide ? kScThreads / 2 : kScThreads;
     A.warps = std::max(1, threads / 32 / (A.perp / 64));
     if (A.perp / 64 > threads / 32) continue;  // a warp has one block of nodes
     // fewer partial sums where the table leaves no room for them
-    while (A.warps > 1 && sc_smem_bytes(C, A.per, k, dmax + 1, A.perp, A.warps) > budget) A.warps /= 2;
-    const size_t fixed = sc_smem_bytes(C, A.per, k, dmax + 1, A.perp, A.warps);
+    while (A.warps > 1 && sc_smem_bytes(C, A.per, k, dmax + 1, A.perp, A.warps, A.hubs) > budget) A.warps /= 2;
+    const size_t fixed = sc_smem_bytes(C, A.per, k, dmax + 1, A.perp, A.warps, A.hubs);
     if (fixed > budget) continue;
     A.ecap = (int32_t)std::min<size_t>((budget - fixed) / 2, (size_t)(2 * m));
+    if (2 * m / C - A.ecap > kScMaxRead) continue;
     const size_t smem = fixed + (size_t)A.ecap * 2;
     A.n = n; A.k = k; A.dmax = dmax; A.iters = iters; A.rowptr = rowptr; A.colidx = colidx; A.pivots = pivots;
     A.cnt_off = cnt_off; A.cnt = cnt; A.dip = dip; A.pos = pos; A.tol = tol; A.iters_done = iters_done;

@@ -282,3 +282,40 @@ def test_sweep_fp32_cluster_of_few_nodes(n):
     y, done, rel = run(400, tol=1e-2)
     assert done == 400 or rel < 1e-2
     assert done < 4 or torch.equal(run(done)[0], y)
+
+
+def _hubs(n, hubs):
+    """Nodes 0 .. hubs - 1 adjacent to every other node."""
+    s = np.repeat(np.arange(hubs), n)
+    d = np.tile(np.arange(n), hubs)
+    keep = s < d
+    return n, s[keep].astype(np.int32), d[keep].astype(np.int32)
+
+
+@pytest.mark.parametrize("name,make,k,cluster", [
+    ("row_of_1024", lambda: _hubs(1025, 1), 5, True),      # one warp's
+    ("row_of_1025", lambda: _hubs(1026, 1), 5, True),      # segments of 256, the last of one entry
+    ("star", lambda: _hubs(8000, 1), 50, True),
+    ("hubs_in_some_ctas", lambda: _hubs(8001, 3), 30, True),
+    ("64_hubs_a_cta", lambda: _clique(1026), 5, True),     # 65 in two CTAs: a warp each there
+    ("rows_partly_kept", lambda: _clique(1300), 20, True),
+    ("too_dense", lambda: _clique(1600), 2, False)])
+def test_sweep_fp32_cluster_hubs_and_dense_rows(name, make, k, cluster):
+    """Rows of more than 1,024 entries, and graphs whose neighbours the cluster
+    keeps in part or not at all: one iteration from the fourth against the
+    oracle at the single step's bound; the same bits again, and without hints."""
+    n, s, d = make()
+    prep = O.prepare(n, s, d, k)
+    x0 = (np.random.default_rng(n).standard_normal((n, 2)) * np.sqrt(n)).astype(np.float32)
+    g, P = _gpu_graph(n, s, d), _gpu_pivots(k, prep)
+    P.dmax = int(prep.dip.max())
+    four, five = torch.from_numpy(x0.copy()).to(DEV), torch.from_numpy(x0.copy()).to(DEV)
+    ssm.ssm_iterate(g, P, four, 4)
+    ssm.ssm_iterate(g, P, five, 5)
+    assert (ssm.ssm_last_sweep_config()["kernel"] == "f32_cluster") == cluster
+    want, _ = O.sweep_jacobi(prep.g, prep.pivots, prep.dip, prep.w, four.cpu().numpy().astype(np.float64))
+    assert _norm_err(five.cpu().numpy(), want) < 1e-5
+    P.dmax = None
+    again = torch.from_numpy(x0.copy()).to(DEV)
+    ssm.ssm_iterate(g, P, again, 5)
+    assert torch.equal(again, five)
