@@ -56,6 +56,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "dip_part.cuh"
 #include "sweep.cuh"
 
 namespace ssm {
@@ -623,54 +624,20 @@ __global__ void __launch_bounds__(kSweepThreads, MODE == 2 ? SSM_SWEEP_FULL_MIN_
 // of the node's entry in the shared-memory table.  A distance above the table
 // (a wrong dmax hint) is recorded as SSM_E_ARG and clamped, so no table read
 // leaves the table
-//
-// loads of d_ip: 16 bytes at a time (2: n a multiple of 8 and dip on 16 bytes),
-// aligned words, shifted where the row starts in the middle of one (1: dip on 4
-// bytes), or single entries (0)
-enum DipLoads : int32_t { kDipEntries = 0, kDipWords = 1, kDipQuads = 2 };
-
-// the 2 W entries of d_ip from entry `first` on, two per word (0 from the left-th on)
-template <int W>
-struct DipPart {
-  unsigned w[W];
-};
-template <int W>
-__device__ __forceinline__ DipPart<W> dip_part(const uint16_t *__restrict__ dip, size_t first, int left, int32_t loads) {
-  DipPart<W> v;
-  if (loads == kDipQuads) {  // all of them are there, or none
+struct DipTable {
+  const uint16_t *__restrict__ p;
+  __device__ __forceinline__ uint16_t entry(size_t i) const { return __ldg(p + i); }
+  __device__ __forceinline__ unsigned word(size_t i) const { return __ldg(reinterpret_cast<const unsigned *>(p) + i); }
+  template <int W>
+  __device__ __forceinline__ void words(size_t first, unsigned (&w)[W]) const {
     if constexpr (W == 4) {
-      const uint4 q = left ? __ldg(reinterpret_cast<const uint4 *>(dip + first)) : make_uint4(0u, 0u, 0u, 0u);
-      v.w[0] = q.x; v.w[1] = q.y; v.w[2] = q.z; v.w[3] = q.w;
+      const uint4 q = __ldg(reinterpret_cast<const uint4 *>(p + first));
+      w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
     } else {
-      v.w[0] = left ? __ldg(reinterpret_cast<const unsigned *>(dip + first)) : 0u;
-    }
-  } else if (loads == kDipWords) {
-    const int odd = (int)(first & 1u);
-    const unsigned *words = reinterpret_cast<const unsigned *>(dip) + (first >> 1);
-    unsigned w[W + 1];
-#pragma unroll
-    for (int t = 0; t < W + 1; ++t) w[t] = left > 0 && 2 * t - odd < left ? __ldg(words + t) : 0u;
-#pragma unroll
-    for (int t = 0; t < W; ++t) {
-      const unsigned x = odd ? __byte_perm(w[t], w[t + 1], 0x5432) : w[t];
-      v.w[t] = 2 * t + 1 < left ? x : 2 * t < left ? x & 0xFFFFu : 0u;
-    }
-  } else {
-#pragma unroll
-    for (int t = 0; t < W; ++t) {
-      const unsigned lo = 2 * t < left ? (unsigned)__ldg(dip + first + 2 * t) : 0u;
-      const unsigned hi = 2 * t + 1 < left ? (unsigned)__ldg(dip + first + 2 * t + 1) : 0u;
-      v.w[t] = lo | (hi << 16);
+      w[0] = word(first >> 1);
     }
   }
-  return v;
-}
-
-// how many of the nodes 2 W g .. 2 W (g + 1) - 1 there are
-template <int W>
-__device__ __forceinline__ int part_left(int n, int64_t g) {
-  return (int)max((int64_t)0, min((int64_t)(2 * W), n - 2 * W * g));
-}
+};
 
 // word (t k + a) P + (p mod P), t = p div P, of the copy holds node pair
 // p = (2p, 2p + 1) of pivot a (P = kTileNodes / 2 pairs per tile); a thread
@@ -693,7 +660,7 @@ __global__ void k_tile_dip(int32_t n, int32_t k, const uint16_t *__restrict__ di
   const int64_t nquads = ((int64_t)(n + kTileNodes - 1) / kTileNodes) * (kTileNodes / 8);
   for (int a = blockIdx.y; a < k; a += gridDim.y)
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < nquads; g += (int64_t)gridDim.x * blockDim.x)
-      tile_store<4>(dtile, k, a, g, dip_part<4>(dip, (size_t)a * n + 8 * g, part_left<4>(n, g), loads));
+      tile_store<4>(dtile, k, a, g, dip_part<4>(DipTable{dip}, (size_t)a * n + 8 * g, part_left<4>(n, g), loads));
 }
 
 // full-table mode: the copy with e(d) the byte offset of the node's entry, and
@@ -736,17 +703,18 @@ __global__ void __launch_bounds__(256) k_tile_den(int32_t n, int32_t k, int32_t 
       tile_store<W>(dtile, k, a, g, out);
     };
     constexpr int kAhead = W == 4 ? 4 : 8;
+    const DipTable table{dip};
     const int left = part_left<W>(n, g);
     size_t first = (size_t)(2 * W * g);
     int a = 0;
     for (; a + kAhead <= k; a += kAhead) {
       DipPart<W> v[kAhead];
 #pragma unroll
-      for (int t = 0; t < kAhead; ++t, first += (size_t)n) v[t] = dip_part<W>(dip, first, left, loads);
+      for (int t = 0; t < kAhead; ++t, first += (size_t)n) v[t] = dip_part<W>(table, first, left, loads);
 #pragma unroll
       for (int t = 0; t < kAhead; ++t) pivot(a + t, v[t]);
     }
-    for (; a < k; ++a, first += (size_t)n) pivot(a, dip_part<W>(dip, first, left, loads));
+    for (; a < k; ++a, first += (size_t)n) pivot(a, dip_part<W>(table, first, left, loads));
 #pragma unroll
     for (int q = 0; q < 2 * W; ++q) {
       const int64_t i = 2 * W * g + q;
