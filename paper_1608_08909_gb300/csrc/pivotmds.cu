@@ -1322,11 +1322,13 @@ __global__ void k_wgram_reduce(int32_t k, int64_t nchunks, const double *__restr
 
 // x_i = C v = -1/2 (sum_a d_ia^2 v_a - rbar_i sigma - kappa): in FP64 for a
 // double layout; for a float one the sum over pivots in two-float FP32 (d^2 as
-// an exact pair, 2^-45 or better, 0.5 ms of FP64 before)
+// an exact pair, 2^-45 or better, 0.5 ms of FP64 before), the distances scaled by
+// a power of two so that the largest lies in [1, 2): neither the squares nor
+// their sums leave FP32's range where a float layout does not
 template <bool F64>
 __global__ void __launch_bounds__(256) k_wproject(int32_t n, int32_t k, const float *__restrict__ dist,
                                                   const double *__restrict__ vv, const EigOut *__restrict__ eo,
-                                                  void *__restrict__ pos) {
+                                                  const unsigned *__restrict__ dmax, void *__restrict__ pos) {
   extern __shared__ __align__(16) double svv[];  // FP64: v0[k], v1[k]; FP32: per pivot (v0 hi, v1 hi, v0 lo, v1 lo)
   float4 *sv = reinterpret_cast<float4 *>(svv);
   if (F64) {
@@ -1340,6 +1342,9 @@ __global__ void __launch_bounds__(256) k_wproject(int32_t n, int32_t k, const fl
   }
   __syncthreads();
   const double sig0 = eo->sigma[0], sig1 = eo->sigma[1], kap0 = eo->kappa[0], kap1 = eo->kappa[1];
+  const int ex = max(-126, min(126, (int)(*dmax >> 23) - 127));
+  const float down = __uint_as_float((unsigned)(127 - ex) << 23);
+  const double up = scalbn(1.0, 2 * ex);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     double x = 0.0, y = 0.0, rs = 0.0;
     if (F64) {
@@ -1356,7 +1361,7 @@ __global__ void __launch_bounds__(256) k_wproject(int32_t n, int32_t k, const fl
       for (int a0 = 0; a0 < k; a0 += 8) {
         float dq[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) dq[q] = a0 + q < k ? __ldg(dist + (size_t)(a0 + q) * n + i) : 0.f;
+        for (int q = 0; q < 8; ++q) dq[q] = a0 + q < k ? down * __ldg(dist + (size_t)(a0 + q) * n + i) : 0.f;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           if (a0 + q >= k) break;
@@ -1370,9 +1375,9 @@ __global__ void __launch_bounds__(256) k_wproject(int32_t n, int32_t k, const fl
           rh = t;
         }
       }
-      x = (double)hi.x + (double)lo.x;
-      y = (double)hi.y + (double)lo.y;
-      rs = (double)rh + (double)rl;
+      x = up * ((double)hi.x + (double)lo.x);
+      y = up * ((double)hi.y + (double)lo.y);
+      rs = up * ((double)rh + (double)rl);
     }
     const double rbar = rs / (double)k;
     x = -0.5 * (x - rbar * sig0 - kap0);
@@ -1458,9 +1463,9 @@ SSM_API int ssm_pivotmds_weighted(int32_t n, const int32_t *rowptr, const int32_
   const int pb = (int)std::min<int64_t>(((int64_t)n + 255) / 256, (int64_t)sms * 8);
   const size_t psm = 2 * (size_t)k * sizeof(double);
   if (precision == 64)
-    note_launch(), k_wproject<true><<<pb, 256, psm, s>>>(n, k, dist, w.vv, w.eo, pos);
+    note_launch(), k_wproject<true><<<pb, 256, psm, s>>>(n, k, dist, w.vv, w.eo, x.wmax, pos);
   else
-    note_launch(), k_wproject<false><<<pb, 256, psm, s>>>(n, k, dist, w.vv, w.eo, pos);
+    note_launch(), k_wproject<false><<<pb, 256, psm, s>>>(n, k, dist, w.vv, w.eo, x.wmax, pos);
   if (rescale) return launch_rescale(n, rowptr, colidx, elen, pos, precision, w, status, s);
   SSM_TRY_CUDA(cudaGetLastError());
   return SSM_OK;

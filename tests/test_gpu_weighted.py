@@ -288,3 +288,24 @@ def test_weighted_counts_of_a_large_region():
     greg, gs = ssm.ssm_weighted_counts(g, torch.from_numpy(piv).to(DEV), torch.from_numpy(dip).to(DEV))
     assert np.array_equal(greg.cpu().numpy(), reg)
     assert np.array_equal(gs.cpu().numpy(), O.wcounts(og, piv, dip, reg, threads=8))
+
+
+@pytest.mark.parametrize("top", [126, 100, -40, -90])
+def test_weighted_pivotmds_float_layout_range(top):
+    """Lengths times a power of two: every step of PivotMDS scales exactly, so
+    the float layout is that of the unscaled lengths times its square, as far
+    as floats hold it (`top`: the exponent of its largest coordinate; at 126
+    the sum of the squared distances to the pivots is above FP32's range)."""
+    n, s, d, l = I.rgg_lengths(3000, 7.0, 3)
+    og = O.build_wcsr(n, s, d, l)
+    dip = O.wpivot_dist(og, O.wmaxmin(og, 200))
+
+    def layout(scale):
+        g = _gpu_wgraph(n, s, d, (l * scale).astype(np.float32))
+        table = torch.from_numpy((dip * scale).astype(np.float32)).to(DEV)
+        return ssm.ssm_pivotmds_weighted(g, table, precision=32, rescale=False)[0].cpu().numpy().astype(np.float64)
+
+    one = layout(np.float32(1))
+    e = int((top - np.frexp(np.abs(one).max())[1]) // 2)
+    assert top < 126 or (dip.astype(np.float64) ** 2).sum(0).max() * 4.0 ** e > 2.0 ** 128
+    assert np.array_equal(layout(np.float32(2) ** np.float32(e)), one * 4.0 ** e)
