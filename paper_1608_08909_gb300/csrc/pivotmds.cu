@@ -1132,10 +1132,9 @@ SSM_API int ssm_pivotmds(int32_t n, const int32_t *rowptr, const int32_t *colidx
 // the column centring applied before the product so that nothing cancels.
 //
 // The squares are taken to fixed point: X_ia = d_ia^2 2^f rounded to an
-// integer (the square of a 24-bit mantissa shifted).  Column sums are exact sums
-// of X below 2^49 (the rounding, unbiased, is 2^-49 / sqrt(n) of the range).  The
-// product is that of the centred integers V = X - C, C the mean rounded: on the
-// tensor cores for up to 208 pivots, X below 2^55 (wgram_tc.cu); for more of
+// integer (the square of a 24-bit mantissa shifted).  Column sums are exact
+// sums of the squares themselves.  The product is that of the centred integers
+// V = X - C, C the mean rounded: on the tensor cores for up to 208 pivots, X below 2^55 (wgram_tc.cu); for more of
 // them here, X below 2^47: V = H 2^20 + L, |L| <= 2^19, and a pair costs three 32 x 32 -> 64-bit
 // integer multiply-adds, H H' and H L' + L H', exact over kWFlush nodes, where
 // FP64 at 1/64 of the FP32 rate costs 16 issue cycles a multiply-add.  L L' is
@@ -1143,7 +1142,7 @@ SSM_API int ssm_pivotmds(int32_t n, const int32_t *rowptr, const int32_t *colidx
 // 2^-52 / sqrt(n) of the entry).  The 64-bit sums go to FP64 per fixed node
 // chunk and the chunk partials are added in chunk order.
 // Measured (262K nodes, k = 200): the FP64 product took 16.2 ms, this one
-// 3.9, the tensor cores 1.7; the column sums 0.26 -> 0.09 (and 0.04 for the largest distance); the
+// 3.9, the tensor cores 1.7; the column sums 0.26 -> 0.10 (and 0.04 for the largest distance); the
 // projection for a float layout 0.50 -> 0.09.
 namespace ssm {
 
@@ -1172,33 +1171,54 @@ __global__ void k_wdmax(int64_t count, const float *__restrict__ dist, unsigned 
   if ((threadIdx.x & 31) == 0) atomicMax(out, m);
 }
 
-// partc[a * nchunks + c] = sum over the nodes of chunk c of d_ia^2 (an exact
-// integer sum, rounded once)
+// d^2 in units of 2^-64 of the largest distance's last place: exact from 2^-32
+// of the largest distance on; below 2^112 for d <= dmax
+__device__ __forceinline__ unsigned __int128 wsquare(float d, unsigned dmax_bits) {
+  const unsigned b = __float_as_uint(d) & 0x7FFFFFFFu;
+  const unsigned long long m = (b & 0x7FFFFFu) | 0x800000u;
+  const int sh = 64 - 2 * ((int)(dmax_bits >> 23) - (int)(b >> 23));
+  if ((b >> 23) == 0u || sh <= -48) return 0;  // zero (or below a normal float)
+  return sh >= 0 ? (unsigned __int128)(m * m) << sh : (unsigned __int128)(m * m >> -sh);
+}
+// the value of such a sum, rounded
+__device__ __forceinline__ double wsquare_sum(unsigned __int128 t, unsigned dmax_bits) {
+  const double v = (double)(unsigned long long)(t >> 64) * 18446744073709551616.0 + (double)(unsigned long long)t;
+  return scalbn(v, 2 * ((int)(dmax_bits >> 23) - 150) - 64);
+}
+
+// partc[a * nchunks + c] = sum over the nodes of chunk c of d_ia^2: an exact
+// 128-bit sum, rounded once (of squares rounded to 49 bits of the range, equal
+// distances' errors added up: on tables with a few far nodes the centring lost
+// some ten bits against FP64 sums)
 __global__ void __launch_bounds__(256) k_wcolsum_part(int32_t n, int32_t k, const float *__restrict__ dist,
                                                       const unsigned *__restrict__ dmax, int64_t chunk, int64_t nchunks,
                                                       double *__restrict__ partc) {
-  __shared__ unsigned long long red[8];
-  const int f = wfix_f(*dmax) + kWfix49;
+  __shared__ unsigned __int128 red[8];
+  const unsigned top = *dmax;
   for (int64_t task = blockIdx.x; task < (int64_t)k * nchunks; task += gridDim.x) {
     const int a = (int)(task / nchunks);
     const int64_t c = task - (int64_t)a * nchunks;
     const int64_t i0 = c * chunk, i1 = min((int64_t)n, i0 + chunk);
     const float *row = dist + (size_t)a * n;
-    unsigned long long acc = 0ull;  // at most 16384 values below 2^49
+    unsigned __int128 acc = 0;  // at most 16384 values below 2^112 in a chunk
     for (int64_t ib = i0 + threadIdx.x; ib < i1; ib += 4 * blockDim.x) {
       float d[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) d[q] = ib + q * blockDim.x < i1 ? __ldg(row + ib + q * blockDim.x) : 0.0f;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc += (unsigned long long)wfix(d[q], f);
+      for (int q = 0; q < 4; ++q) acc += wsquare(d[q], top);
     }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)acc, o);
+      const unsigned long long hi = __shfl_xor_sync(0xffffffffu, (unsigned long long)(acc >> 64), o);
+      acc += (unsigned __int128)hi << 64 | lo;
+    }
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {
-      unsigned long long t = 0ull;
+      unsigned __int128 t = 0;
       for (int w = 0; w < 8; ++w) t += red[w];
-      partc[task] = scalbn((double)t, -f);
+      partc[task] = wsquare_sum(t, top);
     }
     __syncthreads();
   }

@@ -4,6 +4,8 @@ distances, max/min pivots, regions and counts bit-exact (least float32 path
 sums are unique, whatever the search order); PivotMDS to 1e-10 in the
 eigenvalues; the FP64 sweep bit-identical, the FP32 sweep within 1e-5 per
 step; stress to 1e-9."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -309,3 +311,21 @@ def test_weighted_pivotmds_float_layout_range(top):
     e = int((top - np.frexp(np.abs(one).max())[1]) // 2)
     assert top < 126 or (dip.astype(np.float64) ** 2).sum(0).max() * 4.0 ** e > 2.0 ** 128
     assert np.array_equal(layout(np.float32(2) ** np.float32(e)), one * 4.0 ** e)
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_weighted_pivotmds_column_means(seed):
+    """Double layouts have mean zero but for FP64 rounding of the means
+    themselves, also when a few nodes are a thousand times as far as the others
+    and those all equally far.  The squares' projections and the centring each
+    round a handful of terms below the column means: 16 ulp of their sum."""
+    rng = np.random.default_rng(seed)
+    n, near = 4096, rng.uniform(0.5, 1.5, 2).astype(np.float32)
+    dist = np.repeat(near[:, None], n, 1)
+    dist[0, 0] = dist[1, 1] = 0.0
+    dist[0, 2] = dist[1, 3] = 1000.0
+    s, d, l = np.arange(n - 1, dtype=np.int32), np.arange(1, n, dtype=np.int32), np.ones(n - 1, np.float32)
+    pos, _ = ssm.ssm_pivotmds_weighted(_gpu_wgraph(n, s, d, l), torch.from_numpy(dist).to(DEV), precision=64, rescale=False)
+    means = (dist.astype(np.float64) ** 2).mean(1)
+    for axis in pos.cpu().numpy().T:
+        assert abs(math.fsum(axis)) / n < 16 * 2.0 ** -53 * means.sum()
