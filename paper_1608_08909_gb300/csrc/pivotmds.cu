@@ -1142,7 +1142,7 @@ SSM_API int ssm_pivotmds(int32_t n, const int32_t *rowptr, const int32_t *colidx
 // 2^-52 / sqrt(n) of the entry).  The 64-bit sums go to FP64 per fixed node
 // chunk and the chunk partials are added in chunk order.
 // Measured (262K nodes, k = 200): the FP64 product took 16.2 ms, this one
-// 3.9, the tensor cores 1.7; the column sums 0.26 -> 0.10 (and 0.04 for the largest distance); the
+// 3.9, the tensor cores 2.2; the column sums 0.26 -> 0.10 (and 0.04 for the largest distance); the
 // projection for a float layout 0.50 -> 0.09.
 namespace ssm {
 

@@ -5,11 +5,14 @@
 // v_p with -128 <= v_p <= 128 (the bytes of V + 0x80808080808080, less 128 each),
 // all exact in FP16, and
 //   G = sum_s 256^(12-s) sum_{p+q=s} v_p^T v_q.
-// Classes s = 0 .. 6 are formed (28 digit pairs); what is left off is some 2^-60
-// of a diagonal entry / sqrt(n), with random signs.  An FP32
-// accumulator holds an exact integer: it is read out before (s + 1) 2^14 times
-// its nodes passes 2^24, into 32-bit sums, and those go into 64-bit sums in
-// global memory with integer atomics (order-free), three per entry.
+// Classes s = 0 .. 8 are formed (39 digit pairs): what is left off is below
+// 2^-68 of the range's square per node, and below 2^-53 of a diagonal entry also
+// where one of 65,536 nodes is far from the others, those equally far.  (With
+// classes 0 .. 6, 1.7 ms, that table's eigenvalue was 2e-12 off, and with lengths
+// over four decades 4e-15 where an FP64 product is at 4e-16.)  An FP32
+// accumulator holds an exact integer: it is read out before 2^14 times its pairs
+// and nodes passes 2^24, into 32-bit sums, and those go into 64-bit sums in
+// global memory with integer atomics (order-free), four per entry.
 //
 // A CTA has one class and a range of nodes (as many CTAs per class as its work
 // asks for).  Per unit of 32 nodes a warp loads two pivots' rows at a time (128
@@ -20,13 +23,13 @@
 // double-buffered: the MMAs (M = 128 pivots, N = all of them; the second tile,
 // the last 128 pivots, only against those from 128 on) run while the next unit
 // is converted.  Both operands of every pair are planes of the same buffer.
-// Bound by the conversion (about 60 instructions per 64 values and class, so
-// some 1,500-2,000 cycles a unit and CTA) and, for the last classes, the MMAs.
-// Measured (262K nodes, k = 200): 1.7 ms, against 3.9 in integer multiply-adds and
-// 16.2 in FP64.
+// Bound by the conversion (7,400 to 10,000 cycles a unit and CTA at k = 200) and,
+// for the classes of many pairs, the MMAs.  Measured (262K nodes, k = 200): 2.2 ms,
+// against 16.2 in FP64.
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "tc.cuh"
@@ -36,7 +39,7 @@ namespace ssm {
 
 constexpr int kWgThreads = 512;
 constexpr int kWgUnit = 32;     // nodes per unit (two MMAs of K = 16)
-constexpr int kWgClasses = 7;   // s = 0 .. 6
+constexpr int kWgClasses = 9;   // s = 0 .. 8
 constexpr int kWgRowPairs = 7;  // row pairs per warp (104 over 16 warps, rounded up)
 constexpr int kWgSums = 120;    // read-outs per 32-bit sum: 120 2^24 < 2^31
 constexpr unsigned long long kWgBias = 0x80808080808080ull;
@@ -104,7 +107,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgram_tc(int32_t n, int32_t k
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int pad = wg_pad(k), R = wg_rows(k), n1 = max(0, pad - 128);
   const uint32_t group = wg_group(k), plane = wg_plane(k);
-  const int planes = cls + 1;  // digits 0 .. cls
+  const int dlo = max(0, cls - ((int)kWgDigits - 1)), dhi = cls - dlo;  // digits p with a partner cls - p
+  const int planes = dhi - dlo + 1;
   const int flush = 512 / kWgUnit * 2 / planes;                          // units per read-out: planes 2^14 nodes <= 2^24
   const uint32_t base = tc_smem(wg_raw);
   int *const sum1 = reinterpret_cast<int *>(wg_raw + 2u * kWgDigits * plane);        // [n1][128] second tile's sums, a thread's own
@@ -140,9 +144,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgram_tc(int32_t n, int32_t k
   const int q4 = warp & 3, cg = warp >> 2;  // TMEM lanes 32 q4 .. + 31; strips of eight columns cg, cg + 4, ...
   const int row = 32 * q4 + lane;
   const uint32_t tlane = tmem + ((uint32_t)(32 * q4) << 16);
-  // 64-bit sums: classes 0-2 in units of 256^10, 3-4 of 256^8, 5-6 of 256^6
-  const int part = cls < 3 ? 0 : cls < 5 ? 1 : 2;
-  const int up = 8 * (cls < 3 ? 2 - cls : cls < 5 ? 4 - cls : 6 - cls);
+  // 64-bit sums: classes 0-2 in units of 256^10, 3-4 of 256^8, 5-6 of 256^6, 7-8 of 256^4
+  const int part = cls < 3 ? 0 : (cls - 1) / 2;
+  const int up = 8 * (2 + 2 * part - cls);
   auto emit = [&]() {
     unsigned long long *out = acc + (size_t)part * k * k;
     auto add = [&](int a, int b, int v) {
@@ -176,6 +180,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgram_tc(int32_t n, int32_t k
     const bool freed = it < 2 || tc_wait_warp(mb, (unsigned)((it - 2) >> 1) & 1u);
     unsigned char *const dst = wg_raw + (size_t)buf * kWgDigits * plane;
     const bool in = u * kWgUnit + lane < n;
+    auto convert = [&](auto least) {  // digits from `least` on
 #pragma unroll
     for (int i = 0; i < kWgRowPairs; ++i) {
       const int r0 = 2 * (warp + 16 * i);
@@ -193,10 +198,14 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgram_tc(int32_t n, int32_t k
         unsigned char *const at = dst + (unsigned)(lane >> 3) * group + (unsigned)(r0 + (odd ? 1 : 0)) * 16u +
                                   (unsigned)((lane & 7) >> 1) * 4u;
 #pragma unroll
-        for (int p = 0; p < (int)kWgDigits; ++p)
-          if (p < planes) *reinterpret_cast<uint32_t *>(at + (unsigned)p * plane) = wg_digit(a, b, p);
+        for (int p = decltype(least)::value; p < (int)kWgDigits; ++p)
+          if (p <= dhi) *reinterpret_cast<uint32_t *>(at + (unsigned)p * plane) = wg_digit(a, b, p);
       }
     }
+    };
+    if (dlo == 0) convert(std::integral_constant<int, 0>());
+    else if (dlo == 1) convert(std::integral_constant<int, 1>());
+    else convert(std::integral_constant<int, 2>());
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the planes are read by the tensor cores
     asm volatile("tcgen05.fence::before_thread_sync;");
     const int stuck = __syncthreads_or(freed ? 0 : 1);
@@ -208,8 +217,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgram_tc(int32_t n, int32_t k
     if (warp == 0) {
       const uint32_t bs = base + (unsigned)buf * kWgDigits * plane;
       uint32_t add = since > 0 ? 1u : 0u;
-      for (int p = 0; p < planes; ++p) {
-        const uint32_t pa = bs + (unsigned)p * plane, pb = bs + (unsigned)(planes - 1 - p) * plane;
+      for (int p = dlo; p <= dhi; ++p) {
+        const uint32_t pa = bs + (unsigned)p * plane, pb = bs + (unsigned)(cls - p) * plane;
 #pragma unroll
         for (int st = 0; st < 2; ++st) {
           const uint32_t off = (unsigned)st * 2u * group;
@@ -265,24 +274,25 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgram_tc(int32_t n, int32_t k
 __global__ void k_wgram_final(int32_t k, const unsigned *__restrict__ dmax, const unsigned long long *__restrict__ acc,
                               double *__restrict__ G) {
   const int64_t kk = (int64_t)k * k;
-  const double unit = wfix_bad(*dmax) ? __longlong_as_double(0x7FF8000000000000ll) : scalbn(1.0, 48 - 2 * wfix_f(*dmax));
+  const double unit = wfix_bad(*dmax) ? __longlong_as_double(0x7FF8000000000000ll) : scalbn(1.0, 32 - 2 * wfix_f(*dmax));
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < kk; t += (int64_t)gridDim.x * blockDim.x) {
     const int a = (int)(t / k), b = (int)(t - (int64_t)a * k);
     if (a > b) continue;
-    const double g = (scalbn((double)(long long)acc[t], 32) + scalbn((double)(long long)acc[kk + t], 16) +
-                      (double)(long long)acc[2 * kk + t]) *
-                     unit;
+    auto part = [&](int q) { return (double)(long long)acc[q * kk + t]; };
+    const double g = (scalbn(part(0), 48) + (scalbn(part(1), 32) + (scalbn(part(2), 16) + part(3)))) * unit;
     G[(size_t)a * k + b] = g;
     G[(size_t)b * k + a] = g;
   }
 }
 
-size_t wgram_tc_acc_words(int32_t k) { return 3 * (size_t)k * k; }
+size_t wgram_tc_acc_words(int32_t k) { return 4 * (size_t)k * k; }
 
 int launch_wgram_tc(int32_t n, int32_t k, const float *dist, const unsigned *dmax, const long long *centre,
                     unsigned long long *acc, double *G, int32_t *status, cudaStream_t s) {
-  // cycles per unit of a class (conversion, or MMAs where they are more, and its share of a read-out)
-  const int cost[kWgClasses] = {1500, 1640, 1800, 1940, 2100, 2250, 2450};
+  // cycles per unit of a class (conversion, MMAs, its share of a read-out) in
+  // hundredths of the longest one's, from one class at a time at k = 200; at k = 60,
+  // 100 and 128 the shares are the same within 5 %
+  const int cost[kWgClasses] = {74, 80, 82, 88, 91, 95, 100, 92, 86};
   int total = 0;
   for (int c : cost) total += c;
   const int sms = std::max(num_sms(), 2 * kWgClasses);

@@ -329,3 +329,26 @@ def test_weighted_pivotmds_column_means(seed):
     means = (dist.astype(np.float64) ** 2).mean(1)
     for axis in pos.cpu().numpy().T:
         assert abs(math.fsum(axis)) / n < 16 * 2.0 ** -53 * means.sum()
+
+
+@pytest.mark.parametrize("k", [8, 130])
+@pytest.mark.parametrize("seed", range(2))
+def test_weighted_pivotmds_one_far_node(seed, k):
+    """The largest eigenvalue where one node in 65,536 is 32 times as far as the
+    others, which are equally far, against extended precision.  An entry of B
+    is rounded some eight times, at a magnitude up to 60 times lambda_1 / k:
+    errors with random signs reach 8 ulp of lambda_1 (k = 8); 32 are allowed."""
+    rng = np.random.default_rng(seed)
+    n = 65536
+    dist = np.repeat((rng.uniform(0.5, 1.0, (k, 1)) * 31).astype(np.float32), n, 1)
+    dist[:, 0] = 1000 * np.linspace(0.3, 1.0, k)
+    s, d, l = np.arange(n - 1, dtype=np.int32), np.arange(1, n, dtype=np.int32), np.ones(n - 1, np.float32)
+    _, eig = ssm.ssm_pivotmds_weighted(_gpu_wgraph(n, s, d, l), torch.from_numpy(dist).to(DEV), precision=64, rescale=False)
+    c = dist.astype(np.longdouble) ** 2
+    c = (c - c.mean(1, keepdims=True) - c.mean(0) + c.mean()) / 2
+    v = c[:, 0]
+    for _ in range(20):  # the others' eigenvalues are below 1e-2 of this one
+        v = c @ (v @ c)
+        v = v / np.sqrt((v * v).sum())
+    lam = ((v @ c) ** 2).sum()
+    assert abs(eig[0].item() - lam) < 32 * 2.0 ** -53 * lam
