@@ -1134,26 +1134,26 @@ SSM_API int ssm_pivotmds(int32_t n, const int32_t *rowptr, const int32_t *colidx
 // The squares are taken to fixed point: X_ia = d_ia^2 2^f rounded to an
 // integer (the square of a 24-bit mantissa shifted).  Column sums are exact
 // sums of the squares themselves.  The product is that of the centred integers
-// V = X - C, C the mean rounded: on the tensor cores for up to 208 pivots, X below 2^55 (wgram_tc.cu); for more of
-// them here, X below 2^47: V = H 2^20 + L, |L| <= 2^19, and a pair costs three 32 x 32 -> 64-bit
-// integer multiply-adds, H H' and H L' + L H', exact over kWFlush nodes, where
-// FP64 at 1/64 of the FP32 rate costs 16 issue cycles a multiply-add.  L L' is
-// formed on the diagonal only, where it does not average out (elsewhere it is
-// 2^-52 / sqrt(n) of the entry).  The 64-bit sums go to FP64 per fixed node
-// chunk and the chunk partials are added in chunk order.
-// Measured (262K nodes, k = 200): the FP64 product took 16.2 ms, this one
-// 3.9, the tensor cores 2.2; the column sums 0.26 -> 0.10 (and 0.04 for the largest distance); the
-// projection for a float layout 0.50 -> 0.09.
+// V = X - C, C the mean rounded, X below 2^55: on the tensor cores for up to 208
+// pivots (wgram_tc.cu); for more of them here: V = H 2^27 + L, |H| <= 2^28,
+// |L| <= 2^26, and a pair costs four 32 x 32 -> 64-bit integer multiply-adds, H H',
+// H L' + L H' and L L', exact over the kWStage nodes in shared memory, where FP64 at
+// 1/64 of the FP32 rate costs 16 issue cycles a multiply-add.  They are added up in
+// 128 bits, exactly, per fixed node chunk, and the chunk partials in FP64 in chunk
+// order.
+// Measured (262K nodes): k = 240: the FP64 product took 20.0 ms, this one 7.1; k = 200: the
+// FP64 product 16.2, the tensor cores 2.2; the column sums 0.26 -> 0.10 (and 0.04 for
+// the largest distance); the projection for a float layout 0.50 -> 0.09.
 namespace ssm {
 
 constexpr int kWStage = 64;     // nodes staged in shared memory at a time
-constexpr int kWFlush = 512;    // nodes per 64-bit sum: 2^54 2^9 < 2^63
-constexpr int kWSplit = 20;     // bits of L
+constexpr int kWSplit = 27;     // bits of L
+static_assert(2 * 28 + 6 < 63 && kWStage == 64, "64-bit sums of kWStage products");
 
 static int64_t wgram_chunk(int32_t n) {
   int64_t c = ((int64_t)n + 63) / 64;
   c = std::max<int64_t>(1024, std::min<int64_t>(16384, c));
-  return (c + kWFlush - 1) / kWFlush * kWFlush;
+  return (c + 511) / 512 * 512;
 }
 
 __global__ void k_wdmax(int64_t count, const float *__restrict__ dist, unsigned *__restrict__ out) {
@@ -1225,14 +1225,14 @@ __global__ void __launch_bounds__(256) k_wcolsum_part(int32_t n, int32_t k, cons
 }
 
 __global__ void k_wcolsum_final(int32_t n, int32_t k, int64_t nchunks, const double *__restrict__ partc,
-                                const unsigned *__restrict__ dmax, int bits, double *__restrict__ colsum,
-                                long long *__restrict__ centre) {  // the centre in X of exponent f + bits
+                                const unsigned *__restrict__ dmax, double *__restrict__ colsum,
+                                long long *__restrict__ centre) {
   for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < k; a += gridDim.x * blockDim.x) {
     double t = 0.0;
 #pragma unroll 8
     for (int64_t c = 0; c < nchunks; ++c) t += partc[(size_t)a * nchunks + c];
     colsum[a] = t;
-    centre[a] = __double2ll_rn(scalbn(t, wfix_f(*dmax) + bits) / (double)n);
+    centre[a] = __double2ll_rn(scalbn(t, wfix_f(*dmax)) / (double)n);
   }
 }
 
@@ -1250,7 +1250,7 @@ __global__ void __launch_bounds__(T *T / 4) k_wgram(int32_t n, int32_t k, const 
   __shared__ __align__(16) int sh[2][kWStage][T + 2], sl[2][kWStage][T + 2];
   const int tx = threadIdx.x % kHalf, ty = threadIdx.x / kHalf;
   const int64_t npairs = (int64_t)ntiles * (ntiles + 1) / 2;
-  const int f = wfix_f(*dmax) + kWfix47;
+  const int f = wfix_f(*dmax);
   const double unit = wfix_bad(*dmax) ? __longlong_as_double(0x7FF8000000000000ll) : scalbn(1.0, -2 * f);
   for (int64_t task = blockIdx.x; task < npairs * nchunks; task += gridDim.x) {
     const int64_t c = task / npairs;
@@ -1264,56 +1264,45 @@ __global__ void __launch_bounds__(T *T / 4) k_wgram(int32_t n, int32_t k, const 
     const bool diag = ta == tb;
     const int a0 = ta * T, b0 = tb * T;
     const int64_t i0 = c * chunk, i1 = min((int64_t)n, i0 + chunk);
-    double g[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-    for (int64_t fb = i0; fb < i1; fb += kWFlush) {
-      long long hh[2][2] = {{0ll, 0ll}, {0ll, 0ll}}, hl[2][2] = {{0ll, 0ll}, {0ll, 0ll}}, ll[2] = {0ll, 0ll};
-      const int64_t fe = min(i1, fb + kWFlush);
-      for (int64_t ib = fb; ib < fe; ib += kWStage) {
-        __syncthreads();  // the staged nodes are consumed
-        for (int e = threadIdx.x; e < (diag ? 1 : 2) * kWStage * T; e += kThreads) {
-          const int side = e / (kWStage * T), r = e - side * (kWStage * T), pv = r / kWStage, nd = r % kWStage;
-          const int p = (side ? b0 : a0) + pv;
-          const int64_t i = ib + nd;
-          int H = 0, L = 0;
-          if (p < k && i < fe) {
-            const long long v = wfix(__ldg(dist + (size_t)p * n + i), f) - __ldg(centre + p);
-            H = (int)((v + (1ll << (kWSplit - 1))) >> kWSplit);
-            L = (int)(v - ((long long)H << kWSplit));
-          }
-          sh[side][nd][pv] = H;
-          sl[side][nd][pv] = L;
+    __int128 g[2][2] = {{0, 0}, {0, 0}};  // below 2^110 16384
+    for (int64_t ib = i0; ib < i1; ib += kWStage) {
+      __syncthreads();  // the staged nodes are consumed
+      for (int e = threadIdx.x; e < (diag ? 1 : 2) * kWStage * T; e += kThreads) {
+        const int side = e / (kWStage * T), r = e - side * (kWStage * T), pv = r / kWStage, nd = r % kWStage;
+        const int p = (side ? b0 : a0) + pv;
+        const int64_t i = ib + nd;
+        int H = 0, L = 0;
+        if (p < k && i < i1) {
+          const long long v = wfix(__ldg(dist + (size_t)p * n + i), f) - __ldg(centre + p);
+          H = (int)((v + (1ll << (kWSplit - 1))) >> kWSplit);
+          L = (int)(v - ((long long)H << kWSplit));
         }
-        __syncthreads();
-        const int sb = diag ? 0 : 1;
+        sh[side][nd][pv] = H;
+        sl[side][nd][pv] = L;
+      }
+      __syncthreads();
+      const int sb = diag ? 0 : 1;
+      long long hh[2][2] = {{0ll, 0ll}, {0ll, 0ll}}, hl[2][2] = {{0ll, 0ll}, {0ll, 0ll}}, ll[2][2] = {{0ll, 0ll}, {0ll, 0ll}};
 #pragma unroll 4
-        for (int nd = 0; nd < kWStage; ++nd) {
-          const int2 xh = *reinterpret_cast<const int2 *>(&sh[0][nd][2 * ty]), xl = *reinterpret_cast<const int2 *>(&sl[0][nd][2 * ty]);
-          const int2 yh = *reinterpret_cast<const int2 *>(&sh[sb][nd][2 * tx]), yl = *reinterpret_cast<const int2 *>(&sl[sb][nd][2 * tx]);
-          hh[0][0] += (long long)xh.x * yh.x;
-          hh[0][1] += (long long)xh.x * yh.y;
-          hh[1][0] += (long long)xh.y * yh.x;
-          hh[1][1] += (long long)xh.y * yh.y;
-          hl[0][0] += (long long)xh.x * yl.x;
-          hl[0][1] += (long long)xh.x * yl.y;
-          hl[1][0] += (long long)xh.y * yl.x;
-          hl[1][1] += (long long)xh.y * yl.y;
-          hl[0][0] += (long long)xl.x * yh.x;
-          hl[0][1] += (long long)xl.x * yh.y;
-          hl[1][0] += (long long)xl.y * yh.x;
-          hl[1][1] += (long long)xl.y * yh.y;
-        }
-        if (diag && tx == ty)
-          for (int nd = 0; nd < kWStage; ++nd) {
-            ll[0] += (long long)sl[0][nd][2 * tx] * sl[0][nd][2 * tx];
-            ll[1] += (long long)sl[0][nd][2 * tx + 1] * sl[0][nd][2 * tx + 1];
+      for (int nd = 0; nd < kWStage; ++nd) {
+        const int2 xh2 = *reinterpret_cast<const int2 *>(&sh[0][nd][2 * ty]), xl2 = *reinterpret_cast<const int2 *>(&sl[0][nd][2 * ty]);
+        const int2 yh2 = *reinterpret_cast<const int2 *>(&sh[sb][nd][2 * tx]), yl2 = *reinterpret_cast<const int2 *>(&sl[sb][nd][2 * tx]);
+        const int xh[2] = {xh2.x, xh2.y}, xl[2] = {xl2.x, xl2.y}, yh[2] = {yh2.x, yh2.y}, yl[2] = {yl2.x, yl2.y};
+#pragma unroll
+        for (int p = 0; p < 2; ++p)
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            hh[p][q] += (long long)xh[p] * yh[q];
+            hl[p][q] += (long long)xh[p] * yl[q];
+            hl[p][q] += (long long)xl[p] * yh[q];
+            ll[p][q] += (long long)xl[p] * yl[q];
           }
       }
 #pragma unroll
       for (int p = 0; p < 2; ++p)
 #pragma unroll
         for (int q = 0; q < 2; ++q)
-          g[p][q] += ((double)hh[p][q] * (double)(1 << kWSplit) + (double)hl[p][q]) * (double)(1 << kWSplit) +
-                     (p == q ? (double)ll[p] : 0.0);
+          g[p][q] += (__int128)hh[p][q] * (1ll << (2 * kWSplit)) + (__int128)hl[p][q] * (1ll << kWSplit) + ll[p][q];
     }
     double *pg = partg + (size_t)c * k * k;
 #pragma unroll
@@ -1321,7 +1310,9 @@ __global__ void __launch_bounds__(T *T / 4) k_wgram(int32_t n, int32_t k, const 
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         const int a = a0 + 2 * ty + p, b = b0 + 2 * tx + q;
-        if (a < k && b < k) pg[(size_t)a * k + b] = g[p][q] * unit;
+        if (a < k && b < k)
+          pg[(size_t)a * k + b] = ((double)(long long)(g[p][q] >> 64) * 18446744073709551616.0 +
+                                   (double)(unsigned long long)g[p][q]) * unit;
       }
   }
 }
@@ -1458,7 +1449,7 @@ SSM_API int ssm_pivotmds_weighted(int32_t n, const int32_t *rowptr, const int32_
   note_launch(), k_wcolsum_part<<<(unsigned)std::min<int64_t>((int64_t)k * nch, (int64_t)sms * 8), 256, 0, s>>>(
       n, k, dist, x.wmax, ch, nch, x.partc);
   note_launch(), k_wcolsum_final<<<(k + 31) / 32, 32, 0, s>>>(n, k, nch, x.partc, x.wmax,
-                                                       k <= kWgMaxK ? 0 : kWfix47, x.colsum, x.centre);
+                                                       x.colsum, x.centre);
   const int64_t kk = (int64_t)k * k;
   if (k <= kWgMaxK) {
     if (int rc = launch_wgram_tc(n, k, dist, x.wmax, x.centre, x.acc, w.B, status, s)) return rc;

@@ -26,9 +26,6 @@ __device__ __forceinline__ long long wfix(float d, int f) {
   return sh <= 0 ? (long long)((m * m) << -sh) : (long long)((m * m + (1ull << (sh - 1))) >> sh);
 }
 
-// with fewer bits, where 32-bit halves are wanted: X below 2^47
-constexpr int kWfix47 = -8;
-
 // G'_ab = sum_i V_ia V_ib 2^(-2 f), V = X - centre, into the symmetric k x k
 // matrix G for k up to kWgMaxK; acc holds wgram_tc_acc_words(k) 64-bit words.
 constexpr int kWgMaxK = 208;

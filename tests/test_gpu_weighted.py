@@ -331,7 +331,7 @@ def test_weighted_pivotmds_column_means(seed):
         assert abs(math.fsum(axis)) / n < 16 * 2.0 ** -53 * means.sum()
 
 
-@pytest.mark.parametrize("k", [8, 130])
+@pytest.mark.parametrize("k", [8, 130, 240])
 @pytest.mark.parametrize("seed", range(2))
 def test_weighted_pivotmds_one_far_node(seed, k):
     """The largest eigenvalue where one node in 65,536 is 32 times as far as the
@@ -347,7 +347,7 @@ def test_weighted_pivotmds_one_far_node(seed, k):
     c = dist.astype(np.longdouble) ** 2
     c = (c - c.mean(1, keepdims=True) - c.mean(0) + c.mean()) / 2
     v = c[:, 0]
-    for _ in range(20):  # the others' eigenvalues are below 1e-2 of this one
+    for _ in range(3):  # the others' eigenvalues are below 1e-14 of this one
         v = c @ (v @ c)
         v = v / np.sqrt((v * v).sum())
     lam = ((v @ c) ** 2).sum()
