@@ -773,7 +773,7 @@ __global__ void k_dip_max(int64_t count, const uint16_t *__restrict__ dip, unsig
 // FP64 at a 64th of FP32's rate bounds it: a term's count of FP64
 // instructions.  The square root and the divides of a term therefore share
 // one reciprocal square root (over_length), and s / d^2 takes 1 / d^2 from a
-// table: some 33 instructions a term where three IEEE divides and a square
+// table: some 37 instructions a term where three IEEE divides and a square
 // root made it 85.  ba64k, k = 200: 1.05 ms an iteration, 2.1 to 2.2 before.
 struct PivD {
   double x, y;
@@ -792,17 +792,34 @@ __device__ __forceinline__ bool mid_range(double v) {
   return ((unsigned)__double2hiint(v) & 0x7FFFFFFFu) - (623u << 20) < (800u << 20);
 }
 
+// Whether g + c, c = res z, may lie so close to a rounding boundary that a wrong
+// last bit of c shows: c, from the upper 24 bits of res and z, within 2^-17 of half
+// an odd number of units of g's last place, or g next to a power of two, where
+// the unit changes.  (res is a residual: zero where g is exact.)  FP32 and integer
+// instructions: FP64's are the scarce ones.
+__device__ __forceinline__ bool near_boundary(double g, double res, double z) {
+  const int gh = __double2hiint(g), rh = __double2hiint(res), zh = __double2hiint(z);
+  auto upper = [](double v) {  // in [1, 2)
+    return __uint_as_float(0x3F800000u | (__funnelshift_l((unsigned)__double2loint(v), (unsigned)__double2hiint(v), 3) & 0x7FFFFFu));
+  };
+  const int e = (rh >> 20 & 0x7FF) + (zh >> 20 & 0x7FF) - (gh >> 20 & 0x7FF) - 971;  // |c| = upper upper 2^e units of g
+  const float t = __int_as_float(__float_as_int(upper(res) * upper(z)) + (min(max(e, -8), 8) << 23));
+  const float n = __fadd_rn(__fadd_rn(t, 12582912.f), -12582912.f);  // t rounded to an integer
+  const bool near = fabsf(t - n) > 0.5f - 0x1p-17f || (t > 0.2f && (unsigned)((gh + 1) & 0xFFFFF) <= 1u);
+  return near && rh << 1 != 0;
+}
+
 // (qx, qy) = (tx / r, ty / r) with r = sqrt(dx^2 + dy^2), every operation
 // rounded to nearest; false where r is zero.  One reciprocal square root y of
 // h = r^2 serves them: Halley's iteration brings the hardware's approximation
-// (20 bits) to FP64 rounding, r is h y corrected once by its exact residual,
-// 1 / r is y corrected once, and each quotient is the product with it
-// corrected once by its exact residual (Markstein's scheme: a residual by
-// fused multiply-add, one correction).  What is rounded last is within 2^-104
-// of the exact value, so a result differs from the IEEE operation's, by one
-// unit in the last place, only where that lies so close to a rounding
-// boundary: about one operand in 2^50 (none of 15e9 random ones).  Where a value is outside 2^+-400 (or
-// not a number), the IEEE operations.
+// (20 bits) to FP64 rounding (within 1.6 2^-53), r is h y corrected once by its
+// exact residual, 1 / r is y corrected once, and each quotient is the product with
+// it corrected once by its exact residual (Markstein's scheme: a residual by
+// fused multiply-add, one correction).  What is rounded last, g + res z, is then
+// within 2^-48 of g's last place of the exact value, g itself within three
+// units, so the result is the IEEE operation's except where that value lies
+// next to a rounding boundary.  There (one operand in some 20,000: near_boundary), and
+// where a value is outside 2^+-400 or not a number, the IEEE operations.
 __device__ __forceinline__ bool over_length(double dx, double dy, double tx, double ty, double &qx, double &qy) {
   const double h = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
   if (mid_range(h) && (mid_range(tx) || tx == 0.0) && (mid_range(ty) || ty == 0.0)) {
@@ -812,13 +829,14 @@ __device__ __forceinline__ bool over_length(double dx, double dy, double tx, dou
     y = __fma_rn(__dmul_rn(y, e), __fma_rn(e, 0.375, 0.5), y);
     const double g = __dmul_rn(h, y);
     const double half = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));  // y / 2
-    const double r = __fma_rn(__fma_rn(-g, g, h), half, g);
+    const double gres = __fma_rn(-g, g, h);
+    const double r = __fma_rn(gres, half, g);
     const double z = __fma_rn(__fma_rn(-r, y, 1.0), y, y);
-    qx = __dmul_rn(tx, z);
-    qx = __fma_rn(__fma_rn(-r, qx, tx), z, qx);
-    qy = __dmul_rn(ty, z);
-    qy = __fma_rn(__fma_rn(-r, qy, ty), z, qy);
-    return true;
+    const double px = __dmul_rn(tx, z), py = __dmul_rn(ty, z);
+    const double rx = __fma_rn(-r, px, tx), ry = __fma_rn(-r, py, ty);
+    qx = __fma_rn(rx, z, px);
+    qy = __fma_rn(ry, z, py);
+    if (!(near_boundary(g, gres, half) | near_boundary(px, rx, z) | near_boundary(py, ry, z))) return true;
   }
   const double r = __dsqrt_rn(h);
   if (!(r > 0.0)) return false;

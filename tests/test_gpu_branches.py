@@ -319,3 +319,77 @@ def test_sweep_fp32_cluster_hubs_and_dense_rows(name, make, k, cluster):
     again = torch.from_numpy(x0.copy()).to(DEV)
     ssm.ssm_iterate(g, P, again, 5)
     assert torch.equal(again, five)
+
+
+def _hard_quotients(count, seed):
+    """(dx, dy) with r = RN(sqrt(RN(RN(dx^2) + RN(dy^2)))) and dx / r within a
+    relative 2^-105 of a midpoint between two doubles: r odd, 2^54 dx = M r +- 1
+    with M, 54 bits, the inverse of -+r modulo 2^54."""
+    rng = np.random.default_rng(seed)
+    r, dx = [], []
+    while len(r) < count:
+        R = int(rng.integers(1 << 52, 1 << 53)) | 1
+        for sign in (1, -1):
+            M = -sign * pow(R, -1, 1 << 54) % (1 << 54)
+            if M >> 53:
+                r.append(float(R))
+                dx.append(float((M * R + sign) >> 54))
+    r, dx = np.array(r), np.array(dx)
+    dy = np.sqrt((r - dx) * (r + dx))
+    for step in range(1, 40):  # the next dy up and down until r comes out
+        off = np.sqrt(dx * dx + dy * dy) - r
+        dy = np.where(off > 0, np.nextafter(dy, 0), np.where(off < 0, np.nextafter(dy, np.inf), dy))
+    ok = np.sqrt(dx * dx + dy * dy) == r
+    return dx[ok], dy[ok]
+
+
+def _hard_roots():
+    """(dx, dy) whose h = RN(RN(dx^2) + RN(dy^2)) has a root next to a midpoint:
+    h = H 2^(b - 2) with M^2 = 2^b H - delta for an odd M of 54 bits and a small
+    delta, M a root of -delta modulo 2^b."""
+    out = []
+    for b in (54, 55):
+        for delta in list(range(7, 1200, 8)) + list(range(-1, -1200, -8)):
+            M = 1
+            for bits in range(4, b + 1):  # a root modulo 2^bits
+                if (M * M + delta) % (1 << bits):
+                    M += 1 << (bits - 2)
+            for root in (M, -M, M + (1 << (b - 1)), (1 << (b - 1)) - M):
+                root %= 1 << b
+                if root >> 53 != 1:
+                    continue
+                assert (root * root + delta) % (1 << b) == 0
+                H = (root * root + delta) >> b
+                if H >> 52 != 1:
+                    continue
+                h = float(H) * 2.0 ** (b - 2 - 104)
+                for x in np.sqrt(h * np.linspace(0.3, 0.9, 40)):
+                    ys = np.sqrt(h - x * x) + np.arange(-4, 5) * np.spacing(np.sqrt(h - x * x))
+                    hit = ys[x * x + ys * ys == h]
+                    if len(hit):
+                        out.append((x, hit[0]))
+                        break
+    return np.array(out).T
+
+
+def test_sweep_fp64_rounds_as_ieee_operations():
+    """A leaf of a star whose hub is at the origin moves to (dx / r, dy / r), with
+    the square root and the quotients of the shared reciprocal square root:
+    the IEEE operations' bits where the exact values lie next to midpoints of
+    two doubles, and on ordinary ones."""
+    rng = np.random.default_rng(5)
+    xy = [_hard_quotients(20000, 1), _hard_quotients(20000, 2)[::-1], _hard_roots(),
+          rng.standard_normal((2, 100000)) * 10.0 ** rng.integers(-3, 4, 100000)]
+    assert [v.shape[1] if hasattr(v, "shape") else len(v[0]) for v in xy][2] > 100 and len(xy[0][0]) > 15000
+    x0 = np.concatenate([np.zeros((1, 2))] + [np.stack(v, 1) for v in xy])
+    x0[1:] *= rng.choice([-1.0, 1.0], (len(x0) - 1, 2)) * 2.0 ** rng.integers(-60, 60, (len(x0) - 1, 1))
+    n = len(x0)
+    g = _gpu_graph(n, np.zeros(n - 1, np.int32), np.arange(1, n, dtype=np.int32))
+    piv = torch.zeros(1, dtype=torch.int32, device=DEV)
+    dip = ssm.ssm_pivot_bfs(g, piv)
+    P = ssm.Pivots(1, piv, dip, *ssm.ssm_aggregate(dip, ssm.ssm_aggregate_size(dip)))
+    pos = torch.from_numpy(x0.copy()).to(DEV)
+    ssm.ssm_iterate(g, P, pos, 1)
+    d = x0[1:]
+    want = d / np.sqrt(d[:, 0] * d[:, 0] + d[:, 1] * d[:, 1])[:, None]
+    assert np.array_equal(pos.cpu().numpy()[1:], want)
