@@ -476,22 +476,30 @@ __global__ void k_sssp_labels(int64_t count, unsigned *__restrict__ dist, int32_
   if (inf) dev_fail(status, SSM_E_DISCONNECTED);
 }
 
-size_t sssp_ws_bytes(int32_t n, int32_t k) { return 256 + sssp_slot_bytes(n) * (size_t)sssp_blocks(k); }
+// Blocks of half the width, four at once on an SM and not two, where there are
+// many sources and their rounds are narrow: 1024 sources take 2.6 against 3.1 ms on
+// 20K nodes, but 43 against 32 ms on 262K.  As many blocks as run at once: each
+// has its queues in the workspace.
+struct SsspShape {
+  int threads, blocks;
+};
+static SsspShape sssp_shape(int32_t n, int32_t k) {
+  const bool half = k > 2 * num_sms() && n < 65536;
+  return {half ? kSsspThreads / 2 : kSsspThreads, std::max(1, std::min<int>(k, num_sms() * (half ? 4 : 2)))};
+}
+
+size_t sssp_ws_bytes(int32_t n, int32_t k) { return 256 + sssp_slot_bytes(n) * (size_t)sssp_shape(n, k).blocks; }
 
 int launch_sssp(int32_t n, const int32_t *rowptr, const int32_t *colidx, const float *elen, int32_t k,
                 const int32_t *sources, float *dist, int32_t *status, void *ws, size_t ws_bytes, cudaStream_t s) {
-  const int blocks = sssp_blocks(k);
+  const SsspShape shape = sssp_shape(n, k);
   const size_t sb = sssp_slot_bytes(n);
   if (ws_bytes < sssp_ws_bytes(n, k))
     return fail(SSM_E_NOMEM, "sssp: workspace %zu bytes, need %zu", ws_bytes, sssp_ws_bytes(n, k));
   MeanWs *mean = (MeanWs *)ws;
   char *slots = (char *)ws + 256;
   if (int rc = launch_mean_length(n, rowptr, elen, mean, s)) return rc;
-  // blocks of half the width, twice as many at once, where there are many
-  // sources and their rounds are narrow: 1024 sources take 2.6 against 3.1 ms
-  // on 20K nodes, but 43 against 32 ms on 262K
-  const int threads = k > 2 * num_sms() && n < 65536 ? kSsspThreads / 2 : kSsspThreads;
-  note_launch(), k_sssp_multi<<<blocks, threads, 0, s>>>(n, rowptr, colidx, (const unsigned *)elen, k, sources,
+  note_launch(), k_sssp_multi<<<shape.blocks, shape.threads, 0, s>>>(n, rowptr, colidx, (const unsigned *)elen, k, sources,
                                                        (unsigned *)dist, mean, slots, sb, status);
   const int64_t cnt = (int64_t)k * n;
   note_launch(), k_sssp_labels<<<(unsigned)std::min<int64_t>((cnt / 4 + 255) / 256 + 1, (int64_t)num_sms() * 16), 256, 0, s>>>(
@@ -499,8 +507,6 @@ int launch_sssp(int32_t n, const int32_t *rowptr, const int32_t *colidx, const f
   SSM_TRY_CUDA(cudaGetLastError());
   return SSM_OK;
 }
-
-int sssp_blocks(int32_t k) { return std::max(1, std::min<int>(k, num_sms() * 4)); }
 
 // ------------------------------------------------------------ regions and s
 __global__ void k_wregion_keys(int32_t n, int32_t k, const float *__restrict__ dist, int32_t *__restrict__ region,

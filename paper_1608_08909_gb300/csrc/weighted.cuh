@@ -5,10 +5,7 @@
 
 namespace ssm {
 
-// Blocks the multi-source search runs (one source per block at a time) and
-// the workspace bytes of one block's queues.
-int sssp_blocks(int32_t k);
-size_t sssp_slot_bytes(int32_t n);
+size_t sssp_slot_bytes(int32_t n);  // the queues of one search
 size_t sssp_ws_bytes(int32_t n, int32_t k);  // launch_sssp's workspace
 // dist[a*n + v] = least float32 path sum from sources[a] to v, for a < k;
 // an unreachable node flags SSM_E_DISCONNECTED.  ws holds

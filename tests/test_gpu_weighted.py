@@ -352,3 +352,12 @@ def test_weighted_pivotmds_one_far_node(seed, k):
         v = v / np.sqrt((v * v).sum())
     lam = ((v @ c) ** 2).sum()
     assert abs(eig[0].item() - lam) < 32 * 2.0 ** -53 * lam
+
+
+@pytest.mark.parametrize("n,k,per_sm", [(65535, 1024, 4), (65536, 1024, 2), (1 << 20, 1024, 2), (65535, 8, 0)])
+def test_weighted_search_workspace_is_what_runs_at_once(n, k, per_sm):
+    """Queues (four of n words, on 256 bytes) for as many searches as the blocks
+    of the chosen width that an SM holds: no call asks for memory that its
+    kernel cannot use."""
+    slots = min(k, per_sm * torch.cuda.get_device_properties(0).multi_processor_count) if per_sm else k
+    assert ssm.lib().ssm_pivot_sssp_workspace(n, k) == 256 + slots * 4 * ((4 * n + 255) // 256 * 256)
