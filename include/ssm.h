@@ -155,8 +155,15 @@ int ssm_select_pivots(int32_t n, int64_t m, const int32_t *rowptr, const int32_t
  * once).  1 <= k <= min(n, 1024), 1 <= max_iter.  Device error SSM_E_ARG
  * when n * max(d) >= 2^32 or n * k * max(d)^2 >= 2^53 (the bounds of the
  * exact integer arithmetic) or a pivot id is outside 0..n-1.
+ * Workspace: ssm_kmeans_pivots_workspace, which for k <= 208 holds a 16-bit
+ * copy of the whole table (the tensor-core filter's, used while k times half
+ * the largest distance stays below 2^18).  From ssm_kmeans_pivots_workspace_least
+ * (about 20 n bytes) on a smaller one is accepted: the results are the same,
+ * from 64-bit integer products, which take some thirty times as long on a
+ * small-world graph.
  * ------------------------------------------------------------------- */
 size_t ssm_kmeans_pivots_workspace(int32_t n, int32_t k);
+size_t ssm_kmeans_pivots_workspace_least(int32_t n, int32_t k);
 int ssm_kmeans_pivots(int32_t n, int32_t k, const uint16_t *dip, const int32_t *pivots_in, int32_t max_iter,
                       int32_t *pivots_out, int32_t *assign, int32_t *iters, int32_t *status,
                       void *ws, size_t ws_bytes, cudaStream_t stream);

@@ -70,6 +70,7 @@ def lib():
                 "ssm_select_pivots_workspace": (sz, [i32, i64]),
                 "ssm_select_pivots": (ctypes.c_int, [i32, i64, v, v, i32, i32, v, v, v, sz, v]),
                 "ssm_kmeans_pivots_workspace": (sz, [i32, i32]),
+                "ssm_kmeans_pivots_workspace_least": (sz, [i32, i32]),
                 "ssm_kmeans_pivots": (ctypes.c_int, [i32, i32, v, v, i32, v, v, v, v, v, sz, v]),
                 "ssm_pivot_bfs_workspace": (sz, [i32, i64, i32]),
                 "ssm_pivot_bfs": (ctypes.c_int, [i32, i64, v, v, i32, v, v, v, v, sz, v]),
@@ -246,7 +247,10 @@ def ssm_kmeans_pivots(dip: torch.Tensor, pivots: torch.Tensor, max_iter: int = 5
     asg = torch.empty(n, dtype=torch.int32, device=dev)
     it = torch.zeros(1, dtype=torch.int32, device=dev)
     st = _status(dev)
-    ws = _ws(L.ssm_kmeans_pivots_workspace(n, k), dev)
+    try:
+        ws = _ws(L.ssm_kmeans_pivots_workspace(n, k), dev)
+    except torch.cuda.OutOfMemoryError:  # no room for a second copy of the table: the same results without it
+        ws = _ws(L.ssm_kmeans_pivots_workspace_least(n, k), dev)
     _rc(L.ssm_kmeans_pivots(n, k, _ptr(dip), _ptr(pivots.contiguous()), max_iter, _ptr(out), _ptr(asg), _ptr(it),
                             _ptr(st), _ptr(ws), ws.numel(), _stream(stream)), "ssm_kmeans_pivots")
     if check:

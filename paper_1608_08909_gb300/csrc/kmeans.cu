@@ -56,6 +56,8 @@
 // 22-34 us, the moves 85 us (pass 2) to 22 us (pass 50), the centres 6 us.
 // Every pass is launched up front and stops on the device (no host round
 // trip), so the call is asynchronous.
+// The filter's arrays take as much memory as the table itself; a caller who has
+// less than they need gets the integer products instead.
 // Exactness needs n * max(d) < 2^32 (32-bit centre sums) and
 // n * k * max(d)^2 < 2^53 (t and n_a ||y||^2 exact in FP64 / int64); both are
 // checked on the device (SSM_E_ARG).
@@ -167,8 +169,8 @@ __global__ void k_km_dmax(int64_t count, const uint16_t *__restrict__ dip, unsig
 
 // centre a = y of pivot a; the exactness bounds are checked and the filter's
 // width is chosen here
-__global__ void k_km_init(int32_t n, int32_t k, const uint16_t *__restrict__ dip, const int32_t *__restrict__ piv,
-                          KmState W, int32_t *__restrict__ status) {
+__global__ void k_km_init(int32_t n, int32_t k, int tc, const uint16_t *__restrict__ dip,
+                          const int32_t *__restrict__ piv, KmState W, int32_t *__restrict__ status) {
   const unsigned dmx = *W.dmax;
   const double dm = (double)dmx;
   if ((double)n * dm >= 4294967296.0 || (double)n * (double)k * dm * dm >= 9007199254740992.0) {
@@ -186,7 +188,7 @@ __global__ void k_km_init(int32_t n, int32_t k, const uint16_t *__restrict__ dip
     int w = 12;
     while (w > 1 && (int64_t)k * c * (1ll << (w - 1)) > (1ll << 24)) --w;
     F.w = w;
-    F.on = k <= kKtMaxK && c <= 2048 && w >= kKtMinBits ? 1 : 0;
+    F.on = tc && c <= 2048 && w >= kKtMinBits ? 1 : 0;
     int f = 0;
     if (F.on) {  // the largest f with c 2^f <= 2^(2w-1) - 2^w
       const int64_t top = (1ll << (2 * w - 1)) - (1ll << w);
@@ -1008,8 +1010,8 @@ __global__ void k_km_fill(int32_t k, KmState W) {
   }
 }
 
-static size_t carve_kmeans(Carver &c, KmState &W, int32_t **assign_ws, int32_t n, int32_t k) {
-  const bool tc = k <= kKtMaxK;
+// tc: with the filter's arrays, which hold a copy of the whole table
+static size_t carve_kmeans(Carver &c, KmState &W, int32_t **assign_ws, int32_t n, int32_t k, bool tc) {
   W.S = c.take<unsigned>((size_t)k * kt_pad(k));
   W.ST = c.take<unsigned>((size_t)k * k);
   W.M = c.take<unsigned>(km_sum_words(k));
@@ -1025,6 +1027,7 @@ static size_t carve_kmeans(Carver &c, KmState &W, int32_t **assign_ws, int32_t n
   W.open = c.take<unsigned>(2);
   W.wide = c.take<unsigned>(2);
   W.list = c.take<int4>((size_t)n);
+  W.vnode = reinterpret_cast<long long *>(W.list);  // the moves are over when the pivots are chosen
   W.unsure = tc ? c.take<int2>((size_t)n) : nullptr;
   W.tau = tc ? c.take<float>((size_t)n) : nullptr;
   W.hbase = tc ? c.take<float>((size_t)kt_pad(k)) : nullptr;
@@ -1032,7 +1035,6 @@ static size_t carve_kmeans(Carver &c, KmState &W, int32_t **assign_ws, int32_t n
   W.image = tc ? c.take<unsigned char>(((size_t)n + kKtTile - 1) / kKtTile * kt_tile_bytes(k)) : nullptr;
   W.vbest = c.take<long long>((size_t)k);
   W.pbest = c.take<int32_t>((size_t)k);
-  W.vnode = c.take<long long>((size_t)n);
   *assign_ws = c.take<int32_t>((size_t)n);
   return c.size();
 }
@@ -1044,7 +1046,15 @@ SSM_API size_t ssm_kmeans_pivots_workspace(int32_t n, int32_t k) {
   ssm::Carver c(nullptr, 0);
   ssm::KmState W;
   int32_t *a;
-  return ssm::carve_kmeans(c, W, &a, n, k);
+  return ssm::carve_kmeans(c, W, &a, n, k, k <= ssm::kKtMaxK);
+}
+
+SSM_API size_t ssm_kmeans_pivots_workspace_least(int32_t n, int32_t k) {
+  if (n < 1 || k < 1) return 0;
+  ssm::Carver c(nullptr, 0);
+  ssm::KmState W;
+  int32_t *a;
+  return ssm::carve_kmeans(c, W, &a, n, k, false);
 }
 
 SSM_API int ssm_kmeans_pivots(int32_t n, int32_t k, const uint16_t *dip, const int32_t *pivots_in, int32_t max_iter,
@@ -1055,14 +1065,16 @@ SSM_API int ssm_kmeans_pivots(int32_t n, int32_t k, const uint16_t *dip, const i
     return fail(SSM_E_ARG, "ssm_kmeans_pivots: null pointer or bad size");
   if (k < 1 || k > kKmMaxK || k > n) return fail(SSM_E_ARG, "ssm_kmeans_pivots: need 1 <= k <= min(n, %d)", kKmMaxK);
   if (max_iter < 1) return fail(SSM_E_ARG, "ssm_kmeans_pivots: max_iter must be >= 1");
+  // without room for the filter every pass takes the integer products, with the
+  // same results
+  const bool tc = k <= kKtMaxK && ws_bytes >= ssm_kmeans_pivots_workspace(n, k);
   Carver c(ws, ws_bytes);
   KmState W;
   int32_t *asg_ws = nullptr;
-  carve_kmeans(c, W, &asg_ws, n, k);
+  carve_kmeans(c, W, &asg_ws, n, k, tc);
   if (!c.ok) return fail(SSM_E_NOMEM, "ssm_kmeans_pivots: workspace %zu bytes, need %zu", ws_bytes, c.size());
   int32_t *asg = assign ? assign : asg_ws;
   const int sms = num_sms();
-  const bool tc = k <= kKtMaxK;
   SSM_TRY_CUDA(cudaMemsetAsync(W.dmax, 0, sizeof(unsigned), s));
   SSM_TRY_CUDA(cudaMemsetAsync(W.stop, 0, sizeof(int32_t), s));
   SSM_TRY_CUDA(cudaMemsetAsync(iters, 0, sizeof(int32_t), s));
@@ -1070,7 +1082,7 @@ SSM_API int ssm_kmeans_pivots(int32_t n, int32_t k, const uint16_t *dip, const i
   const int64_t kn = (int64_t)k * n;
   note_launch(), k_km_dmax<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((kn / 8 + 255) / 256, sms * 8)), 256, 0, s>>>(
       kn, dip, W.dmax);
-  note_launch(), k_km_init<<<std::min(k, sms * 4), 256, 0, s>>>(n, k, dip, pivots_in, W, status);
+  note_launch(), k_km_init<<<std::min(k, sms * 4), 256, 0, s>>>(n, k, tc ? 1 : 0, dip, pivots_in, W, status);
   const int kt_tiles = (int)(((int64_t)n + kKtTile - 1) / kKtTile);
   const int tiles = (int)(((int64_t)n + kKmNodes - 1) / kKmNodes);
   const size_t smem = tc ? (size_t)kt_digit_bytes(k) + kt_tile_bytes(k) : 0;

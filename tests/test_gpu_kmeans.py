@@ -111,3 +111,30 @@ def test_kmeans_sp_filter_edges(k, n, dmax, passes):
     assert int(got_it.item()) == want_it
     assert np.array_equal(got_a.cpu().numpy(), want_a)
     assert np.array_equal(got_p.cpu().numpy(), want_p)
+
+
+@pytest.mark.parametrize("k", [30, 208, 209])
+def test_kmeans_sp_with_the_least_workspace(k):
+    """A workspace without room for the filter's copy of the table gives the same
+    results; one byte less is refused.  No more than 24 bytes a node beyond
+    the k x k sums."""
+    n, passes = 3001, 6
+    dip = I.distance_table(k, n, 60, 5 + k)
+    piv = np.random.default_rng(k).permutation(n)[:k].astype(np.int32)
+    want_p, want_a, want_it = O.kmeans_sp(dip, piv, passes)
+    L, dt, dp = ssm.lib(), torch.from_numpy(dip).to(DEV), torch.from_numpy(piv).to(DEV)
+    least = L.ssm_kmeans_pivots_workspace_least(n, k)
+    assert least <= L.ssm_kmeans_pivots_workspace(n, k) and least <= 24 * n + 16 * (k + 16) ** 2 + 8192
+    out, asg = torch.empty(k, dtype=torch.int32, device=DEV), torch.empty(n, dtype=torch.int32, device=DEV)
+    it, st = torch.zeros(1, dtype=torch.int32, device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    ws = torch.empty(least, dtype=torch.uint8, device=DEV)
+
+    def call(size):
+        return L.ssm_kmeans_pivots(n, k, dt.data_ptr(), dp.data_ptr(), passes, out.data_ptr(), asg.data_ptr(),
+                                   it.data_ptr(), st.data_ptr(), ws.data_ptr(), size, torch.cuda.current_stream().cuda_stream)
+
+    assert call(least - 256) == -5
+    assert call(least) == 0 and st.item() == 0
+    assert int(it.item()) == want_it
+    assert np.array_equal(asg.cpu().numpy(), want_a)
+    assert np.array_equal(out.cpu().numpy(), want_p)
