@@ -616,6 +616,13 @@ __global__ void __launch_bounds__(kKtThreads, 1) k_km_assign_tc(int32_t n, int32
   if (warp == 16) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
+// Too many nodes are left with all clusters: k_km_assign takes the whole pass, at
+// 8 ns a node (k = 200), where k_km_resolve takes 36 for such a node.  (A star:
+// all leaves are equally far from all centres; 2^18 leaves, two passes: 11.0 -> 3.0 ms.)
+__device__ __forceinline__ bool km_mostly_wide(const KmState &W, int32_t n, int32_t pass) {
+  return __ldcg(W.wide + (pass & 1)) > (unsigned)n / 6u;
+}
+
 // one assignment pass without the filter, 64 nodes at a time: the distances of
 // the tile and the sums of 64 clusters are staged 64 pivots at a time
 __global__ void __launch_bounds__(kKmThreads) k_km_assign(int32_t n, int32_t k, int32_t pass,
@@ -627,7 +634,7 @@ __global__ void __launch_bounds__(kKmThreads) k_km_assign(int32_t n, int32_t k, 
   __shared__ int ba[16][kKmNodes];                             // and its cluster
   __shared__ double s_best[kKmNodes];
   __shared__ int s_arg[kKmNodes];
-  if (__ldcg(W.stop) || W.filt->on) return;
+  if (__ldcg(W.stop) || (W.filt->on && !km_mostly_wide(W, n, pass))) return;
   const int tid = threadIdx.x;
   const int tn = tid & 15, ta = tid >> 4;  // node group (4 nodes), cluster group (4 clusters)
   for (int n0 = blockIdx.x * kKmNodes; n0 < n; n0 += gridDim.x * kKmNodes) {
@@ -740,7 +747,7 @@ __global__ void __launch_bounds__(256, 3) k_km_resolve(int32_t n, int32_t k, int
   __shared__ int s_at[8];
   if (__ldcg(W.stop)) return;
   const KmFilter F = *W.filt;
-  if (!F.on) return;
+  if (!F.on || km_mostly_wide(W, n, pass)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned nopen = __ldcg(W.open + (pass & 1)), nwide = __ldcg(W.wide + (pass & 1));
   constexpr int kRegs = (kKtMaxK + 31) / 32;

@@ -138,3 +138,21 @@ def test_kmeans_sp_with_the_least_workspace(k):
     assert int(it.item()) == want_it
     assert np.array_equal(asg.cpu().numpy(), want_a)
     assert np.array_equal(out.cpu().numpy(), want_p)
+
+
+@pytest.mark.parametrize("share", [0.14, 0.2, 1.0])
+def test_kmeans_sp_ties_with_all_clusters(share):
+    """Nodes equally far from all centres, on both sides of the sixth of the
+    nodes from which the integer products take the whole pass: bit-exact."""
+    n, k, passes = 4000, 40, 5
+    rng = np.random.default_rng(3)
+    dip = rng.integers(1, 9, (k, n)).astype(np.uint16)
+    dip[:, rng.permutation(n)[:int(share * n)]] = 2  # as a star's leaves
+    piv = rng.permutation(n)[:k].astype(np.int32)
+    dip[:, piv] = 2
+    dip[np.arange(k), piv] = 0
+    want_p, want_a, want_it = O.kmeans_sp(dip, piv, passes)
+    got_p, got_a, got_it = ssm.ssm_kmeans_pivots(torch.from_numpy(dip).to(DEV), torch.from_numpy(piv).to(DEV), passes)
+    assert int(got_it.item()) == want_it
+    assert np.array_equal(got_a.cpu().numpy(), want_a)
+    assert np.array_equal(got_p.cpu().numpy(), want_p)
