@@ -618,7 +618,8 @@ __global__ void k_seg_start(int32_t k, const unsigned long long *__restrict__ ke
 
 // s_ia for one pivot (blockIdx.x) and a range of nodes: the entries of region a
 // with 2 d_ja <= d_ia are a prefix of its sorted segment, found by binary search
-// in shared memory (a segment of more than kCountSeg entries: in global memory).
+// in shared memory; of a segment of more than kCountSeg entries, every
+// stride-th is there, and the search ends in global memory between two of them.
 // One search over global memory per (pivot, node), with a binary search of the
 // node's row for the pivot, took 1.62 ms on 52 M pairs, now 0.26; the pivot and its
 // neighbours, where s is 0, are cleared afterwards (k_wcounts_near).
@@ -630,20 +631,35 @@ __global__ void __launch_bounds__(256) k_wcounts(int32_t n, const float *__restr
   const int a = blockIdx.x;
   const int64_t lo = seg[a];
   const int len = (int)(seg[a + 1] - lo);
-  const bool staged = len <= kCountSeg;
-  if (staged)
-    for (int t = threadIdx.x; t < len; t += blockDim.x) sd[t] = __fmul_rn(2.0f, __uint_as_float((unsigned)keys[lo + t]));
+  const int stride = (len + kCountSeg - 1) / kCountSeg, kept = stride > 1 ? (len + stride - 1) / stride : len;
+  auto twice = [&](int t) { return __fmul_rn(2.0f, __uint_as_float((unsigned)__ldg(keys + lo + t))); };
+  for (int t0 = threadIdx.x; t0 < kept; t0 += 8 * (int)blockDim.x) {  // eight loads in flight
+    float v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = twice(min(t0 + q * (int)blockDim.x, kept - 1) * stride);
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (t0 + q * (int)blockDim.x < kept) sd[t0 + q * (int)blockDim.x] = v[q];
+  }
   __syncthreads();
   const float *d = dist + (size_t)a * n;
   uint32_t *out = s_out + (size_t)a * n;
   for (int64_t i = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.y * blockDim.x) {
     const float di = __ldg(d + i);
-    int b = 0, e = len;
+    int b = 0, e = kept;
     while (b < e) {
       const int mid = (b + e) >> 1;
-      const float v = staged ? sd[mid] : __fmul_rn(2.0f, __uint_as_float((unsigned)keys[lo + mid]));
-      if (v <= di) b = mid + 1;
+      if (sd[mid] <= di) b = mid + 1;
       else e = mid;
+    }
+    if (stride > 1 && b > 0) {  // entry (b - 1) stride is below, entry b stride is not
+      e = min(b * stride, len);
+      b = (b - 1) * stride + 1;
+      while (b < e) {
+        const int mid = (b + e) >> 1;
+        if (twice(mid) <= di) b = mid + 1;
+        else e = mid;
+      }
     }
     out[i] = (uint32_t)b;
   }
@@ -1030,7 +1046,10 @@ SSM_API int ssm_weighted_counts(int32_t n, const int32_t *rowptr, const int32_t 
       n, k, dist, region, w.keys, npad);
   if (int rc = launch_sort(w.keys, npad, s)) return rc;
   note_launch(), k_seg_start<<<std::max(1, (k + 256) / 256), 256, 0, s>>>(k, w.keys, npad, w.seg);
-  note_launch(), k_wcounts<<<dim3((unsigned)k, (unsigned)std::min((n + 8191) / 8192, 65535)), 256, 0, s>>>(n, dist, w.keys, w.seg, s_tab);
+  // 2048 nodes a block (a star's one large region is then some n / 2048 blocks' work),
+  // fewer where there would be less than two blocks per SM
+  const int64_t parts = std::max<int64_t>(((int64_t)n + 2047) / 2048, std::min<int64_t>(((int64_t)n + 255) / 256, (2 * sms + k - 1) / k));
+  note_launch(), k_wcounts<<<dim3((unsigned)k, (unsigned)std::min<int64_t>(parts, 65535)), 256, 0, s>>>(n, dist, w.keys, w.seg, s_tab);
   note_launch(), k_wcounts_near<<<k, 128, 0, s>>>(n, rowptr, colidx, pivots, s_tab);
   SSM_TRY_CUDA(cudaGetLastError());
   return SSM_OK;

@@ -361,3 +361,20 @@ def test_weighted_search_workspace_is_what_runs_at_once(n, k, per_sm):
     kernel cannot use."""
     slots = min(k, per_sm * torch.cuda.get_device_properties(0).multi_processor_count) if per_sm else k
     assert ssm.lib().ssm_pivot_sssp_workspace(n, k) == 256 + slots * 4 * ((4 * n + 255) // 256 * 256)
+
+
+@pytest.mark.parametrize("n,k", [(8191, 1), (8193, 1), (20000, 1), (50000, 3)])
+def test_weighted_counts_of_segments_beyond_shared_memory(n, k):
+    """Regions of up to seven times the entries that a block keeps, equal
+    distances among them: the counts by sorting each region's distances."""
+    rng = np.random.default_rng(n)
+    dist = rng.choice(np.concatenate([[1.0, 2.0, 4.0], rng.uniform(0.5, 8.0, n // 2)]), (k, n)).astype(np.float32)
+    s, d, l = np.arange(n - 1, dtype=np.int32), np.arange(1, n, dtype=np.int32), np.ones(n - 1, np.float32)
+    piv = rng.permutation(n)[:k].astype(np.int32)
+    greg, gs = ssm.ssm_weighted_counts(_gpu_wgraph(n, s, d, l), torch.from_numpy(piv).to(DEV), torch.from_numpy(dist).to(DEV))
+    reg = dist.argmin(0)
+    assert np.array_equal(greg.cpu().numpy(), reg)
+    for a in range(k):
+        want = np.searchsorted(np.sort(np.float32(2) * dist[a][reg == a]), dist[a], side="right").astype(np.uint32)
+        want[[i for i in (piv[a] - 1, piv[a], piv[a] + 1) if 0 <= i < n]] = 0
+        assert np.array_equal(gs[a].cpu().numpy().view(np.uint32), want)
