@@ -155,11 +155,12 @@ struct SsspQueues {
 
 // The whole warp: places in a queue (counter in shared memory) for the flagged
 // (lane, slot) pairs, one atomic for all of them; places[q] is set where flag[q]
-__device__ __forceinline__ void sssp_places(const bool (&flag)[kSsspU], unsigned *counter, unsigned (&place)[kSsspU]) {
+template <int U>
+__device__ __forceinline__ void sssp_places(const bool (&flag)[U], unsigned *counter, unsigned (&place)[U]) {
   const unsigned lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
-  unsigned mask[kSsspU], total = 0;
+  unsigned mask[U], total = 0;
 #pragma unroll
-  for (int q = 0; q < kSsspU; ++q) {
+  for (int q = 0; q < U; ++q) {
     mask[q] = __ballot_sync(0xffffffffu, flag[q]);
     total += __popc(mask[q]);
   }
@@ -168,7 +169,7 @@ __device__ __forceinline__ void sssp_places(const bool (&flag)[kSsspU], unsigned
   if (lane == 0) at = atomicAdd(counter, total);
   at = __shfl_sync(0xffffffffu, at, 0);
 #pragma unroll
-  for (int q = 0; q < kSsspU; ++q) {
+  for (int q = 0; q < U; ++q) {
     place[q] = at + __popc(mask[q] & below);
     at += __popc(mask[q]);
   }
@@ -266,6 +267,36 @@ __device__ void sssp_block(int32_t n, const int32_t *__restrict__ rowptr, const 
         if ((int)lane >= o) incl += t;
       }
       const int total = __shfl_sync(0xffffffffu, incl, 31);
+      // up to 32 edges (a path's rounds): no read before the atomicMin, whose
+      // round trip is then the longest in the chain that is left
+      if (total <= 32) {
+        const int t = (int)lane;
+        bool act = t < total;
+        int lo = 0;
+#pragma unroll
+        for (int step = 16; step >= 1; step >>= 1) {
+          const int pv = __shfl_sync(0xffffffffu, incl, lo + step - 1);
+          if (pv <= t) lo += step;
+        }
+        const int at = lo > 31 ? 31 : lo;
+        const int pos = __shfl_sync(0xffffffffu, e, at) - (__shfl_sync(0xffffffffu, incl, at) - t);
+        const int u = act ? __ldg(colidx + pos) : 0;
+        const unsigned len = act ? __ldg(elen + pos) : 0u;
+        const unsigned nb = __float_as_uint(__fadd_rn(__uint_as_float(__shfl_sync(0xffffffffu, dv, at)), __uint_as_float(len)));
+        act = act && nb < kInfBits;
+        const unsigned old = act ? atomicMin(row + u, 2u * nb + 1u) : 0u;
+        const int rb = act ? __ldg(rowptr + u) : 0, re = act ? __ldg(rowptr + u + 1) : 0;
+        const bool lower = act && (old >> 1) > nb, was = (old & 1u) != 0u, below = nb < tbits;
+        const bool near[1] = {lower && below && (!was || (old >> 1) >= tbits)}, far[1] = {lower && !below && !was};
+        unsigned place[1] = {};
+        sssp_places(near, next, place);
+        if (near[0]) Q.put_near(cur ^ 1, place[0], make_int4(u, rb, re, 0));
+        sssp_places(far, &s_far, place);
+        if (far[0]) Q.put_far(fcur, place[0], u);
+        const unsigned least = __reduce_min_sync(0xffffffffu, lower && !below ? nb : 0xFFFFFFFFu);
+        if (lane == 0 && least != 0xFFFFFFFFu) atomicMin(&s_least, least);
+        continue;
+      }
       for (int s0 = 0; s0 < total; s0 += 32 * kSsspU) {
         int u[kSsspU], at[kSsspU];
         unsigned nb[kSsspU], len[kSsspU];
