@@ -618,15 +618,20 @@ __global__ void __launch_bounds__(kEigThreads) k_eigen(int32_t n, int32_t k, con
     // vector's growth over the second below 2^8 (Gram-Schmidt then leaves
     // 2^8 of FP64's rounding in it, far below tol) and over the last below
     // 2^32.  ba1m, k = 200: 0.69 ms, with one product each 1.94 ms.
-    const double g2 = H[0] / H[(P > 1 ? 1 : 0) * (P + 1)], gP = H[0] / H[(P - 1) * (P + 1)];
-    double a2 = g2, aP = gP;
-    for (int p = 1; p < kEigMaxProducts; ++p) {
-      a2 *= g2;
-      aP *= gP;
-      if (!(a2 <= 256.0 && aP <= 4294967296.0)) break;  // (a Ritz value of zero: no)
-      for (int t = threadIdx.x; t < k * P; t += blockDim.x) V[t] = Y[t];
-      __syncthreads();
-      if (!product(M, P)) return;
+    // (Compared by products first: the divisions are 1 us of an iteration.)
+    const double h2 = H[(P > 1 ? 1 : 0) * (P + 1)], hP = H[(P - 1) * (P + 1)];
+    if (H[0] * H[0] <= 256.0 * (h2 * h2) && H[0] * H[0] <= 4294967296.0 * (hP * hP)) {  // (a Ritz value of zero: no)
+      const double g2 = H[0] / h2, gP = H[0] / hP;
+      double a2 = g2 * g2, aP = gP * gP;
+      int steps = 1;
+      do {
+        for (int t = threadIdx.x; t < k * P; t += blockDim.x) V[t] = Y[t];
+        __syncthreads();
+        if (!product(M, P)) return;
+        ++steps;
+        a2 *= g2;
+        aP *= gP;
+      } while (steps < kEigMaxProducts && a2 <= 256.0 && aP <= 4294967296.0);
     }
     for (int t = threadIdx.x; t < k * P; t += blockDim.x) V[t] = Y[t];
     __syncthreads();
