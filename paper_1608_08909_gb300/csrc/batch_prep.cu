@@ -100,7 +100,7 @@ __device__ int block_exclusive_scan(int *a, int len, int *s_part) {
 __global__ void __launch_bounds__(kPrepThreads) k_prep_pivots(PrepArgs A) {
   extern __shared__ __align__(16) unsigned char psm[];
   __shared__ int s_part[kPrepThreads / 32 + 1], s_ecc[kPrepMaxK];
-  __shared__ int s_task, s_len[3];
+  __shared__ int s_task, s_len[3], s_hub[kBsMaxHubs];
   __shared__ unsigned s_key[2];
   const int lane = threadIdx.x & 31;
   for (;;) {
@@ -201,7 +201,8 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_pivots(PrepArgs A) {
     if (threadIdx.x < 3) s_len[threadIdx.x] = 0;
     if (threadIdx.x < 2) s_key[threadIdx.x] = 0u;
     __syncthreads();
-    const BlockSearch B{key, off, nbr, qa, qb, s_len};
+    const BlockSearch B{key, off, nbr, qa, qb, s_len, s_hub};
+    const bool hubs = block_search_hubs(off, n);
     int slot = 0;
     for (int a = 0; a < k; ++a) {
       int p = 0;
@@ -218,7 +219,8 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_pivots(PrepArgs A) {
         A.pivots[D.piv_off + a] = p;
         s_key[(a + 1) & 1] = 0u;
       }
-      block_search(B, p, 7, a, slot);
+      if (hubs) block_search<true>(B, p, 7, a, slot);
+      else block_search<false>(B, p, 7, a, slot);
       if (a == 0)
         for (int i = threadIdx.x; i < n; i += blockDim.x)
           if (key[i] == kBsInf) dev_fail(A.status, SSM_E_DISCONNECTED);

@@ -393,3 +393,25 @@ def test_sweep_fp64_rounds_as_ieee_operations():
     d = x0[1:]
     want = d / np.sqrt(d[:, 0] * d[:, 0] + d[:, 1] * d[:, 1])[:, None]
     assert np.array_equal(pos.cpu().numpy()[1:], want)
+
+
+@pytest.mark.parametrize("n,hubs", [(1025, 1), (1026, 1), (9000, 2), (1100, 31), (1100, 32), (1100, 40)])
+def test_small_graph_hub_rows(n, hubs):
+    """Rows of more than 1,024 entries in the searches of one block's shared
+    memory, up to and beyond the 32 of a level that all warps share, single
+    graph and batch: the oracle's pivots and distances."""
+    n, s, d = _hubs(n, hubs)
+    order = np.random.default_rng(n + hubs).permutation(n).astype(np.int32)
+    s, d = order[s], order[d]
+    k = 20
+    og = O.build_csr(n, s, d)
+    piv = O.maxmin(og, k, 0)
+    dip = O.pivot_dist(og, piv)
+    g = _gpu_graph(n, s, d)
+    got = ssm.ssm_select_pivots(g, k, 0)
+    assert ssm.ssm_last_pivot_config()["cluster"] == 1
+    assert np.array_equal(got.cpu().numpy(), piv)
+    assert np.array_equal(ssm.ssm_pivot_bfs(g, got).cpu().numpy(), dip)
+    b = ssm.ssm_batch_prepare([(n, s, d, k)] * 2)
+    assert np.array_equal(b.pivots.cpu().numpy().reshape(2, k), np.stack([piv, piv]))
+    assert np.array_equal(b.dip.cpu().numpy().reshape(2, k, n), np.stack([dip, dip]))
