@@ -175,3 +175,17 @@ def test_batch_pivots_edges():
         dip = O.pivot_dist(og, piv)
         assert np.array_equal(v["dip"].cpu().numpy(), dip), g
         assert np.array_equal(v["region"].cpu().numpy(), O.regions(dip)), g
+
+
+@pytest.mark.parametrize("make", [lambda: I.path(12288), lambda: I.grid(3, 2000), lambda: I.grid(40, 300),
+                                  lambda: I.random_btree(4097, 3), lambda: I.path(31), lambda: I.grid(33, 31)])
+def test_batch_distances_of_narrow_and_wide_levels(make):
+    """Searches whose levels are a few nodes (marked chunks), many (all chunks)
+    and both in turn: bit-exact distances."""
+    n, s, d = make()
+    k = min(100, n // 2)
+    og = O.build_csr(n, s, d)
+    piv = O.maxmin(og, k, 0)
+    b = ssm.ssm_batch_prepare([(n, s, d, k)])
+    assert np.array_equal(b.pivots.cpu().numpy(), piv)
+    assert np.array_equal(b.dip.cpu().numpy().reshape(k, n), O.pivot_dist(og, piv))
