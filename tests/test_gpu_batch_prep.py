@@ -189,3 +189,20 @@ def test_batch_distances_of_narrow_and_wide_levels(make):
     b = ssm.ssm_batch_prepare([(n, s, d, k)])
     assert np.array_equal(b.pivots.cpu().numpy(), piv)
     assert np.array_equal(b.dip.cpu().numpy().reshape(k, n), O.pivot_dist(og, piv))
+
+
+@pytest.mark.parametrize("n,m,hub", [(2, 300, 0), (32, 900, 0), (33, 900, 40), (33, 1500, 0), (700, 30000, 699),
+                                     (12288, 500, 12287), (5000, 120000, 400)])
+def test_batch_csr_rows_of_all_lengths(n, m, hub):
+    """Rows on both sides of the 48 entries that one thread sorts, repeated edges
+    and self-loops among them, and of graphs of 32 nodes and one more."""
+    rng = np.random.default_rng(n + m)
+    s, d = rng.integers(0, n, m), rng.integers(0, n, m)
+    s = np.concatenate([s, np.zeros(hub, int), np.arange(n - 1)]).astype(np.int32)
+    d = np.concatenate([d, rng.integers(0, n, hub), np.arange(1, n)]).astype(np.int32)
+    og = O.build_csr(n, s, d)
+    b = ssm.ssm_batch_prepare([(n, s, d, min(4, n))] * 2, check=False)
+    for j in range(2):
+        v = b.graph(j)
+        assert np.array_equal(v["rowptr"].cpu().numpy(), og.rowptr)
+        assert np.array_equal(v["colidx"].cpu().numpy(), og.colidx)
