@@ -782,7 +782,12 @@ struct PivD {
 
 // d, d^2 and RN(1 / d^2) for d below kF64Dists
 constexpr int kF64Dists = 1024;
-constexpr int kF64LongRow = 16;  // longer rows: k_f64_long_rows
+// Rows longer than long_row are k_f64_long_rows': long_row is twice the mean degree,
+// at least kF64LongRow and at most kShortDeg (ba64k, k = 200, ten iterations: 16 10.35
+// ms, 32 10.50; geometric graph of 65,536 nodes, mean degree 20, k = 2: 2.4 and 1.5).
+// Where the hints count no row above kShortDeg there is no such launch (path of
+// 14,000 nodes, k = 2: 0.38 -> 0.34).
+constexpr int kF64LongRow = 16;
 struct DistD {
   double d, d2, inv;
 };
@@ -852,7 +857,7 @@ __device__ __forceinline__ double2 f64_neighbour(const double2 &x, const double2
   return over_length(dx, dy, dx, dy, ux, uy) ? make_double2(__dadd_rn(q.x, ux), __dadd_rn(q.y, uy)) : q;
 }
 
-// The neighbour sums of rows above kF64LongRow, a warp per row: the lanes form
+// The neighbour sums of rows above long_row, a warp per row: the lanes form
 // 32 summands at a time, which are added in CSR order (x in even lanes, y in odd
 // ones).  Consecutive rows go to different blocks: in a heavy-tailed graph the
 // first nodes are the hubs.  As part of the sweep a hub's row, in one lane, was
@@ -861,7 +866,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_f64_long_rows(int32_t n, cons
                                                                  const int32_t *__restrict__ colidx,
                                                                  const int32_t *__restrict__ stop,
                                                                  const double2 *__restrict__ pin,
-                                                                 double2 *__restrict__ nb) {
+                                                                 double2 *__restrict__ nb, int32_t long_row) {
   __shared__ double2 s_sum[kSweepThreads / 32][32];
   if (__ldcg(stop)) return;
   const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
@@ -869,7 +874,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_f64_long_rows(int32_t n, cons
   for (int64_t i0 = first; i0 < n; i0 += 32 * warps) {
     const int64_t i = i0 + lane * warps;  // lane's row: every warps-th
     const int b = i < n ? __ldg(rowptr + i) : 0, e = i < n ? __ldg(rowptr + i + 1) : 0;
-    for (unsigned m = __ballot_sync(0xffffffffu, e - b > kF64LongRow); m; m &= m - 1u) {
+    for (unsigned m = __ballot_sync(0xffffffffu, e - b > long_row); m; m &= m - 1u) {
       const int o = __ffs(m) - 1;
       const int ob = __shfl_sync(0xffffffffu, b, o), oe = __shfl_sync(0xffffffffu, e, o);
       const int64_t row = i0 + o * warps;
@@ -892,7 +897,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_f64_long_rows(int32_t n, cons
 template <bool CNT_SMEM>
 __global__ void __launch_bounds__(kSweepThreads) k_sweep_f64(SweepArgs A, const double2 *__restrict__ pin,
                                                               double2 *__restrict__ pout,
-                                                              const double2 *__restrict__ nb) {
+                                                              const double2 *__restrict__ nb, int32_t long_row) {
   extern __shared__ __align__(16) unsigned char smem[];
   PivD *piv = reinterpret_cast<PivD *>(smem);
   DistD *dist = reinterpret_cast<DistD *>(piv + A.k);  // [kF64Dists]
@@ -934,7 +939,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_sweep_f64(SweepArgs A, const 
     double nx = 0.0, ny = 0.0, den = 0.0;
     const int b = live ? __ldg(A.rowptr + i) : 0, e = live ? __ldg(A.rowptr + i + 1) : 0;
     if (live) {
-      if (e - b > kF64LongRow) {
+      if (e - b > long_row) {
         const double2 v = __ldg(nb + i);
         nx = v.x;
         ny = v.y;
@@ -1108,6 +1113,8 @@ SSM_API int ssm_iterate(int32_t n, int64_t m, const int32_t *rowptr, const int32
   int64_t tiles;
   unsigned meta[3] = {0, 0, 0};
   bool tsm = true;
+  const bool f64_long = !(hints && hints[1] == 0 && hints[2] == 0);
+  const int32_t long_row = f64_long ? (int32_t)std::max<int64_t>(kF64LongRow, std::min<int64_t>(kShortDeg, 4 * m / n)) : INT32_MAX;
   if (precision == 64) {
     const size_t piv = (size_t)k * sizeof(PivD) + kF64Dists * sizeof(DistD), tab = (size_t)cnt_len * sizeof(double);
     tsm = piv + tab <= kSmemBudget;
@@ -1248,11 +1255,13 @@ SSM_API int ssm_iterate(int32_t n, int64_t m, const int32_t *rowptr, const int32
       SSM_TRY_CUDA(cudaLaunchKernelExC(&cfg, kern, args));
       continue;
     }
-    note_launch(), k_f64_long_rows<<<(int)std::min<int64_t>(tiles, (int64_t)sms * 8), kSweepThreads, 0, s>>>(
-        n, rowptr, colidx, w.stop, (const double2 *)pin, w.nb64);
-    SSM_TRY_CUDA(cudaGetLastError());
+    if (f64_long) {
+      note_launch(), k_f64_long_rows<<<(int)std::min<int64_t>(tiles, (int64_t)sms * 8), kSweepThreads, 0, s>>>(
+          n, rowptr, colidx, w.stop, (const double2 *)pin, w.nb64, long_row);
+      SSM_TRY_CUDA(cudaGetLastError());
+    }
     const double2 *nb64 = w.nb64;
-    void *args[] = {&A, &pin, &pout, &nb64};
+    void *args[] = {&A, &pin, &pout, &nb64, const_cast<int32_t *>(&long_row)};
     note_launch();
     SSM_TRY_CUDA(cudaLaunchKernel(kern, dim3(blocks), dim3(kSweepThreads), args, smem, s));
   }
