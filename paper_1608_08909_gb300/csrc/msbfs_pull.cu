@@ -57,6 +57,7 @@ struct PullArgs {
   unsigned *fb;     // [kPullMaxLevels + 1][fbw] bit v of level L: F_L[v] is not zero (zeroed by the caller)
   size_t fbw;       // words per level bitmap (a multiple of 32: 128-byte rows)
   const int32_t *long_rows;  // nodes of degree above kPullLong
+  const unsigned *long_bits; // a bit per node: it is one of them
   const unsigned *nlong;     // how many (device)
   unsigned *nlev;   // levels with new bits (written when the pass completes)
   unsigned *flag;   // [6]: new bits seen at level L, nodes left unfinished (both by L mod 3)
@@ -131,7 +132,10 @@ __global__ void __launch_bounds__(kPullThreads, 2) k_msbfs_pull(PullArgs A) {
     unsigned pairs = 0;  // new (source, node) pairs of this lane (counted up to the probe level)
     for (unsigned base = gwarp * 32u; base < n; base += nwarps * 32u) {
       const unsigned v = base + lane;
-      const bool live = v < n;
+      // A long row is the second phase's in every respect, its words too when it
+      // has nothing new: a warp that is there already may have finished the row
+      // before this one comes by, and what it wrote must stay.
+      const bool live = v < n && !(__ldg(A.long_bits + (base >> 5)) >> lane & 1u);
       uint4 miss[kPullW4], acc[kPullW4];
       bool open = false;
 #pragma unroll
@@ -146,9 +150,7 @@ __global__ void __launch_bounds__(kPullThreads, 2) k_msbfs_pull(PullArgs A) {
         rb = __ldg(A.rowptr + v);
         re = __ldg(A.rowptr + v + 1);
       }
-      // rows longer than kPullLong wait for the second phase of the level
-      const bool deferred = open && re - rb > kPullLong;
-      if (open && re - rb <= kPullLong) {
+      if (open) {
         // four neighbours in flight, stop once every missing source turned up
         for (int t = rb; t < re; t += 4) {
           unsigned u[4];
@@ -185,9 +187,9 @@ __global__ void __launch_bounds__(kPullThreads, 2) k_msbfs_pull(PullArgs A) {
         left |= (nw[c].x ^ miss[c].x) | (nw[c].y ^ miss[c].y) | (nw[c].z ^ miss[c].z) | (nw[c].w ^ miss[c].w);
       }
       // this warp's 32 nodes in level L + 1's bitmap (a long row adds its bit later)
-      const unsigned fbits = __ballot_sync(0xffffffffu, live && !deferred && got);
+      const unsigned fbits = __ballot_sync(0xffffffffu, live && got);
       if (lane == 0 && fbits != 0u) atomicOr(fbnext + (base >> 5), fbits);
-      if (live && !deferred) {
+      if (live) {
 #pragma unroll
         for (int c = 0; c < kPullW4; ++c) {
           fnext[(size_t)v * kPullW4 + c] = nw[c];
@@ -201,16 +203,14 @@ __global__ void __launch_bounds__(kPullThreads, 2) k_msbfs_pull(PullArgs A) {
           }
         }
       }
-      if (!deferred) {
-        any_new |= got;
-        unfinished |= left;
-        if (L < kPullProbeLevel)
+      any_new |= got;
+      unfinished |= left;
+      if (L < kPullProbeLevel)
 #pragma unroll
-          for (int c = 0; c < kPullW4; ++c)
-            pairs += __popc(nw[c].x) + __popc(nw[c].y) + __popc(nw[c].z) + __popc(nw[c].w);
-      }
+        for (int c = 0; c < kPullW4; ++c)
+          pairs += __popc(nw[c].x) + __popc(nw[c].y) + __popc(nw[c].z) + __popc(nw[c].w);
     }
-    // second phase: the open long rows (hubs), one per warp across the grid,
+    // second phase: the long rows (hubs), one per warp across the grid,
     // kPullLongBatch entries per lane in flight, stopping once the node has
     // every missing source
     for (unsigned li = gwarp; li < nlong; li += nwarps) {
@@ -224,7 +224,10 @@ __global__ void __launch_bounds__(kPullThreads, 2) k_msbfs_pull(PullArgs A) {
         part[c] = make_uint4(0u, 0u, 0u, 0u);
         open |= (hmiss[c].x | hmiss[c].y | hmiss[c].z | hmiss[c].w) != 0u;
       }
-      if (!open) continue;  // warp-uniform; the first phase wrote its empty frontier word
+      if (!open) {  // warp-uniform
+        if (lane < kPullW4) fnext[(size_t)v * kPullW4 + lane] = make_uint4(0u, 0u, 0u, 0u);
+        continue;
+      }
       const int hb = __ldg(A.rowptr + v), he = __ldg(A.rowptr + v + 1);
       for (int t0 = hb + (int)lane; t0 - (int)lane < he; t0 += 32 * kPullLongBatch) {
         unsigned u[kPullLongBatch];
@@ -373,9 +376,14 @@ __global__ void __launch_bounds__(256) k_pull_distances(PullArgs A) {
 
 // the nodes of degree above kPullLong, in any order (the pass is order-free)
 __global__ void k_pull_long_rows(int32_t n, const int32_t *__restrict__ rowptr, int32_t *__restrict__ out,
-                                 unsigned *__restrict__ count) {
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
-    if (__ldg(rowptr + v + 1) - __ldg(rowptr + v) > kPullLong) out[atomicAdd(count, 1u)] = v;
+                                 unsigned *__restrict__ count, unsigned *__restrict__ bits) {
+  const int64_t padded = ((int64_t)n + 31) / 32 * 32;  // whole warps
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < padded; v += (int64_t)gridDim.x * blockDim.x) {
+    const bool lng = v < n && __ldg(rowptr + v + 1) - __ldg(rowptr + v) > kPullLong;
+    if (lng) out[atomicAdd(count, 1u)] = (int32_t)v;
+    const unsigned m = __ballot_sync(0xffffffffu, lng);
+    if ((threadIdx.x & 31) == 0) bits[v >> 5] = m;
+  }
 }
 
 // words of one level's frontier bitmap, rounded to whole 128-byte rows
@@ -387,6 +395,7 @@ size_t msbfs_pull_workspace(int32_t n) {
   c.take<uint4>((size_t)n * kPullW4 * (kPullMaxLevels + 1));
   c.take<unsigned>(pull_bitmap_words(n) * (kPullMaxLevels + 1));
   c.take<int32_t>((size_t)n);
+  c.take<unsigned>(((size_t)n + 31) / 32);
   c.take<unsigned>(1);
   c.take<unsigned>(1);
   c.take<unsigned>(6);
@@ -406,6 +415,7 @@ int launch_msbfs_pull(int32_t n, const int32_t *rowptr, const int32_t *colidx, i
   A.fbw = pull_bitmap_words(n);
   A.fb = c.take<unsigned>(A.fbw * (kPullMaxLevels + 1));
   int32_t *long_rows = c.take<int32_t>((size_t)n);
+  unsigned *long_bits = c.take<unsigned>(((size_t)n + 31) / 32);
   unsigned *nlong = c.take<unsigned>(1);
   A.nlev = c.take<unsigned>(1);
   A.flag = c.take<unsigned>(6);
@@ -418,9 +428,10 @@ int launch_msbfs_pull(int32_t n, const int32_t *rowptr, const int32_t *colidx, i
   // the long rows (listed on the device; the BFS reads their number there)
   SSM_TRY_CUDA(cudaMemsetAsync(nlong, 0, sizeof(unsigned), s));
   note_launch(), k_pull_long_rows<<<std::max(1, std::min((n + 255) / 256, num_sms() * 8)), 256, 0, s>>>(
-      n, rowptr, long_rows, nlong);
+      n, rowptr, long_rows, nlong, long_bits);
   SSM_TRY_CUDA(cudaGetLastError());
   A.long_rows = long_rows;
+  A.long_bits = long_bits;
   A.nlong = nlong;
   for (int base = 0; base < k; base += kPullSources) {
     A.base = base;

@@ -795,3 +795,19 @@ def test_iterate_rejects_a_dmax_hint_below_the_largest_distance():
     assert e.value.code == -1
     # the context stays usable
     ssm.ssm_iterate(g, P, pos, 1)
+
+
+def test_pivot_bfs_dense_graph_again_and_again():
+    """The pulled search where every row is a long one (two phases of a level
+    write the same nodes' words): the same table from 4,000 calls."""
+    rng = np.random.default_rng(1)
+    n, m = 1000, 150000
+    s, d = rng.integers(0, n, m).astype(np.int32), rng.integers(0, n, m).astype(np.int32)
+    og = O.build_csr(n, s, d)
+    piv = O.maxmin(og, 50, 0)
+    want = torch.from_numpy(O.pivot_dist(og, piv).view(np.int16)).to(DEV)
+    g, p = _gpu_graph(n, s, d), torch.from_numpy(piv).to(DEV)
+    wrong = torch.zeros((), dtype=torch.int64, device=DEV)
+    for _ in range(4000):
+        wrong += (ssm.ssm_pivot_bfs(g, p, check=False).view(torch.int16) != want).any()
+    assert wrong.item() == 0
