@@ -11,7 +11,7 @@
 // CTA: node v at (v mod C) per + v div C.  A lane has two consecutive nodes (packed FP32x2), so a pivot's
 // position is one broadcast and its table row is shared by 64 nodes; the warps
 // of a 64-node block share its pivots and neighbours (warp w every W-th), rows
-// above kScLong entries are a warp's work each (hubs: below), and a node's W + 1 partial sums
+// above `lng` entries are a warp's work each (hubs: below), and a node's W + 1 partial sums
 // are added in order.  (Lanes sharing a node, each with its own pivots, took
 // 1.4 to 5 times as long: every pivot position and table entry was a gather.)
 // A CTA stores its new positions into the other buffer of every CTA (distributed
@@ -32,7 +32,7 @@
 // that all its warps share (star of 8,000 nodes: 20.5, and 21 with a warp per
 // row; 6.9 so).  A CTA keeps the neighbours that its shared memory has room for
 // and reads the others from L2 in every iteration, which 16 SMs of one GPC do at
-// some 0.5 TB/s: the limit to this form on dense graphs (kScMaxRead).
+// some 0.5 TB/s.
 #include <algorithm>
 
 #include "cluster.cuh"
@@ -43,7 +43,12 @@ namespace ssm {
 
 constexpr int kScThreads = 1024;  // half as many where a CTA has fewer than kScWide (node, pivot) pairs
 constexpr int kScWide = 8192;
-constexpr int kScLong = 16;       // longest row that one lane per warp walks
+// The longest row that one lane per warp walks: twice the mean degree (a warp takes
+// 0.03 us over a row whatever its length: 8,000 nodes of degree 60, k = 2: 12.9 us an
+// iteration so, 19.6 with rows above 16 a warp's, 14.5 in two kernels), at least
+// kScLong; kScLong where the mean is above kScLaneMean
+constexpr int kScLong = 16;
+constexpr int kScLaneMean = 64;
 constexpr int kScHub = kMidDeg;   // longest row that one warp walks, if a CTA has few that are longer
 constexpr int kScMaxHubs = 64;    // (above this many they fill the warps as they are)
 constexpr int kScHubSegs = 128;   // a hub's entries per warp: so that these and one per hub are enough,
@@ -52,15 +57,18 @@ constexpr int kScMaxCluster = 16;
 constexpr int kScMaxN = 8192;     // node ids in 16 bits
 constexpr int kScMaxD = 4095;     // d^2 exact in FP32
 constexpr int kScMinIters = 4;    // the tables are formed by every launch
-// Neighbours per CTA, on average, beyond its shared memory: with 55,000 (8,000
-// nodes of degree 200, k = 3) 25 us an iteration against 15 in two kernels; with
-// 45,000 (clique of 1,500, k = 2) 16.0 against 15.5; with 12,000 (clique of 1,300,
-// k = 50) 13.9 against 18.3
-constexpr int64_t kScMaxRead = 49152;
+// Above that mean an iteration takes a CTA some 0.1 us per thousand neighbours and
+// 0.03 a row, two kernels at least 14 (k = 2) to 19 us (k = 50): rows count for
+// kScRowCost neighbours (more than their time, for the tables of a short run), and
+// above kScMaxDense the two kernels are taken.  (Here and there, k = 2 / 50: 4,000
+// nodes of degree 200 12.4 / 12.4 and 13.6 / 19; of degree 400 19 / 19 and 14 / 20;
+// 8,000 of degree 100 23 / 26 and 15 / 19; clique of 1,500 16.5 / 17 and 15.5 / 19.)
+constexpr int64_t kScRowCost = 500, kScMaxDense = 187700;
 constexpr float kScR2Floor = 1e-24f;
 
 struct ScArgs {
   int32_t n, k, dmax, per, perp, warps, iters;  // nodes per CTA (perp: up to whole blocks), warps per 64-node block
+  int32_t lng;   // longest row that one lane per warp walks
   int32_t ecap;  // neighbour ids of a CTA kept in shared memory
   int32_t hubs;  // there are rows above kScHub: the hubs' lists are part of the shared memory
   const int32_t *rowptr, *colidx, *pivots, *cnt_off;
@@ -218,11 +226,23 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
   }
   __syncthreads();
   auto here = [&](int li) { return rows[li + 1] <= A.ecap; };  // a row's neighbours are kept; else read from the graph
+  auto keep = [&](int li, int first, int step) {  // a row's neighbours, eight loads in flight
+    if (!here(li)) return;
+    const int32_t *col = A.colidx + start[li];
+    const int e = rows[li + 1];
+    for (int t = rows[li] + first; t < e; t += 8 * step) {
+      int v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = __ldg(col + min(t + q * step, e - 1));
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (t + q * step < e) cols[t + q * step] = (uint16_t)at(v[q]);
+    }
+  };
   for (int li = tid; li < own; li += T) {
     const int e = __ldg(A.rowptr + li * (int)C + (int)r), t0 = rows[li], len = rows[li + 1] - t0;
     start[li] = e - t0;
-    if (len <= kScLong && here(li))
-      for (int t = 0; t < len; ++t) cols[t0 + t] = (uint16_t)at(__ldg(A.colidx + e + t));
+    if (len <= A.lng) keep(li, 0, 1);
     if (len > kScHub) {
       atomicAdd(&s_nhub, 1);
       atomicAdd(&s_hubsum, len);
@@ -242,24 +262,11 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
       hub->node[h] = li;
       hub->first[h] = first;
       for (int q = 0; q < c; ++q) hub->seg[first + q] = li | q << 16;
-    } else if (len > kScLong) {
+    } else if (len > A.lng) {
       lrows[atomicAdd(&s_nlong, 1)] = li;
     }
   }
   __syncthreads();
-  auto keep = [&](int li, int first, int step) {  // a row's neighbours, eight loads in flight
-    if (!here(li)) return;
-    const int32_t *col = A.colidx + start[li];
-    const int e = rows[li + 1];
-    for (int t = rows[li] + first; t < e; t += 8 * step) {
-      int v[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = __ldg(col + min(t + q * step, e - 1));
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (t + q * step < e) cols[t + q * step] = (uint16_t)at(v[q]);
-    }
-  };
   for (int q = warp; q < s_nlong; q += T / 32) keep(lrows[q], lane, 32);  // long rows, a warp each
   for (int h = 0; h < nhub; ++h) keep(hub->node[h], tid, T);              // hubs, all threads
   for (int t = tid; t < A.perp * k; t += T) {
@@ -309,7 +316,7 @@ __global__ void __launch_bounds__(kScThreads, 1) k_sweep_cluster(ScArgs A) {
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         const int rb = rows[l0 + q], re = rows[l0 + q + 1];
-        if (re - rb <= kScLong) {
+        if (re - rb <= A.lng) {
           const bool in = re <= A.ecap;
           for (int t = rb + wb; t < re; t += W)
             sc_edge(Xc, in ? cols[t] : at(__ldg(A.colidx + start[l0 + q] + t)), q ? x1 : x0, sx[q], sy[q]);
@@ -444,7 +451,9 @@ int launch_sweep_cluster(int32_t n, int64_t m, const int32_t *rowptr, const int3
     const size_t fixed = sc_smem_bytes(C, A.per, k, dmax + 1, A.perp, A.warps, A.hubs);
     if (fixed > budget) continue;
     A.ecap = (int32_t)std::min<size_t>((budget - fixed) / 2, (size_t)(2 * m));
-    if (2 * m / C - A.ecap > kScMaxRead) continue;
+    const int64_t mean = 2 * m / n;
+    A.lng = mean > kScLaneMean ? kScLong : (int32_t)std::max<int64_t>(kScLong, 2 * mean);
+    if (mean > kScLaneMean && kScRowCost * A.per + 2 * m / C > kScMaxDense) continue;
     const size_t smem = fixed + (size_t)A.ecap * 2;
     A.n = n; A.k = k; A.dmax = dmax; A.iters = iters; A.rowptr = rowptr; A.colidx = colidx; A.pivots = pivots;
     A.cnt_off = cnt_off; A.cnt = cnt; A.dip = dip; A.pos = pos; A.tol = tol; A.iters_done = iters_done;

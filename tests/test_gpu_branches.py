@@ -415,3 +415,22 @@ def test_small_graph_hub_rows(n, hubs):
     b = ssm.ssm_batch_prepare([(n, s, d, k)] * 2)
     assert np.array_equal(b.pivots.cpu().numpy().reshape(2, k), np.stack([piv, piv]))
     assert np.array_equal(b.dip.cpu().numpy().reshape(2, k, n), np.stack([dip, dip]))
+
+
+@pytest.mark.parametrize("n,deg,cluster", [(1000, 16, True), (1000, 60, True), (1000, 70, True), (3000, 64, True), (8000, 110, False)])
+def test_sweep_fp32_cluster_mean_degrees(n, deg, cluster):
+    """The limit between rows of one lane per warp and of a warp follows the mean
+    degree up to 64; dense graphs of many rows take two kernels: one iteration
+    from the fourth against the oracle at the single step's bound."""
+    rng = np.random.default_rng(n + deg)
+    s = np.concatenate([np.arange(n - 1), rng.integers(0, n, n * deg // 2)]).astype(np.int32)
+    d = np.concatenate([np.arange(1, n), rng.integers(0, n, n * deg // 2)]).astype(np.int32)
+    prep = O.prepare(n, s, d, 12)
+    x0 = (rng.standard_normal((n, 2)) * np.sqrt(n)).astype(np.float32)
+    g, P = _gpu_graph(n, s, d), _gpu_pivots(12, prep)
+    four, five = torch.from_numpy(x0.copy()).to(DEV), torch.from_numpy(x0.copy()).to(DEV)
+    ssm.ssm_iterate(g, P, four, 4)
+    ssm.ssm_iterate(g, P, five, 5)
+    assert (ssm.ssm_last_sweep_config()["kernel"] == "f32_cluster") == cluster
+    want, _ = O.sweep_jacobi(prep.g, prep.pivots, prep.dip, prep.w, four.cpu().numpy().astype(np.float64))
+    assert _norm_err(five.cpu().numpy(), want) < 1e-5
