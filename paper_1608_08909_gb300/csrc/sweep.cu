@@ -666,7 +666,7 @@ __global__ void k_tile_dip(int32_t n, int32_t k, const uint16_t *__restrict__ di
 // full-table mode: the copy with e(d) the byte offset of the node's entry, and
 // den[i] = deg(i) + sum_{a = 0..k-1} w'_ia in FP32, pivots in order (the sum the
 // clamped mode forms inside every sweep): one pass over d_ip for both, a thread
-// per 2 W nodes with four or eight pivots' loads in flight, -w in shared memory.  HBM
+// per 2 W nodes with four or sixteen pivots' loads in flight, -w in shared memory.  HBM
 // bounds it with W = 4: ba1m, k = 200: 133 us for 838 MB = 6.3 TB/s (copy and sum apart: 165 + 81)
 // W = 1 below this many nodes, where the chain over the pivots is the bound and
 // threads are few: n = 20,000: 19 against 37 us, 100,000: 30 against 54, 2^20:
@@ -679,7 +679,14 @@ __global__ void __launch_bounds__(256) k_tile_den(int32_t n, int32_t k, int32_t 
                                                   const int32_t *__restrict__ rowptr, float *__restrict__ den) {
   extern __shared__ __align__(16) unsigned char td_smem[];
   float *mw = reinterpret_cast<float *>(td_smem);  // [k][row]
-  for (int t = threadIdx.x; t < k * row; t += blockDim.x) mw[t] = __ldg(wtab + t);
+  for (int t0 = threadIdx.x; t0 < k * row; t0 += 8 * (int)blockDim.x) {  // eight loads in flight
+    float w[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) w[q] = __ldg(wtab + min(t0 + q * (int)blockDim.x, k * row - 1));
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (t0 + q * (int)blockDim.x < k * row) mw[t0 + q * (int)blockDim.x] = w[q];
+  }
   __syncthreads();
   const int64_t parts = ((int64_t)(n + kTileNodes - 1) / kTileNodes) * (kTileNodes / (2 * W));
   const unsigned top = (unsigned)row - 1u;
@@ -702,7 +709,7 @@ __global__ void __launch_bounds__(256) k_tile_den(int32_t n, int32_t k, int32_t 
       }
       tile_store<W>(dtile, k, a, g, out);
     };
-    constexpr int kAhead = W == 4 ? 4 : 8;
+    constexpr int kAhead = W == 4 ? 4 : 16;
     const DipTable table{dip};
     const int left = part_left<W>(n, g);
     size_t first = (size_t)(2 * W * g);
