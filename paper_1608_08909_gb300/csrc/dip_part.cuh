@@ -39,6 +39,11 @@ SSM_HD DipPart<W> dip_part(const T &dip, size_t first, int left, int32_t loads) 
 #endif
       for (int t = 0; t < W; ++t) v.w[t] = 0u;
     }
+  } else if (loads == kDipWords && left == 2 * W && (first & 1u) == 0) {  // whole words
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int t = 0; t < W; ++t) v.w[t] = dip.word((first >> 1) + t);
   } else if (loads == kDipWords) {
     const int odd = (int)(first & 1u);
     unsigned w[W + 1];
