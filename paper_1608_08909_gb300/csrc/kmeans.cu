@@ -634,7 +634,11 @@ __global__ void __launch_bounds__(kKmThreads) k_km_assign(int32_t n, int32_t k, 
   __shared__ int ba[16][kKmNodes];                             // and its cluster
   __shared__ double s_best[kKmNodes];
   __shared__ int s_arg[kKmNodes];
-  if (__ldcg(W.stop) || (W.filt->on && !km_mostly_wide(W, n, pass))) return;
+  {
+    const bool wide = km_mostly_wide(W, n, pass);  // the three loads together
+    const int stop = __ldcg(W.stop), on = W.filt->on;
+    if (stop || (on && !wide)) return;
+  }
   const int tid = threadIdx.x;
   const int tn = tid & 15, ta = tid >> 4;  // node group (4 nodes), cluster group (4 clusters)
   for (int n0 = blockIdx.x * kKmNodes; n0 < n; n0 += gridDim.x * kKmNodes) {
@@ -745,11 +749,10 @@ __global__ void __launch_bounds__(256, 3) k_km_resolve(int32_t n, int32_t k, int
                                                     int32_t *__restrict__ assign) {
   __shared__ double s_best[8];
   __shared__ int s_at[8];
-  if (__ldcg(W.stop)) return;
   const KmFilter F = *W.filt;
-  if (!F.on || km_mostly_wide(W, n, pass)) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned nopen = __ldcg(W.open + (pass & 1)), nwide = __ldcg(W.wide + (pass & 1));
+  if (__ldcg(W.stop) || !F.on || km_mostly_wide(W, n, pass)) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int kRegs = (kKtMaxK + 31) / 32;
   unsigned y[kRegs];
   auto load = [&](int i) {
