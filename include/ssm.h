@@ -305,7 +305,12 @@ int ssm_gram(int32_t n, int32_t k, const uint16_t *dip, uint64_t *g_lo, uint64_t
  * synchronous anyway, or from ssm_iterate_hints (synchronous); with hints
  * the call is asynchronous, with hints == NULL it computes them and waits
  * once for `stream`.  Wrong hints give SSM_E_ARG where they are out of
- * range and wrong results otherwise. 
+ * range and wrong results otherwise.
+ * Up to 8192 nodes, four or more FP32 iterations run in one thread-block
+ * cluster, fewer in two kernels per iteration, which add up a node's terms in
+ * another order: the same run cut into calls of other lengths may differ in
+ * the last bits (calls of four or more on one side, calls of one to three on
+ * the other, can be cut at will).  ssm_last_sweep_config tells which ran.
  * ------------------------------------------------------------------- */
 size_t ssm_iterate_workspace(int32_t n, int64_t m, int32_t k, int64_t cnt_len, int32_t precision);
 int ssm_iterate(int32_t n, int64_t m, const int32_t *rowptr, const int32_t *colidx, int32_t k,
@@ -392,7 +397,7 @@ typedef struct {
 } ssm_batch_graph;
 size_t ssm_batch_iterate_workspace(int32_t G, const ssm_batch_graph *graphs);
 /* Batched preparation of the graphs above (Algorithm 1 lines 1-4 for G
- * small graphs in three launches): from edge lists to
+ * small graphs in four launches): from edge lists to
  * the packed arrays ssm_batch_iterate reads.  Graph g has n nodes (1..12288),
  * k max/min-sp pivots (2 <= k <= min(n, 100); start node 0), and m_in edges
  * src/dst[edge_off .. edge_off + m_in) with local ids.
